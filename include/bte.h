@@ -53,6 +53,14 @@ typedef enum {
                           refinement residuals, FP64 x step and moments */
 } bte_precision;
 
+/* How the velocity systems are factored. By default, with at most 32 harmonics, refinement on
+ * (refine_max != 0) and a window of at most 512 columns (nr <= 320 with more than 16 harmonics, up to
+ * 544 with fewer), through a windowed LU with partial pivoting: the system in the harmonic basis with
+ * the speed index slowest, which is a band matrix but for the l = 0 columns that inelastic gain
+ * reaches (Section 3.3; csrc/bte_window.cu). Otherwise, and with any of the flags below that select a
+ * variant of it, through a dense LU per point. Both eliminate with partial pivoting and are refined
+ * against the same system. */
+
 /* flags for bte_config.flags */
 #define BTE_FLAG_HOST_ONLY 1u   /* assemble the operators on the host only: no CUDA call is made;
                                    bte_get_operator works, device entry points return BTE_ESTATE */
@@ -71,10 +79,10 @@ typedef enum {
 #define BTE_FLAG_FULL_V 16u     /* with nl < ntheta, factor the full Nv x Nv matrix A_i per point. By
                                    default such a handle factors the reduced matrix I - dt B_i of order
                                    nl * nr (B = C + E A_v in the harmonic basis, Section 3.3; both
-                                   multiplied by I (x) M_v, see bte_step) and solves
-                                   through A^-1 f = f + P_O((I - dt B)^-1 - I) P_S f: the same solution,
+                                   multiplied by I (x) M_v, see bte_step; windowed or dense, as
+                                   above) and solves through A^-1 f = f + P_O((I - dt B)^-1 - I) P_S f: the same solution,
                                    (nv / (nl nr))^3 fewer factorisation flops and (nv / (nl nr))^2 less
-                                   factor memory. bte_step_adjoint needs the full factors. */
+                                   factor memory. bte_step_adjoint needs nl = ntheta or this flag. */
 #define BTE_FLAG_TC_ONE_CTA 64u  /* BTE_MIXED on the tensor cores, panels in pairs: run the K = 256 update
                                    on 128 x 128 tiles of single CTAs instead of 256 x 256 tiles of CTA
                                    pairs (same products, twice the operand bytes staged per flop) */
@@ -86,7 +94,8 @@ typedef enum {
                                    launch first waits (about 1 ms, before it issues any copy or MMA)
                                    on a barrier that nothing signals, so the bounded wait expires,
                                    the launch does no work and the step returns BTE_ECUDA with F
-                                   unchanged. Never set it for real work. */
+                                   unchanged. Selects the dense LU, whose kernels it tests. Never set it for
+                                   real work. */
 
 typedef struct {
   int nx;            /* Chebyshev-Gauss-Lobatto points, >= 3 */
@@ -154,8 +163,8 @@ typedef struct {
   unsigned last_flags;    /* device status bits of the last step (1 zero pivot, 2 non-finite result,
                              4 not converged, 8 expired device wait, 16 non-finite input) */
   unsigned long long launches; /* kernels launched by this handle so far */
-  int tensor_cores;       /* 1 if the trailing updates run on tcgen05 (TF32x3) */
-  int solve_n;            /* order of the per-point factorisation: nv, or nl * nr for the reduced
+  int tensor_cores;       /* 1 if the trailing (or window) updates run on tcgen05 (TF32x3) */
+  int solve_n;            /* order of the per-point systems factored: nv, or nl * nr for the reduced
                              system (nl < ntheta without BTE_FLAG_FULL_V); 0 with BTE_FLAG_STRUCTURED */
   double last_refine_evals; /* refinement residuals evaluated per point and step of the last bte_step /
                              bte_run, averaged over points and steps (not rounded); each evaluation
@@ -190,8 +199,9 @@ bte_status bte_init_maxwellian(bte_handle* h, double* F_dev, const double* ne_de
 /* One semi-implicit step t -> t + dt of F_dev (device, in/out), eqs. "bte_semi_implicit".
  * The field of the velocity step is E_dev[nx] (device, V/m) if non-NULL, else the uniform
  * E = (V0/L) sin(2 pi freq (t + dt/2)). The velocity step solves A_i x = b at every point
- * (eq. "vspace_batched_system"); the dense paths factor (I (x) M_v) A_i = I (x) M_v -
- * dt (P_O C P_S + E_i P_O A_v P_S), the same system before the mass scaling of Section 3.4 (LU with
+ * (eq. "vspace_batched_system"); the LU paths factor (I (x) M_v) A_i = I (x) M_v -
+ * dt (P_O C P_S + E_i P_O A_v P_S), or the same in the harmonic basis: the system before the mass
+ * scaling of Section 3.4 (LU with
  * partial pivoting on the scaled A_i meets element growth of order 1e15 on speed grids of a few
  * hundred B-splines), and refine against A_i itself in FP64 (Algorithm 2).
  * On BTE_ESINGULAR/ENOCONV/ENONFINITE F is left unchanged.
@@ -270,7 +280,7 @@ bte_status bte_init_maxwellian_static(const bte_handle* h, double* F_dev, const 
  * mu_i = A_i^-T (X^T lambda)_i the adjoint after the velocity step and F*_i = A_i^-1 (X F^n)_i the
  * state after it (both at point i, nv entries). The transposed x step uses U^T, the transposed
  * Q_ij blocks and U^-T (copied to the device on the first call); A_i^T is solved with the same LU
- * factors (recomputed from F^n). Synchronises the handle's stream. */
+ * factors (recomputed for the step's field). Synchronises the handle's stream. */
 bte_status bte_step_adjoint(bte_handle* h, const double* F_dev, double* lambda_dev, double t_s, double V0,
                             double freq_Hz, const double* g_dev, double g_weight, double* SC_dev,
                             double* SA_dev);
@@ -360,7 +370,8 @@ bte_status bte_step_implicit(bte_handle* h, double* F_dev, const double* ni_dev,
 typedef struct bte_batch bte_batch;
 
 /* flags for bte_batch_create */
-#define BTE_BATCH_AUTOTUNE 1u  /* per distinct instance shape (nx, nr, ntheta, nl, precision), time
+#define BTE_BATCH_AUTOTUNE 1u  /* for instances on the dense LU (the windowed one has no variants):
+                                  per distinct instance shape (nx, nr, ntheta, nl, precision), time
                                   one short run of every algorithm variant (tensor-core or CUDA-core
                                   trailing update; on the tensor cores panels in pairs on CTA-pair or
                                   single-CTA tiles, or one panel at a time; panel column-block

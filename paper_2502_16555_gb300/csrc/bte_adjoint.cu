@@ -5,7 +5,8 @@
 // S_n^T = X^T V_n^T X^T: X^T applies U^T, the transposed Q_ij blocks and U^-T in place of U^-1, Q_ij
 // and U; V_n^T solves with A_i^T through the same LU factors. The factors are those of
 // (I (x) M_v) A_i, so A_i^-1 g = LU^-1 (I (x) M_v) g and A_i^-T g = (I (x) M_v) LU^-T g (M_v is
-// symmetric). A parameter theta enters only through
+// symmetric); with the windowed LU the factors are those of the harmonic system and the transposed
+// passes run in reverse (window_solve_t_kernel). A parameter theta enters only through
 // A_i, and d(A^-1 G)/dtheta = -A^-1 (dA/dtheta) F*, so a step contributes
 //     dJ/dtheta += mu^T (dt dK/dtheta) F*,   mu = A^-T X^T lambda^{n+1},  F* = A^-1 X F^n,
 // per point; the library accumulates SC = sum mu F*^T (and SA with the weight dE/dV0) and contracts
@@ -131,9 +132,16 @@ bte_status bte_step_adjoint(bte_handle* h, const double* F_dev, double* lambda_d
   bte::launch_x_apply_q(h->Q, h->Y, h->Y2, nx, nt, nr, st);
   bte::launch_x_from_eigen(h->Y2, h->U, h->Fa, nx, nt, nr, nullptr, st);
   const bte::MassBand mass{h->Mband, nr, o.mw};
-  bte::launch_v_form<double>(h->KCg, h->KAg, mass, nullptr, Eu, o.dt, fac, nx, nv, st);
-  nl += 4;
-  for (int k0 = 0; k0 < n; k0 += nb) {
+  nl += 3;
+  if (h->windowed) {
+    // counted by the handle; refined, so that F* is as accurate as the dense solve's
+    if ((s = bte::handle_window_factor(h, Eu)) != BTE_OK) return s;
+    if ((s = bte::handle_window_solve(h, h->Fa, h->Fb, Eu)) != BTE_OK) return s;
+  } else {
+    bte::launch_v_form<double>(h->KCg, h->KAg, mass, nullptr, Eu, o.dt, fac, nx, nv, st);
+    ++nl;
+  }
+  for (int k0 = 0; k0 < n && !h->windowed; k0 += nb) {
     const int kb = std::min(nb, n - k0);
     bte::launch_lu_panel<double>(fac, h->piv, h->perm, static_cast<double*>(h->linv), nullptr, nx, n, k0, kb, nb,
                                  h->status, nullptr, nullptr, nullptr, nullptr, h->panel_w, st);
@@ -145,13 +153,19 @@ bte_status bte_step_adjoint(bte_handle* h, const double* F_dev, double* lambda_d
       nl += 2;
     }
   }
-  bte::launch_lu_solve<double>(fac, h->piv, h->Fa, h->Fb, nx, n, nb, nullptr, 0, st, mass);
+  if (!h->windowed) {
+    bte::launch_lu_solve<double>(fac, h->piv, h->Fa, h->Fb, nx, n, nb, nullptr, 0, st, mass);
+    ++nl;
+  }
   // nu = X^T lambda (R), mu = A^-T nu (Fw), sensitivities, lambda <- X^T mu + w g
   bte::launch_x_to_eigen(lambda_dev, h->Ut, h->Y, nx, nt, nr, h->status, st);
   bte::launch_x_apply_q(h->Qt, h->Y, h->Y2, nx, nt, nr, st);
   bte::launch_x_from_eigen(h->Y2, h->Uinvt, h->R, nx, nt, nr, nullptr, st);
-  bte::launch_lu_solve_t(fac, h->piv, h->R, h->Fw, nx, n, nb, st, mass);
-  nl += 5;
+  if (h->windowed)
+    BA_CUDA(h, bte::launch_window_solve_t(h->win, h->R, h->Fw, mass, h->TO, h->TS, nx, nt, st));
+  else
+    bte::launch_lu_solve_t(fac, h->piv, h->R, h->Fw, nx, n, nb, st, mass);
+  nl += 4;
   if (SC_dev || SA_dev) {
     dim3 grid((nv + 31) / 32, (nv + 31) / 32);
     sens_accumulate_kernel<<<grid, 256, 0, st>>>(h->Fw, h->Fb, nx, nv, SC_dev, SA_dev, std::sin(arg) / o.L);

@@ -154,6 +154,7 @@ bte_status autotune(bte_batch* b) {
   std::map<Key, bte::Variant> best;
   for (size_t i = 0; i < b->hs.size(); ++i) {
     bte_handle* h = b->hs[i];
+    if (bte::handle_windowed(h)) continue;  // one algorithm: keeps its variant
     const bte::HostOps& o = *bte::handle_ops(h);
     bte_info info;
     bte_get_info(h, &info);

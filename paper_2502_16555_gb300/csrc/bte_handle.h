@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "bte_internal.h"
+#include "bte_kernels.h"
 
 struct bte_handle {
   bte_config cfg{};
@@ -26,6 +27,9 @@ struct bte_handle {
   bool reduced = false;     // dense LU of I - dt B_i (order nl * nr) instead of A_i (order nv)
   int nlu = 0;              // order of the per-point factorisation (nv, or nl * nr when reduced)
   double *yred = nullptr, *zred = nullptr;  // P_S f and the reduced solution (nx * nlu each)
+  bool windowed = false;    // windowed LU of the harmonic system (bte_window.cu): no dense factors
+  bte::WindowBuffers win;
+  double ts_inf = 0.0, to_inf = 0.0;  // infinity norms of T_S and T_O
   bool use_tc = false;    // tcgen05 trailing update (FP32 storage only)
   bool have_tc = false;   // the tensor-core workspace exists (use_tc may be switched on)
   int panel_w = 0;        // preferred column-block width of the panel kernel (0: by shape)

@@ -99,6 +99,10 @@ bte_status handle_enqueue_sc_step(bte_handle* h, double* F_dev, const double* ni
 // the field E_dev (factor: form and factor first; else reuse the last factors, no refinement).
 bte_status handle_enqueue_xhalf(bte_handle* h, const double* in, double* out);
 bte_status handle_enqueue_vsolve(bte_handle* h, const double* in, double* out, const double* E_dev, bool factor);
+// The windowed LU's pieces for the adjoint: the factors with the uniform field Eu, and the refined
+// solves of in into out through them.
+bte_status handle_window_factor(bte_handle* h, double Eu);
+bte_status handle_window_solve(bte_handle* h, const double* in, double* out, double Eu);
 // The field of eq. "hybrid_discrete_c" (bte_hybrid.cu): E = L (ni - u^T F) + V0 sin(2 pi f t) E_1
 // into E_dev on the handle's stream (ni_dev NULL: no ions; V0 = 0: no electrode voltage).
 bte_status enqueue_field(bte_handle* h, const double* F_dev, const double* ni_dev, double t, double V0,
@@ -117,6 +121,7 @@ struct Variant {
   int cg = 2;
 };
 bool handle_has_tc(const bte_handle* h);
+bool handle_windowed(const bte_handle* h);  // the windowed LU: none of these variants applies
 void handle_set_variant(bte_handle* h, const Variant& v);
 Variant handle_get_variant(const bte_handle* h);
 

@@ -175,6 +175,63 @@ void launch_residual(const double* x, const double* b, const double* E, double E
                      cudaStream_t st);
 void launch_check_conv(const int* conv, int nx, unsigned* status, cudaStream_t st);
 
+// ---- the windowed LU of the harmonic system with the speed index slowest (bte_window.cu)
+// Shapes of the window for nl harmonics and nr B-splines; ok = false where it does not apply (nl > 32,
+// or a window wider than the 512 columns of tensor memory).
+struct WindowPlan {
+  int nr = 0, nl = 0;
+  int nlp = 0, g = 0;   // power of two >= nl; speed indices per 32-column chunk
+  int np = 0;           // chunks (panels)
+  int RC = 0, RS = 0;   // chunks that enter ahead of the panel; ring chunks right of it
+  int NS = 0;           // row slots in use, 32 (1 + RC)
+  int kf0 = 0, NF = 0;  // first speed index kept as a far column; far columns (a multiple of 32)
+  int NU = 0, NW = 0;   // window columns RS 32 + NF; row template length (RS + 1) 32 + NF
+  int tmem_cols = 0;
+  bool ok = false;
+};
+struct WindowBuffers {
+  WindowPlan w;
+  bool fp64 = false;
+  void *base = nullptr, *slope = nullptr;  // row templates: values without and per unit of the field
+  void *T = nullptr, *U = nullptr;         // factors, window_t_count / window_u_count values a point
+  signed char* slotj = nullptr;            // window_slot_count a point
+  double* W = nullptr;                     // FP64: 128 (NU + 32) values a point
+  int* rows = nullptr;                     // FP64: 128 values a point
+  double* vec = nullptr;                   // 3 nl nr values a point
+  double* fmax_ = nullptr;                 // one value a point
+};
+WindowPlan window_plan(int nr, int nl);
+// Templates [np 32][NW] and [np 32][(RS + 1) 32] from the unscaled blocks (M, Cg, Ag_lo, Ag_up).
+void window_tables(const WindowPlan& w, const HostOps& o, std::vector<double>& base, std::vector<double>& slope);
+size_t window_t_count(const WindowPlan& w);
+size_t window_u_count(const WindowPlan& w);
+size_t window_slot_count(const WindowPlan& w);
+// FP32 buffers: forms and factors H_i at every point with the field E[i] (Eu when E is NULL).
+cudaError_t launch_window_factor(const WindowBuffers& b, const double* E, double Eu, int nx, unsigned* status,
+                                 cudaStream_t st);
+// FP64 buffers: the same as a sequence of launches, init, then panel s and update s for s = 0 .. np - 1.
+cudaError_t launch_window_init_f64(const WindowBuffers& b, const double* E, double Eu, int nx, unsigned* status,
+                                   cudaStream_t st);
+cudaError_t launch_window_panel_f64(const WindowBuffers& b, int s, int nx, unsigned* status, cudaStream_t st);
+cudaError_t launch_window_update_f64(const WindowBuffers& b, const double* E, double Eu, int s, int nx, unsigned* status,
+                                     cudaStream_t st);
+// The solves out_i = A_i^-1 in_i through the last factors, in the harmonic basis with the vectors y, z,
+// rho of the buffers: project in, then substitute (z += H^-1 rho; points with conv[i] != 0 skipped, conv
+// NULL: none) and residual in turn. residual with check: rho, the test of launch_residual (ratio,
+// conv and the count in status[1] as it writes them; always made when last) and out where the test was
+// made; without check: out alone. ts_inf, to_inf: infinity norms of T_S and T_O. The buffers' U must
+// have been zeroed once.
+cudaError_t launch_window_project(const WindowBuffers& b, const double* in, MassBand mass, const double* TS, int* conv,
+                                  int nx, int nt, cudaStream_t st);
+cudaError_t launch_window_substitute(const WindowBuffers& b, const int* conv, int nx, unsigned* status, cudaStream_t st);
+cudaError_t launch_window_residual(const WindowBuffers& b, const double* in, double* out, const double* E, double Eu,
+                                   double dt, const ResidualOps& ro, MassBand mass, const double* TO, double ts_inf,
+                                   double to_inf, double* ratio, int* conv, double tol, double kc_inf, double ka_inf,
+                                   int nx, int nt, bool check, bool last, unsigned* status, cudaStream_t st);
+// out_i = A_i^-T in_i through the last factors (FP64 buffers only).
+cudaError_t launch_window_solve_t(const WindowBuffers& b, const double* in, double* out, MassBand mass,
+                                  const double* TO, const double* TS, int nx, int nt, cudaStream_t st);
+
 // ---- misc
 void launch_commit(const double* src, double* dst, size_t n, const unsigned* status, cudaStream_t st);
 void launch_moments(const double* F, const double* mom_n, const double* mom_e, const double* mom_r,

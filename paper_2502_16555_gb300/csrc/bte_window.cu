@@ -1,0 +1,1535 @@
+// The per-point velocity solves of eq. "vspace_batched_system" (arXiv 2502.16555) through a windowed
+// LU with partial pivoting, one CTA per collocation point from formation to the last factor.
+//
+// The system. With P_S P_O = T_S T_O = I, A_i^-1 f = f + P_O (G_i^-1 - I) P_S f, G_i = I - dt B_i in the
+// harmonic basis (Section 3.3), and H_i = (I (x) M_v) G_i = I (x) M_v - dt (C + E_i A_v) has the same
+// solutions. Its blocks are banded in the speed index (cubic B-splines couple |p - k| <= 3) and couple
+// only l and l +- 1; the one exception is the gain of the inelastic processes, which reaches from row
+// (p, l = 0) to columns (k, l = 0) far above p. Taken with the speed index slowest, H_i is a band
+// matrix of half width 3 nl + 1 plus, for the l = 0 columns, entries far to the right: order
+// n = nl nr, but 2 n (4 nl) (6 nl + nr) operations instead of 2 n^3 / 3 (medium grid 0.27 against
+// 5.7 Gflop a point), with partial pivoting over every row that has an entry in the column, exactly as
+// in a dense LU of the same matrix.
+//
+// The window. Columns are taken 32 at a time ("chunks": g = 32 / nlp speed indices, nlp the power of
+// two >= nl, unused columns skipped). While chunk s is eliminated, the rows that can have an entry in
+// it are those of chunks <= s + RC (RC = ceil(3 / g) <= 3): at most 128 live rows, held in 128 fixed
+// slots; the 32 rows chosen as pivots leave their slots to the 32 rows of the chunk that enters, so
+// no row is ever moved. Their columns are those of the next RS = 2 RC chunks (a ring of RS x 32) and
+// the far l = 0 columns, one per speed index; when a chunk enters the ring, its l = 0 columns take over
+// what the far columns held.
+//
+// In a panel every eliminated row keeps, in the place of the eliminated column, the running product
+// of the elimination (the in-place form of Gauss elimination that carries its own inverse): after
+// 32 columns a pivot row holds its row of inv(L11) left of the diagonal and of U11 from it on, and
+// any other row holds t = -L21 inv(L11). The whole window is then updated by one product,
+// D += T B with B the pivot rows (T's pivot rows: inv(L11) - I), and the forward substitution is
+// one matrix-vector product with T per panel.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cmath>
+#include <cstdint>
+#include <string>
+#include <vector>
+
+#include "bte_handle.h"
+#include "bte_kernels.h"
+#include "bte_tf32.cuh"
+
+namespace bte {
+namespace {
+
+constexpr int kPW = 32;      // panel (chunk) width
+constexpr int kSlots = 128;  // row slots: the tensor cores' M
+constexpr int kThreads = 256;
+constexpr long long kWaitCycles = 1ll << 32;  // bounded device waits, about 2 s
+constexpr double kBackwardFloor = 256.0 * 1.1102230246251565e-16;  // as in launch_residual
+
+__host__ __device__ inline int imin(int a, int b) { return a < b ? a : b; }
+__host__ __device__ inline int imax(int a, int b) { return a > b ? a : b; }
+
+// columns of chunk s that are unknowns of the system
+__device__ __forceinline__ unsigned chunk_mask(const WindowPlan& w, int s) {
+  unsigned m = 0;
+  for (int i = 0; i < w.g; ++i)
+    if (s * w.g + i < w.nr) m |= ((w.nl < 32 ? (1u << w.nl) : 0u) - 1u) << (i * w.nlp);
+  return m;
+}
+
+__device__ __forceinline__ uint32_t saddr(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
+
+__device__ __forceinline__ void mbar_init(uint64_t* b, uint32_t count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(saddr(b)), "r"(count));
+}
+
+__device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+      : "=r"(ok)
+      : "r"(saddr(b)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+
+// Bounded: on expiry the status bit is set, later waits of the CTA return at once and the kernel runs
+// to its end on whatever the buffers hold (every access stays in bounds); the step reports it.
+__device__ __forceinline__ void mbar_wait(uint64_t* b, uint32_t parity, volatile int* gave_up, unsigned* status) {
+  if (mbar_try(b, parity)) return;
+  const long long t0 = clock64();
+  while (!mbar_try(b, parity)) {
+    if (*gave_up) return;
+    if (clock64() - t0 > kWaitCycles) {
+      *gave_up = 1;
+      atomicOr(status, kTimeout);
+      return;
+    }
+  }
+}
+
+__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+
+// shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups 1024 B apart
+__device__ __forceinline__ uint64_t sdesc(uint32_t addr) {
+  uint64_t d = 0;
+  d |= static_cast<uint64_t>((addr & 0x3FFFFu) >> 4);
+  d |= static_cast<uint64_t>(1) << 16;
+  d |= static_cast<uint64_t>(1024 >> 4) << 32;
+  d |= static_cast<uint64_t>(1) << 46;
+  d |= static_cast<uint64_t>(2) << 61;
+  return d;
+}
+
+__device__ __forceinline__ void mma_tf32(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, 1, 0;\n"
+      " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}"
+      ::"r"(tmem_d), "l"(a), "l"(b), "r"(idesc));
+}
+
+__device__ __forceinline__ void mma_commit(uint64_t* bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(saddr(bar))
+               : "memory");
+}
+
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
+  uint32_t r[32];
+  __syncwarp();
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
+        "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]),
+        "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),
+        "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const float (&v)[32]) {
+  uint32_t r[32];
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(v[i]);
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,"
+      "%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};"
+      ::"r"(taddr),
+      "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+      "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]),
+      "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]),
+      "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
+      : "memory");
+}
+
+__device__ __forceinline__ float tmem_ld1(uint32_t taddr) {
+  uint32_t r;
+  __syncwarp();
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+  return __uint_as_float(r);
+}
+
+__device__ __forceinline__ void tmem_st1(uint32_t taddr, float v) {
+  __syncwarp();
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x1.b32 [%0], {%1};" ::"r"(taddr), "r"(__float_as_uint(v)) : "memory");
+}
+
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+// 32 consecutive template values of a row: base + E slope (slope NULL: base)
+__device__ __forceinline__ void row_values(const float* __restrict__ base, const float* __restrict__ slope, float E,
+                                           float (&v)[32]) {
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const float4 b = __ldg(reinterpret_cast<const float4*>(base) + q);
+    v[4 * q] = b.x, v[4 * q + 1] = b.y, v[4 * q + 2] = b.z, v[4 * q + 3] = b.w;
+  }
+  if (slope) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const float4 s = __ldg(reinterpret_cast<const float4*>(slope) + q);
+      v[4 * q] = fmaf(E, s.x, v[4 * q]), v[4 * q + 1] = fmaf(E, s.y, v[4 * q + 1]);
+      v[4 * q + 2] = fmaf(E, s.z, v[4 * q + 2]), v[4 * q + 3] = fmaf(E, s.w, v[4 * q + 3]);
+    }
+  }
+}
+
+__device__ __forceinline__ void store32(float* dst, const float (&v)[32]) {
+#pragma unroll
+  for (int q = 0; q < 8; ++q)
+    reinterpret_cast<float4*>(dst)[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+}
+
+// 1 / p to FP32 rounding: the hardware's approximation and one Newton-Raphson step (the IEEE division
+// is a call with special cases, about 250 cycles in the panel's chain)
+__device__ __forceinline__ float recip(float p) {
+  float r;
+  asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(p));
+  return fmaf(r, fmaf(-p, r, 1.f), r);
+}
+
+// The same in FP64, with two steps (the approximation has about 20 bits).
+__device__ __forceinline__ double recip(double p) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(p));
+  r = fma(r, fma(-p, r, 1.0), r);
+  return fma(r, fma(-p, r, 1.0), r);
+}
+
+struct FactorArgs {
+  WindowPlan w;
+  const void* base;    // [np 32][NW] row templates (T)
+  const void* slope;   // [np 32][(RS + 1) 32]
+  const double* E;
+  double Eu;
+  void* T;             // [nx][np][32][NS]
+  void* U;             // [nx][np][1024 + 32 NU]: inv(U11), then the pivot rows over the window
+  signed char* slotj;  // [nx][np][NS]: the pivot index of each slot, -1 if its row stays
+  double* W;           // FP64: the window [nx][128][NU + 32]
+  int* rows;           // FP64: the padded row in each slot [nx][128]
+  unsigned* status;
+};
+
+// Mixed path. The window D (128 slots x NU columns) lives in tensor memory in FP32; T and B are split
+// into TF32 heads and remainders in shared memory (the split and the three products of the dense
+// path's trailing updates) and D += T B runs as tcgen05.mma with M = 128, K = 32.
+// Warps 0-3 (one thread a slot) hold the panel's 32 columns in registers and eliminate them: per
+// column one warp-wide argmax, each warp's candidate row posted to shared memory, one barrier of
+// the panel's warps. Warps 4-7 meanwhile finish the panel before: the pivot rows' updated window is
+// written out as U, the rows of the entering chunk take the freed slots. The next panel waits only for
+// the update of its own 32 columns, which is issued first.
+// Bound by the latency of the 32 dependent columns of a panel (13.5 us a panel, 9.5 of them in the
+// columns), not by the tensor cores (5000 cycles a panel, hidden) or memory. Medium grid (128 points,
+// order 2048): 0.88 ms for formation and factors, where the dense LU took 10.9 ms.
+__global__ void __launch_bounds__(kThreads, 2) window_lu_tc_kernel(const FactorArgs a) {
+  extern __shared__ __align__(1024) unsigned char raw[];
+  const WindowPlan& w = a.w;
+  unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
+  float* Thi = reinterpret_cast<float*>(sm);
+  float* Tlo = Thi + kSlots * kPW;
+  float* Bhi = Tlo + kSlots * kPW;
+  float* Blo = Bhi + w.NU * kPW;
+  __shared__ __align__(16) float prow[2][4][8];    // each warp's candidate row in the current sub-block
+  __shared__ __align__(16) uint2 keys[2][4];       // its magnitude and lane, and 1 / its pivot
+  __shared__ __align__(16) float pblk[2][8][24];   // a sub-block's pivot rows over the other columns
+  __shared__ signed char slotj[2][kSlots];
+  __shared__ float u11[2][64 * 33];  // rows 0 .. 31 stay zero: the back substitution reads above the block
+  __shared__ __align__(8) uint64_t bar_next, bar_rest;
+  __shared__ uint32_t tmem_base;
+  __shared__ int gave_up;
+
+  const int pt = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, quad = warp & 3;
+  const int slot = quad * 32 + lane, np = w.np, NW = w.NW, NS = w.NS, RS = w.RS, RC = w.RC, g = w.g;
+  const int NWR = (RS + 1) * 32;
+  const bool panel_warp = warp < 4;
+  const int npw = NS / 32;  // panel warps that hold rows
+  const float* base = static_cast<const float*>(a.base);
+  const float* slope = static_cast<const float*>(a.slope);
+  const float E = static_cast<float>(a.E ? a.E[pt] : a.Eu);
+  float* Tg = static_cast<float*>(a.T) + static_cast<size_t>(pt) * np * 32 * NS;
+  const size_t ustride = 1024 + 32 * static_cast<size_t>(w.NU);
+  float* Ug = static_cast<float*>(a.U) + static_cast<size_t>(pt) * np * ustride;
+  signed char* sjg = a.slotj + static_cast<size_t>(pt) * np * NS;
+
+  if (tid == 0) {
+    mbar_init(&bar_next, 1);
+    mbar_init(&bar_rest, 1);
+    gave_up = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(saddr(&tmem_base)),
+                 "r"(static_cast<uint32_t>(w.tmem_cols)));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  // K columns of unused unknowns stay zero in B for the whole factorisation
+  for (int i = tid; i < w.NU * kPW; i += kThreads) Bhi[i] = Blo[i] = 0.f;
+  for (int i = tid; i < 2 * 64 * 33; i += kThreads) (&u11[0][0])[i] = 0.f;
+  for (int i = tid; i < 2 * 8 * 24; i += kThreads) (&pblk[0][0][0])[i] = 0.f;
+  if (tid < 8) (&keys[0][0])[tid] = make_uint2(0u, 0u);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_base + (static_cast<uint32_t>(quad * 32) << 16);  // this warp's lanes
+  const int nfar = imax(0, w.nr - w.kf0);
+
+  float v[32];
+#pragma unroll
+  for (int i = 0; i < 32; ++i) v[i] = 0.f;
+  // rows of chunks 0 .. RC enter at panel 0, slot by slot
+  const bool valid0 = slot < NS && slot / 32 < np && ((chunk_mask(w, slot / 32) >> lane) & 1u);
+  bool act = panel_warp && valid0;
+  if (panel_warp) {
+    if (act) row_values(base + static_cast<size_t>(slot) * NW, slope + static_cast<size_t>(slot) * NWR, E, v);
+  } else {
+    for (int d = 1; d <= RS; ++d) {
+      float r[32];
+      if (valid0) row_values(base + static_cast<size_t>(slot) * NW + d * 32, slope + static_cast<size_t>(slot) * NWR + d * 32, E, r);
+      else
+#pragma unroll
+        for (int i = 0; i < 32; ++i) r[i] = 0.f;
+      tmem_st32(tmem + (d % RS) * 32, r);
+    }
+    for (int c = 0; c < w.NF / 32; ++c) {
+      float r[32];
+      if (valid0) row_values(base + static_cast<size_t>(slot) * NW + NWR + c * 32, nullptr, 0.f, r);
+      else
+#pragma unroll
+        for (int i = 0; i < 32; ++i) r[i] = 0.f;
+      tmem_st32(tmem + (RS + c) * 32, r);
+    }
+    tmem_wait_st();
+    tc_fence_before();
+  }
+  bool bad = false;
+
+  for (int s = 0; s < np; ++s) {
+    const int par = s & 1;
+    const int dmax = imin(RS, np - 1 - s);                       // ring chunks right of the panel
+    const int fc0 = (s * g) / 32, nfc = s * g < nfar ? w.NF / 32 : fc0;  // far chunks [fc0, nfc)
+    int pj = -1;
+    if (panel_warp) {
+      // ---- the panel: 32 columns in registers, one thread a row
+      if (warp < npw) {
+        const unsigned mask = chunk_mask(w, s);
+        bool cand = act;
+        int b = 0;  // posting buffer: alternates from one eliminated column to the next
+        // Four sub-blocks of 8 columns. Inside one, only its 8 columns follow every pivot; the other 24
+        // (T entries of earlier columns, values of later ones) take the 8 pivots at once from the
+        // pivot rows as they were (D += T B again). The registers turn by one place per column and
+        // by 8 per sub-block, so that the column being eliminated is always v[0] and the loops stay
+        // rolled (unrolled over 32 columns they ran from instruction memory: 1600 cycles a column).
+#pragma unroll 1
+        for (int q = 0; q < 4; ++q) {
+          int pq = -1;  // this row's pivot index within the sub-block
+#pragma unroll 1
+          for (int c = 0; c < 8; ++c) {
+            float f = 0.f, last = v[0];
+            float4 r0 = make_float4(0.f, 0.f, 0.f, 0.f), r1 = r0;
+            if ((mask >> (8 * q + c)) & 1u) {
+              b ^= 1;
+              // the low 5 bits of the magnitude give way to the lane: the largest entry to 2^-18
+              const unsigned key = cand ? (__float_as_uint(v[0]) & 0x7fffffe0u) + 32u + lane : 0u;
+              const float inv = recip(v[0]);
+              const unsigned best = __reduce_max_sync(0xffffffffu, key);
+              if (key == best && cand) {
+                float4* post = reinterpret_cast<float4*>(prow[b][warp]);
+                post[0] = make_float4(v[0], v[1], v[2], v[3]);
+                post[1] = make_float4(v[4], v[5], v[6], v[7]);
+                keys[b][warp] = make_uint2(key, __float_as_uint(inv));
+              } else if (best == 0u && lane == 0) {
+                keys[b][warp] = make_uint2(0u, 0u);
+              }
+              __syncwarp();
+              asm volatile("bar.sync 1, %0;" ::"r"(npw * 32) : "memory");
+              const uint4 k01 = *reinterpret_cast<const uint4*>(&keys[b][0]), k23 = *reinterpret_cast<const uint4*>(&keys[b][2]);
+              unsigned kb = k01.x, iv = k01.y;
+              int wb = 0;
+              if (k01.z > kb) kb = k01.z, iv = k01.w, wb = 1;
+              if (k23.x > kb) kb = k23.x, iv = k23.y, wb = 2;
+              if (k23.z > kb) kb = k23.z, iv = k23.w, wb = 3;
+              r0 = *reinterpret_cast<const float4*>(&prow[b][wb][0]);
+              r1 = *reinterpret_cast<const float4*>(&prow[b][wb][4]);
+              if (wb == warp && key == kb && cand) {
+                pq = c;
+                cand = false;
+                if (kb < 64u || kb >= 0x7f800020u) bad = true;  // zero, infinite or NaN
+              }
+              if (cand) f = v[0] * __uint_as_float(iv), last = -f;
+            }
+            v[0] = fmaf(-f, r0.y, v[1]), v[1] = fmaf(-f, r0.z, v[2]), v[2] = fmaf(-f, r0.w, v[3]);
+            v[3] = fmaf(-f, r1.x, v[4]), v[4] = fmaf(-f, r1.y, v[5]), v[5] = fmaf(-f, r1.z, v[6]);
+            v[6] = fmaf(-f, r1.w, v[7]);
+            v[7] = last;
+          }
+          if (pq >= 0) {
+            pj = 8 * q + pq;
+#pragma unroll
+            for (int k = 0; k < 6; ++k)
+              *reinterpret_cast<float4*>(&pblk[q & 1][pq][4 * k]) =
+                  make_float4(v[8 + 4 * k], v[9 + 4 * k], v[10 + 4 * k], v[11 + 4 * k]);
+          }
+          __syncwarp();
+          asm volatile("bar.sync 1, %0;" ::"r"(npw * 32) : "memory");
+          // rows eliminated before this sub-block and slots without a row do not change
+          const bool live = cand || pq >= 0;
+          float t[8], w8[8];
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            w8[k] = v[k];
+            t[k] = live && (pq < 0 || k < pq) && ((mask >> (8 * q + k)) & 1u) ? v[k] : 0.f;
+          }
+#pragma unroll
+          for (int k4 = 0; k4 < 6; ++k4) {
+            float4 acc = make_float4(v[8 + 4 * k4], v[9 + 4 * k4], v[10 + 4 * k4], v[11 + 4 * k4]);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+              const float4 r = *reinterpret_cast<const float4*>(&pblk[q & 1][k][4 * k4]);
+              acc.x = fmaf(t[k], r.x, acc.x), acc.y = fmaf(t[k], r.y, acc.y);
+              acc.z = fmaf(t[k], r.z, acc.z), acc.w = fmaf(t[k], r.w, acc.w);
+            }
+            v[4 * k4] = acc.x, v[4 * k4 + 1] = acc.y, v[4 * k4 + 2] = acc.z, v[4 * k4 + 3] = acc.w;
+          }
+#pragma unroll
+          for (int k = 0; k < 8; ++k) v[24 + k] = w8[k];
+        }
+        if (pj >= 0) {
+#pragma unroll
+          for (int k = 0; k < 32; ++k) u11[par][(32 + pj) * 33 + k] = k >= pj ? v[k] : 0.f;
+#pragma unroll
+          for (int k = 0; k < 32; ++k)
+            if (k >= pj) v[k] = 0.f;
+        }
+        if (warp == 0 && !((mask >> lane) & 1u))
+          for (int k = 0; k < 32; ++k) u11[par][(32 + lane) * 33 + k] = k == lane ? 1.f : 0.f;
+        // T of this panel: global (column k of the 32, slots contiguous) and the split operand
+#pragma unroll
+        for (int k = 0; k < 32; ++k) Tg[(static_cast<size_t>(s) * 32 + k) * NS + slot] = v[k];
+        sjg[static_cast<size_t>(s) * NS + slot] = static_cast<signed char>(pj);
+      }
+      slotj[par][slot] = static_cast<signed char>(pj);
+      if (s > 0) mbar_wait(&bar_rest, (s - 1) & 1, &gave_up, a.status);  // T and B are free again
+      if (dmax > 0) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          float4 h, l;
+          split_tf32(v[4 * q], h.x, l.x);
+          split_tf32(v[4 * q + 1], h.y, l.y);
+          split_tf32(v[4 * q + 2], h.z, l.z);
+          split_tf32(v[4 * q + 3], h.w, l.w);
+          const int o = slot * 32 + ((q ^ (slot & 7)) << 2);
+          *reinterpret_cast<float4*>(Thi + o) = h;
+          *reinterpret_cast<float4*>(Tlo + o) = l;
+        }
+      }
+    }
+    __syncthreads();  // pivots known; the window of the panel before is complete in tensor memory
+    tc_fence_after();
+    const int j = slotj[par][slot];
+    const int tnew = s + 1 + RC, rnew = tnew * 32 + j;  // the row that takes this slot
+    const bool fresh = j >= 0 && tnew < np && ((chunk_mask(w, tnew) >> j) & 1u);
+    if (dmax > 0) {
+      // the pivot rows' window, split, as the K-major B operand; chunks alternate between the halves
+      const int cnt = dmax + (nfc - fc0);
+      for (int c = panel_warp ? 0 : 1; c < cnt; c += 2) {
+        const int col = c < dmax ? ((s + 1 + c) % RS) * 32 : (RS + fc0 + c - dmax) * 32;
+        float r[32];
+        tmem_ld32(tmem + col, r);
+        if (j >= 0) {
+          float* bh = Bhi + col * 32 + (j & 3);
+          float* bl = Blo + col * 32 + (j & 3);
+#pragma unroll
+          for (int i = 0; i < 32; ++i) {
+            float h, l;
+            split_tf32(r[i], h, l);
+            const int o = i * 32 + (((j >> 2) ^ (i & 7)) << 2);
+            bh[o] = h;
+            bl[o] = l;
+          }
+        }
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      tc_fence_before();
+      __syncthreads();
+      tc_fence_after();
+      if (warp == 5) {  // not a panel warp: the tensor cores' queue holds the issuing thread up
+        const uint64_t dah = sdesc(saddr(Thi)), dal = sdesc(saddr(Tlo)), dbh = sdesc(saddr(Bhi)), dbl = sdesc(saddr(Blo));
+        // ranges of window columns: chunk s + 1; then the other ring chunks, slots (s + 2) % RS ..
+        // (s + dmax) % RS, wrapping; then the far columns (at most 256 columns an instruction)
+        const int q1 = (s + 1) % RS, q2 = (s + 2) % RS, m = dmax - 1, m1 = imin(m, RS - q2);
+#pragma unroll 1
+        for (int r = 0; r < 5; ++r) {
+          int col = q1 * 32, n = 32;
+          if (r == 1) col = q2 * 32, n = m1 * 32;
+          if (r == 2) col = 0, n = (m - m1) * 32;
+          if (r >= 3) col = (RS + fc0) * 32 + (r - 3) * 256, n = imin(256, (nfc - fc0) * 32 - (r - 3) * 256);
+          if (n <= 0) continue;
+          const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | (static_cast<uint32_t>(n >> 3) << 17) |
+                                 (static_cast<uint32_t>(kSlots >> 4) << 24);
+          const uint64_t off = static_cast<uint64_t>(col) * 8;  // 128-byte rows in units of 16 bytes
+          const uint32_t d = tmem_base + col;
+          if (lane == 0) {
+#pragma unroll 1
+            for (int k = 0; k < 4; ++k) {  // 8 TF32 columns = 32 bytes inside the swizzle row
+              mma_tf32(d, dal + 2 * k, dbh + off + 2 * k, idesc);
+              mma_tf32(d, dah + 2 * k, dbl + off + 2 * k, idesc);
+              mma_tf32(d, dah + 2 * k, dbh + off + 2 * k, idesc);
+            }
+            if (r == 0) mma_commit(&bar_next);
+          }
+          __syncwarp();
+        }
+        if (lane == 0) mma_commit(&bar_rest);
+        __syncwarp();
+      }
+    }
+    float* Up = Ug + s * ustride;
+    if (warp == 4) {
+      // inv(U11): one lane a column; row k of the inverse leaves the turning registers at x[31]
+      float x[32];
+#pragma unroll
+      for (int r = 0; r < 32; ++r) x[r] = r == lane ? 1.f : 0.f;
+      const float dl = u11[par][(32 + lane) * 33 + lane], rd = dl != 0.f ? recip(dl) : 0.f;
+#pragma unroll 1
+      for (int k = 31; k >= 0; --k) {
+        const float* u = &u11[par][(32 + k) * 33 + k];
+        const float xk = x[31] * __shfl_sync(0xffffffffu, rd, k);
+        Up[k * 32 + lane] = xk;
+#pragma unroll
+        for (int i = 31; i > 0; --i) x[i] = fmaf(-u[-33 * (32 - i)], xk, x[i - 1]);
+        x[0] = 0.f;
+      }
+    }
+    if (dmax == 0) break;
+    float* urow = Up + 1024 + static_cast<size_t>(imax(j, 0)) * w.NU;
+    const float* nb = base + static_cast<size_t>(imax(rnew, 0)) * NW;
+    const float* ns = slope + static_cast<size_t>(imax(rnew, 0)) * NWR;
+    if (panel_warp) {
+      // the next panel's columns: updated rows from tensor memory, the entering rows from the templates
+      float r[32];
+      if (fresh) row_values(nb, ns, E, v);
+      else
+#pragma unroll
+        for (int i = 0; i < 32; ++i) v[i] = 0.f;
+      mbar_wait(&bar_next, par, &gave_up, a.status);
+      tc_fence_after();
+      tmem_ld32(tmem + ((s + 1) % RS) * 32, r);
+      tc_fence_before();
+      __syncwarp();
+      asm volatile("bar.arrive 2, %0;" ::"r"(kThreads) : "memory");
+      if (j >= 0) {
+        store32(urow, r);
+        act = fresh;
+      } else {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) v[i] = r[i];
+      }
+    } else {
+      if (fresh) {  // the entering row's templates into L1 while the tensor cores work
+        for (int d = 1; d <= RS; ++d) {
+          asm volatile("prefetch.global.L1 [%0];" ::"l"(nb + d * 32));
+          asm volatile("prefetch.global.L1 [%0];" ::"l"(ns + d * 32));
+        }
+        for (int c = fc0; c < nfc; ++c) asm volatile("prefetch.global.L1 [%0];" ::"l"(nb + NWR + c * 32));
+      }
+      mbar_wait(&bar_rest, par, &gave_up, a.status);
+      tc_fence_after();
+      for (int d = 2; d <= dmax; ++d) {
+        const uint32_t t = tmem + ((s + d) % RS) * 32;
+        float r[32];
+        tmem_ld32(t, r);
+        if (j >= 0) {
+          store32(urow + (d - 1) * 32, r);
+          if (fresh) row_values(nb + (d - 1) * 32, ns + (d - 1) * 32, E, r);
+          else
+#pragma unroll
+            for (int i = 0; i < 32; ++i) r[i] = 0.f;
+        }
+        tmem_st32(t, r);
+      }
+      for (int c = fc0; c < nfc; ++c) {
+        const uint32_t t = tmem + (RS + c) * 32;
+        float r[32];
+        tmem_ld32(t, r);
+        if (j >= 0) {
+          store32(urow + (RS + c) * 32, r);
+          if (fresh) row_values(nb + NWR + c * 32, nullptr, 0.f, r);
+          else
+#pragma unroll
+            for (int i = 0; i < 32; ++i) r[i] = 0.f;
+        }
+        tmem_st32(t, r);
+      }
+      tmem_wait_st();
+      __syncwarp();
+      asm volatile("bar.sync 2, %0;" ::"r"(kThreads) : "memory");  // the panel warps have read chunk s + 1
+      tc_fence_after();
+      if (s + 1 + RS < np) {
+        // chunk s + 1 + RS enters the ring in the place of chunk s + 1: the rows that stay have
+        // entries only in its l = 0 columns, so far kept apart
+        const uint32_t t = tmem + ((s + 1) % RS) * 32;
+        float r[32];
+        if (fresh) row_values(nb + RS * 32, ns + RS * 32, E, r);
+        else
+#pragma unroll
+          for (int i = 0; i < 32; ++i) r[i] = 0.f;
+        tmem_st32(t, r);
+        tmem_wait_st();
+        for (int i = 0; i < g; ++i) {
+          if ((s + 1 + RS) * g + i >= w.nr) break;
+          const uint32_t tf = tmem + RS * 32 + s * g + i;
+          float x = tmem_ld1(tf);
+          if (fresh) x = fmaf(E, __ldg(ns + RS * 32 + i * w.nlp), __ldg(nb + RS * 32 + i * w.nlp));
+          else if (j >= 0) x = 0.f;
+          tmem_st1(t + i * w.nlp, x);
+          tmem_st1(tf, 0.f);
+        }
+        tmem_wait_st();
+      }
+      tc_fence_before();
+    }
+  }
+  if (bad) atomicOr(a.status, kZeroPivot);
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base),
+                 "r"(static_cast<uint32_t>(w.tmem_cols)));
+}
+
+// FP64 path: the same elimination as two launches per panel, the window in a global scratch that stays
+// in L2 ([nx][128][NU + 32]: the ring holds one chunk more than in tensor memory, the panel's own). The
+// products run on the FP64 units, whose rate bounds them (7.2 GFLOP/s an SM), so the update of a
+// panel is spread over all SMs, one CTA per point and 32-column chunk, whatever the number of
+// points. (One CTA per point for the whole factorisation took 1.77 ms on the 32-point small grid and
+// 23.7 ms on the medium one.)
+struct PanelArgs {
+  FactorArgs f;
+  int s;
+};
+
+__device__ __forceinline__ int ring_col(const WindowPlan& w, int chunk) { return (chunk % (w.RS + 1)) * 32; }
+
+// Rows of chunks 0 .. RC into the window: one CTA per point and slot.
+__global__ void window_f64_init_kernel(const FactorArgs a) {
+  const WindowPlan& w = a.w;
+  const int pt = blockIdx.y, r = blockIdx.x, ldw = w.NU + 32, NWR = (w.RS + 1) * 32;
+  double* D = a.W + (static_cast<size_t>(pt) * kSlots + r) * ldw;
+  const double E = a.E ? a.E[pt] : a.Eu;
+  if (threadIdx.x == 0) a.rows[pt * kSlots + r] = r;
+  const bool valid = r < w.NS && r / 32 < w.np && ((chunk_mask(w, r / 32) >> (r & 31)) & 1u);
+  const double* base = static_cast<const double*>(a.base) + static_cast<size_t>(r) * w.NW;
+  const double* slope = static_cast<const double*>(a.slope) + static_cast<size_t>(r) * NWR;
+  for (int c = threadIdx.x; c < ldw; c += blockDim.x) {
+    // at panel 0 ring slot d holds chunk d
+    double x = 0.0;
+    if (valid) x = c < NWR ? fma(E, __ldg(slope + c), __ldg(base + c)) : __ldg(base + c);
+    D[c] = x;
+  }
+}
+
+// The 32 columns of panel s, one thread a slot: T, U11 and the pivots. Bound by the FP64 units of one SM
+// (31 FMAs a column and thread) and the latency of the columns; nothing else runs on them here: the
+// pivot's checks are made on its bits and its reciprocal takes two Newton steps.
+__global__ void __launch_bounds__(kSlots) window_f64_panel_kernel(const PanelArgs pa) {
+  const FactorArgs& a = pa.f;
+  const WindowPlan& w = a.w;
+  __shared__ __align__(16) double prow[2][4][32];
+  __shared__ unsigned long long kval[2][4];
+  const int pt = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, s = pa.s;
+  const int np = w.np, NS = w.NS, npw = NS / 32;
+  for (int i = tid; i < 256; i += kSlots) (&prow[0][0][0])[i] = 0.0;
+  __syncthreads();
+  const unsigned mask = chunk_mask(w, s);
+  int pj = -1;
+  bool bad = false;
+  if (warp < npw) {
+    const int row = a.rows[pt * kSlots + tid];  // the padded row in this slot
+    bool cand = row < np * 32 && ((chunk_mask(w, row / 32) >> (row & 31)) & 1u);
+    const double* D = a.W + (static_cast<size_t>(pt) * kSlots + tid) * (w.NU + 32) + ring_col(w, s);
+    double v[32];
+#pragma unroll
+    for (int k = 0; k < 32; k += 2) {
+      const double2 x = *reinterpret_cast<const double2*>(D + k);
+      v[k] = cand ? x.x : 0.0, v[k + 1] = cand ? x.y : 0.0;
+    }
+    int b = 0;
+#pragma unroll 1
+    for (int j = 0; j < 32; ++j) {  // the registers turn as in window_lu_tc_kernel
+      double f = 0.0, last = v[0];
+      const double* pr = prow[0][0];
+      if ((mask >> j) & 1u) {
+        b ^= 1;
+        // |v| as an ordered integer, candidates above the rest (NaN above all: reported below)
+        const unsigned long long key =
+            cand ? static_cast<unsigned long long>(__double_as_longlong(v[0]) & 0x7fffffffffffffffll) + 1ull : 0ull;
+        const unsigned hi = static_cast<unsigned>(key >> 32), bh = __reduce_max_sync(0xffffffffu, hi);
+        const unsigned lo = hi == bh ? static_cast<unsigned>(key) : 0u, bl = __reduce_max_sync(0xffffffffu, lo);
+        const int src = __ffs(__ballot_sync(0xffffffffu, hi == bh && static_cast<unsigned>(key) == bl)) - 1;
+        if (lane == src) {
+#pragma unroll
+          for (int k = 0; k < 32; k += 2) *reinterpret_cast<double2*>(&prow[b][warp][k]) = make_double2(v[k], v[k + 1]);
+          kval[b][warp] = (static_cast<unsigned long long>(bh) << 32) | bl;
+        }
+        __syncwarp();
+        asm volatile("bar.sync 1, %0;" ::"r"(npw * 32) : "memory");
+        unsigned long long kb = kval[b][0];
+        int wb = 0;
+        for (int q = 1; q < npw; ++q)
+          if (kval[b][q] > kb) kb = kval[b][q], wb = q;
+        pr = prow[b][wb];
+        if (wb == warp && lane == src) {
+          pj = j;
+          cand = false;
+          if (kb < 2ull || kb > 0x7ff0000000000000ull) bad = true;  // zero, infinite or NaN
+        }
+        const double m = v[0] * recip(pr[0]);
+        if (cand) f = m, last = -m;
+      }
+#pragma unroll
+      for (int k = 0; k < 32; k += 2) {
+        const double2 r = *reinterpret_cast<const double2*>(pr + k);
+        if (k > 0) v[k - 1] = fma(-f, r.x, v[k]);
+        v[k] = fma(-f, r.y, v[k + 1]);
+      }
+      v[31] = last;
+    }
+    // U11 goes where its inverse will be (window_f64_update_kernel inverts it in place)
+    double* u11 = static_cast<double*>(a.U) + (static_cast<size_t>(pt) * np + s) * (1024 + 32 * static_cast<size_t>(w.NU));
+    if (pj >= 0) {
+#pragma unroll
+      for (int k = 0; k < 32; ++k) {
+        u11[pj * 32 + k] = k >= pj ? v[k] : 0.0;
+        if (k >= pj) v[k] = 0.0;
+      }
+    }
+    if (warp == 0 && !((mask >> lane) & 1u))
+      for (int k = 0; k < 32; ++k) u11[lane * 32 + k] = k == lane ? 1.0 : 0.0;
+    double* T = static_cast<double*>(a.T) + (static_cast<size_t>(pt) * np + s) * 32 * NS;
+#pragma unroll
+    for (int k = 0; k < 32; ++k) T[k * NS + tid] = v[k];
+    a.slotj[(static_cast<size_t>(pt) * np + s) * NS + tid] = static_cast<signed char>(pj);
+    if (pj >= 0) a.rows[pt * kSlots + tid] = (s + 1 + w.RC) * 32 + pj;
+  }
+  if (bad) atomicOr(a.status, kZeroPivot);
+}
+
+// U11 (32 x 32, row-major, upper triangular) <- its inverse, 128 threads, sm 3 x 16 x 17 values: the two
+// 16 x 16 diagonal blocks at once (one lane a column, the rows in turning registers), then
+// -inv(A) B inv(D) by 16 x 16 products.
+__device__ void invert_u11(double* u, double* sm, int tid) {
+  double* x = sm;               // [2][16][17]: the diagonal blocks' inverses
+  double* t = sm + 2 * 16 * 17; // [16][17]: B inv(D)
+  if (tid < 32) {
+    const int blk = tid >> 4, c = tid & 15;
+    const double* d = u + blk * 16 * 33;  // the block's corner
+    const double rd = recip(d[c * 33]);
+    double v[16];
+#pragma unroll
+    for (int r = 0; r < 16; ++r) v[r] = r == c ? 1.0 : 0.0;
+#pragma unroll 1
+    for (int k = 15; k >= 0; --k) {
+      const double xk = v[15] * __shfl_sync(0xffffffffu, rd, (tid & 16) + k);
+      x[(blk * 16 + k) * 17 + c] = xk;
+#pragma unroll
+      for (int i = 15; i > 0; --i) {
+        const int r = k - 16 + i;  // the row now moving into place i
+        v[i] = fma(r >= 0 ? -d[r * 32 + k] : 0.0, xk, v[i - 1]);
+      }
+      v[0] = 0.0;
+    }
+  }
+  __syncthreads();
+  for (int e = tid; e < 256; e += kSlots) {
+    const int r = e >> 4, c = e & 15;
+    double s = 0.0;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) s = fma(u[r * 32 + 16 + k], x[(16 + k) * 17 + c], s);
+    t[r * 17 + c] = s;
+  }
+  __syncthreads();
+  for (int e = tid; e < 1024; e += kSlots) {
+    const int r = e >> 5, c = e & 31;
+    double s = 0.0;
+    if (r >= 16 || c < 16) {
+      s = (r >> 4) == (c >> 4) ? x[r * 17 + (c & 15)] : 0.0;
+    } else {
+#pragma unroll
+      for (int k = 0; k < 16; ++k) s = fma(-x[r * 17 + k], t[k * 17 + c - 16], s);
+    }
+    u[r * 32 + c] = s;
+  }
+}
+
+// D += T B on one chunk of the window after panel s; the pivot rows go out as U and the rows that
+// enter take their slots. blockIdx.x: the ring chunks s + 1 .. s + dmax, the far chunks from the
+// first that still has a live column, and last the chunk that enters the ring, whose l = 0 columns
+// are the g far columns it takes over. Pivot rows that are zero on the chunk are left out of the
+// product (on the outer half of the ring all but the rows that pivoting brought forward). One more CTA per
+// point inverts U11 meanwhile.
+__global__ void __launch_bounds__(kSlots) window_f64_update_kernel(const PanelArgs pa, int dmax, int fc0, int nfc) {
+  const FactorArgs& a = pa.f;
+  const WindowPlan& w = a.w;
+  extern __shared__ __align__(1024) unsigned char raw[];
+  double* Ts = reinterpret_cast<double*>(raw);  // [32][128], rows of T in use, in the order of ks
+  double* Bs = Ts + kPW * kSlots;               // [32][32]
+  __shared__ signed char slotj[kSlots];
+  __shared__ int pslot[32], ks[32], nk;
+  const int pt = blockIdx.y, tid = threadIdx.x, lane = tid & 31, s = pa.s;
+  const int np = w.np, NS = w.NS, RS = w.RS, g = w.g, NU = w.NU, ldw = NU + 32, NWR = (RS + 1) * 32;
+  const double* base = static_cast<const double*>(a.base);
+  const double* slope = static_cast<const double*>(a.slope);
+  const double E = a.E ? a.E[pt] : a.Eu;
+  double* D = a.W + static_cast<size_t>(pt) * kSlots * ldw;
+  const double* T = static_cast<const double*>(a.T) + (static_cast<size_t>(pt) * np + s) * 32 * NS;
+  double* U = static_cast<double*>(a.U) + (static_cast<size_t>(pt) * np + s) * (1024 + 32 * static_cast<size_t>(NU)) + 1024;
+  if (blockIdx.x == gridDim.x - 1) {
+    invert_u11(U - 1024, Ts, tid);
+    return;
+  }
+  const int bx = blockIdx.x;
+  const bool ring = bx < dmax, far = !ring && bx < dmax + nfc - fc0;
+  // D's column for column i of the product: a ring chunk, a far chunk without the columns already taken
+  // over, or the far columns s g + i that the entering chunk takes over
+  const int fc = fc0 + bx - dmax, nfar = w.nr - w.kf0;
+  const int col = ring ? ring_col(w, s + 1 + bx) : NWR + (far ? fc * 32 : s * g);
+  const int ilo = far ? imax(0, (s + 1) * g - fc * 32) : 0;
+  const int ihi = ring ? 32 : far ? imin(32, nfar - fc * 32) : imax(0, imin(g, nfar - s * g));
+  auto dcol = [&](int i) -> int { return i >= ilo && i < ihi ? col + i : -1; };
+  if (tid < 32) pslot[tid] = -1;
+  __syncthreads();
+  {
+    const int j = tid < NS ? a.slotj[(static_cast<size_t>(pt) * np + s) * NS + tid] : -1;
+    slotj[tid] = static_cast<signed char>(j);
+    if (j >= 0) pslot[j] = tid;
+  }
+  __syncthreads();
+  // the pivot rows with an entry on the chunk, 32 rows by four warps
+  for (int k = tid >> 5; k < 32; k += 4) {
+    const int ps = pslot[k], dc = dcol(lane);
+    const double x = ps >= 0 && dc >= 0 ? D[static_cast<size_t>(ps) * ldw + dc] : 0.0;
+    const bool any = __any_sync(0xffffffffu, (__double_as_longlong(x) & 0x7fffffffffffffffll) != 0);
+    Bs[k * 32 + lane] = x;
+    if (lane == 0) ks[k] = any ? 1 : 0;
+  }
+  __syncthreads();
+  if (tid < 32) {
+    const bool has = ks[tid] != 0;
+    const unsigned m = __ballot_sync(0xffffffffu, has);
+    __syncwarp();
+    if (has) ks[__popc(m & ((1u << tid) - 1u))] = tid;
+    if (tid == 0) nk = __popc(m);
+  }
+  __syncthreads();
+  const int cnt = nk;
+  for (int q = 0; q < cnt; ++q) Ts[q * kSlots + tid] = tid < NS ? __ldg(T + ks[q] * NS + tid) : 0.0;
+  // 4 rows (lane + 32 q) x 8 columns (of the warp) a thread: a warp whose columns are not in use has no
+  // FP64 work
+  const int c0 = 8 * (tid >> 5);
+  const bool work = c0 < ihi && c0 + 8 > ilo, entering = !ring && !far;
+  double acc[4][8];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const double* dr = D + static_cast<size_t>(lane + 32 * q) * ldw;
+#pragma unroll
+    for (int c = 0; c < 8; c += 2) {
+      acc[q][c] = acc[q][c + 1] = 0.0;
+      if (!work) continue;
+      if (entering) {  // its far columns start anywhere
+        const int d0 = dcol(c0 + c), d1 = dcol(c0 + c + 1);
+        if (d0 >= 0) acc[q][c] = dr[d0];
+        if (d1 >= 0) acc[q][c + 1] = dr[d1];
+      } else {
+        const double2 x = *reinterpret_cast<const double2*>(dr + col + c0 + c);
+        acc[q][c] = x.x, acc[q][c + 1] = x.y;
+      }
+    }
+  }
+  __syncthreads();
+  if (work) {
+#pragma unroll 2
+    for (int k = 0; k < cnt; ++k) {
+      const double* b = Bs + ks[k] * 32 + c0;
+      const double2 b0 = *reinterpret_cast<const double2*>(b), b1 = *reinterpret_cast<const double2*>(b + 2);
+      const double2 b2 = *reinterpret_cast<const double2*>(b + 4), b3 = *reinterpret_cast<const double2*>(b + 6);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        if (32 * q >= NS) break;  // slots not in use
+        const double t = Ts[k * kSlots + lane + 32 * q];
+        acc[q][0] = fma(t, b0.x, acc[q][0]), acc[q][1] = fma(t, b0.y, acc[q][1]);
+        acc[q][2] = fma(t, b1.x, acc[q][2]), acc[q][3] = fma(t, b1.y, acc[q][3]);
+        acc[q][4] = fma(t, b2.x, acc[q][4]), acc[q][5] = fma(t, b2.y, acc[q][5]);
+        acc[q][6] = fma(t, b3.x, acc[q][6]), acc[q][7] = fma(t, b3.y, acc[q][7]);
+      }
+    }
+  }
+  const int tnew = s + 1 + w.RC;
+  const unsigned mnew = tnew < np ? chunk_mask(w, tnew) : 0u;
+  const int ecol = ring_col(w, s + 1 + RS);  // where the entering chunk goes: the panel's own place
+  const int uoff = ring ? bx * 32 : col - 32;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int r = lane + 32 * q, j = slotj[r];
+    const bool fresh = j >= 0 && ((mnew >> j) & 1u);
+    const size_t row = static_cast<size_t>(tnew) * 32 + (j >= 0 ? j : 0);
+    double* dr = D + static_cast<size_t>(r) * ldw;
+    if (entering) {
+      // columns 0, nlp, 2 nlp .. of the chunk are the far columns; a fresh row brings its own values
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        const int i = c0 + c;
+        if (dcol(i) >= 0) {
+          if (j >= 0) U[static_cast<size_t>(j) * NU + uoff + i] = acc[q][c];
+          else dr[ecol + i * w.nlp] = acc[q][c];
+        }
+        const int b = i / w.nlp;  // column i of the chunk is not a far column, or the row is fresh or gone
+        if (j >= 0)
+          dr[ecol + i] = fresh ? fma(E, __ldg(slope + row * NWR + RS * 32 + i), __ldg(base + row * w.NW + RS * 32 + i)) : 0.0;
+        else if (i % w.nlp != 0 || b >= ihi)
+          dr[ecol + i] = 0.0;
+      }
+    } else if (work) {
+      if (j >= 0) {
+        double* ur = U + static_cast<size_t>(j) * NU + uoff + c0;
+#pragma unroll
+        for (int c = 0; c < 8; c += 2)
+          if (c0 + c >= ilo) *reinterpret_cast<double2*>(ur + c) = make_double2(acc[q][c], acc[q][c + 1]);
+          else if (c0 + c + 1 >= ilo) ur[c + 1] = acc[q][c + 1];
+        const double* bp = base + row * w.NW + (ring ? bx * 32 : col) + c0;
+        const double* sp = slope + row * NWR + bx * 32 + c0;
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          acc[q][c] = 0.0;
+          if (fresh) acc[q][c] = ring ? fma(E, __ldg(sp + c), __ldg(bp + c)) : __ldg(bp + c);
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < 8; c += 2)
+        if (c0 + c >= ilo)
+          *reinterpret_cast<double2*>(dr + col + c0 + c) = make_double2(acc[q][c], acc[q][c + 1]);
+        else if (c0 + c + 1 >= ilo)
+          dr[col + c0 + c + 1] = acc[q][c + 1];
+    }
+  }
+}
+
+// ---------------------------------------------------------------- solves and refinement
+
+struct SolveArgs {
+  WindowPlan w;
+  const void* T;
+  const void* U;
+  const signed char* slotj;
+  const double* in;         // right-hand sides and results [nx][nt nr]
+  double* out;
+  const double* E;
+  double Eu, dt;
+  ResidualOps ro;
+  MassBand mass;
+  const double *TO, *TS;
+  double ts_inf, to_inf;    // infinity norms of T_S and T_O
+  double* vec;              // [nx][3 n]: y, z, rho
+  double* fmax_;            // [nx] max|f|
+  double* ratio;
+  int* conv;
+  double tol, kc_inf, ka_inf;
+  int nt;
+  int stages;
+  unsigned stage_bytes;
+  unsigned* status;
+};
+
+template <typename T>
+struct Vec4;
+template <>
+struct Vec4<float> {
+  static __device__ __forceinline__ float dot(const float* a, const float* b) {
+    const float4 x = *reinterpret_cast<const float4*>(a), y = *reinterpret_cast<const float4*>(b);
+    return fmaf(x.w, y.w, fmaf(x.z, y.z, fmaf(x.y, y.y, x.x * y.x)));
+  }
+};
+template <>
+struct Vec4<double> {
+  static __device__ __forceinline__ double dot(const double* a, const double* b) {
+    const double2 x = *reinterpret_cast<const double2*>(a), y = *reinterpret_cast<const double2*>(b);
+    const double2 z = *reinterpret_cast<const double2*>(a + 2), u = *reinterpret_cast<const double2*>(b + 2);
+    return fma(z.y, u.y, fma(z.x, u.x, fma(x.y, y.y, x.x * y.x)));
+  }
+};
+
+constexpr int kEval = 512;  // threads of the projection and residual kernels
+
+// Block-wide maximum of two values; every thread gets the result.
+__device__ __forceinline__ void block_max2(double& p, double& q, double* red) {
+  for (int o = 16; o > 0; o >>= 1) {
+    p = fmax(p, __shfl_xor_sync(0xffffffffu, p, o));
+    q = fmax(q, __shfl_xor_sync(0xffffffffu, q, o));
+  }
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = p, red[kEval / 32 + (threadIdx.x >> 5)] = q;
+  __syncthreads();
+  p = red[0], q = red[kEval / 32];
+  for (int i = 1; i < kEval / 32; ++i) p = fmax(p, red[i]), q = fmax(q, red[kEval / 32 + i]);
+}
+
+// The solves run in the harmonic basis: y = P_S f, z the harmonic solution (x = f + P_O (z - y)); the
+// residual of the system that was factored, rho = M (y - z) + dt (C + E A_v) z, needs only banded
+// products, and r = P_O M^-1 rho is the residual of A_i x = f (P_S x = z).
+
+// y = P_S f, z = 0, rho = M y, max|f|. By parity: Y_l(-mu) = (-1)^l Y_l(mu) and the ordinates are
+// symmetric, so the sums over a half of them with f(a) +- f(nt - 1 - a) give the even and the odd
+// harmonics: half the FP64 operations, which bound it.
+__global__ void __launch_bounds__(kEval) window_project_kernel(const SolveArgs a) {
+  extern __shared__ __align__(1024) unsigned char raw[];
+  const int nr = a.w.nr, nl = a.w.nl, nt = a.nt, n = nl * nr, nv = nt * nr, hf = nt / 2, hc = (nt + 1) / 2;
+  double* fold = reinterpret_cast<double*>(raw);  // 2 hc nr
+  double* ys = fold + 2 * hc * nr;                // n
+  __shared__ double red[2 * kEval / 32];
+  const int pt = blockIdx.x, tid = threadIdx.x;
+  const double* f = a.in + static_cast<size_t>(pt) * nv;
+  double* y = a.vec + static_cast<size_t>(pt) * 3 * n;
+  double mb = 0.0, unused = 0.0;
+  for (int i = tid; i < hc * nr; i += kEval) {
+    const int q = i / nr, k = i % nr;
+    const double p = f[i], m = q < hf ? f[(nt - 1 - q) * nr + k] : 0.0;
+    fold[i] = p + m;
+    fold[hc * nr + i] = q < hf ? p - m : 0.0;
+    mb = fmax(mb, fmax(fabs(p), fabs(m)));
+  }
+  block_max2(mb, unused, red);
+  if (tid == 0) {
+    a.fmax_[pt] = mb;
+    if (a.conv) a.conv[pt] = 0;
+  }
+  for (int i = tid; i < n; i += kEval) {
+    const int l = i / nr, k = i % nr;
+    const double* src = fold + (l & 1 ? hc * nr : 0) + k;
+    const double* ts = a.TS + l * nt;
+    double s0 = 0.0, s1 = 0.0;
+    int q = 0;
+    for (; q + 1 < hc; q += 2) {
+      s0 = fma(__ldg(ts + q), src[q * nr], s0);
+      s1 = fma(__ldg(ts + q + 1), src[(q + 1) * nr], s1);
+    }
+    if (q < hc) s0 = fma(__ldg(ts + q), src[q * nr], s0);
+    ys[i] = s0 + s1;
+    y[i] = s0 + s1;
+    y[n + i] = 0.0;
+  }
+  __syncthreads();
+  const int mw = a.mass.w, bw = 2 * mw + 1;
+  for (int i = tid; i < n; i += kEval) {
+    const int l = i / nr, p = i % nr;
+    const double* mr = a.mass.m + static_cast<size_t>(p) * bw + mw - p;
+    double s = 0.0;
+    for (int k = imax(0, p - mw); k <= imin(nr - 1, p + mw); ++k) s = fma(__ldg(mr + k), ys[l * nr + k], s);
+    y[2 * n + i] = s;
+  }
+}
+
+// z += H^-1 rho through the window factors, one CTA per point. The factors are streamed once, panel by
+// panel (the T forwards, then inv(U11) and U backwards), through a ring of shared-memory stages
+// filled by bulk copies: bound by the copy rate of one SM (3.4 MB a point and solve on the medium
+// grid). Converged points return at once.
+template <typename T>
+__global__ void __launch_bounds__(kThreads) window_substitute_kernel(const SolveArgs a) {
+  extern __shared__ __align__(1024) unsigned char raw[];
+  const WindowPlan& w = a.w;
+  const int pt = blockIdx.x, tid = threadIdx.x;
+  if (a.conv && a.conv[pt]) return;
+  const int np = w.np, NS = w.NS, NU = w.NU, RS = w.RS, RC = w.RC, g = w.g, nl = w.nl, nr = w.nr, nlp = w.nlp;
+  const int n = nl * nr, S = a.stages;
+  const unsigned fbytes = 32u * NS * sizeof(T), bbytes = (1024u + 32u * NU) * sizeof(T);
+  unsigned char* stage = raw;
+  T* b = reinterpret_cast<T*>(raw + static_cast<size_t>(S) * a.stage_bytes);  // padded unknowns, chunk by chunk
+  const int npad = (np + RS) * 32;
+  T* bp = b + npad;  // [2][32] pivot values; the backward pass's 32 partial results
+  double* z = a.vec + static_cast<size_t>(pt) * 3 * n + n;
+  const double* rho = z + n;
+  __shared__ __align__(8) uint64_t full[8];
+  __shared__ int gave_up;
+  const T* Tg = static_cast<const T*>(a.T) + static_cast<size_t>(pt) * np * 32 * NS;
+  const size_t ustride = 1024 + 32 * static_cast<size_t>(NU);
+  const T* Ug = static_cast<const T*>(a.U) + static_cast<size_t>(pt) * np * ustride;
+  const signed char* sj = a.slotj + static_cast<size_t>(pt) * np * NS;
+  const int nfar = imax(0, nr - w.kf0);
+  // the q-th copy: the T of panels 0 .. np - 1, then the U of panels np - 1 .. 0
+  auto issue = [&](int q) {
+    const T* src = q < np ? Tg + static_cast<size_t>(q) * 32 * NS : Ug + static_cast<size_t>(2 * np - 1 - q) * ustride;
+    const unsigned bytes = q < np ? fbytes : bbytes;
+    uint64_t* bar = &full[q % S];
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(saddr(bar)), "r"(bytes) : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                     saddr(stage + static_cast<size_t>(q % S) * a.stage_bytes)),
+                 "l"(src), "r"(bytes), "r"(saddr(bar))
+                 : "memory");
+  };
+  if (tid == 0) {
+    for (int i = 0; i < S; ++i) mbar_init(&full[i], 1);
+    gave_up = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    for (int q = 0; q < imin(S, 2 * np); ++q) issue(q);
+  }
+  for (int i = tid; i < npad; i += kThreads) {
+    const int k = i / nlp, l = i % nlp;
+    b[i] = k < nr && l < nl ? static_cast<T>(rho[l * nr + k]) : T(0);
+  }
+  if (tid < 64) bp[tid] = T(0);  // unused unknowns stay zero
+  __syncthreads();
+  // forward: one thread a slot
+  if (tid < NS) {
+    T wv = tid < npad ? b[tid] : T(0);
+    int jn = sj[tid];
+    for (int s = 0; s < np; ++s) {
+      const int j = jn;
+      if (s + 1 < np) jn = sj[static_cast<size_t>(s + 1) * NS + tid];
+      if (j >= 0) bp[(s & 1) * 32 + j] = wv;
+      asm volatile("bar.sync 1, %0;" ::"r"(NS) : "memory");
+      // every slot's thread is past panel s - 1: its stage can be filled again
+      if (tid == 0 && s > 0 && s - 1 + S < 2 * np) issue(s - 1 + S);
+      mbar_wait(&full[s % S], (s / S) & 1, &gave_up, a.status);
+      const T* t = reinterpret_cast<const T*>(stage + static_cast<size_t>(s % S) * a.stage_bytes) + tid;
+      const T* q = bp + (s & 1) * 32;
+      T acc[4] = {wv, T(0), T(0), T(0)};
+#pragma unroll
+      for (int k = 0; k < 32; ++k) acc[k & 3] = fma(t[k * NS], q[k], acc[k & 3]);
+      wv = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+      if (j >= 0) {
+        b[s * 32 + j] = wv;  // y of this panel; the chunk that enters takes the slot
+        wv = s + 1 + RC < np ? b[(s + 1 + RC) * 32 + j] : T(0);
+      }
+    }
+  }
+  __syncthreads();
+  if (tid == 0 && np - 1 + S < 2 * np) issue(np - 1 + S);
+  // backward: eight threads a row
+  const int row = tid >> 3, sub = tid & 7;
+  for (int s = np - 1; s >= 0; --s) {
+    const int q = 2 * np - 1 - s;
+    mbar_wait(&full[q % S], (q / S) & 1, &gave_up, a.status);
+    const T* ui = reinterpret_cast<const T*>(stage + static_cast<size_t>(q % S) * a.stage_bytes);
+    const T* u = ui + 1024 + static_cast<size_t>(row) * NU;
+    const T* x = b + (s + 1) * 32;
+    const int wr = imin(RS, np - 1 - s) * 32;
+    T s0 = T(0), s1 = T(0);
+    for (int c = 4 * sub; c < wr; c += 32) s0 += Vec4<T>::dot(u + c, x + c);
+    const T* uf = u + RS * 32;
+    if (s * g < nfar && s + 1 < np)
+      for (int k = ((s * g) / 32) * 32 + sub; k < nfar; k += 8)
+        if (k >= s * g) s1 = fma(uf[k], b[(w.kf0 + k) * nlp], s1);
+    T acc = s0 + s1;
+    acc += __shfl_xor_sync(0xffffffffu, acc, 4);
+    acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+    T* t = bp + (s & 1) * 32;
+    if (sub == 0) t[row] = b[s * 32 + row] - acc;
+    __syncthreads();
+    T e = Vec4<T>::dot(ui + row * 32 + 4 * sub, t + 4 * sub);
+    e += __shfl_xor_sync(0xffffffffu, e, 4);
+    e += __shfl_xor_sync(0xffffffffu, e, 2);
+    e += __shfl_xor_sync(0xffffffffu, e, 1);
+    if (sub == 0) b[s * 32 + row] = e;
+    __syncthreads();
+    if (tid == 0 && q + S < 2 * np) issue(q + S);
+  }
+  for (int i = tid; i < n; i += kThreads) z[i] += static_cast<double>(b[(i % nr) * nlp + i / nr]);
+}
+
+// With check: rho of the iterate, the convergence test of launch_residual (max|r| and max|x| at the
+// ordinates; ratio, conv and the count in status[1] as it writes them) and, where the test was
+// made, x into out. As long as a bound that costs one reduction (|rho_p| <= sum_k |M_pk| max|M^-1 rho|
+// and |M^-1 rho| <= |T_S| max|r|) already shows a point to be short of the tolerance, neither the
+// Cholesky substitution nor the projections are made, except at the last sweep. Without check: x alone.
+__global__ void __launch_bounds__(kEval) window_residual_kernel(const SolveArgs a, int check, int last) {
+  extern __shared__ __align__(1024) unsigned char raw[];
+  const int nr = a.w.nr, nl = a.w.nl, nt = a.nt, n = nl * nr, nv = nt * nr, hf = nt / 2, hc = (nt + 1) / 2;
+  const int pt = blockIdx.x, tid = threadIdx.x;
+  if (check && a.conv[pt]) return;
+  double* z = reinterpret_cast<double*>(raw);  // n
+  double* dz = z + n;                          // z - y
+  double* q = dz + n;                          // rho, then M^-1 rho
+  __shared__ double red[2 * kEval / 32];
+  const double* f = a.in + static_cast<size_t>(pt) * nv;
+  double* out = a.out + static_cast<size_t>(pt) * nv;
+  double* vec = a.vec + static_cast<size_t>(pt) * 3 * n;
+  const double Ei = a.E ? a.E[pt] : a.Eu;
+  for (int i = tid; i < n; i += kEval) {
+    const double zi = vec[n + i];
+    z[i] = zi;
+    dz[i] = zi - vec[i];
+  }
+  __syncthreads();
+  double mb = 0.0, nA = 0.0;
+  const double floor_ = fmin(kBackwardFloor, a.tol);
+  if (check) {
+    mb = a.fmax_[pt];
+    nA = 1.0 + a.dt * (a.kc_inf + fabs(Ei) * a.ka_inf);
+    const int mw = a.mass.w, bw = 2 * mw + 1;
+    double lb = 0.0, mz = 0.0;
+    for (int i = tid; i < n; i += kEval) {
+      const int l = i / nr, p = i % nr;
+      const int k0 = imax(0, p - mw), k1 = imin(nr - 1, p + mw);
+      const double* zl = z + l * nr;
+      const double* dl = dz + l * nr;
+      const double* mr = a.mass.m + static_cast<size_t>(p) * bw + mw - p;
+      double m = 0.0, c = 0.0, fl = 0.0, rs = 0.0;
+      for (int k = k0; k <= k1; ++k) {
+        const double t = __ldg(mr + k);
+        m = fma(-t, dl[k], m);
+        rs += fabs(t);
+      }
+      if (l > 0) {
+        const double* row = a.ro.band + static_cast<size_t>(p) * bw + mw - p;
+        const double* fr = a.ro.fband + (static_cast<size_t>(l) * nr + p) * bw + mw - p;
+        for (int k = k0; k <= k1; ++k) {
+          c = fma(__ldg(row + k), zl[k], c);
+          fl = fma(__ldg(fr + k), zl[k - nr], fl);
+        }
+      } else {
+        const double* row = a.ro.c0 + static_cast<size_t>(p) * nr;
+        for (int k = k0; k < nr; ++k) c = fma(__ldg(row + k), zl[k], c);
+      }
+      if (l + 1 < nl) {
+        const double* fr = a.ro.fband + (static_cast<size_t>(nl + l) * nr + p) * bw + mw - p;
+        for (int k = k0; k <= k1; ++k) fl = fma(__ldg(fr + k), zl[k + nr], fl);
+      }
+      const double r = m + a.dt * (c + Ei * fl);
+      q[i] = r;
+      vec[2 * n + i] = r;
+      lb = fmax(lb, fabs(r) / rs);
+      mz = fmax(mz, fabs(dl[p]));
+    }
+    block_max2(lb, mz, red);
+    if (tid == 0) atomicAdd(a.status + 1, 1u);  // residual evaluations
+    const double least = lb / a.ts_inf;
+    if (!last && least > a.tol * mb && least > floor_ * (nA * (mb + a.to_inf * mz) + mb)) return;
+    // q_l <- M^-1 q_l by the banded Cholesky factor, one thread a harmonic
+    for (int l = tid; l < nl; l += kEval) {
+      double* gl = q + l * nr;
+      if (mw == 3) {
+        double y1 = 0.0, y2 = 0.0, y3 = 0.0;
+        for (int p = 0; p < nr; ++p) {
+          const double* r = a.ro.chol + static_cast<size_t>(p) * 4;
+          const double y = fma(-__ldg(r + 2), y1, fma(-__ldg(r + 1), y2, fma(-__ldg(r), y3, gl[p]))) * __ldg(a.ro.cinv + p);
+          gl[p] = y;
+          y3 = y2, y2 = y1, y1 = y;
+        }
+        double z1 = 0.0, z2 = 0.0, z3 = 0.0;
+        for (int p = nr - 1; p >= 0; --p) {
+          double s = gl[p];
+          if (p + 1 < nr) s = fma(-__ldg(a.ro.chol + static_cast<size_t>(p + 1) * 4 + 2), z1, s);
+          if (p + 2 < nr) s = fma(-__ldg(a.ro.chol + static_cast<size_t>(p + 2) * 4 + 1), z2, s);
+          if (p + 3 < nr) s = fma(-__ldg(a.ro.chol + static_cast<size_t>(p + 3) * 4), z3, s);
+          const double zz = s * __ldg(a.ro.cinv + p);
+          gl[p] = zz;
+          z3 = z2, z2 = z1, z1 = zz;
+        }
+      } else {
+        for (int p = 0; p < nr; ++p) {
+          const double* r = a.ro.chol + static_cast<size_t>(p) * (mw + 1);
+          double s = gl[p];
+          for (int j = imax(0, mw - p); j < mw; ++j) s = fma(-__ldg(r + j), gl[p - mw + j], s);
+          gl[p] = s * __ldg(a.ro.cinv + p);
+        }
+        for (int p = nr - 1; p >= 0; --p) {
+          double s = gl[p];
+          for (int k = p + 1; k <= imin(nr - 1, p + mw); ++k)
+            s = fma(-__ldg(a.ro.chol + static_cast<size_t>(k) * (mw + 1) + p - k + mw), gl[k], s);
+          gl[p] = s * __ldg(a.ro.cinv + p);
+        }
+      }
+    }
+    __syncthreads();
+  }
+  // x = f + P_O (z - y) and, with check, r = P_O q, both by parity
+  double mr = 0.0, mx = 0.0;
+  for (int i = tid; i < hc * nr; i += kEval) {
+    const int o = i / nr, k = i % nr;
+    const double* to = a.TO + o * nl;
+    double xe = 0.0, xo = 0.0, re = 0.0, ro = 0.0;
+    for (int l = 0; l < nl; l += 2) {
+      const double t0 = __ldg(to + l);
+      xe = fma(t0, dz[l * nr + k], xe);
+      if (check) re = fma(t0, q[l * nr + k], re);
+      if (l + 1 < nl) {
+        const double t1 = __ldg(to + l + 1);
+        xo = fma(t1, dz[(l + 1) * nr + k], xo);
+        if (check) ro = fma(t1, q[(l + 1) * nr + k], ro);
+      }
+    }
+    const double x1 = f[i] + (xe + xo);
+    mr = fmax(mr, fabs(re + ro)), mx = fmax(mx, fabs(x1));
+    if (o < hf) {
+      const size_t i2 = static_cast<size_t>(nt - 1 - o) * nr + k;
+      const double x2 = f[i2] + (xe - xo);
+      out[i2] = x2;
+      mr = fmax(mr, fabs(re - ro)), mx = fmax(mx, fabs(x2));
+    }
+    out[i] = x1;
+  }
+  if (!check) return;
+  block_max2(mr, mx, red);
+  if (tid == 0) {
+    const double ratio = mb > 0.0 ? mr / mb : (mr > 0.0 ? INFINITY : 0.0);
+    a.ratio[pt] = ratio;
+    a.conv[pt] = ratio <= a.tol || mr <= floor_ * (nA * mx + mb) ? 1 : 0;
+  }
+}
+
+// out = A^-T in for the adjoint (FP64 factors, no refinement): the transposed passes of
+// window_solve_kernel in reverse order. A^-1 = I + P_O (H^-1 M - I) P_S, so
+// A^-T g = g + P_S^T (M H^-T - I) P_O^T g (M symmetric).
+__global__ void __launch_bounds__(kThreads) window_solve_t_kernel(const SolveArgs a) {
+  extern __shared__ __align__(1024) unsigned char raw[];
+  const WindowPlan& w = a.w;
+  const int pt = blockIdx.x, tid = threadIdx.x;
+  const int np = w.np, NS = w.NS, NU = w.NU, RS = w.RS, RC = w.RC, g = w.g, nl = w.nl, nr = w.nr, nlp = w.nlp, nt = a.nt;
+  const int nv = nt * nr, npad = (np + RS) * 32, n = nl * nr;
+  double* x = reinterpret_cast<double*>(raw);  // npad: cotangents, then pivot results, then H^-T
+  double* wv = x + npad;                       // kSlots
+  double* v = wv + kSlots;                     // 32
+  const double* f = a.in + static_cast<size_t>(pt) * nv;
+  double* out = a.out + static_cast<size_t>(pt) * nv;
+  double* gh = a.vec + static_cast<size_t>(pt) * 3 * n;
+  const double* Tg = static_cast<const double*>(a.T) + static_cast<size_t>(pt) * np * 32 * NS;
+  const size_t ustride = 1024 + 32 * static_cast<size_t>(NU);
+  const double* Ug = static_cast<const double*>(a.U) + static_cast<size_t>(pt) * np * ustride;
+  const signed char* sj = a.slotj + static_cast<size_t>(pt) * np * NS;
+  const int nfar = imax(0, nr - w.kf0);
+  for (int i = tid; i < npad; i += kThreads) x[i] = 0.0;
+  if (tid < kSlots) wv[tid] = 0.0;
+  __syncthreads();
+  for (int i = tid; i < n; i += kThreads) {
+    const int l = i / nr, k = i % nr;
+    double s = 0.0;
+    for (int q = 0; q < nt; ++q) s = fma(__ldg(a.TO + q * nl + l), f[q * nr + k], s);
+    gh[i] = s;
+    x[k * nlp + l] = s;
+  }
+  __syncthreads();
+  const int row = tid >> 3, sub = tid & 7;
+  for (int s = 0; s < np; ++s) {
+    const double* ui = Ug + s * ustride;
+    double e = 0.0;
+    for (int r = sub; r < 32; r += 8) e = fma(__ldg(ui + r * 32 + row), x[s * 32 + r], e);
+    e += __shfl_xor_sync(0xffffffffu, e, 4);
+    e += __shfl_xor_sync(0xffffffffu, e, 2);
+    e += __shfl_xor_sync(0xffffffffu, e, 1);
+    if (sub == 0) v[row] = e;
+    __syncthreads();
+    if (tid < 32) x[s * 32 + tid] = v[tid];
+    const int wr = imin(RS, np - 1 - s) * 32;
+    const int f0 = s * g, nf = s + 1 < np ? imax(0, nfar - f0) : 0;
+    for (int c = tid; c < wr + nf; c += kThreads) {
+      const double* u = ui + 1024 + (c < wr ? c : RS * 32 + f0 + c - wr);
+      double t = 0.0;
+#pragma unroll 8
+      for (int j = 0; j < 32; ++j) t = fma(__ldg(u + static_cast<size_t>(j) * NU), v[j], t);
+      x[c < wr ? (s + 1) * 32 + c : (w.kf0 + f0 + c - wr) * nlp] -= t;
+    }
+    __syncthreads();
+  }
+  for (int s = np - 1; s >= 0; --s) {
+    const int j = tid < NS ? sj[static_cast<size_t>(s) * NS + tid] : -1;
+    if (j >= 0) {
+      const double keep = x[s * 32 + j];
+      // the row that entered this slot after panel s: its cotangent is complete
+      if (s + 1 + RC < np) x[(s + 1 + RC) * 32 + j] = wv[tid];
+      wv[tid] = keep;
+    }
+    __syncthreads();
+    double e = 0.0;
+    for (int q = sub; q < NS; q += 8) e = fma(__ldg(Tg + (static_cast<size_t>(s) * 32 + row) * NS + q), wv[q], e);
+    e += __shfl_xor_sync(0xffffffffu, e, 4);
+    e += __shfl_xor_sync(0xffffffffu, e, 2);
+    e += __shfl_xor_sync(0xffffffffu, e, 1);
+    if (sub == 0) v[row] = e;
+    __syncthreads();
+    if (j >= 0) wv[tid] += v[j];
+    __syncthreads();
+  }
+  if (tid < NS && tid < np * 32) x[tid] = wv[tid];
+  __syncthreads();
+  const int mw = a.mass.w, bw = 2 * mw + 1;
+  for (int i = tid; i < n; i += kThreads) {
+    const int l = i / nr, p = i % nr;
+    const double* mr = a.mass.m + static_cast<size_t>(p) * bw + mw - p;
+    double s = 0.0;
+    for (int k = imax(0, p - mw); k <= imin(nr - 1, p + mw); ++k) s = fma(__ldg(mr + k), x[k * nlp + l], s);
+    gh[i] = s - gh[i];
+  }
+  __syncthreads();
+  for (int i = tid; i < nv; i += kThreads) {
+    const int q = i / nr, k = i % nr;
+    double s = f[i];
+    for (int l = 0; l < nl; ++l) s = fma(__ldg(a.TS + l * nt + q), gh[l * nr + k], s);
+    out[i] = s;
+  }
+}
+
+int round_up(int a, int b) { return (a + b - 1) / b * b; }
+
+}  // namespace
+
+WindowPlan window_plan(int nr, int nl) {
+  WindowPlan w;
+  if (nl < 1 || nl > 32) return w;
+  w.nr = nr, w.nl = nl;
+  w.nlp = 1;
+  while (w.nlp < nl) w.nlp *= 2;
+  w.g = kPW / w.nlp;
+  w.np = (nr + w.g - 1) / w.g;
+  w.RC = (3 + w.g - 1) / w.g;
+  w.RS = 2 * w.RC;
+  w.NS = 32 * (1 + w.RC);
+  w.kf0 = (w.RS + 1) * w.g;
+  w.NF = nr > w.kf0 ? round_up(nr - w.kf0, 32) : 0;
+  w.NU = w.RS * 32 + w.NF;
+  w.NW = (w.RS + 1) * 32 + w.NF;
+  w.tmem_cols = 32;
+  while (w.tmem_cols < w.NU) w.tmem_cols *= 2;
+  w.ok = w.NU <= 512;
+  return w;
+}
+
+void window_tables(const WindowPlan& w, const HostOps& o, std::vector<double>& base, std::vector<double>& slope) {
+  const int nr = o.nr, nl = o.nl, NWR = (w.RS + 1) * 32;
+  base.assign(static_cast<size_t>(w.np) * 32 * w.NW, 0.0);
+  slope.assign(static_cast<size_t>(w.np) * 32 * NWR, 0.0);
+  for (int p = 0; p < nr; ++p)
+    for (int l = 0; l < nl; ++l) {
+      const int t = p / w.g, row = t * 32 + (p % w.g) * w.nlp + l;
+      const int c0 = std::max(0, t - w.RC);  // the panel at which the row enters
+      double* br = base.data() + static_cast<size_t>(row) * w.NW;
+      double* sr = slope.data() + static_cast<size_t>(row) * NWR;
+      // splines overlap for |p - k| <= 3 only; the gain couples l = 0 to any k above
+      const int hi = l == 0 ? nr - 1 : std::min(nr - 1, p + 3);
+      for (int k = std::max(0, p - 3); k <= hi; ++k) {
+        const int d = k / w.g - c0, col = d <= w.RS ? d * 32 + (k % w.g) * w.nlp : -1;
+        const size_t e = (static_cast<size_t>(l) * nr + p) * nr + k;
+        const double m = std::abs(p - k) <= 3 ? o.M[p * nr + k] : 0.0;
+        const double v = m - o.dt * o.Cg[e];
+        if (col >= 0) br[col + l] = v;
+        else br[NWR + k - w.kf0] = v;
+        if (k <= p + 3) {
+          if (l > 0) sr[col + l - 1] = -o.dt * o.Ag_lo[e];
+          if (l + 1 < nl) sr[col + l + 1] = -o.dt * o.Ag_up[e];
+        }
+      }
+    }
+}
+
+size_t window_t_count(const WindowPlan& w) { return static_cast<size_t>(w.np) * 32 * w.NS; }
+size_t window_u_count(const WindowPlan& w) { return static_cast<size_t>(w.np) * (1024 + 32 * static_cast<size_t>(w.NU)); }
+size_t window_slot_count(const WindowPlan& w) { return static_cast<size_t>(w.np) * w.NS; }
+
+static FactorArgs factor_args(const WindowBuffers& b, const double* E, double Eu, unsigned* status) {
+  FactorArgs a;
+  a.w = b.w, a.base = b.base, a.slope = b.slope, a.E = E, a.Eu = Eu, a.T = b.T, a.U = b.U, a.slotj = b.slotj;
+  a.W = b.W, a.rows = b.rows, a.status = status;
+  return a;
+}
+
+static SolveArgs solve_args(const WindowBuffers& b, MassBand mass, int nt) {
+  SolveArgs a{};
+  a.w = b.w, a.T = b.T, a.U = b.U, a.slotj = b.slotj, a.vec = b.vec, a.fmax_ = b.fmax_, a.mass = mass, a.nt = nt;
+  return a;
+}
+
+cudaError_t launch_window_factor(const WindowBuffers& b, const double* E, double Eu, int nx, unsigned* status,
+                                 cudaStream_t st) {
+  const FactorArgs a = factor_args(b, E, Eu, status);
+  const int smem = 1024 + static_cast<int>(sizeof(float)) * kPW * 2 * (kSlots + b.w.NU);
+  const cudaError_t e = cudaFuncSetAttribute(window_lu_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  window_lu_tc_kernel<<<nx, kThreads, smem, st>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_window_init_f64(const WindowBuffers& b, const double* E, double Eu, int nx, unsigned* status,
+                                   cudaStream_t st) {
+  window_f64_init_kernel<<<dim3(kSlots, nx), 128, 0, st>>>(factor_args(b, E, Eu, status));
+  return cudaGetLastError();
+}
+
+cudaError_t launch_window_panel_f64(const WindowBuffers& b, int s, int nx, unsigned* status, cudaStream_t st) {
+  window_f64_panel_kernel<<<nx, kSlots, 0, st>>>(PanelArgs{factor_args(b, nullptr, 0.0, status), s});
+  return cudaGetLastError();
+}
+
+cudaError_t launch_window_update_f64(const WindowBuffers& b, const double* E, double Eu, int s, int nx, unsigned* status,
+                                     cudaStream_t st) {
+  const WindowPlan& w = b.w;
+  const int dmax = std::min(w.RS, w.np - 1 - s), nfar = std::max(0, w.nr - w.kf0);
+  // far columns s g .. s g + g - 1 belong to the entering chunk; the chunk after them has the next live one
+  const int fc0 = ((s + 1) * w.g) / 32, nfc = (s + 1) * w.g < nfar ? w.NF / 32 : fc0;
+  const int smem = static_cast<int>(sizeof(double)) * (kPW * kSlots + kPW * kPW);
+  const int grid = dmax + nfc - fc0 + (s + 1 + w.RS < w.np ? 1 : 0) + 1;
+  window_f64_update_kernel<<<dim3(grid, nx), kSlots, smem, st>>>(PanelArgs{factor_args(b, E, Eu, status), s}, dmax, fc0, nfc);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_window_project(const WindowBuffers& b, const double* in, MassBand mass, const double* TS, int* conv,
+                                  int nx, int nt, cudaStream_t st) {
+  SolveArgs a = solve_args(b, mass, nt);
+  a.in = in, a.TS = TS, a.conv = conv;
+  const int smem = static_cast<int>(sizeof(double)) * (2 * ((nt + 1) / 2) + b.w.nl) * b.w.nr;
+  const cudaError_t e = cudaFuncSetAttribute(window_project_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  window_project_kernel<<<nx, kEval, smem, st>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_window_substitute(const WindowBuffers& b, const int* conv, int nx, unsigned* status, cudaStream_t st) {
+  SolveArgs a = solve_args(b, MassBand{}, 0);
+  a.conv = const_cast<int*>(conv), a.status = status;
+  const size_t ts = b.fp64 ? sizeof(double) : sizeof(float);
+  const size_t fb = ts * 32 * b.w.NS, bb = ts * (1024 + 32 * static_cast<size_t>(b.w.NU));
+  a.stage_bytes = static_cast<unsigned>(round_up(static_cast<int>(std::max(fb, bb)), 128));
+  const size_t fixed = ts * (static_cast<size_t>(b.w.np + b.w.RS) * 32 + 64);
+  // one CTA an SM takes up to 8 stages; with more points than SMs two CTAs share one where both can
+  // have two stages
+  size_t room = 224 * 1024 - fixed;
+  if (nx > 152 && fixed + 2 * static_cast<size_t>(a.stage_bytes) <= 112 * 1024) room = 112 * 1024 - fixed;
+  a.stages = static_cast<int>(std::max<size_t>(1, std::min<size_t>(8, room / a.stage_bytes)));
+  const int smem = static_cast<int>(a.stages * static_cast<size_t>(a.stage_bytes) + fixed);
+  auto k = b.fp64 ? window_substitute_kernel<double> : window_substitute_kernel<float>;
+  const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  k<<<nx, kThreads, smem, st>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_window_residual(const WindowBuffers& b, const double* in, double* out, const double* E, double Eu,
+                                   double dt, const ResidualOps& ro, MassBand mass, const double* TO, double ts_inf,
+                                   double to_inf, double* ratio, int* conv, double tol, double kc_inf, double ka_inf,
+                                   int nx, int nt, bool check, bool last, unsigned* status, cudaStream_t st) {
+  SolveArgs a = solve_args(b, mass, nt);
+  a.in = in, a.out = out, a.E = E, a.Eu = Eu, a.dt = dt, a.ro = ro, a.TO = TO, a.ts_inf = ts_inf, a.to_inf = to_inf;
+  a.ratio = ratio, a.conv = conv, a.tol = tol, a.kc_inf = kc_inf, a.ka_inf = ka_inf, a.status = status;
+  const int smem = static_cast<int>(sizeof(double)) * 3 * b.w.nl * b.w.nr;
+  const cudaError_t e = cudaFuncSetAttribute(window_residual_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  window_residual_kernel<<<nx, kEval, smem, st>>>(a, check ? 1 : 0, last ? 1 : 0);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_window_solve_t(const WindowBuffers& b, const double* in, double* out, MassBand mass,
+                                  const double* TO, const double* TS, int nx, int nt, cudaStream_t st) {
+  SolveArgs a = solve_args(b, mass, nt);
+  a.in = in, a.out = out, a.TO = TO, a.TS = TS;
+  const int smem = static_cast<int>(sizeof(double)) * ((b.w.np + b.w.RS) * 32 + kSlots + 32);
+  const cudaError_t e = cudaFuncSetAttribute(window_solve_t_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  window_solve_t_kernel<<<nx, kThreads, smem, st>>>(a);
+  return cudaGetLastError();
+}
+
+}  // namespace bte
