@@ -194,21 +194,52 @@ bte_status window_factor(bte_handle* h, const double* E_dev, double Eu) {
   return BTE_OK;
 }
 
-// out_i = A_i^-1 in_i through the last window factors, with up to `sweeps` refinement sweeps (conv
-// tells afterwards which points converged; with 0 sweeps nothing is checked).
-bte_status window_solve(bte_handle* h, const double* in, double* out, const double* E_dev, double Eu, int sweeps) {
+// The inverses of the block-tridiagonal elimination at every point.
+bte_status struct_factor(bte_handle* h, const double* E_dev, double Eu) {
+  const HostOps& o = h->ops;
+  const bte::MassBand mass{h->Mband, o.nr, o.mw};
+  if (h->precision == BTE_FP64)
+    BTE_LAUNCH(BTE_K_LU_GEMM, bte::launch_struct_factor<double>(E_dev, Eu, o.dt, residual_ops(h), mass,
+                                                                static_cast<double*>(h->xs), o.nx, o.nr, o.nl, h->st));
+  else
+    BTE_LAUNCH(BTE_K_LU_GEMM, bte::launch_struct_factor<float>(E_dev, Eu, o.dt, residual_ops(h), mass,
+                                                               static_cast<float*>(h->xs), o.nx, o.nr, o.nl, h->st));
+  return BTE_OK;
+}
+
+// z += H_i^-1 rho through the last factors of either harmonic path.
+bte_status harmonic_substitute(bte_handle* h, const double* E_dev, double Eu, const int* conv) {
+  const HostOps& o = h->ops;
+  const bte::MassBand mass{h->Mband, o.nr, o.mw};
+  if (!h->structured)
+    BTE_LAUNCH(BTE_K_LU_SOLVE, bte::launch_window_substitute(h->win, conv, o.nx, h->status, h->st));
+  else if (h->precision == BTE_FP64)
+    BTE_LAUNCH(BTE_K_LU_SOLVE, bte::launch_struct_substitute<double>(E_dev, Eu, o.dt, residual_ops(h), mass,
+                                                                     static_cast<double*>(h->xs), h->win.vec, conv,
+                                                                     o.nx, o.nr, o.nl, h->st));
+  else
+    BTE_LAUNCH(BTE_K_LU_SOLVE, bte::launch_struct_substitute<float>(E_dev, Eu, o.dt, residual_ops(h), mass,
+                                                                    static_cast<float*>(h->xs), h->win.vec, conv, o.nx,
+                                                                    o.nr, o.nl, h->st));
+  return BTE_OK;
+}
+
+// out_i = A_i^-1 in_i through the last factors of either harmonic path (windowed, block tridiagonal),
+// with up to `sweeps` refinement sweeps (conv tells afterwards which points converged; with 0 sweeps
+// nothing is checked).
+bte_status harmonic_solve(bte_handle* h, const double* in, double* out, const double* E_dev, double Eu, int sweeps) {
   const HostOps& o = h->ops;
   const bte::MassBand mass{h->Mband, o.nr, o.mw};
   const bte::ResidualOps ro = residual_ops(h);
   int* conv = sweeps > 0 ? h->conv : nullptr;
   BTE_LAUNCH(BTE_K_LU_SOLVE, bte::launch_window_project(h->win, in, mass, h->TS, conv, o.nx, o.nt, h->st));
-  BTE_LAUNCH(BTE_K_LU_SOLVE, bte::launch_window_substitute(h->win, conv, o.nx, h->status, h->st));
+  BTE_TRY(harmonic_substitute(h, E_dev, Eu, conv));
   for (int s = 0; s <= sweeps; ++s) {
     BTE_LAUNCH(BTE_K_RESIDUAL,
                bte::launch_window_residual(h->win, in, out, E_dev, Eu, o.dt, ro, mass, h->TO, h->ts_inf, h->to_inf,
                                            h->ratio, conv, h->tol, o.kc_inf, o.ka_inf, o.nx, o.nt, sweeps > 0,
                                            s == sweeps, h->status, h->st));
-    if (s < sweeps) BTE_LAUNCH(BTE_K_LU_SOLVE, bte::launch_window_substitute(h->win, conv, o.nx, h->status, h->st));
+    if (s < sweeps) BTE_TRY(harmonic_substitute(h, E_dev, Eu, conv));
   }
   return BTE_OK;
 }
@@ -220,23 +251,14 @@ bte_status window_solve(bte_handle* h, const double* in, double* out, const doub
 bte_status enqueue_vsolve(bte_handle* h, const double* in, double* out, const double* E_dev, double Eu,
                           bool factor) {
   const HostOps& o = h->ops;
-  const int nx = o.nx, nt = o.nt, nr = o.nr, nl = o.nl;
+  const int nx = o.nx;
   cudaStream_t st = h->st;
   const int n = h->nlu, nb = h->nb;
-  if (h->windowed) {
-    if (factor) BTE_TRY(window_factor(h, E_dev, Eu));
-    return window_solve(h, in, out, E_dev, Eu, 0);
+  if (h->windowed || h->structured) {
+    if (factor) BTE_TRY(h->structured ? struct_factor(h, E_dev, Eu) : window_factor(h, E_dev, Eu));
+    return harmonic_solve(h, in, out, E_dev, Eu, 0);
   }
-  if (h->structured) {
-    if (h->precision == BTE_FP64)
-      BTE_LAUNCH(BTE_K_LU_SOLVE, bte::launch_vsolve_struct<double>(in, out, E_dev, Eu, o.dt, h->Cs, h->Alo, h->Aup,
-                                                                   h->TO, h->TS, static_cast<double*>(h->xs), nx, nt,
-                                                                   nr, nl, nullptr, 0, h->status, st));
-    else
-      BTE_LAUNCH(BTE_K_LU_SOLVE, bte::launch_vsolve_struct<float>(in, out, E_dev, Eu, o.dt, h->Cs, h->Alo, h->Aup,
-                                                                  h->TO, h->TS, static_cast<float*>(h->xs), nx, nt,
-                                                                  nr, nl, nullptr, 0, h->status, st));
-  } else if (h->precision == BTE_FP64) {
+  if (h->precision == BTE_FP64) {
     double* fac = static_cast<double*>(h->fac);
     if (factor) {
       BTE_LAUNCH(BTE_K_V_FORM, form_v<double>(h, E_dev, Eu, fac));
@@ -322,8 +344,7 @@ bte_status enqueue_vsolve(bte_handle* h, const double* in, double* out, const do
         BTE_LAUNCH(BTE_K_LU_PANEL, bte::launch_lu_uinv<float>(fac, static_cast<float*>(h->uinv), nx, n, nb, st));
     }
   }
-  if (!h->structured) BTE_TRY(enqueue_lu_solve(h, in, out, nullptr, 0));
-  return BTE_OK;
+  return enqueue_lu_solve(h, in, out, nullptr, 0);
 }
 
 // Residual evaluations of the mixed path's FP64 escalation (the first follows the fresh FP64 solve,
@@ -353,9 +374,10 @@ bte_status enqueue_step(bte_handle* h, const double* F_in, double* F_out, const 
   // velocity step (eq. "bte_semi_implicit_vspace" / "vspace_batched_system"); a caller's field
   // array is checked like the state
   if (E_dev && !ni_dev) BTE_LAUNCH(BTE_K_OTHER, bte::launch_check_field(E_dev, nx, h->status, st));
-  if (h->windowed) {
-    BTE_TRY(window_factor(h, E_dev, Eu));
-    BTE_TRY(window_solve(h, h->Fa, h->Fb, E_dev, Eu, h->refine_max));
+  const bool harmonic = h->windowed || h->structured;
+  if (harmonic) {
+    BTE_TRY(h->structured ? struct_factor(h, E_dev, Eu) : window_factor(h, E_dev, Eu));
+    BTE_TRY(harmonic_solve(h, h->Fa, h->Fb, E_dev, Eu, h->refine_max));
   } else {
     const bte_status vs = enqueue_vsolve(h, h->Fa, h->Fb, E_dev, Eu, true);
     if (vs != BTE_OK) return vs;
@@ -363,22 +385,13 @@ bte_status enqueue_step(bte_handle* h, const double* F_in, double* F_out, const 
   // FP64 iterative refinement: residual through Algorithm 2, correction through the factors
   if (h->refine_max > 0) {
     const bte::ResidualOps ro = residual_ops(h);
-    if (!h->windowed) BTE_CUDA(h, cudaMemsetAsync(h->conv, 0, sizeof(int) * nx, st));
-    for (int s = 0; s <= h->refine_max && !h->windowed; ++s) {
+    if (!harmonic) BTE_CUDA(h, cudaMemsetAsync(h->conv, 0, sizeof(int) * nx, st));
+    for (int s = 0; s <= h->refine_max && !harmonic; ++s) {
       BTE_LAUNCH(BTE_K_RESIDUAL, bte::launch_residual(h->Fb, h->Fa, E_dev, Eu, o.dt, ro, h->TO, h->TS, h->R, h->ratio,
                                                       h->conv, h->tol, o.kc_inf, o.ka_inf, nx, nt, nr, nl, h->status,
                                                       st));
       if (s == h->refine_max) break;
-      if (h->structured && h->precision == BTE_FP64)
-        BTE_LAUNCH(BTE_K_LU_SOLVE, bte::launch_vsolve_struct<double>(h->R, h->Fb, E_dev, Eu, o.dt, h->Cs, h->Alo, h->Aup,
-                                                                     h->TO, h->TS, static_cast<double*>(h->xs), nx,
-                                                                     nt, nr, nl, h->conv, 1, nullptr, st));
-      else if (h->structured)
-        BTE_LAUNCH(BTE_K_LU_SOLVE, bte::launch_vsolve_struct<float>(h->R, h->Fb, E_dev, Eu, o.dt, h->Cs, h->Alo, h->Aup,
-                                                                    h->TO, h->TS, static_cast<float*>(h->xs), nx, nt,
-                                                                    nr, nl, h->conv, 1, nullptr, st));
-      else
-        BTE_TRY(enqueue_lu_solve(h, h->R, h->Fb, h->conv, 1));
+      BTE_TRY(enqueue_lu_solve(h, h->R, h->Fb, h->conv, 1));
     }
     if (h->xs64) {
       // points whose refinement with the FP32 factors has not converged (cond(A_i) * eps_32 near or
@@ -530,6 +543,24 @@ bte_status read_status(bte_handle* h, int steps = 1) {
   return BTE_OK;
 }
 
+// What the solves in the harmonic basis share: their vectors and the norms of the projections.
+bte_status alloc_harmonic(bte_handle* h) {
+  const HostOps& o = h->ops;
+  BTE_TRY(dalloc(h, &h->win.vec, static_cast<size_t>(o.nx) * 3 * o.nl * o.nr));
+  BTE_TRY(dalloc(h, &h->win.fmax_, o.nx));
+  for (int l = 0; l < o.nl; ++l) {
+    double s = 0.0;
+    for (int a = 0; a < o.nt; ++a) s += std::fabs(o.TS[static_cast<size_t>(l) * o.nt + a]);
+    h->ts_inf = std::max(h->ts_inf, s);
+  }
+  for (int a = 0; a < o.nt; ++a) {
+    double s = 0.0;
+    for (int l = 0; l < o.nl; ++l) s += std::fabs(o.TO[static_cast<size_t>(a) * o.nl + l]);
+    h->to_inf = std::max(h->to_inf, s);
+  }
+  return BTE_OK;
+}
+
 // Buffers of the windowed LU (U starts at zero: the rows of unused unknowns are never written).
 bte_status alloc_window(bte_handle* h) {
   bte::WindowBuffers& b = h->win;
@@ -542,24 +573,13 @@ bte_status alloc_window(bte_handle* h) {
   BTE_TRY(dalloc(h, &T, ts * nx * bte::window_t_count(w)));
   BTE_TRY(dalloc(h, &U, ts * nx * bte::window_u_count(w)));
   BTE_TRY(dalloc(h, &b.slotj, nx * bte::window_slot_count(w)));
-  BTE_TRY(dalloc(h, &b.vec, nx * 3 * o.nl * o.nr));
-  BTE_TRY(dalloc(h, &b.fmax_, nx));
+  BTE_TRY(alloc_harmonic(h));
   if (b.fp64) {
     BTE_TRY(dalloc(h, &b.W, nx * 128 * (w.NU + 32)));
     BTE_TRY(dalloc(h, &b.rows, nx * 128));
   }
   b.base = base, b.slope = slope, b.T = T, b.U = U;
   BTE_CUDA(h, cudaMemsetAsync(U, 0, ts * nx * bte::window_u_count(w), h->st));
-  for (int l = 0; l < o.nl; ++l) {
-    double s = 0.0;
-    for (int a = 0; a < o.nt; ++a) s += std::fabs(o.TS[static_cast<size_t>(l) * o.nt + a]);
-    h->ts_inf = std::max(h->ts_inf, s);
-  }
-  for (int a = 0; a < o.nt; ++a) {
-    double s = 0.0;
-    for (int l = 0; l < o.nl; ++l) s += std::fabs(o.TO[static_cast<size_t>(a) * o.nl + l]);
-    h->to_inf = std::max(h->to_inf, s);
-  }
   return BTE_OK;
 }
 
@@ -633,7 +653,7 @@ bte_status handle_enqueue_vsolve(bte_handle* h, const double* in, double* out, c
 }
 bte_status handle_window_factor(bte_handle* h, double Eu) { return window_factor(h, nullptr, Eu); }
 bte_status handle_window_solve(bte_handle* h, const double* in, double* out, double Eu) {
-  return window_solve(h, in, out, nullptr, Eu, h->refine_max);
+  return harmonic_solve(h, in, out, nullptr, Eu, h->refine_max);
 }
 bte_status handle_reset_status(bte_handle* h, cudaStream_t st) {
   BTE_CUDA(h, cudaMemsetAsync(h->status, 0, 2 * sizeof(unsigned), st));
@@ -740,7 +760,7 @@ bte_status bte_create(const bte_config* cfg, bte_handle** out) {
                             chk(dalloc(h, &h->KAg, static_cast<size_t>(o.nv) * o.nv)))) &&
               (!dense_r || (chk(dalloc(h, &h->Cg, blk)) && chk(dalloc(h, &h->Aglo, blk)) &&
                                chk(dalloc(h, &h->Agup, blk)))) &&
-              (h->structured || chk(dalloc(h, &h->Mband, o.Mband.size()))) &&
+              chk(dalloc(h, &h->Mband, o.Mband.size())) &&
               chk(dalloc(h, &h->rc0, static_cast<size_t>(o.nr) * o.nr)) &&
               chk(dalloc(h, &h->rband, static_cast<size_t>(o.nr) * (2 * o.mw + 1))) &&
               chk(dalloc(h, &h->rfband, static_cast<size_t>(2) * o.nl * o.nr * (2 * o.mw + 1))) &&
@@ -759,13 +779,15 @@ bte_status bte_create(const bte_config* cfg, bte_handle** out) {
               chk(dalloc(h, &h->conv, o.nx)) && chk(dalloc(h, &h->status, 2));
     if (ok && h->structured) {
       const size_t xsz = static_cast<size_t>(o.nx) * o.nl * o.nr * o.nr;
-      if (h->precision == BTE_FP64) {
+      const size_t ssz = static_cast<size_t>(o.nx) * o.nl * bte::struct_stride(o.nr);
+      ok = chk(alloc_harmonic(h));
+      if (ok && h->precision == BTE_FP64) {
         double* x = nullptr;
-        ok = chk(dalloc(h, &x, xsz));
+        ok = chk(dalloc(h, &x, ssz));
         h->xs = x;
       } else {
         float* x = nullptr;
-        ok = chk(dalloc(h, &x, xsz));
+        ok = ok && chk(dalloc(h, &x, ssz));
         h->xs = x;
         if (ok && bte::struct_smem_bytes(o.nr, o.nl, sizeof(double)) <= 200 * 1024)
           ok = chk(dalloc(h, &h->xs64, xsz));
@@ -810,7 +832,7 @@ bte_status bte_create(const bte_config* cfg, bte_handle** out) {
     }
     if (ok) ok = chk(upload(h, h->U, o.U)) && chk(upload(h, h->Uinv, o.Uinv)) && chk(upload(h, h->Q, o.Q)) &&
                  chk(upload(h, h->TO, o.TO)) && chk(upload(h, h->TS, o.TS)) &&
-                 (!h->Mband || chk(upload(h, h->Mband, o.Mband)));
+                 chk(upload(h, h->Mband, o.Mband));
     if (ok) {
       cudaError_t ce = cudaMemsetAsync(h->status, 0, 2 * sizeof(unsigned), h->st);
       if (ce == cudaSuccess) ce = cudaStreamSynchronize(h->st);

@@ -24,6 +24,19 @@ struct MassBand {
   int w = 0;
 };
 
+// The operators of the FP64 refinement residual, all before the mass scaling: C_0 dense ([nr][nr]);
+// the band ([nr][2 w + 1], band[p][k - p + w]) of the loss part of C (the whole C_l for l >= 1);
+// the bands of the field blocks (A_v)_{q,q-1} and (A_v)_{q,q+1} ([2][nl][nr][2 w + 1], zero where
+// a block does not exist); the band of the Cholesky factor R of M_v ([nr][w + 1],
+// chol[p][j] = R[p][p - w + j]) and 1 / R[p][p].
+struct ResidualOps {
+  const double* c0 = nullptr;
+  const double* band = nullptr;
+  const double* fband = nullptr;
+  const double* chol = nullptr;
+  const double* cinv = nullptr;
+  int w = 0;
+};
 // tensor-core (tcgen05) trailing updates of the FP32 LU; workspace of tc_workspace_bytes(), parts
 // 0-1 L21 split, 2-3 (P A12)^T split, 4-5 one panel's inv(L11) split, 6-7 U12^T split, 8-9 a
 // two-panel block's inv(L11) split (layout in bte_tc.cu)
@@ -112,7 +125,18 @@ template <typename T>
 void launch_lu_solve_blocked(const T* fac, const int* perm, const T* linv, const T* uinv, const double* b,
                              double* x, int nx, int n, int nb, const int* conv, int accumulate, cudaStream_t st,
                              MassBand mass = {});
-// ---- structure-exploiting velocity solve (block tridiagonal in l): Fout = A_i^-1 Fin per point
+// ---- structure-exploiting velocity solve (block tridiagonal in l), nr <= 64. struct_factor: the
+// inverses S_l^-1 of the block elimination, nl blocks of struct_stride(nr) values a point; substitute:
+// z += H^-1 rho on the vectors of WindowBuffers (points with conv[i] != 0 skipped, conv NULL: none).
+size_t struct_stride(int nr);
+template <typename T>
+cudaError_t launch_struct_factor(const double* E, double E_uniform, double dt, const ResidualOps& ro, MassBand mass,
+                                 T* S, int nx, int nr, int nl, cudaStream_t st);
+template <typename T>
+cudaError_t launch_struct_substitute(const double* E, double E_uniform, double dt, const ResidualOps& ro, MassBand mass,
+                                     const T* S, double* vec, const int* conv, int nx, int nr, int nl,
+                                     cudaStream_t st);
+// The mixed paths' FP64 escalation, factors and solve in one launch: Fout = A_i^-1 Fin per point
 // (Fout += when accumulate); T is the arithmetic of the block elimination; Xscratch holds
 // nx * nl * nr * nr values of T.
 size_t struct_smem_bytes(int nr, int nl, size_t tsize);
@@ -152,19 +176,6 @@ template <typename T>
 void launch_lu_solve(const T* fac, const int* piv, const double* b, double* x, int nx, int n, int nb,
                      const int* conv, int accumulate, cudaStream_t st, MassBand mass = {});
 
-// The operators of the FP64 refinement residual, all before the mass scaling: C_0 dense ([nr][nr]);
-// the band ([nr][2 w + 1], band[p][k - p + w]) of the loss part of C (the whole C_l for l >= 1);
-// the bands of the field blocks (A_v)_{q,q-1} and (A_v)_{q,q+1} ([2][nl][nr][2 w + 1], zero where
-// a block does not exist); the band of the Cholesky factor R of M_v ([nr][w + 1],
-// chol[p][j] = R[p][p - w + j]) and 1 / R[p][p].
-struct ResidualOps {
-  const double* c0 = nullptr;
-  const double* band = nullptr;
-  const double* fband = nullptr;
-  const double* chol = nullptr;
-  const double* cinv = nullptr;
-  int w = 0;
-};
 // FP64 residual r = b - (x - dt P_O M_v^-1 (C + E_i A_v) P_S x) (Algorithm 2's structured
 // evaluation: the products with C and A_v are banded except C_0, and M_v^-1 is applied by banded
 // Cholesky substitution), per-point ratio max|r|/max|b|; marks conv[i] = 1 when ratio <= tol or the

@@ -3,22 +3,24 @@
 // eqs. "proj_ops", "bte_1d_discrete"), where C is block diagonal in l and A_v block tridiagonal
 // (couplings l -> l +- 1 only, Section 3.3). Because P_S P_O = T_S T_O = I,
 //     A_i^-1 f = f + P_O ( (I - dt B_i)^-1 - I ) P_S f,
-// so one dense Nv x Nv solve becomes one block-tridiagonal solve of N_l blocks of Nr x Nr:
-// y = P_S f; block elimination over l (S_0 = D_0, S_q = D_q - L_q S_{q-1}^-1 U_{q-1}, blocks
-// D_q = I - dt Cs_q, L_q = -dt E As_lo[q], U_q = -dt E As_up[q]); back substitution; f* = f + P_O (z - y).
-// The blocks are inverted by Gauss-Jordan without pivoting: S_q stays diagonally dominant enough
-// (in-block growth 1.0 and pivots >= 0.2 on the workloads' field range), and the FP64 refinement
-// that follows (Algorithm 2 residual) removes what rounding leaves.
+// so one dense Nv x Nv solve becomes one block-tridiagonal solve of N_l blocks of Nr x Nr.
 //
-// One CTA of 256 threads per point, a 16 x 16 thread grid over the Nr x Nr blocks (Nr <= 64):
-// thread (ty, tx) owns the elements (ty + 16 a, tx + 16 b), a, b < 4, of the block being inverted and
-// keeps them in registers for the whole Gauss-Jordan sweep; only the pivot row and column go
-// through shared memory. Inverses are stored transposed, couplings transposed where they are the
-// left factor, so every shared-memory read is a broadcast or conflict-free. The X_q of the
-// forward sweep go to a per-point global scratch for the back substitution.
+// BTE_FLAG_STRUCTURED (struct_factor_kernel, struct_substitute_kernel): the system multiplied by the
+// mass matrix, H_i = (I (x) M_v)(I - dt B_i), whose blocks are banded but for the gain in the block
+// (0, 0). It is eliminated from the highest harmonic down, S_l = D_l - U_l S_{l+1}^-1 L_{l+1} with
+// D_l = M_v - dt C_l, L_l = -dt E (A_v)_{l,l-1}, U_l = -dt E (A_v)_{l,l+1}: A_v is skew-symmetric and
+// M_v - dt C_l symmetric positive definite for l >= 1, so every S_l, l >= 1, is D_l plus a positive
+// semidefinite matrix and its inversion needs no pivoting; S_0 comes last. The products with L and U
+// cost 7 operations an element. The inverses are kept for the refinement's solves.
+//
+// The mixed paths' escalation (vsolve_struct_kernel, FP64): the mass-scaled blocks, eliminated upwards
+// and solved in one launch for the points whose refinement has not converged.
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "bte_kernels.h"
+#include "bte_recip.cuh"
 
 namespace bte {
 namespace {
@@ -226,6 +228,195 @@ __global__ void __launch_bounds__(kST) vsolve_struct_kernel(const double* __rest
   if (bad && status) atomicOr(status, kNonFinite);
 }
 
+// S_l^-1 of every harmonic of one point (CTA), l = nl - 1 .. 0, into Sg[pt][l] (row-major, stride
+// `stride` values). A 16 x 16 thread grid holds the block being inverted in registers, thread
+// (ty, tx) the elements (ty + 16 a, tx + 16 b); the Gauss-Jordan step k reads the pivot row, column
+// and reciprocal that their owners posted in step k - 1: one barrier a step. In FP64 the units'
+// rate bounds it (a step is 16 FMAs and 4 products a thread; the reciprocal is the owner's alone),
+// in FP32 the latency of the nl nr dependent steps.
+template <typename T>
+__global__ void __launch_bounds__(kST) struct_factor_kernel(const double* __restrict__ E, double E_uniform, double dt,
+                                                            ResidualOps ro, MassBand mass, T* __restrict__ Sg,
+                                                            size_t stride, int n, int nl) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const int w = mass.w, bw = 2 * w + 1, nn = n * n;
+  const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
+  T* Sinv = reinterpret_cast<T*>(smraw);  // [n][n]
+  T* Y = Sinv + nn;                       // [n][n]
+  T* Lb = Y + nn;                         // [n][bw], dt E (A_v)_{l+1,l}
+  T* Ub = Lb + n * bw;                    // [n][bw], dt E (A_v)_{l,l+1}
+  T* prow2 = Ub + n * bw;                 // 2 x 64 pivot rows
+  T* pcol2 = prow2 + 128;                 // 2 x 64 pivot columns
+  __shared__ T pinv2[2];
+  const int pt = blockIdx.x;
+  const double dtE = dt * (E ? E[pt] : E_uniform);
+  T* out = Sg + static_cast<size_t>(pt) * nl * stride;
+  for (int l = nl - 1; l >= 0; --l) {
+    T s[kG][kG];
+#pragma unroll
+    for (int a = 0; a < kG; ++a)
+#pragma unroll
+      for (int b = 0; b < kG; ++b) {
+        const int i = ty + 16 * a, j = tx + 16 * b, d = j - i + w;
+        double v = i == j ? 1.0 : 0.0;  // past the block: the identity
+        if (i < n && j < n) {
+          const bool in = d >= 0 && d < bw;
+          v = in ? __ldg(mass.m + i * bw + d) : 0.0;
+          if (l == 0) v -= dt * __ldg(ro.c0 + i * n + j);
+          else if (in) v -= dt * __ldg(ro.band + i * bw + d);
+        }
+        s[a][b] = static_cast<T>(v);
+      }
+    if (l + 1 < nl) {
+      for (int e = threadIdx.x; e < n * bw; e += kST) {
+        Lb[e] = static_cast<T>(dtE * __ldg(ro.fband + static_cast<size_t>(l + 1) * n * bw + e));
+        Ub[e] = static_cast<T>(dtE * __ldg(ro.fband + static_cast<size_t>(nl + l) * n * bw + e));
+      }
+      __syncthreads();
+      for (int e = threadIdx.x; e < nn; e += kST) {  // Y = S_{l+1}^-1 L_{l+1} (up to sign)
+        const int i = e / n, j = e % n;
+        T acc = T(0);
+        for (int t = -w; t <= w; ++t)
+          if (j + t >= 0 && j + t < n) acc = fma(Sinv[i * n + j + t], Lb[(j + t) * bw + w - t], acc);
+        Y[e] = acc;
+      }
+      __syncthreads();
+#pragma unroll
+      for (int a = 0; a < kG; ++a) {
+        const int i = ty + 16 * a;
+        if (i >= n) break;
+        for (int t = -w; t <= w; ++t) {
+          if (i + t < 0 || i + t >= n) continue;
+          const T u = Ub[i * bw + w + t];
+#pragma unroll
+          for (int b = 0; b < kG; ++b) {
+            const int j = tx + 16 * b;
+            if (j < n) s[a][b] = fma(-u, Y[(i + t) * n + j], s[a][b]);
+          }
+        }
+      }
+    }
+    // in-place inverse; the identity beyond n needs no steps. Steps kb, 16 + kb, .. by blocks of 16, so
+    // that the pivot's register index is known
+    auto post = [&](int o, auto q, int buf) {  // row and column 16 q + o, and the reciprocal of the pivot
+      constexpr int Q = decltype(q)::value;
+      if (ty == o)
+#pragma unroll
+        for (int b = 0; b < kG; ++b) prow2[64 * buf + tx + 16 * b] = s[Q][b];
+      if (tx == o) {
+#pragma unroll
+        for (int a = 0; a < kG; ++a) pcol2[64 * buf + ty + 16 * a] = s[a][Q];
+        if (ty == o) pinv2[buf] = recip(s[Q][Q]);
+      }
+    };
+    auto sweep = [&](auto q) {
+      constexpr int Q = decltype(q)::value;
+      const int kn = min(16, n - 16 * Q);
+#pragma unroll 1
+      for (int o = 0; o < kn; ++o) {
+        const int c = o & 1;
+        const T p = pinv2[c];
+        T pr[kG], fc[kG];
+#pragma unroll
+        for (int u = 0; u < kG; ++u) {
+          pr[u] = prow2[64 * c + tx + 16 * u];
+          fc[u] = pcol2[64 * c + ty + 16 * u] * p;
+        }
+#pragma unroll
+        for (int a = 0; a < kG; ++a)
+#pragma unroll
+          for (int b = 0; b < kG; ++b) s[a][b] = fma(-fc[a], pr[b], s[a][b]);
+        if (tx == o)
+#pragma unroll
+          for (int a = 0; a < kG; ++a) s[a][Q] = -fc[a];
+        if (ty == o)  // the pivot row: scaled instead
+#pragma unroll
+          for (int b = 0; b < kG; ++b) s[Q][b] = b == Q && tx == o ? p : pr[b] * p;
+        if (o + 1 < kn) post(o + 1, q, c ^ 1);
+        else if (Q + 1 < kG && kn == 16 && 16 * (Q + 1) < n) post(0, std::integral_constant<int, (Q + 1) % kG>{}, 0);
+        __syncthreads();
+      }
+    };
+    post(0, std::integral_constant<int, 0>{}, 0);
+    __syncthreads();
+    sweep(std::integral_constant<int, 0>{});
+    sweep(std::integral_constant<int, 1>{});
+    sweep(std::integral_constant<int, 2>{});
+    sweep(std::integral_constant<int, 3>{});
+    T* o = out + static_cast<size_t>(l) * stride;
+#pragma unroll
+    for (int a = 0; a < kG; ++a)
+#pragma unroll
+      for (int b = 0; b < kG; ++b) {
+        const int i = ty + 16 * a, j = tx + 16 * b;
+        if (i < n && j < n) Sinv[i * n + j] = s[a][b], o[i * n + j] = s[a][b];
+      }
+    __syncthreads();
+  }
+}
+
+// z += H^-1 rho (vectors [nx][3 nl n]: y, z, rho) through the inverses: downwards g_l = S_l^-1 r_l with
+// r_l = rho_l - U_l g_{l+1}, then upwards z_l = g_l - S_l^-1 L_l z_{l-1}. Four lanes a row; the next
+// block's row is loaded while this one is used. Converged points return at once.
+template <typename T>
+__global__ void __launch_bounds__(kST) struct_substitute_kernel(const double* __restrict__ E, double E_uniform,
+                                                                double dt, ResidualOps ro, MassBand mass,
+                                                                const T* __restrict__ Sg, size_t stride,
+                                                                double* __restrict__ vec, const int* conv, int n,
+                                                                int nl) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const int pt = blockIdx.x, tid = threadIdx.x;
+  if (conv && conv[pt]) return;
+  const int w = mass.w, bw = 2 * w + 1, m = nl * n;
+  T* g = reinterpret_cast<T*>(smraw);  // [nl][n]
+  T* r = g + m;                        // [64]
+  double* z = vec + static_cast<size_t>(pt) * 3 * m + m;
+  const double* rho = z + m;
+  const T* S = Sg + static_cast<size_t>(pt) * nl * stride;
+  const T dtE = static_cast<T>(dt * (E ? E[pt] : E_uniform));
+  const int row = tid >> 2, sub = tid & 3;  // 64 rows, lanes take columns sub + 4 c
+  T buf[16];
+  auto load = [&](int l) {
+#pragma unroll
+    for (int c = 0; c < 16; ++c) {
+      const int j = sub + 4 * c;
+      buf[c] = row < n && j < n ? S[static_cast<size_t>(l) * stride + row * n + j] : T(0);
+    }
+  };
+  load(nl - 1);
+  for (int i = tid; i < 64; i += kST) r[i] = i < n ? static_cast<T>(rho[(nl - 1) * n + i]) : T(0);
+  __syncthreads();
+  for (int step = 0; step < 2 * nl - 1; ++step) {
+    const bool down = step < nl;
+    const int l = down ? nl - 1 - step : step - nl + 1;
+    T acc = T(0);
+#pragma unroll
+    for (int c = 0; c < 16; ++c) acc = fma(buf[c], r[sub + 4 * c], acc);
+    if (step + 1 < 2 * nl - 1) load(step + 1 < nl ? nl - 2 - step : step + 2 - nl);
+    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+    acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+    if (sub == 0 && row < n) g[l * n + row] = down ? acc : g[l * n + row] + acc;
+    __syncthreads();
+    // the next vector: rho_{l-1} + dt E Aup_{l-1} g_l downwards, dt E Alo_{l+1} z_l upwards
+    const int ln = down ? l - 1 : l + 1;
+    const bool turn = down && l == 0;  // z_0 = g_0: the way up starts with harmonic 1
+    const int src = l, dst = turn ? 1 : ln;
+    if (dst >= 0 && dst < nl && tid < 64) {
+      T v = T(0);
+      if (tid < n) {
+        const bool up = !down || turn;
+        const double* fr = ro.fband + (static_cast<size_t>(up ? dst : nl + dst) * n + tid) * bw + w - tid;
+        for (int k = max(0, tid - w); k <= min(n - 1, tid + w); ++k) v = fma(static_cast<T>(__ldg(fr + k)), g[src * n + k], v);
+        v *= dtE;
+        if (!up) v += static_cast<T>(rho[dst * n + tid]);
+      }
+      r[tid] = v;
+    }
+    __syncthreads();
+  }
+  for (int i = tid; i < m; i += kST) z[i] += static_cast<double>(g[i]);
+}
+
 // ---- the reduced dense system (N_l < N_theta): the same identity with I - dt B_i factored as a
 // dense m x m matrix, m = N_l Nr, by the LU kernels of the full system, in its unscaled form
 // (I (x) M_v)(I - dt B_i) (LU with partial pivoting on the mass-scaled form meets large element
@@ -335,11 +526,40 @@ void launch_vsolve_struct(const double* Fin, double* Fout, const double* E, doub
                                                  conv, accumulate, status);
 }
 
-template void launch_vsolve_struct<float>(const double*, double*, const double*, double, double, const double*,
-                                          const double*, const double*, const double*, const double*, float*, int, int,
-                                          int, int, const int*, int, unsigned*, cudaStream_t);
 template void launch_vsolve_struct<double>(const double*, double*, const double*, double, double, const double*,
                                            const double*, const double*, const double*, const double*, double*, int,
                                            int, int, int, const int*, int, unsigned*, cudaStream_t);
+
+size_t struct_stride(int nr) { return (static_cast<size_t>(nr) * nr + 3) / 4 * 4; }
+
+template <typename T>
+cudaError_t launch_struct_factor(const double* E, double E_uniform, double dt, const ResidualOps& ro, MassBand mass,
+                                 T* S, int nx, int nr, int nl, cudaStream_t st) {
+  const int smem = static_cast<int>(sizeof(T)) * (2 * nr * nr + 2 * nr * (2 * mass.w + 1) + 4 * 64);
+  const cudaError_t e = cudaFuncSetAttribute(struct_factor_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  struct_factor_kernel<T><<<nx, kST, smem, st>>>(E, E_uniform, dt, ro, mass, S, struct_stride(nr), nr, nl);
+  return cudaGetLastError();
+}
+template cudaError_t launch_struct_factor<float>(const double*, double, double, const ResidualOps&, MassBand, float*,
+                                                 int, int, int, cudaStream_t);
+template cudaError_t launch_struct_factor<double>(const double*, double, double, const ResidualOps&, MassBand, double*,
+                                                  int, int, int, cudaStream_t);
+
+template <typename T>
+cudaError_t launch_struct_substitute(const double* E, double E_uniform, double dt, const ResidualOps& ro, MassBand mass,
+                                     const T* S, double* vec, const int* conv, int nx, int nr, int nl,
+                                     cudaStream_t st) {
+  const int smem = static_cast<int>(sizeof(T)) * (nl * nr + 64);
+  const cudaError_t e =
+      cudaFuncSetAttribute(struct_substitute_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  struct_substitute_kernel<T><<<nx, kST, smem, st>>>(E, E_uniform, dt, ro, mass, S, struct_stride(nr), vec, conv, nr, nl);
+  return cudaGetLastError();
+}
+template cudaError_t launch_struct_substitute<float>(const double*, double, double, const ResidualOps&, MassBand,
+                                                     const float*, double*, const int*, int, int, int, cudaStream_t);
+template cudaError_t launch_struct_substitute<double>(const double*, double, double, const ResidualOps&, MassBand,
+                                                      const double*, double*, const int*, int, int, int, cudaStream_t);
 
 }  // namespace bte

@@ -35,6 +35,7 @@
 
 #include "bte_handle.h"
 #include "bte_kernels.h"
+#include "bte_recip.cuh"
 #include "bte_tf32.cuh"
 
 namespace bte {
@@ -184,22 +185,6 @@ __device__ __forceinline__ void store32(float* dst, const float (&v)[32]) {
 #pragma unroll
   for (int q = 0; q < 8; ++q)
     reinterpret_cast<float4*>(dst)[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-}
-
-// 1 / p to FP32 rounding: the hardware's approximation and one Newton-Raphson step (the IEEE division
-// is a call with special cases, about 250 cycles in the panel's chain)
-__device__ __forceinline__ float recip(float p) {
-  float r;
-  asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(p));
-  return fmaf(r, fmaf(-p, r, 1.f), r);
-}
-
-// The same in FP64, with two steps (the approximation has about 20 bits).
-__device__ __forceinline__ double recip(double p) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(p));
-  r = fma(r, fma(-p, r, 1.0), r);
-  return fma(r, fma(-p, r, 1.0), r);
 }
 
 struct FactorArgs {
@@ -1380,8 +1365,8 @@ int round_up(int a, int b) { return (a + b - 1) / b * b; }
 
 WindowPlan window_plan(int nr, int nl) {
   WindowPlan w;
-  if (nl < 1 || nl > 32) return w;
   w.nr = nr, w.nl = nl;
+  if (nl < 1 || nl > 32) return w;
   w.nlp = 1;
   while (w.nlp < nl) w.nlp *= 2;
   w.g = kPW / w.nlp;
