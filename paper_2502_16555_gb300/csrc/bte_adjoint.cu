@@ -85,21 +85,17 @@ bte_status dalloc(bte_handle* h, T** p, size_t count) {
 bte_status ensure_transposed(bte_handle* h) {
   if (h->Qt) return BTE_OK;
   const bte::HostOps& o = h->ops;
-  const int nr = o.nr, nx = o.nx;
-  std::vector<double> ut(nr * nr), uit(nr * nr), qt(o.Q.size());
+  const int nr = o.nr;
+  std::vector<double> ut(nr * nr), uit(nr * nr);
   for (int i = 0; i < nr; ++i)
     for (int k = 0; k < nr; ++k) ut[i * nr + k] = o.U[k * nr + i], uit[i * nr + k] = o.Uinv[k * nr + i];
-  const size_t blocks = static_cast<size_t>(o.nt) * nr;
-  for (size_t bk = 0; bk < blocks; ++bk)
-    for (int r = 0; r < nx; ++r)
-      for (int c = 0; c < nx; ++c) qt[bk * nx * nx + static_cast<size_t>(r) * nx + c] = o.Q[bk * nx * nx + static_cast<size_t>(c) * nx + r];
   bte_status s;
   if ((s = dalloc(h, &h->Ut, ut.size())) != BTE_OK || (s = dalloc(h, &h->Uinvt, uit.size())) != BTE_OK ||
-      (s = dalloc(h, &h->Qt, qt.size())) != BTE_OK)
+      (s = dalloc(h, &h->Qt, o.Q.size())) != BTE_OK)
     return s;
   BA_CUDA(h, cudaMemcpy(h->Ut, ut.data(), sizeof(double) * ut.size(), cudaMemcpyHostToDevice));
   BA_CUDA(h, cudaMemcpy(h->Uinvt, uit.data(), sizeof(double) * uit.size(), cudaMemcpyHostToDevice));
-  BA_CUDA(h, cudaMemcpy(h->Qt, qt.data(), sizeof(double) * qt.size(), cudaMemcpyHostToDevice));
+  BA_CUDA(h, cudaMemcpy(h->Qt, o.Q.data(), sizeof(double) * o.Q.size(), cudaMemcpyHostToDevice));
   return BTE_OK;
 }
 

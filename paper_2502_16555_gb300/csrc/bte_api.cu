@@ -665,6 +665,7 @@ bool handle_profiling(const bte_handle* h) { return h->prof; }
 unsigned long long handle_launches(const bte_handle* h) { return h->launches; }
 void handle_add_launches(bte_handle* h, unsigned long long n) { h->launches += n; }
 bool handle_has_tc(const bte_handle* h) { return h->have_tc; }
+ResidualOps handle_residual_ops(const bte_handle* h) { return residual_ops(h); }
 bool handle_windowed(const bte_handle* h) { return h->windowed; }
 void handle_set_variant(bte_handle* h, const Variant& v) {
   release_run_graph(h);
@@ -834,6 +835,7 @@ bte_status bte_create(const bte_config* cfg, bte_handle** out) {
                  chk(upload(h, h->TO, o.TO)) && chk(upload(h, h->TS, o.TS)) &&
                  chk(upload(h, h->Mband, o.Mband));
     if (ok) {
+      bte::launch_transpose_blocks(h->Q, o.nx, static_cast<size_t>(o.nt) * o.nr, h->st);
       cudaError_t ce = cudaMemsetAsync(h->status, 0, 2 * sizeof(unsigned), h->st);
       if (ce == cudaSuccess) ce = cudaStreamSynchronize(h->st);
       if (ce != cudaSuccess) ok = false, s = cuda_fail(h, ce, "initialising device buffers");

@@ -41,7 +41,7 @@ struct bte_handle {
   std::vector<void*> allocs;
 
   // x-step operators
-  double *U = nullptr, *Uinv = nullptr, *Q = nullptr;
+  double *U = nullptr, *Uinv = nullptr, *Q = nullptr;  // Q: the blocks transposed (launch_x_matvec)
   // velocity operators: KCg, KAg = P_O C P_S, P_O A_v P_S (Nv x Nv, before the mass scaling; the
   // dense form only), Cs, Alo, Aup the mass-scaled harmonic blocks (residual, structured solve),
   // Cg, Aglo, Agup the same blocks before the mass scaling (reduced form only), Mband the band of M
@@ -62,12 +62,13 @@ struct bte_handle {
   unsigned* status = nullptr;
   unsigned* status_host = nullptr;  // pinned
   std::vector<bte::Process> procs;  // the cross sections of the last bte_set_cross_sections
-  // transposed x-step operators for the adjoint (allocated on its first use)
+  // x-step operators of the adjoint (allocated on its first use): U^T, U^-T, and Q_ij by rows, which are
+  // the transposes of its Q_ij^T
   double *Ut = nullptr, *Uinvt = nullptr, *Qt = nullptr;
   // self-consistent field, ions and the fully-implicit step (allocated on their first use)
   bool hybrid = false;
   double n0_mu_i = 4.65e21, n0_D_i = 2.07e20;   // n0 times ion mobility and diffusion
-  double *Lop = nullptr, *E1 = nullptr, *Dxd = nullptr, *mud = nullptr, *lamd = nullptr, *rion = nullptr;
+  double *Lop = nullptr, *E1 = nullptr, *Dxd = nullptr, *DxT = nullptr, *D2 = nullptr, *mud = nullptr, *lamd = nullptr, *rion = nullptr;
   double *Esc = nullptr, *Ek = nullptr, *ned = nullptr, *ionA = nullptr, *ionb = nullptr;
   int gm = 0;                                   // GMRES basis size allocated
   double *Fk = nullptr, *Fn = nullptr, *Rv = nullptr, *Zx = nullptr, *VX = nullptr, *KAF = nullptr;

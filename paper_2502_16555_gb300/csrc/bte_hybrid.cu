@@ -25,11 +25,17 @@
 
 #include "bte_handle.h"
 #include "bte_kernels.h"
+#include "bte_mass.cuh"
+#include "bte_recip.cuh"
 
 namespace {
 
 constexpr int kDotBlock = 256;   // threads of the reduction kernels
-constexpr int kDotGrid = 304;    // blocks of the partial dot products (2 per SM)
+constexpr int kDotGrid = 152;    // blocks of the partial dot products (at most; one per SM)
+// blocks for n elements: at least four elements a thread
+int dot_grid(size_t n) {
+  return static_cast<int>(std::max<size_t>(1, std::min<size_t>(kDotGrid, n / (4 * kDotBlock))));
+}
 
 __device__ __forceinline__ double block_sum(double v, double* red) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -70,7 +76,19 @@ __global__ void field_kernel(const double* __restrict__ Lop, const double* __res
 // The ion system of eq. "fluid_step", row i per CTA: A = I/dt + D_x diag(mu E) - d D_x D_x,
 // b = ni/dt + src; the wall rows are the flux conditions J(0) = n max(0, -mu E(0)) and
 // J(L) = -n max(0, mu E(L)) with J = mu E n - d D_x n (right-hand side 0).
-__global__ void ion_assemble_kernel(const double* __restrict__ Dx, const double* __restrict__ E,
+// D2 = D_x D_x, once per handle (row i per CTA).
+__global__ void square_kernel(const double* __restrict__ Dx, int nx, double* __restrict__ D2) {
+  const int i = blockIdx.x;
+  const double* di = Dx + static_cast<size_t>(i) * nx;
+  for (int j = threadIdx.x; j < nx; j += blockDim.x) {
+    double dd = 0.0;
+    for (int k = 0; k < nx; ++k) dd = fma(di[k], Dx[static_cast<size_t>(k) * nx + j], dd);
+    D2[static_cast<size_t>(i) * nx + j] = dd;
+  }
+}
+
+__global__ void ion_assemble_kernel(const double* __restrict__ Dx, const double* __restrict__ D2,
+                                    const double* __restrict__ E,
                                     const double* __restrict__ ni, const double* __restrict__ src, double mu,
                                     double d, double dt, int nx, double* __restrict__ A, double* __restrict__ b) {
   const int i = blockIdx.x;
@@ -83,9 +101,7 @@ __global__ void ion_assemble_kernel(const double* __restrict__ Dx, const double*
       v = -d * di[j] + (i == j ? mu * E[i] : 0.0);
       if (i == j) v += i == 0 ? -fmax(0.0, -mu * E[i]) : fmax(0.0, mu * E[i]);
     } else {
-      double dd = 0.0;  // (D_x D_x)[i][j]
-      for (int k = 0; k < nx; ++k) dd = fma(di[k], Dx[static_cast<size_t>(k) * nx + j], dd);
-      v = di[j] * mu * E[j] - d * dd + (i == j ? 1.0 / dt : 0.0);
+      v = di[j] * mu * E[j] - d * D2[static_cast<size_t>(i) * nx + j] + (i == j ? 1.0 / dt : 0.0);
     }
     a[j] = v;
   }
@@ -109,172 +125,164 @@ __global__ void ion_assemble_kernel(const double* __restrict__ Dx, const double*
   }
 }
 
-// x = A^-1 b by Gaussian elimination with partial pivoting, one CTA, A and b in global memory
-// (overwritten). A zero or non-finite pivot sets kZeroPivot in status.
-__global__ void dense_solve_kernel(double* __restrict__ A, double* __restrict__ b, int n, double* __restrict__ x,
-                                   unsigned* status) {
-  __shared__ double rv[32];
-  __shared__ int ri[32];
-  __shared__ int piv;
-  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
-  for (int k = 0; k < n; ++k) {
-    double best = -1.0;
-    int bi = k;
-    for (int i = k + tid; i < n; i += nt) {
-      const double v = fabs(A[static_cast<size_t>(i) * n + k]);
-      if (v > best) best = v, bi = i;
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      const double ov = __shfl_xor_sync(0xffffffffu, best, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (ov > best || (ov == best && oi < bi)) best = ov, bi = oi;
-    }
-    if (lane == 0) rv[warp] = best, ri[warp] = bi;
-    __syncthreads();
-    if (tid == 0) {
-      for (int w = 1; w < nt / 32; ++w)
-        if (rv[w] > rv[0] || (rv[w] == rv[0] && ri[w] < ri[0])) rv[0] = rv[w], ri[0] = ri[w];
-      piv = ri[0];
-      if (!(rv[0] > 0.0) || !isfinite(rv[0])) atomicOr(status, bte::kZeroPivot);
-    }
-    __syncthreads();
-    const int p = piv;
-    if (p != k) {
-      for (int j = tid; j < n; j += nt) {
-        const double t = A[static_cast<size_t>(k) * n + j];
-        A[static_cast<size_t>(k) * n + j] = A[static_cast<size_t>(p) * n + j];
-        A[static_cast<size_t>(p) * n + j] = t;
-      }
-      if (tid == 0) {
-        const double t = b[k];
-        b[k] = b[p];
-        b[p] = t;
-      }
-    }
-    __syncthreads();
-    const double inv = 1.0 / A[static_cast<size_t>(k) * n + k];
-    // rows below the pivot: a warp per row, lanes over the columns (lane 0 also takes b)
-    for (int i = k + 1 + warp; i < n; i += nt >> 5) {
-      const double l = A[static_cast<size_t>(i) * n + k] * inv;
-      for (int j = k + 1 + lane; j < n; j += 32) A[static_cast<size_t>(i) * n + j] -= l * A[static_cast<size_t>(k) * n + j];
-      if (lane == 0) b[i] -= l * b[k];
-    }
-    __syncthreads();
-  }
-  __shared__ double red[32];
-  for (int i = n - 1; i >= 0; --i) {
-    double s = 0.0;
-    for (int j = i + 1 + tid; j < n; j += nt) s = fma(A[static_cast<size_t>(i) * n + j], x[j], s);
-    s = block_sum(s, red);
-    if (tid == 0) x[i] = (b[i] - s) / A[static_cast<size_t>(i) * n + i];
-    __syncthreads();
-  }
-}
-
-// The same elimination with A and b staged in shared memory (n <= kSmemSolve): one CTA, the
-// pivot column scanned by warp 0, rows exchanged and updated in shared memory.
+// x = A^-1 b by Gaussian elimination with partial pivoting, one CTA. A ([n][ld], column n holds b) is
+// in shared memory for n <= kSmemSolve, in global memory above (overwritten). Rows are marked, not
+// exchanged: every warp finds the pivot of a column for itself (the magnitudes as ordered integers, so
+// that the FP64 units, whose rate bounds the kernel, do products only) and takes the rows i = warp,
+// warp + nw, ..; one barrier a column. A zero or non-finite pivot sets kZeroPivot in status.
+// n = 100: the version with row exchanges, a division and FP64 comparisons per column took 470 us.
 constexpr int kSmemSolve = 150;
-__global__ void dense_solve_smem_kernel(const double* __restrict__ Ag, const double* __restrict__ bg, int n,
-                                        double* __restrict__ x, unsigned* status) {
+template <bool kShared>
+__global__ void __launch_bounds__(512) dense_solve_kernel(double* __restrict__ Ag, const double* __restrict__ bg, int n,
+                                                          double* __restrict__ x, unsigned* status) {
   extern __shared__ double sm[];
-  const int ld = n + 1;          // padded rows; column n holds b
-  double* A = sm;
-  __shared__ int piv;
-  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
-  for (int i = tid >> 5; i < n; i += nt >> 5)
-    for (int j = lane; j < n; j += 32) A[i * ld + j] = Ag[static_cast<size_t>(i) * n + j];
-  for (int i = tid; i < n; i += nt) A[i * ld + n] = bg[i];
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
+  const int ld = kShared ? (n + 1) | 1 : n;  // odd: a column's entries lie in different banks
+  double* A = kShared ? sm : Ag;
+  double* b = sm + (kShared ? n * ld : 0);   // n
+  double* pin = b + n;                       // n: reciprocals of the pivots
+  int* slot = reinterpret_cast<int*>(pin + n);  // n: the column a row was the pivot of, -1 before
+  __shared__ unsigned used_w[128];           // bit per row
+  for (int i = tid; i < n; i += nt) b[i] = bg[i], slot[i] = -1;
+  for (int i = tid; i < 128; i += nt) used_w[i] = 0u;
+  if (kShared)
+    for (int i = warp; i < n; i += nw)
+      for (int j = lane; j < n; j += 32) A[i * ld + j] = Ag[static_cast<size_t>(i) * n + j];
   __syncthreads();
   for (int k = 0; k < n; ++k) {
-    if (tid < 32) {
-      double best = -1.0;
-      int bi = k;
-      for (int i = k + lane; i < n; i += 32) {
-        const double v = fabs(A[i * ld + k]);
-        if (v > best) best = v, bi = i;
-      }
-      for (int o = 16; o > 0; o >>= 1) {
-        const double ov = __shfl_xor_sync(0xffffffffu, best, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (ov > best || (ov == best && oi < bi)) best = ov, bi = oi;
-      }
-      if (lane == 0) {
-        piv = bi;
-        if (!(best > 0.0) || !isfinite(best)) atomicOr(status, bte::kZeroPivot);
-      }
+    unsigned long long best = 0ull;
+    int bi = -1;
+    for (int i = lane, q = 0; i < n; i += 32, ++q) {
+      if ((used_w[q] >> lane) & 1u) continue;
+      const unsigned long long key =
+          static_cast<unsigned long long>(__double_as_longlong(A[static_cast<size_t>(i) * ld + k]) & 0x7fffffffffffffffll) + 1ull;
+      if (key > best) best = key, bi = i;
     }
-    __syncthreads();
-    const int p = piv;
-    if (p != k)
-      for (int j = k + tid; j <= n; j += nt) {
-        const double t = A[k * ld + j];
-        A[k * ld + j] = A[p * ld + j];
-        A[p * ld + j] = t;
-      }
-    __syncthreads();
-    const double inv = 1.0 / A[k * ld + k];
-    // rows below the pivot: a warp per row, lanes over the columns (column n: right-hand side)
-    for (int i = k + 1 + (tid >> 5); i < n; i += nt >> 5) {
-      const double l = A[i * ld + k] * inv;
-      for (int j = k + 1 + lane; j <= n; j += 32) A[i * ld + j] -= l * A[k * ld + j];
+    const unsigned hi = static_cast<unsigned>(best >> 32), mh = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned lo = hi == mh ? static_cast<unsigned>(best) : 0u, ml = __reduce_max_sync(0xffffffffu, lo);
+    const unsigned row = hi == mh && static_cast<unsigned>(best) == ml && bi >= 0 ? static_cast<unsigned>(bi) : 0xffffffffu;
+    const int p = static_cast<int>(__reduce_min_sync(0xffffffffu, row));
+    const unsigned long long pk = (static_cast<unsigned long long>(mh) << 32) | ml;
+    const double* ap = A + static_cast<size_t>(p) * ld;
+    const double inv = bte::recip(ap[k]), bp = b[p];
+    for (int i = warp; i < n; i += nw) {
+      if (i == p || ((used_w[i >> 5] >> (i & 31)) & 1u)) continue;
+      double* ai = A + static_cast<size_t>(i) * ld;
+      const double l = ai[k] * inv;
+      for (int j = k + 1 + lane; j < n; j += 32) ai[j] = fma(-l, ap[j], ai[j]);
+      if (lane == 0) b[i] = fma(-l, bp, b[i]);
+    }
+    __syncthreads();  // every warp has read the marks and the pivot row's marker of this column
+    if (tid == 0) {
+      if (pk < 2ull || pk > 0x7ff0000000000000ull) atomicOr(status, bte::kZeroPivot);
+      used_w[p >> 5] |= 1u << (p & 31);
+      slot[k] = p;
+      pin[k] = inv;
     }
     __syncthreads();
   }
-  // back substitution by warp 0 alone (lanes over the row, shuffle sums): no block barriers
-  if (tid < 32) {
-    for (int i = n - 1; i >= 0; --i) {
-      double s = 0.0;
-      for (int j = i + 1 + lane; j < n; j += 32) s = fma(A[i * ld + j], A[j * ld + n], s);
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (lane == 0) A[i * ld + n] = (A[i * ld + n] - s) / A[i * ld + i];
+  // back substitution by columns, warp 0: x_k, then every earlier pivot row's right-hand side
+  if (warp == 0) {
+    for (int k = n - 1; k >= 0; --k) {
+      const double xk = b[slot[k]] * pin[k];
+      __syncwarp();
+      for (int q = lane; q < k; q += 32) {
+        const int r = slot[q];
+        b[r] = fma(-A[static_cast<size_t>(r) * ld + k], xk, b[r]);
+      }
+      if (lane == 0) x[k] = xk;
       __syncwarp();
     }
   }
-  __syncthreads();
-  for (int i = tid; i < n; i += nt) x[i] = A[i * ld + n];
 }
 
-// out_i = P_O (c C_s + e_i A_s) P_S X_i per point (one CTA per point): c = 1 and e_i = E[i] for
-// the velocity operator at a field, c = 0 and e_i = 1 for P_O A_v P_S alone. Structured operators
-// as in the refinement residual (Algorithm 2).
-__global__ void v_apply_kernel(const double* __restrict__ X, const double* __restrict__ E, double c,
+// out_i = P_O M_v^-1 (c C + e_i A_v) P_S X_i per point (one CTA per point): c = 1 and e_i = E[i] for
+// the velocity operator at a field, c = 0 and e_i = 1 for P_O A_v P_S alone. Banded operators as in the
+// refinement residual (Algorithm 2), or, with few unknowns, the dense mass-scaled blocks (Cs not NULL): the
+// Cholesky substitution is 2 nr dependent steps of one warp (25 us at nr = 64 whatever nl, on FP64 units
+// that take a warp's FMA in about 70 cycles), the dense products 3 nl nr^2 FMAs over all warps (8 us at
+// nl = 3); they meet near nl nr = 400. The projections by parity (Y_l(-mu) = (-1)^l Y_l(mu), symmetric
+// ordinates): half their FP64 operations, which bound it.
+__global__ void v_apply_kernel(const double* __restrict__ X, const double* __restrict__ E, double c, bte::ResidualOps ro,
                                const double* __restrict__ Cs, const double* __restrict__ Alo,
-                               const double* __restrict__ Aup, const double* __restrict__ TO,
-                               const double* __restrict__ TS, double* __restrict__ out, int nt, int nr, int nl) {
+                               const double* __restrict__ Aup, const double* __restrict__ TO, const double* __restrict__ TS, double* __restrict__ out,
+                               int nt, int nr, int nl) {
   extern __shared__ double sm[];
-  const int i = blockIdx.x, nv = nt * nr;
-  double* xs = sm;             // nv
-  double* xS = xs + nv;        // nl*nr
-  double* g = xS + nl * nr;    // nl*nr
+  const int i = blockIdx.x, nv = nt * nr, hf = nt / 2, hc = (nt + 1) / 2, w = ro.w, bw = 2 * w + 1;
+  double* fold = sm;                 // 2 hc nr
+  double* xS = fold + 2 * hc * nr;   // nl nr
+  double* g = xS + nl * nr;          // nl nr
   const double* x = X + static_cast<size_t>(i) * nv;
   const double e = E ? E[i] : 1.0;
-  for (int v = threadIdx.x; v < nv; v += blockDim.x) xs[v] = x[v];
+  for (int v = threadIdx.x; v < hc * nr; v += blockDim.x) {
+    const int q = v / nr, k = v % nr;
+    const double p = x[v], m = q < hf ? x[(nt - 1 - q) * nr + k] : 0.0;
+    fold[v] = p + m;
+    fold[hc * nr + v] = q < hf ? p - m : 0.0;
+  }
   __syncthreads();
   for (int idx = threadIdx.x; idx < nl * nr; idx += blockDim.x) {
     const int l = idx / nr, k = idx % nr;
-    double s = 0.0;
-    for (int a = 0; a < nt; ++a) s = fma(__ldg(TS + l * nt + a), xs[a * nr + k], s);
-    xS[idx] = s;
+    const double* src = fold + (l & 1 ? hc * nr : 0) + k;
+    double s0 = 0.0, s1 = 0.0;
+    int q = 0;
+    for (; q + 1 < hc; q += 2) {
+      s0 = fma(__ldg(TS + l * nt + q), src[q * nr], s0);
+      s1 = fma(__ldg(TS + l * nt + q + 1), src[(q + 1) * nr], s1);
+    }
+    if (q < hc) s0 = fma(__ldg(TS + l * nt + q), src[q * nr], s0);
+    xS[idx] = s0 + s1;
   }
   __syncthreads();
   for (int idx = threadIdx.x; idx < nl * nr; idx += blockDim.x) {
-    const int l = idx / nr, p = idx % nr;
-    const size_t off = (static_cast<size_t>(l) * nr + p) * nr;
+    const int l = idx / nr, p = idx % nr, k0 = max(0, p - w), k1 = min(nr - 1, p + w);
+    const double* z = xS + l * nr;
     double cc = 0.0, f = 0.0;
-    if (c != 0.0)
-      for (int k = 0; k < nr; ++k) cc = fma(__ldg(Cs + off + k), xS[l * nr + k], cc);
-    if (l >= 1)
-      for (int k = 0; k < nr; ++k) f = fma(__ldg(Alo + off + k), xS[(l - 1) * nr + k], f);
-    if (l + 1 < nl)
-      for (int k = 0; k < nr; ++k) f = fma(__ldg(Aup + off + k), xS[(l + 1) * nr + k], f);
+    if (Cs) {
+      const size_t off = (static_cast<size_t>(l) * nr + p) * nr;
+      if (c != 0.0)
+        for (int k = 0; k < nr; ++k) cc = fma(__ldg(Cs + off + k), z[k], cc);
+      if (l >= 1)
+        for (int k = 0; k < nr; ++k) f = fma(__ldg(Alo + off + k), z[k - nr], f);
+      if (l + 1 < nl)
+        for (int k = 0; k < nr; ++k) f = fma(__ldg(Aup + off + k), z[k + nr], f);
+      g[idx] = c * cc + e * f;
+      continue;
+    }
+    if (c != 0.0) {
+      if (l > 0) {
+        const double* row = ro.band + static_cast<size_t>(p) * bw + w - p;
+        for (int k = k0; k <= k1; ++k) cc = fma(__ldg(row + k), z[k], cc);
+      } else {
+        const double* row = ro.c0 + static_cast<size_t>(p) * nr;
+        for (int k = k0; k < nr; ++k) cc = fma(__ldg(row + k), z[k], cc);
+      }
+    }
+    if (l >= 1) {
+      const double* row = ro.fband + (static_cast<size_t>(l) * nr + p) * bw + w - p;
+      for (int k = k0; k <= k1; ++k) f = fma(__ldg(row + k), z[k - nr], f);
+    }
+    if (l + 1 < nl) {
+      const double* row = ro.fband + (static_cast<size_t>(nl + l) * nr + p) * bw + w - p;
+      for (int k = k0; k <= k1; ++k) f = fma(__ldg(row + k), z[k + nr], f);
+    }
     g[idx] = c * cc + e * f;
   }
   __syncthreads();
-  for (int v = threadIdx.x; v < nv; v += blockDim.x) {
+  if (!Cs) {
+    for (int l = threadIdx.x; l < nl; l += blockDim.x) bte::mass_solve(g + l * nr, ro.chol, ro.cinv, nr, w);
+    __syncthreads();
+  }
+  double* o = out + static_cast<size_t>(i) * nv;
+  for (int v = threadIdx.x; v < hc * nr; v += blockDim.x) {
     const int a = v / nr, p = v % nr;
-    double s = 0.0;
-    for (int l = 0; l < nl; ++l) s = fma(__ldg(TO + a * nl + l), g[l * nr + p], s);
-    out[static_cast<size_t>(i) * nv + v] = s;
+    double se = 0.0, so = 0.0;
+    for (int l = 0; l < nl; l += 2) {
+      se = fma(__ldg(TO + a * nl + l), g[l * nr + p], se);
+      if (l + 1 < nl) so = fma(__ldg(TO + a * nl + l + 1), g[(l + 1) * nr + p], so);
+    }
+    o[v] = se + so;
+    if (a < hf) o[(nt - 1 - a) * nr + p] = se - so;
   }
 }
 
@@ -302,18 +310,38 @@ __global__ void implicit_combine_kernel(const double* __restrict__ X, const doub
   }
 }
 
-// partial[blk][j] = sum over this block's elements of V_j . w, j < k (V_j = V + j ld)
-__global__ void multi_dot_kernel(const double* __restrict__ V, size_t ld, int k, const double* __restrict__ w,
-                                 size_t n, double* __restrict__ partial) {
-  __shared__ double red[32];
-  for (int j = 0; j < k; ++j) {
-    const double* v = V + j * ld;
-    double s = 0.0;
-    for (size_t e = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; e < n;
-         e += static_cast<size_t>(gridDim.x) * blockDim.x)
-      s = fma(v[e], w[e], s);
-    s = block_sum(s, red);
-    if (threadIdx.x == 0) partial[static_cast<size_t>(blockIdx.x) * k + j] = s;
+// partial[blk][j] = sum over this block's elements of V_j . w, j < k (V_j = V + j ld). blockIdx.y takes
+// eight of the vectors: w is read once for them and their block sums share the barriers.
+constexpr int kDotVec = 8;
+static_assert(kDotVec == kDotBlock / 32, "one warp per vector");
+__global__ void __launch_bounds__(kDotBlock) multi_dot_kernel(const double* __restrict__ V, size_t ld, int k,
+                                                              const double* __restrict__ w, size_t n,
+                                                              double* __restrict__ partial) {
+  __shared__ double red[kDotVec][kDotBlock];
+  const int j0 = blockIdx.y * kDotVec, nj = min(kDotVec, k - j0), lane = threadIdx.x & 31;
+  const double* v = V + j0 * ld;
+  double s[kDotVec];
+#pragma unroll
+  for (int j = 0; j < kDotVec; ++j) s[j] = 0.0;
+  for (size_t e = blockIdx.x * static_cast<size_t>(kDotBlock) + threadIdx.x; e < n;
+       e += static_cast<size_t>(gridDim.x) * kDotBlock) {
+    const double we = w[e];
+#pragma unroll
+    for (int j = 0; j < kDotVec; ++j)
+      if (j < nj) s[j] = fma(v[j * ld + e], we, s[j]);
+  }
+#pragma unroll
+  for (int j = 0; j < kDotVec; ++j) red[j][threadIdx.x] = s[j];
+  __syncthreads();
+  // warp j sums vector j: FP64 additions bound this part, so it takes 13 of them where a shuffle tree
+  // in every warp takes 40
+  const int j = threadIdx.x >> 5;
+  if (j < nj) {
+    double t = 0.0;
+#pragma unroll
+    for (int q = 0; q < kDotBlock / 32; ++q) t += red[j][lane + 32 * q];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane == 0) partial[static_cast<size_t>(blockIdx.x) * k + j0 + j] = t;
   }
 }
 
@@ -380,7 +408,8 @@ template <typename T>
 bte_status hupload(bte_handle* h, T** p, const std::vector<T>& v) {
   bte_status s = halloc(h, p, v.size());
   if (s != BTE_OK) return s;
-  BH_CUDA(h, cudaMemcpy(*p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice));
+  BH_CUDA(h, cudaMemcpyAsync(*p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice, h->st));
+  BH_CUDA(h, cudaStreamSynchronize(h->st));
   return BTE_OK;
 }
 
@@ -404,9 +433,13 @@ bte_status hybrid_setup(bte_handle* h) {
   if (s == BTE_OK) s = hupload(h, &h->Lop, Lop);
   if (s == BTE_OK) s = hupload(h, &h->E1, E1);
   if (s == BTE_OK) s = hupload(h, &h->Dxd, o.Dx);
+  if (s == BTE_OK) s = hupload(h, &h->DxT, o.Dx);
+  if (s == BTE_OK) launch_transpose_blocks(h->DxT, o.nx, 1, h->st);
   if (s == BTE_OK) s = hupload(h, &h->mud, o.mu);
   if (s == BTE_OK) s = hupload(h, &h->lamd, o.lam);
   if (s == BTE_OK) s = hupload(h, &h->rion, rion);
+  if (s == BTE_OK) s = halloc(h, &h->D2, static_cast<size_t>(o.nx) * o.nx);
+  if (s == BTE_OK) square_kernel<<<o.nx, 256, 0, h->st>>>(h->Dxd, o.nx, h->D2);
   if (s == BTE_OK) s = halloc(h, &h->Esc, o.nx);
   if (s == BTE_OK) s = halloc(h, &h->ned, o.nx);
   if (s == BTE_OK) s = halloc(h, &h->Ek, o.nx);
@@ -430,6 +463,7 @@ bte_status implicit_setup(bte_handle* h, int m, bool full_q) {
     std::vector<double> Q;
     if (!assemble_q(h->ops, h->ops.dt, Q)) return hfail(h, BTE_EINVAL, "a full-step x operator is singular");
     if ((s = hupload(h, &h->Qfull, Q)) != BTE_OK) return s;
+    launch_transpose_blocks(h->Qfull, h->ops.nx, static_cast<size_t>(h->ops.nt) * h->ops.nr, h->st);
   }
   if (h->gm >= m) return BTE_OK;
   const size_t D = static_cast<size_t>(h->ops.nx) * h->ops.nv;
@@ -449,33 +483,39 @@ bte_status implicit_setup(bte_handle* h, int m, bool full_q) {
   return BTE_OK;
 }
 
-// A_x X D_x^T (per ordinate mu_a D_x X_a G^T, G = M_v^-1 G_v) through the eigen basis of G
+// A_x X D_x^T (per ordinate mu_a D_x X_a G^T, G = M_v^-1 G_v) through the eigen basis of G; X NULL: of
+// the vector whose eigen coefficients are in Y2
 void enqueue_xop(bte_handle* h, const double* X, double* out) {
   const HostOps& o = h->ops;
   cudaStream_t st = h->st;
-  launch_x_to_eigen(X, h->Uinv, h->Y, o.nx, o.nt, o.nr, h->status, st);
-  launch_x_matvec(h->Dxd, false, h->lamd, h->mud, h->Y, h->Y2, o.nx, o.nt, o.nr, st);  // lam_i mu_a D_x Y
-  launch_x_from_eigen(h->Y2, h->U, out, o.nx, o.nt, o.nr, nullptr, st);
+  double *in = h->Y2, *mid = h->Y;
+  if (X) {
+    std::swap(in, mid);
+    launch_x_to_eigen(X, h->Uinv, in, o.nx, o.nt, o.nr, h->status, st);
+  }
+  launch_x_matvec(h->DxT, false, h->lamd, h->mud, in, mid, o.nx, o.nt, o.nr, st);  // lam_i mu_a D_x Y
+  launch_x_from_eigen(mid, h->U, out, o.nx, o.nt, o.nr, nullptr, st);
 }
 
 void enqueue_vapply(bte_handle* h, const double* X, const double* E, double c, double* out) {
   const HostOps& o = h->ops;
-  const size_t smem = sizeof(double) * (static_cast<size_t>(o.nv) + 2 * o.nl * o.nr);
-  v_apply_kernel<<<o.nx, 256, smem, h->st>>>(X, E, c, h->Cs, h->Alo, h->Aup, h->TO, h->TS, out, o.nt, o.nr, o.nl);
+  const size_t smem = sizeof(double) * o.nr * (2 * ((o.nt + 1) / 2) + 2 * static_cast<size_t>(o.nl));
+  v_apply_kernel<<<o.nx, 256, smem, h->st>>>(X, E, c, handle_residual_ops(h), o.nl * o.nr <= 400 ? h->Cs : nullptr, h->Alo,
+                                          h->Aup, h->TO, h->TS, out, o.nt, o.nr, o.nl);
 }
 
 // out_dev[j] = V_j . w for j < k on the device (stream-ordered; no host synchronisation)
 void enqueue_dots(bte_handle* h, const double* V, size_t ld, int k, const double* w, double* out_dev) {
   const size_t D = static_cast<size_t>(h->ops.nx) * h->ops.nv;
-  multi_dot_kernel<<<kDotGrid, kDotBlock, 0, h->st>>>(V, ld, k, w, D, h->part);
-  sum_partials_kernel<<<k, 128, 0, h->st>>>(h->part, kDotGrid, k, out_dev);
+  multi_dot_kernel<<<dim3(dot_grid(D), (k + kDotVec - 1) / kDotVec), kDotBlock, 0, h->st>>>(V, ld, k, w, D, h->part);
+  sum_partials_kernel<<<k, 128, 0, h->st>>>(h->part, dot_grid(D), k, out_dev);
 }
 
 // dots[j] = V_j . w for j < k into the pinned host array (synchronises the stream)
 bte_status host_dots(bte_handle* h, const double* V, size_t ld, int k, const double* w, std::vector<double>& out) {
   const size_t D = static_cast<size_t>(h->ops.nx) * h->ops.nv;
-  multi_dot_kernel<<<kDotGrid, kDotBlock, 0, h->st>>>(V, ld, k, w, D, h->part);
-  sum_partials_kernel<<<k, 128, 0, h->st>>>(h->part, kDotGrid, k, h->dsum);
+  multi_dot_kernel<<<dim3(dot_grid(D), (k + kDotVec - 1) / kDotVec), kDotBlock, 0, h->st>>>(V, ld, k, w, D, h->part);
+  sum_partials_kernel<<<k, 128, 0, h->st>>>(h->part, dot_grid(D), k, h->dsum);
   BH_CUDA(h, cudaMemcpyAsync(h->dsum_host, h->dsum, k * sizeof(double), cudaMemcpyDeviceToHost, h->st));
   BH_CUDA(h, cudaStreamSynchronize(h->st));
   out.assign(h->dsum_host, h->dsum_host + k);
@@ -543,18 +583,14 @@ bte_status bte_ion_step(bte_handle* h, double* ni_dev, const double* F_dev, doub
   if (s != BTE_OK) return s;
   point_dot_kernel<<<o.nx, 256, 0, st>>>(F_dev, h->rion, o.nv, h->ned);
   scale_kernel<<<(o.nx + 255) / 256, 256, 0, st>>>(h->ned, o.n0, o.nx);
-  ion_assemble_kernel<<<o.nx, 256, 0, st>>>(h->Dxd, h->Esc, ni_dev, h->ned, h->n0_mu_i / o.n0, h->n0_D_i / o.n0,
+  ion_assemble_kernel<<<o.nx, 256, 0, st>>>(h->Dxd, h->D2, h->Esc, ni_dev, h->ned, h->n0_mu_i / o.n0, h->n0_D_i / o.n0,
                                            o.dt, o.nx, h->ionA, h->ionb);
-  if (o.nx <= kSmemSolve) {
-    const size_t smem = sizeof(double) * o.nx * (o.nx + 1);
-    static bool attr = false;
-    if (!attr) {
-      cudaFuncSetAttribute(dense_solve_smem_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-      attr = true;
-    }
-    dense_solve_smem_kernel<<<1, 1024, smem, st>>>(h->ionA, h->ionb, o.nx, h->ned, h->status);
-  } else {
-    dense_solve_kernel<<<1, 1024, 0, st>>>(h->ionA, h->ionb, o.nx, h->ned, h->status);
+  {
+    const bool fits = o.nx <= kSmemSolve;
+    const size_t smem = (fits ? sizeof(double) * o.nx * ((o.nx + 1) | 1) : 0) + o.nx * (2 * sizeof(double) + sizeof(int));
+    auto solve = fits ? dense_solve_kernel<true> : dense_solve_kernel<false>;
+    BH_CUDA(h, cudaFuncSetAttribute(solve, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+    solve<<<1, fits ? 256 : 512, smem, st>>>(h->ionA, h->ionb, o.nx, h->ned, h->status);
   }
   bte::launch_commit(h->ned, ni_dev, o.nx, h->status, st);
   bte::handle_add_launches(h, 5);
@@ -661,11 +697,12 @@ bte_status bte_step_implicit(bte_handle* h, double* F_dev, const double* ni_dev,
     }
     return r;
   };
-  // Jacobian action at F_k (eq. "1dbte_jac_action" with the inflow rows as identity)
-  auto jac = [&](const double* X, double* out) {
+  // Jacobian action at F_k (eq. "1dbte_jac_action" with the inflow rows as identity). in_eigen: X is the
+  // x step's last result, whose eigen coefficients are still in Y2 (the transform there and back is left out)
+  auto jac = [&](const double* X, double* out, bool in_eigen = false) {
     point_dot_kernel<<<nx, 256, 0, st>>>(X, h->mom_n, o.nv, h->ned);
     field_kernel<<<(nx * 32 + 255) / 256, 256, 0, st>>>(h->Lop, h->E1, nullptr, h->ned, 0.0, nx, h->El);
-    bte::enqueue_xop(h, X, h->Zx);
+    bte::enqueue_xop(h, in_eigen ? nullptr : X, h->Zx);
     bte::enqueue_vapply(h, X, h->Ek, 1.0, h->VX);
     implicit_combine_kernel<<<vg, 256, 0, st>>>(X, nullptr, 0.0, h->Zx, h->VX, h->El, h->KAF, h->mud, dt, nx, nt,
                                                 nr, out);
@@ -716,7 +753,7 @@ bte_status bte_step_implicit(bte_handle* h, double* F_dev, const double* ni_dev,
         double* Vn = h->Vb + static_cast<size_t>(j + 1) * D;
         double* Zj = h->Zb + static_cast<size_t>(j) * D;
         if ((s = pinv(Vj, Zj)) != BTE_OK) return s;
-        jac(Zj, Vn);
+        jac(Zj, Vn, precond == 0);
         // classical Gram-Schmidt twice, then the norm: the projections stay on the device (the
         // axpys read them there), so the host waits once per iteration for all three results
         const size_t stride = static_cast<size_t>(m) + 1;

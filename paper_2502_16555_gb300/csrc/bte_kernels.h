@@ -61,14 +61,17 @@ void tc_lu_u12_pair(float* fac, int nx, int n, int k0, void* ws, unsigned* statu
 void tc_lu_gemm_pair(float* fac, int nx, int n, int k0, void* ws, unsigned* status, cudaStream_t st, int probe = 0,
                      int cg = 2);
 
-// Y2[b] = s_b M_b Y[b] for the nt * nr pairs b = a nr + i: M_b = M + b nx^2 (per_pair) or the one
-// matrix M; s_b = lam[i] mu[a] when lam is given (device arrays), else 1. Y, Y2 are [nt][nr][nx].
-void launch_x_matvec(const double* M, bool per_pair, const double* lam, const double* mu, const double* Y,
+// Y2[b] = s_b M_b Y[b] for the nt * nr pairs b = a nr + i, from the transposes: M_b^T = MT + b nx^2
+// (per_pair) or the one matrix MT; s_b = lam[i] mu[a] when lam is given (device arrays), else 1. Y, Y2
+// are [nt][nr][nx].
+void launch_x_matvec(const double* MT, bool per_pair, const double* lam, const double* mu, const double* Y,
                      double* Y2, int nx, int nt, int nr, cudaStream_t st);
-// ---- x half step (Algorithm 1): eigen-basis transform, Q_ij apply, back transform
+// Transposes `count` consecutive n x n matrices in place.
+void launch_transpose_blocks(double* M, int n, size_t count, cudaStream_t st);
+// ---- x half step (Algorithm 1): eigen-basis transform, Q_ij apply (QT: the transposes), back transform
 void launch_x_to_eigen(const double* F, const double* Uinv, double* Y, int nx, int nt, int nr,
                        unsigned* status, cudaStream_t st);
-void launch_x_apply_q(const double* Q, const double* Y, double* Y2, int nx, int nt, int nr,
+void launch_x_apply_q(const double* QT, const double* Y, double* Y2, int nx, int nt, int nr,
                       cudaStream_t st);
 void launch_x_from_eigen(const double* Y2, const double* U, double* F, int nx, int nt, int nr,
                          unsigned* status, cudaStream_t st);
@@ -251,6 +254,7 @@ void launch_moments(const double* F, const double* mom_n, const double* mom_e, c
 void launch_fill_maxwellian(double* F, const double* ne, const double* coef, int nx, int nt, int nr,
                             cudaStream_t st);
 
+ResidualOps handle_residual_ops(const bte_handle* h);
 inline cudaStream_t handle_stream(const bte_handle* h) { return static_cast<cudaStream_t>(handle_stream_ptr(h)); }
 
 }  // namespace bte

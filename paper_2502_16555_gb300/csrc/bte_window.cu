@@ -35,6 +35,7 @@
 
 #include "bte_handle.h"
 #include "bte_kernels.h"
+#include "bte_mass.cuh"
 #include "bte_recip.cuh"
 #include "bte_tf32.cuh"
 
@@ -187,6 +188,17 @@ __device__ __forceinline__ void store32(float* dst, const float (&v)[32]) {
     reinterpret_cast<float4*>(dst)[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
 }
 
+// Where p: the 8 values v[0 .. 7] to row, (key, inv) to rec (shared-memory addresses), without a branch.
+__device__ __forceinline__ void post_row(bool p, uint32_t row, const float (&v)[32], uint32_t rec, unsigned key, float inv) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.u32 p, %0, 0;\n"
+      " @p st.shared.v4.f32 [%1], {%2, %3, %4, %5};\n @p st.shared.v4.f32 [%1 + 16], {%6, %7, %8, %9};\n"
+      " @p st.shared.v2.b32 [%10], {%11, %12};\n}"
+      ::"r"(static_cast<unsigned>(p)), "r"(row), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]),
+      "f"(v[6]), "f"(v[7]), "r"(rec), "r"(key), "f"(inv)
+      : "memory");
+}
+
 struct FactorArgs {
   WindowPlan w;
   const void* base;    // [np 32][NW] row templates (T)
@@ -224,7 +236,8 @@ __global__ void __launch_bounds__(kThreads, 2) window_lu_tc_kernel(const FactorA
   __shared__ __align__(16) uint2 keys[2][4];       // its magnitude and lane, and 1 / its pivot
   __shared__ __align__(16) float pblk[2][8][24];   // a sub-block's pivot rows over the other columns
   __shared__ signed char slotj[2][kSlots];
-  __shared__ float u11[2][64 * 33];  // rows 0 .. 31 stay zero: the back substitution reads above the block
+  __shared__ float u11[2][32 * 33];
+  __shared__ float ui[32 * 17];  // inverses of U11's 16 x 16 diagonal blocks
   __shared__ __align__(8) uint64_t bar_next, bar_rest;
   __shared__ uint32_t tmem_base;
   __shared__ int gave_up;
@@ -255,7 +268,6 @@ __global__ void __launch_bounds__(kThreads, 2) window_lu_tc_kernel(const FactorA
   }
   // K columns of unused unknowns stay zero in B for the whole factorisation
   for (int i = tid; i < w.NU * kPW; i += kThreads) Bhi[i] = Blo[i] = 0.f;
-  for (int i = tid; i < 2 * 64 * 33; i += kThreads) (&u11[0][0])[i] = 0.f;
   for (int i = tid; i < 2 * 8 * 24; i += kThreads) (&pblk[0][0][0])[i] = 0.f;
   if (tid < 8) (&keys[0][0])[tid] = make_uint2(0u, 0u);
   tc_fence_before();
@@ -319,34 +331,28 @@ __global__ void __launch_bounds__(kThreads, 2) window_lu_tc_kernel(const FactorA
             float4 r0 = make_float4(0.f, 0.f, 0.f, 0.f), r1 = r0;
             if ((mask >> (8 * q + c)) & 1u) {
               b ^= 1;
-              // the low 5 bits of the magnitude give way to the lane: the largest entry to 2^-18
+              // the low 5 bits of the magnitude give way to the lane: the largest entry to 2^-18. No
+              // branches in a column's chain (each cost 50 to 100 cycles): the store is predicated.
               const unsigned key = cand ? (__float_as_uint(v[0]) & 0x7fffffe0u) + 32u + lane : 0u;
               const float inv = recip(v[0]);
               const unsigned best = __reduce_max_sync(0xffffffffu, key);
-              if (key == best && cand) {
-                float4* post = reinterpret_cast<float4*>(prow[b][warp]);
-                post[0] = make_float4(v[0], v[1], v[2], v[3]);
-                post[1] = make_float4(v[4], v[5], v[6], v[7]);
-                keys[b][warp] = make_uint2(key, __float_as_uint(inv));
-              } else if (best == 0u && lane == 0) {
-                keys[b][warp] = make_uint2(0u, 0u);
-              }
-              __syncwarp();
+              post_row(best ? key == best : lane == 0, saddr(prow[b][warp]), v, saddr(&keys[b][warp]), key, inv);
               asm volatile("bar.sync 1, %0;" ::"r"(npw * 32) : "memory");
               const uint4 k01 = *reinterpret_cast<const uint4*>(&keys[b][0]), k23 = *reinterpret_cast<const uint4*>(&keys[b][2]);
-              unsigned kb = k01.x, iv = k01.y;
-              int wb = 0;
-              if (k01.z > kb) kb = k01.z, iv = k01.w, wb = 1;
-              if (k23.x > kb) kb = k23.x, iv = k23.y, wb = 2;
-              if (k23.z > kb) kb = k23.z, iv = k23.w, wb = 3;
+              const bool s1 = k01.z > k01.x, s2 = k23.z > k23.x;
+              const unsigned ka = s1 ? k01.z : k01.x, kc = s2 ? k23.z : k23.x;
+              const bool s3 = kc > ka;
+              const unsigned kb = s3 ? kc : ka;
+              const unsigned iv = s3 ? (s2 ? k23.w : k23.y) : (s1 ? k01.w : k01.y);
+              const int wb = s3 ? (s2 ? 3 : 2) : (s1 ? 1 : 0);
               r0 = *reinterpret_cast<const float4*>(&prow[b][wb][0]);
               r1 = *reinterpret_cast<const float4*>(&prow[b][wb][4]);
-              if (wb == warp && key == kb && cand) {
-                pq = c;
-                cand = false;
-                if (kb < 64u || kb >= 0x7f800020u) bad = true;  // zero, infinite or NaN
-              }
-              if (cand) f = v[0] * __uint_as_float(iv), last = -f;
+              const bool win = wb == warp && key == kb;
+              pq = win ? c : pq;
+              cand = cand && !win;
+              bad |= kb < 64u || kb >= 0x7f800020u;  // zero, infinite or NaN
+              f = cand ? v[0] * __uint_as_float(iv) : 0.f;
+              last = cand ? -f : last;
             }
             v[0] = fmaf(-f, r0.y, v[1]), v[1] = fmaf(-f, r0.z, v[2]), v[2] = fmaf(-f, r0.w, v[3]);
             v[3] = fmaf(-f, r1.x, v[4]), v[4] = fmaf(-f, r1.y, v[5]), v[5] = fmaf(-f, r1.z, v[6]);
@@ -386,13 +392,13 @@ __global__ void __launch_bounds__(kThreads, 2) window_lu_tc_kernel(const FactorA
         }
         if (pj >= 0) {
 #pragma unroll
-          for (int k = 0; k < 32; ++k) u11[par][(32 + pj) * 33 + k] = k >= pj ? v[k] : 0.f;
+          for (int k = 0; k < 32; ++k) u11[par][pj * 33 + k] = k >= pj ? v[k] : 0.f;
 #pragma unroll
           for (int k = 0; k < 32; ++k)
             if (k >= pj) v[k] = 0.f;
         }
         if (warp == 0 && !((mask >> lane) & 1u))
-          for (int k = 0; k < 32; ++k) u11[par][(32 + lane) * 33 + k] = k == lane ? 1.f : 0.f;
+          for (int k = 0; k < 32; ++k) u11[par][lane * 33 + k] = k == lane ? 1.f : 0.f;
         // T of this panel: global (column k of the 32, slots contiguous) and the split operand
 #pragma unroll
         for (int k = 0; k < 32; ++k) Tg[(static_cast<size_t>(s) * 32 + k) * NS + slot] = v[k];
@@ -412,17 +418,19 @@ __global__ void __launch_bounds__(kThreads, 2) window_lu_tc_kernel(const FactorA
           *reinterpret_cast<float4*>(Thi + o) = h;
           *reinterpret_cast<float4*>(Tlo + o) = l;
         }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       }
     }
-    __syncthreads();  // pivots known; the window of the panel before is complete in tensor memory
+    __syncthreads();  // T in place, pivots known; the window of the panel before is complete in tensor memory
     tc_fence_after();
     const int j = slotj[par][slot];
     const int tnew = s + 1 + RC, rnew = tnew * 32 + j;  // the row that takes this slot
     const bool fresh = j >= 0 && tnew < np && ((chunk_mask(w, tnew) >> j) & 1u);
     if (dmax > 0) {
-      // the pivot rows' window, split, as the K-major B operand; chunks alternate between the halves
+      // the pivot rows' window, split, as the K-major B operand: chunk s + 1, which the next panel needs,
+      // by the panel warps, whose product is issued at once, the others by the other half
       const int cnt = dmax + (nfc - fc0);
-      for (int c = panel_warp ? 0 : 1; c < cnt; c += 2) {
+      auto convert = [&](int c) {
         const int col = c < dmax ? ((s + 1 + c) % RS) * 32 : (RS + fc0 + c - dmax) * 32;
         float r[32];
         tmem_ld32(tmem + col, r);
@@ -438,58 +446,110 @@ __global__ void __launch_bounds__(kThreads, 2) window_lu_tc_kernel(const FactorA
             bl[o] = l;
           }
         }
-      }
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      tc_fence_before();
-      __syncthreads();
-      tc_fence_after();
-      if (warp == 5) {  // not a panel warp: the tensor cores' queue holds the issuing thread up
+      };
+      // warp 0 issues the first product, warp 5 the rest (not a panel warp: the tensor cores' queue holds
+      // the issuing thread up)
+      auto issue = [&](int col, int ncol) {
         const uint64_t dah = sdesc(saddr(Thi)), dal = sdesc(saddr(Tlo)), dbh = sdesc(saddr(Bhi)), dbl = sdesc(saddr(Blo));
-        // ranges of window columns: chunk s + 1; then the other ring chunks, slots (s + 2) % RS ..
-        // (s + dmax) % RS, wrapping; then the far columns (at most 256 columns an instruction)
-        const int q1 = (s + 1) % RS, q2 = (s + 2) % RS, m = dmax - 1, m1 = imin(m, RS - q2);
+        const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | (static_cast<uint32_t>(ncol >> 3) << 17) |
+                               (static_cast<uint32_t>(kSlots >> 4) << 24);
+        const uint64_t off = static_cast<uint64_t>(col) * 8;  // 128-byte rows in units of 16 bytes
+        const uint32_t d = tmem_base + col;
+        if (lane == 0) {
 #pragma unroll 1
-        for (int r = 0; r < 5; ++r) {
-          int col = q1 * 32, n = 32;
-          if (r == 1) col = q2 * 32, n = m1 * 32;
-          if (r == 2) col = 0, n = (m - m1) * 32;
-          if (r >= 3) col = (RS + fc0) * 32 + (r - 3) * 256, n = imin(256, (nfc - fc0) * 32 - (r - 3) * 256);
-          if (n <= 0) continue;
-          const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | (static_cast<uint32_t>(n >> 3) << 17) |
-                                 (static_cast<uint32_t>(kSlots >> 4) << 24);
-          const uint64_t off = static_cast<uint64_t>(col) * 8;  // 128-byte rows in units of 16 bytes
-          const uint32_t d = tmem_base + col;
-          if (lane == 0) {
-#pragma unroll 1
-            for (int k = 0; k < 4; ++k) {  // 8 TF32 columns = 32 bytes inside the swizzle row
-              mma_tf32(d, dal + 2 * k, dbh + off + 2 * k, idesc);
-              mma_tf32(d, dah + 2 * k, dbl + off + 2 * k, idesc);
-              mma_tf32(d, dah + 2 * k, dbh + off + 2 * k, idesc);
-            }
-            if (r == 0) mma_commit(&bar_next);
+          for (int k = 0; k < 4; ++k) {  // 8 TF32 columns = 32 bytes inside the swizzle row
+            mma_tf32(d, dal + 2 * k, dbh + off + 2 * k, idesc);
+            mma_tf32(d, dah + 2 * k, dbl + off + 2 * k, idesc);
+            mma_tf32(d, dah + 2 * k, dbh + off + 2 * k, idesc);
           }
+        }
+        __syncwarp();
+      };
+      auto converted = [&]() {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        tc_fence_before();
+        __syncwarp();
+      };
+#pragma unroll 1
+      for (int c = panel_warp ? 0 : 1; c < (panel_warp ? 1 : cnt); ++c) {
+        convert(c);
+        if (c == 0) {
+          converted();
+          asm volatile("bar.sync 3, 128;" ::: "memory");
+          if (warp == 0) {
+            tc_fence_after();
+            issue(((s + 1) % RS) * 32, 32);
+            if (lane == 0) mma_commit(&bar_next);
+            __syncwarp();
+          }
+        }
+      }
+      if (!panel_warp) {
+        converted();
+        asm volatile("bar.sync 4, 128;" ::: "memory");  // the other chunks are in place
+        tc_fence_after();
+        if (warp == 5) {
+          // the other ring chunks, slots (s + 2) % RS .. (s + dmax) % RS, wrapping, then the far columns
+          // (at most 256 columns an instruction)
+          const int q2 = (s + 2) % RS, m = dmax - 1, m1 = imin(m, RS - q2);
+#pragma unroll 1
+          for (int r = 1; r < 5; ++r) {
+            int col = q2 * 32, n = m1 * 32;
+            if (r == 2) col = 0, n = (m - m1) * 32;
+            if (r >= 3) col = (RS + fc0) * 32 + (r - 3) * 256, n = imin(256, (nfc - fc0) * 32 - (r - 3) * 256);
+            if (n > 0) issue(col, n);
+          }
+          if (lane == 0) mma_commit(&bar_rest);
           __syncwarp();
         }
-        if (lane == 0) mma_commit(&bar_rest);
-        __syncwarp();
       }
     }
     float* Up = Ug + s * ustride;
     if (warp == 4) {
-      // inv(U11): one lane a column; row k of the inverse leaves the turning registers at x[31]
-      float x[32];
+      // inv(U11) by one warp: the two 16 x 16 diagonal blocks at once (one lane a column, the rows in
+      // turning registers), then -inv(A) B inv(D)
+      const float* u = u11[par];
+      const int blk = lane >> 4, c = lane & 15;
+      const float* d = u + blk * 16 * 34;
+      const float rd = recip(d[c * 34]);
+      float x[16];
 #pragma unroll
-      for (int r = 0; r < 32; ++r) x[r] = r == lane ? 1.f : 0.f;
-      const float dl = u11[par][(32 + lane) * 33 + lane], rd = dl != 0.f ? recip(dl) : 0.f;
+      for (int r = 0; r < 16; ++r) x[r] = r == c ? 1.f : 0.f;
 #pragma unroll 1
-      for (int k = 31; k >= 0; --k) {
-        const float* u = &u11[par][(32 + k) * 33 + k];
-        const float xk = x[31] * __shfl_sync(0xffffffffu, rd, k);
-        Up[k * 32 + lane] = xk;
+      for (int k = 15; k >= 0; --k) {
+        const float xk = x[15] * __shfl_sync(0xffffffffu, rd, (lane & 16) + k);
+        ui[(blk * 16 + k) * 17 + c] = xk;
+        const float* dk = d + (k - 16) * 33 + k;  // row k - 16 + i, column k; rows above the block are not used
 #pragma unroll
-        for (int i = 31; i > 0; --i) x[i] = fmaf(-u[-33 * (32 - i)], xk, x[i - 1]);
+        for (int i = 15; i > 0; --i) x[i] = fmaf(-dk[max(i, 16 - k) * 33], xk, x[i - 1]);
         x[0] = 0.f;
       }
+      __syncwarp();
+      // rows blk * 8 .. + 7 of the upper right block, column c
+      float t[16], y[8];
+#pragma unroll
+      for (int r = 0; r < 16; ++r) t[r] = 0.f;
+#pragma unroll 1
+      for (int k = 0; k < 16; ++k) {
+        const float z = ui[(16 + k) * 17 + c];
+#pragma unroll
+        for (int r = 0; r < 16; ++r) t[r] = fmaf(u[r * 33 + 16 + k], z, t[r]);
+      }
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        float acc = 0.f;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) acc = fmaf(-ui[(blk * 8 + r) * 17 + k], t[k], acc);
+        y[r] = acc;
+      }
+#pragma unroll
+      for (int r = 0; r < 16; ++r) {
+        Up[r * 32 + lane] = lane < 16 ? ui[r * 17 + c] : 0.f;
+        Up[(16 + r) * 32 + lane] = lane < 16 ? 0.f : ui[(16 + r) * 17 + c];
+      }
+      __syncwarp();
+#pragma unroll
+      for (int r = 0; r < 8; ++r) Up[(blk * 8 + r) * 32 + 16 + c] = y[r];
     }
     if (dmax == 0) break;
     float* urow = Up + 1024 + static_cast<size_t>(imax(j, 0)) * w.NU;
@@ -1196,41 +1256,7 @@ __global__ void __launch_bounds__(kEval) window_residual_kernel(const SolveArgs 
     const double least = lb / a.ts_inf;
     if (!last && least > a.tol * mb && least > floor_ * (nA * (mb + a.to_inf * mz) + mb)) return;
     // q_l <- M^-1 q_l by the banded Cholesky factor, one thread a harmonic
-    for (int l = tid; l < nl; l += kEval) {
-      double* gl = q + l * nr;
-      if (mw == 3) {
-        double y1 = 0.0, y2 = 0.0, y3 = 0.0;
-        for (int p = 0; p < nr; ++p) {
-          const double* r = a.ro.chol + static_cast<size_t>(p) * 4;
-          const double y = fma(-__ldg(r + 2), y1, fma(-__ldg(r + 1), y2, fma(-__ldg(r), y3, gl[p]))) * __ldg(a.ro.cinv + p);
-          gl[p] = y;
-          y3 = y2, y2 = y1, y1 = y;
-        }
-        double z1 = 0.0, z2 = 0.0, z3 = 0.0;
-        for (int p = nr - 1; p >= 0; --p) {
-          double s = gl[p];
-          if (p + 1 < nr) s = fma(-__ldg(a.ro.chol + static_cast<size_t>(p + 1) * 4 + 2), z1, s);
-          if (p + 2 < nr) s = fma(-__ldg(a.ro.chol + static_cast<size_t>(p + 2) * 4 + 1), z2, s);
-          if (p + 3 < nr) s = fma(-__ldg(a.ro.chol + static_cast<size_t>(p + 3) * 4), z3, s);
-          const double zz = s * __ldg(a.ro.cinv + p);
-          gl[p] = zz;
-          z3 = z2, z2 = z1, z1 = zz;
-        }
-      } else {
-        for (int p = 0; p < nr; ++p) {
-          const double* r = a.ro.chol + static_cast<size_t>(p) * (mw + 1);
-          double s = gl[p];
-          for (int j = imax(0, mw - p); j < mw; ++j) s = fma(-__ldg(r + j), gl[p - mw + j], s);
-          gl[p] = s * __ldg(a.ro.cinv + p);
-        }
-        for (int p = nr - 1; p >= 0; --p) {
-          double s = gl[p];
-          for (int k = p + 1; k <= imin(nr - 1, p + mw); ++k)
-            s = fma(-__ldg(a.ro.chol + static_cast<size_t>(k) * (mw + 1) + p - k + mw), gl[k], s);
-          gl[p] = s * __ldg(a.ro.cinv + p);
-        }
-      }
-    }
+    for (int l = tid; l < nl; l += kEval) mass_solve(q + l * nr, a.ro.chol, a.ro.cinv, nr, mw);
     __syncthreads();
   }
   // x = f + P_O (z - y) and, with check, r = P_O q, both by parity

@@ -2,66 +2,86 @@
 // (Algorithm 2), moments and small helpers. All FP64 unless templated on the storage type.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "bte_kernels.h"
+#include "bte_mass.cuh"
 
 namespace bte {
 namespace {
 
-constexpr int kXT = 32;  // x points per CTA in the eigen-basis transforms
-constexpr int kIC = 32;  // eigen (to) or B-spline (from) indices per CTA: a third grid dimension
+constexpr int kXT = 32;  // rows (ordinate, point) per CTA in the eigen-basis transforms
+constexpr int kIC = 32;  // eigen (to) or B-spline (from) indices per CTA
 constexpr int kG = 4;    // output indices per thread in the transforms (one staged operand, four FMAs)
 
 __device__ __forceinline__ bool finite(double v) { return isfinite(v); }
 
+// The rows of both transforms are the pairs m = a nx + x, taken 32 at a time without regard to where an
+// ordinate ends (a tile per ordinate and 32 points left up to 31 of 32 lanes idle in the last tile: 72
+// against 47 us of FP64 work at nx = 100, nr = 128).
+
 // Y[a][i][x] = sum_k Uinv[i][k] F[x][a][k]  (the U^-1 contraction of Algorithm 1) for the kXT
-// points and kIC eigen indices of this CTA: a thread takes kG consecutive i at one x, a warp shares
-// them (the Uinv rows are broadcasts) and its lanes run over x. Flags non-finite inputs (blockIdx.z == 0 only), which is where a NaN handed in
-// by the caller is first seen.
+// rows and kIC eigen indices of this CTA: a thread takes kG consecutive i at one row, a warp shares
+// them (the Uinv rows are broadcasts) and its lanes run over the rows. Bound by the FP64 units. Flags
+// non-finite inputs (blockIdx.y == 0 only), which is where a NaN handed in by the caller is first seen.
 __global__ void x_to_eigen_kernel(const double* __restrict__ F, const double* __restrict__ Uinv,
                                   double* __restrict__ Y, int nx, int nt, int nr,
                                   unsigned* status) {
   extern __shared__ double sm[];
-  const int a = blockIdx.x, x0 = blockIdx.y * kXT, i0 = blockIdx.z * kIC;
-  const int nxt = min(kXT, nx - x0), nit = min(kIC, nr - i0);
+  const int m0 = blockIdx.x * kXT, i0 = blockIdx.y * kIC;
+  const int nmt = min(kXT, nx * nt - m0), nit = min(kIC, nr - i0);
   const int ld = nr + 1;  // padded row
-  const bool check = status && blockIdx.z == 0;
-  for (int idx = threadIdx.x; idx < nxt * nr; idx += blockDim.x) {
-    const int xx = idx / nr, k = idx % nr;
-    const double v = F[(static_cast<size_t>(x0 + xx) * nt + a) * nr + k];
-    if (check && !finite(v)) atomicOr(status, kNonFiniteIn);
-    sm[xx * ld + k] = v;
+  const bool check = status && blockIdx.y == 0;
+  bool bad = false;
+  for (int r = threadIdx.x >> 5; r < nmt; r += blockDim.x >> 5) {
+    const int a = (m0 + r) / nx, x = (m0 + r) % nx;
+    const double* f = F + (static_cast<size_t>(x) * nt + a) * nr;
+    for (int k = threadIdx.x & 31; k < nr; k += 32) {
+      const double v = f[k];
+      bad |= !finite(v);
+      sm[r * ld + k] = v;
+    }
   }
+  if (check && bad) atomicOr(status, kNonFiniteIn);
   __syncthreads();
-  const int ngr = (nit + kG - 1) / kG;
-  for (int idx = threadIdx.x; idx < ngr * kXT; idx += blockDim.x) {
-    const int ib = i0 + (idx / kXT) * kG, xx = idx % kXT;
-    if (xx >= nxt) continue;
-    const int nu = min(kG, i0 + nit - ib);
+  const int ngr = (nit + kG - 1) / kG, xx = threadIdx.x % kXT;
+  if (xx >= nmt) return;
+  const int a = (m0 + xx) / nx, x = (m0 + xx) % nx;
+  double* y = Y + static_cast<size_t>(a) * nr * nx + x;
+  const double* f = sm + xx * ld;
+  for (int grp = threadIdx.x / kXT; grp < ngr; grp += blockDim.x / kXT) {
+    const int ib = i0 + grp * kG, nu = min(kG, i0 + nit - ib);
     const double* u = Uinv + static_cast<size_t>(ib) * nr;
     double s[kG];
 #pragma unroll
     for (int g = 0; g < kG; ++g) s[g] = 0.0;
-    for (int k = 0; k < nr; ++k) {
-      const double f = sm[xx * ld + k];
+    if (nu == kG) {
+#pragma unroll 4
+      for (int k = 0; k < nr; ++k) {
+        const double fv = f[k];
 #pragma unroll
-      for (int g = 0; g < kG; ++g)
-        if (g < nu) s[g] = fma(__ldg(u + static_cast<size_t>(g) * nr + k), f, s[g]);
+        for (int g = 0; g < kG; ++g) s[g] = fma(__ldg(u + static_cast<size_t>(g) * nr + k), fv, s[g]);
+      }
+    } else {
+      for (int k = 0; k < nr; ++k)
+#pragma unroll
+        for (int g = 0; g < kG; ++g)
+          if (g < nu) s[g] = fma(__ldg(u + static_cast<size_t>(g) * nr + k), f[k], s[g]);
     }
 #pragma unroll
     for (int g = 0; g < kG; ++g)
-      if (g < nu) Y[(static_cast<size_t>(a) * nr + ib + g) * nx + x0 + xx] = s[g];
+      if (g < nu) y[static_cast<size_t>(ib + g) * nx] = s[g];
   }
 }
 
-// Y2[b] = s_b M_b Y[b] for every (ordinate, eigen-index) pair b = a nr + i, M_b = M + b mstride
-// (mstride = nx^2: the per-pair Q_ij of Algorithm 1; 0: one shared matrix), s_b = lam[i] mu[a]
-// when lam is given, else 1. One CTA per pair; a warp owns 32 consecutive rows, lane l sums the
-// columns c = l + 32 k of all 32 rows (each Q row chunk a coalesced 256-byte load), and a
-// transpose reduction (shuffle offsets 16, 8, 4, 2, 1 exchanging half of the remaining rows) leaves
-// row r0 + l's sum on lane l: 31 FP64 additions per lane for 32 rows instead of 5 per row and lane.
-__global__ void x_matvec_kernel(const double* __restrict__ M, size_t mstride, const double* __restrict__ lam,
+// Y2[b] = s_b M_b Y[b] for every (ordinate, eigen-index) pair b = a nr + i; MT holds the transposes,
+// M_b^T = MT + b mstride (mstride = nx^2: the per-pair Q_ij of Algorithm 1; 0: one shared matrix),
+// s_b = lam[i] mu[a] when lam is given, else 1. One CTA per pair, one thread per row: a column of M is
+// one coalesced read and every FP64 instruction is an FMA of the product (with M by rows a warp spent
+// a fifth of them on its transposing reduction: 105 us on the medium grid, where the FMAs take 61
+// at 1.1 TFLOP/s and the 268 MB 40).
+__global__ void x_matvec_kernel(const double* __restrict__ MT, size_t mstride, const double* __restrict__ lam,
                                 const double* __restrict__ mu, const double* __restrict__ Y,
                                 double* __restrict__ Y2, int nx, int nr) {
   extern __shared__ double ys[];
@@ -69,70 +89,84 @@ __global__ void x_matvec_kernel(const double* __restrict__ M, size_t mstride, co
   const double* y = Y + b * nx;
   for (int i = threadIdx.x; i < nx; i += blockDim.x) ys[i] = y[i];
   __syncthreads();
-  const double sb = lam ? lam[b % nr] * mu[b / nr] : 1.0;
-  const double* Mb = M + b * mstride;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  for (int r0 = 32 * warp; r0 < nx; r0 += 32 * nw) {
-    const int nrow = min(32, nx - r0);
-    const double* q = Mb + static_cast<size_t>(r0) * nx;
-    double acc[32];
+  const double* Mb = MT + b * mstride;
+  for (int r = threadIdx.x; r < nx; r += blockDim.x) {
+    const double* q = Mb + r;
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    int c = 0;
+    for (; c + 16 <= nx; c += 16) {
+      double v[16];
 #pragma unroll
-    for (int rr = 0; rr < 32; ++rr) acc[rr] = 0.0;
-    for (int c = lane; c < nx; c += 32) {
-      const double yc = ys[c];
+      for (int k = 0; k < 16; ++k) v[k] = __ldg(q + static_cast<size_t>(c + k) * nx);
 #pragma unroll
-      for (int rr = 0; rr < 32; ++rr)
-        if (rr < nrow) acc[rr] = fma(__ldg(q + static_cast<size_t>(rr) * nx + c), yc, acc[rr]);
+      for (int k = 0; k < 16; ++k) acc[k & 3] = fma(v[k], ys[c + k], acc[k & 3]);
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const bool hi = (lane & o) != 0;
-#pragma unroll
-      for (int k = 0; k < o; ++k) {
-        const double send = hi ? acc[k] : acc[k + o];
-        const double keep = hi ? acc[k + o] : acc[k];
-        acc[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-      }
-    }
-    if (lane < nrow) Y2[b * nx + r0 + lane] = sb * acc[0];
+    for (; c < nx; ++c) acc[0] = fma(__ldg(q + static_cast<size_t>(c) * nx), ys[c], acc[0]);
+    const double s = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+    Y2[b * nx + r] = lam ? lam[b % nr] * mu[b / nr] * s : s;
   }
 }
 
-// F[x][a][k] = sum_i U[k][i] Y2[a][i][x] for the kXT points and kIC B-spline indices of this CTA:
-// a thread takes kG consecutive k at one x, a warp shares them (the U rows are broadcasts) and its
-// lanes run over x (consecutive shared-memory words); flags non-finite results.
+// In-place transpose of consecutive n x n matrices: tile pair (blockIdx.x <= blockIdx.y) of matrix
+// blockIdx.z + z0.
+__global__ void transpose_blocks_kernel(double* __restrict__ M, int n, size_t z0) {
+  if (blockIdx.x > blockIdx.y) return;
+  __shared__ double a[32][33], b[32][33];
+  double* m = M + (z0 + blockIdx.z) * n * n;
+  const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32, tx = threadIdx.x & 31;
+  for (int ty = threadIdx.x >> 5; ty < 32; ty += blockDim.x >> 5) {
+    if (r0 + ty < n && c0 + tx < n) a[ty][tx] = m[static_cast<size_t>(r0 + ty) * n + c0 + tx];
+    if (c0 + ty < n && r0 + tx < n) b[ty][tx] = m[static_cast<size_t>(c0 + ty) * n + r0 + tx];
+  }
+  __syncthreads();
+  for (int ty = threadIdx.x >> 5; ty < 32; ty += blockDim.x >> 5) {
+    if (r0 + ty < n && c0 + tx < n) m[static_cast<size_t>(r0 + ty) * n + c0 + tx] = b[tx][ty];
+    if (c0 + ty < n && r0 + tx < n) m[static_cast<size_t>(c0 + ty) * n + r0 + tx] = a[tx][ty];
+  }
+}
+
+// F[x][a][k] = sum_i U[k][i] Y2[a][i][x] for the kXT rows and kIC B-spline indices of this CTA:
+// a thread takes kG consecutive k at one row, a warp shares them (the U rows are broadcasts) and its
+// lanes run over the rows (consecutive shared-memory words); flags non-finite results.
 __global__ void x_from_eigen_kernel(const double* __restrict__ Y2, const double* __restrict__ U,
                                     double* __restrict__ F, int nx, int nt, int nr,
                                     unsigned* status) {
   extern __shared__ double sm[];
-  const int a = blockIdx.x, x0 = blockIdx.y * kXT, k0 = blockIdx.z * kIC;
-  const int nxt = min(kXT, nx - x0), nkt = min(kIC, nr - k0);
-  for (int idx = threadIdx.x; idx < nr * kXT; idx += blockDim.x) {
-    const int i = idx / kXT, xx = idx % kXT;
-    sm[i * (kXT + 1) + xx] = xx < nxt ? Y2[(static_cast<size_t>(a) * nr + i) * nx + x0 + xx] : 0.0;
-  }
+  const int m0 = blockIdx.x * kXT, k0 = blockIdx.y * kIC;
+  const int nmt = min(kXT, nx * nt - m0), nkt = min(kIC, nr - k0), xx = threadIdx.x % kXT;
+  const int a = (m0 + xx) / nx, x = (m0 + xx) % nx;
+  const double* y2 = Y2 + static_cast<size_t>(a) * nr * nx + x;
+  for (int i = threadIdx.x / kXT; i < nr; i += blockDim.x / kXT)
+    sm[i * (kXT + 1) + xx] = xx < nmt ? y2[static_cast<size_t>(i) * nx] : 0.0;
   __syncthreads();
+  if (xx >= nmt) return;
   bool bad = false;
   const int ngr = (nkt + kG - 1) / kG;
-  for (int idx = threadIdx.x; idx < ngr * kXT; idx += blockDim.x) {
-    const int kb = k0 + (idx / kXT) * kG, xx = idx % kXT;
-    if (xx >= nxt) continue;
-    const int nu = min(kG, k0 + nkt - kb);
+  double* f = F + (static_cast<size_t>(x) * nt + a) * nr;
+  for (int grp = threadIdx.x / kXT; grp < ngr; grp += blockDim.x / kXT) {
+    const int kb = k0 + grp * kG, nu = min(kG, k0 + nkt - kb);
     const double* u = U + static_cast<size_t>(kb) * nr;
     double s[kG];
 #pragma unroll
     for (int g = 0; g < kG; ++g) s[g] = 0.0;
-    for (int i = 0; i < nr; ++i) {
-      const double y = sm[i * (kXT + 1) + xx];
+    if (nu == kG) {
+#pragma unroll 4
+      for (int i = 0; i < nr; ++i) {
+        const double y = sm[i * (kXT + 1) + xx];
 #pragma unroll
-      for (int g = 0; g < kG; ++g)
-        if (g < nu) s[g] = fma(__ldg(u + static_cast<size_t>(g) * nr + i), y, s[g]);
+        for (int g = 0; g < kG; ++g) s[g] = fma(__ldg(u + static_cast<size_t>(g) * nr + i), y, s[g]);
+      }
+    } else {
+      for (int i = 0; i < nr; ++i)
+#pragma unroll
+        for (int g = 0; g < kG; ++g)
+          if (g < nu) s[g] = fma(__ldg(u + static_cast<size_t>(g) * nr + i), sm[i * (kXT + 1) + xx], s[g]);
     }
 #pragma unroll
     for (int g = 0; g < kG; ++g)
       if (g < nu) {
         bad |= !finite(s[g]);
-        F[(static_cast<size_t>(x0 + xx) * nt + a) * nr + kb + g] = s[g];
+        f[kb + g] = s[g];
       }
   }
   if (status && bad) atomicOr(status, kNonFinite);
@@ -253,46 +287,8 @@ __global__ void residual_kernel(const double* __restrict__ X, const double* __re
     }
   }
   __syncthreads();
-  // g_l <- M_v^-1 g_l, M_v = R R^T: R y = g_l (p ascending), then R^T z = y (p descending), one
-  // thread per harmonic; for the cubic band (w = 3) the last three values stay in registers
-  for (int l = threadIdx.x; l < nl; l += blockDim.x) {
-    double* gl = g + l * nr;
-    if (w == 3) {
-      double y1 = 0.0, y2 = 0.0, y3 = 0.0;   // y[p-1], y[p-2], y[p-3]
-      for (int p = 0; p < nr; ++p) {
-        const double* rrow = ro.chol + static_cast<size_t>(p) * 4;   // R[p][p-3], R[p][p-2], R[p][p-1], R[p][p]
-        double s = fma(-__ldg(rrow + 2), y1, gl[p]);
-        s = fma(-__ldg(rrow + 1), y2, s);
-        s = fma(-__ldg(rrow), y3, s);
-        const double y = s * __ldg(ro.cinv + p);
-        gl[p] = y;
-        y3 = y2, y2 = y1, y1 = y;
-      }
-      double z1 = 0.0, z2 = 0.0, z3 = 0.0;   // z[p+1], z[p+2], z[p+3]
-      for (int p = nr - 1; p >= 0; --p) {
-        double s = gl[p];
-        if (p + 1 < nr) s = fma(-__ldg(ro.chol + static_cast<size_t>(p + 1) * 4 + 2), z1, s);
-        if (p + 2 < nr) s = fma(-__ldg(ro.chol + static_cast<size_t>(p + 2) * 4 + 1), z2, s);
-        if (p + 3 < nr) s = fma(-__ldg(ro.chol + static_cast<size_t>(p + 3) * 4), z3, s);
-        const double z = s * __ldg(ro.cinv + p);
-        gl[p] = z;
-        z3 = z2, z2 = z1, z1 = z;
-      }
-    } else {
-      for (int p = 0; p < nr; ++p) {
-        const double* rrow = ro.chol + static_cast<size_t>(p) * (w + 1);   // rrow[j] = R[p][p - w + j]
-        double s = gl[p];
-        for (int j = max(0, w - p); j < w; ++j) s = fma(-__ldg(rrow + j), gl[p - w + j], s);
-        gl[p] = s * __ldg(ro.cinv + p);
-      }
-      for (int p = nr - 1; p >= 0; --p) {
-        double s = gl[p];
-        const int kmax = min(nr - 1, p + w);
-        for (int k = p + 1; k <= kmax; ++k) s = fma(-__ldg(ro.chol + static_cast<size_t>(k) * (w + 1) + p - k + w), gl[k], s);
-        gl[p] = s * __ldg(ro.cinv + p);
-      }
-    }
-  }
+  // g_l <- M_v^-1 g_l, one thread per harmonic
+  for (int l = threadIdx.x; l < nl; l += blockDim.x) mass_solve(g + l * nr, ro.chol, ro.cinv, nr, w);
   __syncthreads();
   double mr = 0.0, mb = 0.0, mx = 0.0;
   for (int v = threadIdx.x; v < nv; v += blockDim.x) {
@@ -410,28 +406,33 @@ static void set_x_transform_smem() {
 void launch_x_to_eigen(const double* F, const double* Uinv, double* Y, int nx, int nt, int nr,
                        unsigned* status, cudaStream_t st) {
   set_x_transform_smem();
-  dim3 grid(nt, (nx + kXT - 1) / kXT, (nr + kIC - 1) / kIC);
+  dim3 grid((nx * nt + kXT - 1) / kXT, (nr + kIC - 1) / kIC);
   const size_t smem = sizeof(double) * kXT * (nr + 1);
   x_to_eigen_kernel<<<grid, 256, smem, st>>>(F, Uinv, Y, nx, nt, nr, status);
 }
 
-void launch_x_matvec(const double* M, bool per_pair, const double* lam, const double* mu, const double* Y,
+void launch_x_matvec(const double* MT, bool per_pair, const double* lam, const double* mu, const double* Y,
                      double* Y2, int nx, int nt, int nr, cudaStream_t st) {
-  const int groups = (nx + 31) / 32;
-  const int threads = 32 * (groups < 8 ? groups : 8);
+  const int threads = std::min(256, (nx + 31) / 32 * 32);
   x_matvec_kernel<<<nt * nr, threads, sizeof(double) * nx, st>>>(
-      M, per_pair ? static_cast<size_t>(nx) * nx : 0, lam, mu, Y, Y2, nx, nr);
+      MT, per_pair ? static_cast<size_t>(nx) * nx : 0, lam, mu, Y, Y2, nx, nr);
 }
 
-void launch_x_apply_q(const double* Q, const double* Y, double* Y2, int nx, int nt, int nr,
+void launch_x_apply_q(const double* QT, const double* Y, double* Y2, int nx, int nt, int nr,
                       cudaStream_t st) {
-  launch_x_matvec(Q, true, nullptr, nullptr, Y, Y2, nx, nt, nr, st);
+  launch_x_matvec(QT, true, nullptr, nullptr, Y, Y2, nx, nt, nr, st);
+}
+
+void launch_transpose_blocks(double* M, int n, size_t count, cudaStream_t st) {
+  const unsigned t = static_cast<unsigned>((n + 31) / 32);
+  for (size_t z = 0; z < count; z += 32768)
+    transpose_blocks_kernel<<<dim3(t, t, static_cast<unsigned>(std::min<size_t>(32768, count - z))), 256, 0, st>>>(M, n, z);
 }
 
 void launch_x_from_eigen(const double* Y2, const double* U, double* F, int nx, int nt, int nr,
                          unsigned* status, cudaStream_t st) {
   set_x_transform_smem();
-  dim3 grid(nt, (nx + kXT - 1) / kXT, (nr + kIC - 1) / kIC);
+  dim3 grid((nx * nt + kXT - 1) / kXT, (nr + kIC - 1) / kIC);
   const size_t smem = sizeof(double) * nr * (kXT + 1);
   x_from_eigen_kernel<<<grid, 256, smem, st>>>(Y2, U, F, nx, nt, nr, status);
 }
