@@ -569,7 +569,7 @@ bte_status alloc_window(bte_handle* h) {
   const size_t ts = b.fp64 ? sizeof(double) : sizeof(float), nx = o.nx, rows = static_cast<size_t>(w.np) * 32;
   unsigned char *base = nullptr, *slope = nullptr, *T = nullptr, *U = nullptr;
   BTE_TRY(dalloc(h, &base, ts * rows * w.NW));
-  BTE_TRY(dalloc(h, &slope, ts * rows * (w.RS + 1) * 32));
+  if (b.fp64) BTE_TRY(dalloc(h, &slope, ts * rows * (w.RS + 1) * 32));
   BTE_TRY(dalloc(h, &T, ts * nx * bte::window_t_count(w)));
   BTE_TRY(dalloc(h, &U, ts * nx * bte::window_u_count(w)));
   BTE_TRY(dalloc(h, &b.slotj, nx * bte::window_slot_count(w)));
@@ -587,19 +587,16 @@ bte_status alloc_window(bte_handle* h) {
 bte_status upload_window(bte_handle* h) {
   std::vector<double> base, slope;
   bte::window_tables(h->win.w, h->ops, base, slope);
-  auto put = [&](void* dst, const std::vector<double>& src) -> bte_status {
-    if (h->win.fp64) {
-      BTE_CUDA(h, cudaMemcpyAsync(dst, src.data(), sizeof(double) * src.size(), cudaMemcpyHostToDevice, h->st));
-      BTE_CUDA(h, cudaStreamSynchronize(h->st));
-    } else {
-      const std::vector<float> f(src.begin(), src.end());
-      BTE_CUDA(h, cudaMemcpyAsync(dst, f.data(), sizeof(float) * f.size(), cudaMemcpyHostToDevice, h->st));
-      BTE_CUDA(h, cudaStreamSynchronize(h->st));
-    }
-    return BTE_OK;
-  };
-  BTE_TRY(put(h->win.base, base));
-  return put(h->win.slope, slope);
+  if (h->win.fp64) {
+    BTE_TRY(upload(h, static_cast<double*>(h->win.base), base));
+    BTE_TRY(upload(h, static_cast<double*>(h->win.slope), slope));
+    BTE_CUDA(h, cudaStreamSynchronize(h->st));
+  } else {
+    const std::vector<float> blocks = bte::window_blocks(h->win.w, base, slope);
+    BTE_TRY(upload(h, static_cast<float*>(h->win.base), blocks));
+    BTE_CUDA(h, cudaStreamSynchronize(h->st));
+  }
+  return BTE_OK;
 }
 
 bool valid_cfg(const bte_config* c, std::string& why) {

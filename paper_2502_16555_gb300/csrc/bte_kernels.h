@@ -207,6 +207,7 @@ struct WindowBuffers {
   WindowPlan w;
   bool fp64 = false;
   void *base = nullptr, *slope = nullptr;  // row templates: values without and per unit of the field
+                                           // (FP32: window_blocks in base)
   void *T = nullptr, *U = nullptr;         // factors, window_t_count / window_u_count values a point
   signed char* slotj = nullptr;            // window_slot_count a point
   double* W = nullptr;                     // FP64: 128 (NU + 32) values a point
@@ -217,6 +218,9 @@ struct WindowBuffers {
 WindowPlan window_plan(int nr, int nl);
 // Templates [np 32][NW] and [np 32][(RS + 1) 32] from the unscaled blocks (M, Cg, Ag_lo, Ag_up).
 void window_tables(const WindowPlan& w, const HostOps& o, std::vector<double>& base, std::vector<double>& slope);
+// The FP32 kernel's form of the templates: [np][RS + 1 + NF / 32] blocks of 32 rows x 32 columns, the
+// 16-byte pieces of row r exchanged by r & 7; a column of another harmonic holds the value per unit field.
+std::vector<float> window_blocks(const WindowPlan& w, const std::vector<double>& base, const std::vector<double>& slope);
 size_t window_t_count(const WindowPlan& w);
 size_t window_u_count(const WindowPlan& w);
 size_t window_slot_count(const WindowPlan& w);

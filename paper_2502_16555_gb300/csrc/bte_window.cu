@@ -164,28 +164,40 @@ __device__ __forceinline__ void tmem_st1(uint32_t taddr, float v) {
 
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
-// 32 consecutive template values of a row: base + E slope (slope NULL: base)
-__device__ __forceinline__ void row_values(const float* __restrict__ base, const float* __restrict__ slope, float E,
-                                           float (&v)[32]) {
+// Row r of a 32 x 32 block stored with its 16-byte pieces exchanged (piece q of row r at place
+// q ^ (r & 7), so that a warp's lanes, one row each, meet different banks).
+__device__ __forceinline__ void load_row(const float* block, int r, float (&v)[32]) {
+  const float4* p = reinterpret_cast<const float4*>(block + r * 32);
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
-    const float4 b = __ldg(reinterpret_cast<const float4*>(base) + q);
-    v[4 * q] = b.x, v[4 * q + 1] = b.y, v[4 * q + 2] = b.z, v[4 * q + 3] = b.w;
-  }
-  if (slope) {
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const float4 s = __ldg(reinterpret_cast<const float4*>(slope) + q);
-      v[4 * q] = fmaf(E, s.x, v[4 * q]), v[4 * q + 1] = fmaf(E, s.y, v[4 * q + 1]);
-      v[4 * q + 2] = fmaf(E, s.z, v[4 * q + 2]), v[4 * q + 3] = fmaf(E, s.w, v[4 * q + 3]);
-    }
+    const float4 x = p[q ^ (r & 7)];
+    v[4 * q] = x.x, v[4 * q + 1] = x.y, v[4 * q + 2] = x.z, v[4 * q + 3] = x.w;
   }
 }
-
-__device__ __forceinline__ void store32(float* dst, const float (&v)[32]) {
+__device__ __forceinline__ void store_row(float* block, int r, const float (&v)[32]) {
+  float4* p = reinterpret_cast<float4*>(block + r * 32);
 #pragma unroll
-  for (int q = 0; q < 8; ++q)
-    reinterpret_cast<float4*>(dst)[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+  for (int q = 0; q < 8; ++q) p[q ^ (r & 7)] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+}
+// A template row at the field E: the columns of its own harmonic (bits of own) stand as they are, the
+// others are per unit of the field.
+__device__ __forceinline__ void scale_row(float (&v)[32], unsigned own, float E) {
+#pragma unroll
+  for (int c = 0; c < 32; ++c) v[c] = (own >> c) & 1u ? v[c] : E * v[c];
+}
+
+// global -> shared, completion counted on bar; shared -> global in this thread's bulk group
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(saddr(dst)),
+               "l"(src), "r"(bytes), "r"(saddr(bar))
+               : "memory");
+}
+__device__ __forceinline__ void bulk_store(void* dst, const void* src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(saddr(src)), "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ void expect_tx(uint64_t* bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(saddr(bar)), "r"(bytes) : "memory");
 }
 
 // Where p: the 8 values v[0 .. 7] to row, (key, inv) to rec (shared-memory addresses), without a branch.
@@ -201,12 +213,13 @@ __device__ __forceinline__ void post_row(bool p, uint32_t row, const float (&v)[
 
 struct FactorArgs {
   WindowPlan w;
-  const void* base;    // [np 32][NW] row templates (T)
-  const void* slope;   // [np 32][(RS + 1) 32]
+  const void* base;    // row templates: FP64 [np 32][NW], FP32 window_blocks
+  const void* slope;   // FP64 [np 32][(RS + 1) 32]
   const double* E;
   double Eu;
   void* T;             // [nx][np][32][NS]
-  void* U;             // [nx][np][1024 + 32 NU]: inv(U11), then the pivot rows over the window
+  void* U;             // [nx][np][1024 + 32 NU]: inv(U11), then the pivot rows over the window (FP64 by
+                       // rows, FP32 in 32 x 32 blocks)
   signed char* slotj;  // [nx][np][NS]: the pivot index of each slot, -1 if its row stays
   double* W;           // FP64: the window [nx][128][NU + 32]
   int* rows;           // FP64: the padded row in each slot [nx][128]
@@ -232,23 +245,25 @@ __global__ void __launch_bounds__(kThreads, 2) window_lu_tc_kernel(const FactorA
   float* Tlo = Thi + kSlots * kPW;
   float* Bhi = Tlo + kSlots * kPW;
   float* Blo = Bhi + w.NU * kPW;
+  float* t0 = Blo + w.NU * kPW;  // the entering rows' template of the next panel's columns
   __shared__ __align__(16) float prow[2][4][8];    // each warp's candidate row in the current sub-block
   __shared__ __align__(16) uint2 keys[2][4];       // its magnitude and lane, and 1 / its pivot
   __shared__ __align__(16) float pblk[2][8][24];   // a sub-block's pivot rows over the other columns
   __shared__ signed char slotj[2][kSlots];
-  __shared__ float u11[2][32 * 33];
+  __shared__ float u11[32 * 33];
   __shared__ float ui[32 * 17];  // inverses of U11's 16 x 16 diagonal blocks
-  __shared__ __align__(8) uint64_t bar_next, bar_rest;
+  // products of chunk s + 1, of the rest; templates of the ring and far columns, of the panel's; U11 inverted
+  __shared__ __align__(8) uint64_t bar_next, bar_rest, bar_tmpl, bar_t0, bar_u;
   __shared__ uint32_t tmem_base;
   __shared__ int gave_up;
 
   const int pt = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, quad = warp & 3;
-  const int slot = quad * 32 + lane, np = w.np, NW = w.NW, NS = w.NS, RS = w.RS, RC = w.RC, g = w.g;
-  const int NWR = (RS + 1) * 32;
+  const int slot = quad * 32 + lane, np = w.np, NS = w.NS, RS = w.RS, RC = w.RC, g = w.g;
+  const int nch = RS + 1 + w.NF / 32;  // template chunks of a row: the panel's, the ring's, the far ones
   const bool panel_warp = warp < 4;
   const int npw = NS / 32;  // panel warps that hold rows
-  const float* base = static_cast<const float*>(a.base);
-  const float* slope = static_cast<const float*>(a.slope);
+  const float* tmpl = static_cast<const float*>(a.base);
+  auto block = [&](int t, int ch) { return tmpl + (static_cast<size_t>(t) * nch + ch) * 1024; };
   const float E = static_cast<float>(a.E ? a.E[pt] : a.Eu);
   float* Tg = static_cast<float*>(a.T) + static_cast<size_t>(pt) * np * 32 * NS;
   const size_t ustride = 1024 + 32 * static_cast<size_t>(w.NU);
@@ -258,6 +273,9 @@ __global__ void __launch_bounds__(kThreads, 2) window_lu_tc_kernel(const FactorA
   if (tid == 0) {
     mbar_init(&bar_next, 1);
     mbar_init(&bar_rest, 1);
+    mbar_init(&bar_tmpl, 1);
+    mbar_init(&bar_t0, 1);
+    mbar_init(&bar_u, 1);
     gave_up = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -279,27 +297,28 @@ __global__ void __launch_bounds__(kThreads, 2) window_lu_tc_kernel(const FactorA
   float v[32];
 #pragma unroll
   for (int i = 0; i < 32; ++i) v[i] = 0.f;
+  unsigned rep = 0;  // bit of every harmonic 0 column in a chunk
+  for (int i = 0; i < g; ++i) rep |= 1u << (i * w.nlp);
+  auto own = [&](int j) { return rep << (j & (w.nlp - 1)); };  // columns of row j's harmonic
   // rows of chunks 0 .. RC enter at panel 0, slot by slot
-  const bool valid0 = slot < NS && slot / 32 < np && ((chunk_mask(w, slot / 32) >> lane) & 1u);
+  const int t_in = slot / 32;
+  const bool valid0 = slot < NS && t_in < np && ((chunk_mask(w, t_in) >> lane) & 1u);
   bool act = panel_warp && valid0;
   if (panel_warp) {
-    if (act) row_values(base + static_cast<size_t>(slot) * NW, slope + static_cast<size_t>(slot) * NWR, E, v);
-  } else {
-    for (int d = 1; d <= RS; ++d) {
-      float r[32];
-      if (valid0) row_values(base + static_cast<size_t>(slot) * NW + d * 32, slope + static_cast<size_t>(slot) * NWR + d * 32, E, r);
-      else
-#pragma unroll
-        for (int i = 0; i < 32; ++i) r[i] = 0.f;
-      tmem_st32(tmem + (d % RS) * 32, r);
+    if (act) {
+      load_row(block(t_in, 0), lane, v);
+      scale_row(v, own(lane), E);
     }
-    for (int c = 0; c < w.NF / 32; ++c) {
+  } else {
+    for (int ch = 1; ch < nch; ++ch) {
       float r[32];
-      if (valid0) row_values(base + static_cast<size_t>(slot) * NW + NWR + c * 32, nullptr, 0.f, r);
-      else
 #pragma unroll
-        for (int i = 0; i < 32; ++i) r[i] = 0.f;
-      tmem_st32(tmem + (RS + c) * 32, r);
+      for (int i = 0; i < 32; ++i) r[i] = 0.f;
+      if (valid0) {
+        load_row(block(t_in, ch), lane, r);
+        if (ch <= RS) scale_row(r, own(lane), E);
+      }
+      tmem_st32(tmem + (ch <= RS ? ch % RS : ch - 1) * 32, r);
     }
     tmem_wait_st();
     tc_fence_before();
@@ -390,15 +409,16 @@ __global__ void __launch_bounds__(kThreads, 2) window_lu_tc_kernel(const FactorA
 #pragma unroll
           for (int k = 0; k < 8; ++k) v[24 + k] = w8[k];
         }
+        if (s > 0) mbar_wait(&bar_u, (s - 1) & 1, &gave_up, a.status);
         if (pj >= 0) {
 #pragma unroll
-          for (int k = 0; k < 32; ++k) u11[par][pj * 33 + k] = k >= pj ? v[k] : 0.f;
+          for (int k = 0; k < 32; ++k) u11[pj * 33 + k] = k >= pj ? v[k] : 0.f;
 #pragma unroll
           for (int k = 0; k < 32; ++k)
             if (k >= pj) v[k] = 0.f;
         }
         if (warp == 0 && !((mask >> lane) & 1u))
-          for (int k = 0; k < 32; ++k) u11[par][lane * 33 + k] = k == lane ? 1.f : 0.f;
+          for (int k = 0; k < 32; ++k) u11[lane * 33 + k] = k == lane ? 1.f : 0.f;
         // T of this panel: global (column k of the 32, slots contiguous) and the split operand
 #pragma unroll
         for (int k = 0; k < 32; ++k) Tg[(static_cast<size_t>(s) * 32 + k) * NS + slot] = v[k];
@@ -424,9 +444,14 @@ __global__ void __launch_bounds__(kThreads, 2) window_lu_tc_kernel(const FactorA
     __syncthreads();  // T in place, pivots known; the window of the panel before is complete in tensor memory
     tc_fence_after();
     const int j = slotj[par][slot];
-    const int tnew = s + 1 + RC, rnew = tnew * 32 + j;  // the row that takes this slot
-    const bool fresh = j >= 0 && tnew < np && ((chunk_mask(w, tnew) >> j) & 1u);
+    const int tnew = s + 1 + RC;  // a row of chunk tnew takes this slot
+    const bool enter = tnew < np, fresh = j >= 0 && enter && ((chunk_mask(w, tnew) >> j) & 1u);
+    const unsigned mine = own(j & 31);
     if (dmax > 0) {
+      if (tid == 32 && enter) {
+        expect_tx(&bar_t0, 4096);
+        bulk_load(t0, block(tnew, 0), 4096, &bar_t0);
+      }
       // the pivot rows' window, split, as the K-major B operand: chunk s + 1, which the next panel needs,
       // by the panel warps, whose product is issued at once, the others by the other half
       const int cnt = dmax + (nfc - fc0);
@@ -499,7 +524,19 @@ __global__ void __launch_bounds__(kThreads, 2) window_lu_tc_kernel(const FactorA
             if (r >= 3) col = (RS + fc0) * 32 + (r - 3) * 256, n = imin(256, (nfc - fc0) * 32 - (r - 3) * 256);
             if (n > 0) issue(col, n);
           }
-          if (lane == 0) mma_commit(&bar_rest);
+          if (lane == 0) {
+            mma_commit(&bar_rest);
+            mbar_wait(&bar_next, par, &gave_up, a.status);
+            mbar_wait(&bar_rest, par, &gave_up, a.status);
+            if (enter) {
+              // the products are done: B's remainders give way to the entering rows' templates, chunk d of
+              // the ring to template chunk d - 1, the chunk that enters (in the place of chunk s + 1) to RS
+              const int far = nfc - fc0, last = s + 1 + RS < np ? RS + 1 : dmax;
+              expect_tx(&bar_tmpl, 4096u * (last - 1 + far));
+              for (int d = 2; d <= last; ++d) bulk_load(Blo + ((s + d) % RS) * 1024, block(tnew, d - 1), 4096, &bar_tmpl);
+              for (int c = fc0; c < nfc; ++c) bulk_load(Blo + (RS + c) * 1024, block(tnew, RS + 1 + c), 4096, &bar_tmpl);
+            }
+          }
           __syncwarp();
         }
       }
@@ -508,7 +545,7 @@ __global__ void __launch_bounds__(kThreads, 2) window_lu_tc_kernel(const FactorA
     if (warp == 4) {
       // inv(U11) by one warp: the two 16 x 16 diagonal blocks at once (one lane a column, the rows in
       // turning registers), then -inv(A) B inv(D)
-      const float* u = u11[par];
+      const float* u = u11;
       const int blk = lane >> 4, c = lane & 15;
       const float* d = u + blk * 16 * 34;
       const float rd = recip(d[c * 34]);
@@ -550,96 +587,104 @@ __global__ void __launch_bounds__(kThreads, 2) window_lu_tc_kernel(const FactorA
       __syncwarp();
 #pragma unroll
       for (int r = 0; r < 8; ++r) Up[(blk * 8 + r) * 32 + 16 + c] = y[r];
+      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(&bar_u)) : "memory");
     }
     if (dmax == 0) break;
-    float* urow = Up + 1024 + static_cast<size_t>(imax(j, 0)) * w.NU;
-    const float* nb = base + static_cast<size_t>(imax(rnew, 0)) * NW;
-    const float* ns = slope + static_cast<size_t>(imax(rnew, 0)) * NWR;
     if (panel_warp) {
-      // the next panel's columns: updated rows from tensor memory, the entering rows from the templates
+      // the next panel's columns: updated rows from tensor memory, the entering rows from the template; the
+      // pivot rows go to the place of B's heads as U, from where they are copied out below
       float r[32];
-      if (fresh) row_values(nb, ns, E, v);
-      else
 #pragma unroll
-        for (int i = 0; i < 32; ++i) v[i] = 0.f;
+      for (int i = 0; i < 32; ++i) v[i] = 0.f;
+      if (enter) {
+        mbar_wait(&bar_t0, par, &gave_up, a.status);
+        if (fresh) {
+          load_row(t0, j, v);
+          scale_row(v, mine, E);
+        }
+      }
       mbar_wait(&bar_next, par, &gave_up, a.status);
       tc_fence_after();
       tmem_ld32(tmem + ((s + 1) % RS) * 32, r);
-      tc_fence_before();
-      __syncwarp();
-      asm volatile("bar.arrive 2, %0;" ::"r"(kThreads) : "memory");
       if (j >= 0) {
-        store32(urow, r);
+        store_row(Bhi + ((s + 1) % RS) * 1024, j, r);
         act = fresh;
       } else {
 #pragma unroll
         for (int i = 0; i < 32; ++i) v[i] = r[i];
       }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      tc_fence_before();
+      __syncwarp();
+      asm volatile("bar.arrive 2, %0;" ::"r"(kThreads) : "memory");
     } else {
-      if (fresh) {  // the entering row's templates into L1 while the tensor cores work
-        for (int d = 1; d <= RS; ++d) {
-          asm volatile("prefetch.global.L1 [%0];" ::"l"(nb + d * 32));
-          asm volatile("prefetch.global.L1 [%0];" ::"l"(ns + d * 32));
-        }
-        for (int c = fc0; c < nfc; ++c) asm volatile("prefetch.global.L1 [%0];" ::"l"(nb + NWR + c * 32));
-      }
       mbar_wait(&bar_rest, par, &gave_up, a.status);
       tc_fence_after();
-      for (int d = 2; d <= dmax; ++d) {
-        const uint32_t t = tmem + ((s + d) % RS) * 32;
+      if (enter) mbar_wait(&bar_tmpl, par, &gave_up, a.status);
+      const int cnt = dmax - 1 + nfc - fc0;
+#pragma unroll 1
+      for (int q = 0; q < cnt; ++q) {
+        const bool ring = q < dmax - 1;
+        const int at = ring ? (s + 2 + q) % RS : RS + fc0 + q - (dmax - 1);
         float r[32];
-        tmem_ld32(t, r);
+        tmem_ld32(tmem + at * 32, r);
         if (j >= 0) {
-          store32(urow + (d - 1) * 32, r);
-          if (fresh) row_values(nb + (d - 1) * 32, ns + (d - 1) * 32, E, r);
-          else
+          store_row(Bhi + at * 1024, j, r);
 #pragma unroll
-            for (int i = 0; i < 32; ++i) r[i] = 0.f;
+          for (int i = 0; i < 32; ++i) r[i] = 0.f;
+          if (fresh) {
+            load_row(Blo + at * 1024, j, r);
+            if (ring) scale_row(r, mine, E);
+          }
         }
-        tmem_st32(t, r);
-      }
-      for (int c = fc0; c < nfc; ++c) {
-        const uint32_t t = tmem + (RS + c) * 32;
-        float r[32];
-        tmem_ld32(t, r);
-        if (j >= 0) {
-          store32(urow + (RS + c) * 32, r);
-          if (fresh) row_values(nb + NWR + c * 32, nullptr, 0.f, r);
-          else
-#pragma unroll
-            for (int i = 0; i < 32; ++i) r[i] = 0.f;
-        }
-        tmem_st32(t, r);
+        tmem_st32(tmem + at * 32, r);
       }
       tmem_wait_st();
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
-      asm volatile("bar.sync 2, %0;" ::"r"(kThreads) : "memory");  // the panel warps have read chunk s + 1
+      asm volatile("bar.sync 2, %0;" ::"r"(kThreads) : "memory");  // U is complete; chunk s + 1 has been read
       tc_fence_after();
+      if (tid == 160) {
+        for (int d = 1; d <= dmax; ++d) bulk_store(Up + d * 1024, Bhi + ((s + d) % RS) * 1024, 4096);
+        for (int c = fc0; c < nfc; ++c) bulk_store(Up + (1 + RS + c) * 1024, Bhi + (RS + c) * 1024, 4096);
+        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+      }
       if (s + 1 + RS < np) {
         // chunk s + 1 + RS enters the ring in the place of chunk s + 1: the rows that stay have
         // entries only in its l = 0 columns, so far kept apart
-        const uint32_t t = tmem + ((s + 1) % RS) * 32;
+        const int at = (s + 1) % RS;
+        const uint32_t t = tmem + at * 32;
         float r[32];
-        if (fresh) row_values(nb + RS * 32, ns + RS * 32, E, r);
-        else
 #pragma unroll
-          for (int i = 0; i < 32; ++i) r[i] = 0.f;
+        for (int i = 0; i < 32; ++i) r[i] = 0.f;
+        if (fresh) {
+          load_row(Blo + at * 1024, j, r);
+          scale_row(r, mine, E);
+        }
         tmem_st32(t, r);
         tmem_wait_st();
         for (int i = 0; i < g; ++i) {
           if ((s + 1 + RS) * g + i >= w.nr) break;
           const uint32_t tf = tmem + RS * 32 + s * g + i;
           float x = tmem_ld1(tf);
-          if (fresh) x = fmaf(E, __ldg(ns + RS * 32 + i * w.nlp), __ldg(nb + RS * 32 + i * w.nlp));
-          else if (j >= 0) x = 0.f;
+          if (fresh) {
+            const int c = i * w.nlp;
+            x = Blo[at * 1024 + j * 32 + ((((c >> 2) ^ (j & 7)) << 2) | (c & 3))] * ((mine >> c) & 1u ? 1.f : E);
+          } else if (j >= 0) {
+            x = 0.f;
+          }
           tmem_st1(t + i * w.nlp, x);
           tmem_st1(tf, 0.f);
         }
         tmem_wait_st();
       }
+      // B's heads are written again after the next barrier
+      if (tid == 160) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+      __syncwarp();
       tc_fence_before();
     }
   }
+  if (tid == 160) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
   if (bad) atomicOr(a.status, kZeroPivot);
   tc_fence_before();
   __syncthreads();
@@ -1094,6 +1139,8 @@ __global__ void __launch_bounds__(kThreads) window_substitute_kernel(const Solve
   unsigned char* stage = raw;
   T* b = reinterpret_cast<T*>(raw + static_cast<size_t>(S) * a.stage_bytes);  // padded unknowns, chunk by chunk
   const int npad = (np + RS) * 32;
+  // U's rows: FP64 [32][NU]; FP32 32 x 32 blocks, one per chunk of the window, as load_row reads them
+  constexpr bool blocks = sizeof(T) == 4;
   T* bp = b + npad;  // [2][32] pivot values; the backward pass's 32 partial results
   double* z = a.vec + static_cast<size_t>(pt) * 3 * n + n;
   const double* rho = z + n;
@@ -1160,15 +1207,30 @@ __global__ void __launch_bounds__(kThreads) window_substitute_kernel(const Solve
     const int q = 2 * np - 1 - s;
     mbar_wait(&full[q % S], (q / S) & 1, &gave_up, a.status);
     const T* ui = reinterpret_cast<const T*>(stage + static_cast<size_t>(q % S) * a.stage_bytes);
-    const T* u = ui + 1024 + static_cast<size_t>(row) * NU;
     const T* x = b + (s + 1) * 32;
     const int wr = imin(RS, np - 1 - s) * 32;
     T s0 = T(0), s1 = T(0);
-    for (int c = 4 * sub; c < wr; c += 32) s0 += Vec4<T>::dot(u + c, x + c);
-    const T* uf = u + RS * 32;
-    if (s * g < nfar && s + 1 < np)
-      for (int k = ((s * g) / 32) * 32 + sub; k < nfar; k += 8)
-        if (k >= s * g) s1 = fma(uf[k], b[(w.kf0 + k) * nlp], s1);
+    if constexpr (blocks) {
+      const T* u = ui + 1024 + row * 32 + 4 * sub;
+      const int c4 = 4 * (sub ^ (row & 7));
+      for (int c = 0; c < wr; c += 32) s0 += Vec4<T>::dot(u + c * 32, x + c + c4);
+      if (s * g < nfar && s + 1 < np)
+        for (int k = ((s * g) / 32) * 32; k < nfar; k += 32) {
+          const T* uf = u + (RS * 32 + k) * 32;
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int kk = k + c4 + e;
+            if (kk >= s * g && kk < nfar) s1 = fma(uf[e], b[(w.kf0 + kk) * nlp], s1);
+          }
+        }
+    } else {
+      const T* u = ui + 1024 + static_cast<size_t>(row) * NU;
+      for (int c = 4 * sub; c < wr; c += 32) s0 += Vec4<T>::dot(u + c, x + c);
+      const T* uf = u + RS * 32;
+      if (s * g < nfar && s + 1 < np)
+        for (int k = ((s * g) / 32) * 32 + sub; k < nfar; k += 8)
+          if (k >= s * g) s1 = fma(uf[k], b[(w.kf0 + k) * nlp], s1);
+    }
     T acc = s0 + s1;
     acc += __shfl_xor_sync(0xffffffffu, acc, 4);
     acc += __shfl_xor_sync(0xffffffffu, acc, 2);
@@ -1180,7 +1242,7 @@ __global__ void __launch_bounds__(kThreads) window_substitute_kernel(const Solve
     e += __shfl_xor_sync(0xffffffffu, e, 4);
     e += __shfl_xor_sync(0xffffffffu, e, 2);
     e += __shfl_xor_sync(0xffffffffu, e, 1);
-    if (sub == 0) b[s * 32 + row] = e;
+    if (sub == 0) b[s * 32 + row] = (chunk_mask(w, s) >> row) & 1u ? e : T(0);
     __syncthreads();
     if (tid == 0 && q + S < 2 * np) issue(q + S);
   }
@@ -1437,6 +1499,21 @@ void window_tables(const WindowPlan& w, const HostOps& o, std::vector<double>& b
     }
 }
 
+std::vector<float> window_blocks(const WindowPlan& w, const std::vector<double>& base, const std::vector<double>& slope) {
+  const int nch = w.RS + 1 + w.NF / 32, NWR = (w.RS + 1) * 32;
+  std::vector<float> out(static_cast<size_t>(w.np) * nch * 1024);
+  for (int t = 0; t < w.np; ++t)
+    for (int ch = 0; ch < nch; ++ch)
+      for (int r = 0; r < 32; ++r)
+        for (int c = 0; c < 32; ++c) {
+          const size_t row = static_cast<size_t>(t) * 32 + r;
+          const bool ring = ch <= w.RS, mine = !ring || (c & (w.nlp - 1)) == (r & (w.nlp - 1));
+          const double v = mine ? base[row * w.NW + ch * 32 + c] : slope[row * NWR + ch * 32 + c];
+          out[((static_cast<size_t>(t) * nch + ch) * 32 + r) * 32 + (((c >> 2) ^ (r & 7)) << 2) + (c & 3)] = static_cast<float>(v);
+        }
+  return out;
+}
+
 size_t window_t_count(const WindowPlan& w) { return static_cast<size_t>(w.np) * 32 * w.NS; }
 size_t window_u_count(const WindowPlan& w) { return static_cast<size_t>(w.np) * (1024 + 32 * static_cast<size_t>(w.NU)); }
 size_t window_slot_count(const WindowPlan& w) { return static_cast<size_t>(w.np) * w.NS; }
@@ -1457,7 +1534,7 @@ static SolveArgs solve_args(const WindowBuffers& b, MassBand mass, int nt) {
 cudaError_t launch_window_factor(const WindowBuffers& b, const double* E, double Eu, int nx, unsigned* status,
                                  cudaStream_t st) {
   const FactorArgs a = factor_args(b, E, Eu, status);
-  const int smem = 1024 + static_cast<int>(sizeof(float)) * kPW * 2 * (kSlots + b.w.NU);
+  const int smem = 1024 + 4096 + static_cast<int>(sizeof(float)) * kPW * 2 * (kSlots + b.w.NU);
   const cudaError_t e = cudaFuncSetAttribute(window_lu_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   window_lu_tc_kernel<<<nx, kThreads, smem, st>>>(a);
