@@ -548,6 +548,15 @@ bte_status alloc_harmonic(bte_handle* h) {
   const HostOps& o = h->ops;
   BTE_TRY(dalloc(h, &h->win.vec, static_cast<size_t>(o.nx) * 3 * o.nl * o.nr));
   BTE_TRY(dalloc(h, &h->win.fmax_, o.nx));
+  BTE_TRY(dalloc(h, &h->win.minv, o.nr));
+  std::vector<double> minv(o.nr);
+  for (int p = 0; p < o.nr; ++p) {
+    double s = 0.0;
+    for (int k = 0; k < o.nr; ++k) s += std::fabs(o.M[static_cast<size_t>(p) * o.nr + k]);
+    minv[p] = 1.0 / s;
+  }
+  BTE_TRY(upload(h, h->win.minv, minv));
+  BTE_CUDA(h, cudaStreamSynchronize(h->st));
   for (int l = 0; l < o.nl; ++l) {
     double s = 0.0;
     for (int a = 0; a < o.nt; ++a) s += std::fabs(o.TS[static_cast<size_t>(l) * o.nt + a]);

@@ -214,6 +214,7 @@ struct WindowBuffers {
   int* rows = nullptr;                     // FP64: 128 values a point
   double* vec = nullptr;                   // 3 nl nr values a point
   double* fmax_ = nullptr;                 // one value a point
+  double* minv = nullptr;                  // [nr] 1 / sum_k |M_v[p][k]|
 };
 WindowPlan window_plan(int nr, int nl);
 // Templates [np 32][NW] and [np 32][(RS + 1) 32] from the unscaled blocks (M, Cg, Ag_lo, Ag_up).

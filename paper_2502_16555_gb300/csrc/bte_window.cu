@@ -33,6 +33,7 @@
 #include <string>
 #include <vector>
 
+#include "bte_async.cuh"
 #include "bte_handle.h"
 #include "bte_kernels.h"
 #include "bte_mass.cuh"
@@ -45,7 +46,6 @@ namespace {
 constexpr int kPW = 32;      // panel (chunk) width
 constexpr int kSlots = 128;  // row slots: the tensor cores' M
 constexpr int kThreads = 256;
-constexpr long long kWaitCycles = 1ll << 32;  // bounded device waits, about 2 s
 constexpr double kBackwardFloor = 256.0 * 1.1102230246251565e-16;  // as in launch_residual
 
 __host__ __device__ inline int imin(int a, int b) { return a < b ? a : b; }
@@ -57,37 +57,6 @@ __device__ __forceinline__ unsigned chunk_mask(const WindowPlan& w, int s) {
   for (int i = 0; i < w.g; ++i)
     if (s * w.g + i < w.nr) m |= ((w.nl < 32 ? (1u << w.nl) : 0u) - 1u) << (i * w.nlp);
   return m;
-}
-
-__device__ __forceinline__ uint32_t saddr(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
-
-__device__ __forceinline__ void mbar_init(uint64_t* b, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(saddr(b)), "r"(count));
-}
-
-__device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-      : "=r"(ok)
-      : "r"(saddr(b)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
-// Bounded: on expiry the status bit is set, later waits of the CTA return at once and the kernel runs
-// to its end on whatever the buffers hold (every access stays in bounds); the step reports it.
-__device__ __forceinline__ void mbar_wait(uint64_t* b, uint32_t parity, volatile int* gave_up, unsigned* status) {
-  if (mbar_try(b, parity)) return;
-  const long long t0 = clock64();
-  while (!mbar_try(b, parity)) {
-    if (*gave_up) return;
-    if (clock64() - t0 > kWaitCycles) {
-      *gave_up = 1;
-      atomicOr(status, kTimeout);
-      return;
-    }
-  }
 }
 
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -184,20 +153,6 @@ __device__ __forceinline__ void store_row(float* block, int r, const float (&v)[
 __device__ __forceinline__ void scale_row(float (&v)[32], unsigned own, float E) {
 #pragma unroll
   for (int c = 0; c < 32; ++c) v[c] = (own >> c) & 1u ? v[c] : E * v[c];
-}
-
-// global -> shared, completion counted on bar; shared -> global in this thread's bulk group
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(saddr(dst)),
-               "l"(src), "r"(bytes), "r"(saddr(bar))
-               : "memory");
-}
-__device__ __forceinline__ void bulk_store(void* dst, const void* src, uint32_t bytes) {
-  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(saddr(src)), "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ void expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(saddr(bar)), "r"(bytes) : "memory");
 }
 
 // Where p: the 8 values v[0 .. 7] to row, (key, inv) to rec (shared-memory addresses), without a branch.
@@ -579,14 +534,16 @@ __global__ void __launch_bounds__(kThreads, 2) window_lu_tc_kernel(const FactorA
         for (int k = 0; k < 16; ++k) acc = fmaf(-ui[(blk * 8 + r) * 17 + k], t[k], acc);
         y[r] = acc;
       }
+      // by rows, the pieces of a row exchanged like a block's
+      auto at = [&](int r, int col) { return Up + r * 32 + ((((col >> 2) ^ (r & 7)) << 2) | (col & 3)); };
 #pragma unroll
       for (int r = 0; r < 16; ++r) {
-        Up[r * 32 + lane] = lane < 16 ? ui[r * 17 + c] : 0.f;
-        Up[(16 + r) * 32 + lane] = lane < 16 ? 0.f : ui[(16 + r) * 17 + c];
+        *at(r, lane) = lane < 16 ? ui[r * 17 + c] : 0.f;
+        *at(16 + r, lane) = lane < 16 ? 0.f : ui[(16 + r) * 17 + c];
       }
       __syncwarp();
 #pragma unroll
-      for (int r = 0; r < 8; ++r) Up[(blk * 8 + r) * 32 + 16 + c] = y[r];
+      for (int r = 0; r < 8; ++r) *at(blk * 8 + r, 16 + c) = y[r];
       if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(&bar_u)) : "memory");
     }
     if (dmax == 0) break;
@@ -1026,6 +983,7 @@ struct SolveArgs {
   double ts_inf, to_inf;    // infinity norms of T_S and T_O
   double* vec;              // [nx][3 n]: y, z, rho
   double* fmax_;            // [nx] max|f|
+  const double* minv;       // [nr] 1 / sum_k |M_pk|
   double* ratio;
   int* conv;
   double tol, kc_inf, ka_inf;
@@ -1043,6 +1001,7 @@ struct Vec4<float> {
     const float4 x = *reinterpret_cast<const float4*>(a), y = *reinterpret_cast<const float4*>(b);
     return fmaf(x.w, y.w, fmaf(x.z, y.z, fmaf(x.y, y.y, x.x * y.x)));
   }
+  static __device__ __forceinline__ float4 load(const float* a) { return *reinterpret_cast<const float4*>(a); }
 };
 template <>
 struct Vec4<double> {
@@ -1051,21 +1010,36 @@ struct Vec4<double> {
     const double2 z = *reinterpret_cast<const double2*>(a + 2), u = *reinterpret_cast<const double2*>(b + 2);
     return fma(z.y, u.y, fma(z.x, u.x, fma(x.y, y.y, x.x * y.x)));
   }
+  struct Four {
+    double x, y, z, w;
+  };
+  static __device__ __forceinline__ Four load(const double* a) {
+    const double2 p = *reinterpret_cast<const double2*>(a), q = *reinterpret_cast<const double2*>(a + 2);
+    return {p.x, p.y, q.x, q.y};
+  }
 };
 
 constexpr int kEval = 512;  // threads of the projection and residual kernels
 
-// Block-wide maximum of two values; every thread gets the result.
-__device__ __forceinline__ void block_max2(double& p, double& q, double* red) {
+// Running maxima of magnitudes as ordered integers: the FP64 units, whose rate bounds these kernels, take
+// no part (a NaN is above everything and stays).
+using Mag = unsigned long long;
+__device__ __forceinline__ Mag mag(double v) { return static_cast<Mag>(__double_as_longlong(v) & 0x7fffffffffffffffll); }
+__device__ __forceinline__ Mag mag_max(Mag a, Mag b) { return a > b ? a : b; }
+
+// Block-wide maximum of two magnitudes; every thread gets the result.
+__device__ __forceinline__ void block_max2(Mag p, Mag q, Mag* red, double& pm, double& qm) {
   for (int o = 16; o > 0; o >>= 1) {
-    p = fmax(p, __shfl_xor_sync(0xffffffffu, p, o));
-    q = fmax(q, __shfl_xor_sync(0xffffffffu, q, o));
+    p = mag_max(p, __shfl_xor_sync(0xffffffffu, p, o));
+    q = mag_max(q, __shfl_xor_sync(0xffffffffu, q, o));
   }
   __syncthreads();
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = p, red[kEval / 32 + (threadIdx.x >> 5)] = q;
   __syncthreads();
   p = red[0], q = red[kEval / 32];
-  for (int i = 1; i < kEval / 32; ++i) p = fmax(p, red[i]), q = fmax(q, red[kEval / 32 + i]);
+  for (int i = 1; i < kEval / 32; ++i) p = mag_max(p, red[i]), q = mag_max(q, red[kEval / 32 + i]);
+  pm = __longlong_as_double(static_cast<long long>(p));
+  qm = __longlong_as_double(static_cast<long long>(q));
 }
 
 // The solves run in the harmonic basis: y = P_S f, z the harmonic solution (x = f + P_O (z - y)); the
@@ -1080,19 +1054,20 @@ __global__ void __launch_bounds__(kEval) window_project_kernel(const SolveArgs a
   const int nr = a.w.nr, nl = a.w.nl, nt = a.nt, n = nl * nr, nv = nt * nr, hf = nt / 2, hc = (nt + 1) / 2;
   double* fold = reinterpret_cast<double*>(raw);  // 2 hc nr
   double* ys = fold + 2 * hc * nr;                // n
-  __shared__ double red[2 * kEval / 32];
+  __shared__ Mag red[2 * kEval / 32];
   const int pt = blockIdx.x, tid = threadIdx.x;
   const double* f = a.in + static_cast<size_t>(pt) * nv;
   double* y = a.vec + static_cast<size_t>(pt) * 3 * n;
-  double mb = 0.0, unused = 0.0;
+  Mag mf = 0;
   for (int i = tid; i < hc * nr; i += kEval) {
     const int q = i / nr, k = i % nr;
     const double p = f[i], m = q < hf ? f[(nt - 1 - q) * nr + k] : 0.0;
     fold[i] = p + m;
     fold[hc * nr + i] = q < hf ? p - m : 0.0;
-    mb = fmax(mb, fmax(fabs(p), fabs(m)));
+    mf = mag_max(mf, mag_max(mag(p), mag(m)));
   }
-  block_max2(mb, unused, red);
+  double mb, unused;
+  block_max2(mf, 0, red, mb, unused);
   if (tid == 0) {
     a.fmax_[pt] = mb;
     if (a.conv) a.conv[pt] = 0;
@@ -1125,10 +1100,15 @@ __global__ void __launch_bounds__(kEval) window_project_kernel(const SolveArgs a
 
 // z += H^-1 rho through the window factors, one CTA per point. The factors are streamed once, panel by
 // panel (the T forwards, then inv(U11) and U backwards), through a ring of shared-memory stages
-// filled by bulk copies: bound by the copy rate of one SM (3.4 MB a point and solve on the medium
-// grid). Converged points return at once.
+// filled by bulk copies; of the far blocks only those still to come are copied. On the medium grid
+// (128 points of 64 x 32, FP32) 0.40 GB a solve, 58 us at the copy bandwidth; measured 88 us, one CTA an
+// SM bound by the panels' chain (a panel 1000 cycles forwards, 1200 backwards). It was 119 us with the
+// stage found by a division, the ranks read one panel ahead and the far columns gathered from the
+// unknowns. 256 points of 128 x 32: 315 us of 295 us at the copy bandwidth (it was 366), two CTAs an
+// SM; one CTA with twice the stages 352 us. Vectors are read and written by rows: 1.4 times the solve
+// when each lane wrote a row of its own. Converged points return at once.
 template <typename T>
-__global__ void __launch_bounds__(kThreads) window_substitute_kernel(const SolveArgs a) {
+__global__ void __launch_bounds__(kThreads, 2) window_substitute_kernel(const SolveArgs a) {
   extern __shared__ __align__(1024) unsigned char raw[];
   const WindowPlan& w = a.w;
   const int pt = blockIdx.x, tid = threadIdx.x;
@@ -1141,7 +1121,8 @@ __global__ void __launch_bounds__(kThreads) window_substitute_kernel(const Solve
   const int npad = (np + RS) * 32;
   // U's rows: FP64 [32][NU]; FP32 32 x 32 blocks, one per chunk of the window, as load_row reads them
   constexpr bool blocks = sizeof(T) == 4;
-  T* bp = b + npad;  // [2][32] pivot values; the backward pass's 32 partial results
+  T* x0 = b + npad + 64;  // [NF] the solution at the far columns
+  T* bp = b + npad;       // [2][32] pivot values; the backward pass's 32 partial results
   double* z = a.vec + static_cast<size_t>(pt) * 3 * n + n;
   const double* rho = z + n;
   __shared__ __align__(8) uint64_t full[8];
@@ -1151,102 +1132,135 @@ __global__ void __launch_bounds__(kThreads) window_substitute_kernel(const Solve
   const T* Ug = static_cast<const T*>(a.U) + static_cast<size_t>(pt) * np * ustride;
   const signed char* sj = a.slotj + static_cast<size_t>(pt) * np * NS;
   const int nfar = imax(0, nr - w.kf0);
-  // the q-th copy: the T of panels 0 .. np - 1, then the U of panels np - 1 .. 0
-  auto issue = [&](int q) {
-    const T* src = q < np ? Tg + static_cast<size_t>(q) * 32 * NS : Ug + static_cast<size_t>(2 * np - 1 - q) * ustride;
-    const unsigned bytes = q < np ? fbytes : bbytes;
-    uint64_t* bar = &full[q % S];
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(saddr(bar)), "r"(bytes) : "memory");
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     saddr(stage + static_cast<size_t>(q % S) * a.stage_bytes)),
-                 "l"(src), "r"(bytes), "r"(saddr(bar))
-                 : "memory");
+  // the far blocks of panel s that are still to be taken over
+  auto far0 = [&](int s) { return imin((s * g) >> 5, w.NF >> 5); };
+  auto far1 = [&](int s) { return s * g < nfar && s + 1 < np ? w.NF >> 5 : far0(s); };
+  // the q-th copy: the T of panels 0 .. np - 1, then the U of panels np - 1 .. 0, into stage q mod S
+  auto issue = [&](int q, int st) {
+    T* dst = reinterpret_cast<T*>(stage + static_cast<size_t>(st) * a.stage_bytes);
+    if (q < np) {
+      expect_tx(&full[st], fbytes);
+      bulk_load(dst, Tg + static_cast<size_t>(q) * 32 * NS, fbytes, &full[st]);
+      return;
+    }
+    const int s = 2 * np - 1 - q;
+    const T* src = Ug + static_cast<size_t>(s) * ustride;
+    if constexpr (!blocks) {
+      expect_tx(&full[st], bbytes);
+      bulk_load(dst, src, bbytes, &full[st]);
+    } else {  // the blocks that the panel's row reads
+      const unsigned near = 4096u * (1 + imin(RS, np - 1 - s)), off = 1024u * (1 + RS + far0(s));
+      const unsigned far = 4096u * (far1(s) - far0(s));
+      expect_tx(&full[st], near + far);
+      bulk_load(dst, src, near, &full[st]);
+      if (far) bulk_load(dst + off, src + off, far, &full[st]);
+    }
   };
   if (tid == 0) {
     for (int i = 0; i < S; ++i) mbar_init(&full[i], 1);
     gave_up = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    for (int q = 0; q < imin(S, 2 * np); ++q) issue(q);
+    for (int q = 0; q < imin(S, 2 * np); ++q) issue(q, q);
   }
-  for (int i = tid; i < npad; i += kThreads) {
-    const int k = i / nlp, l = i % nlp;
-    b[i] = k < nr && l < nl ? static_cast<T>(rho[l * nr + k]) : T(0);
-  }
-  if (tid < 64) bp[tid] = T(0);  // unused unknowns stay zero
+  const int sh = 31 - __clz(nlp);
+  for (int i = tid; i < npad + 64 + w.NF; i += kThreads) b[i] = T(0);  // unused unknowns stay zero
   __syncthreads();
+  // rho and z by rows, whole lines at a time; the columns' conflicts in shared memory cost less
+  for (int i = tid; i < n; i += kThreads) {
+    const int l = i / nr, k = i - l * nr;
+    b[(k << sh) + l] = static_cast<T>(rho[i]);
+  }
+  __syncthreads();
+  // the stage and phase of the copy in use, advanced by hand (a division by S costs as much as the product)
+  int st = 0;
+  uint32_t ph = 0;
+  auto advance = [&]() {
+    if (++st == S) st = 0, ph ^= 1u;
+  };
   // forward: one thread a slot
   if (tid < NS) {
     T wv = tid < npad ? b[tid] : T(0);
-    int jn = sj[tid];
+    // the slots' ranks are read four panels ahead: a panel is shorter than a load from memory
+    auto rank_of = [&](int s) { return s < np ? static_cast<int>(sj[static_cast<size_t>(s) * NS + tid]) : -1; };
+    int j1 = rank_of(0), j2 = rank_of(1), j3 = rank_of(2), j4 = rank_of(3), freed = 0;
     for (int s = 0; s < np; ++s) {
-      const int j = jn;
-      if (s + 1 < np) jn = sj[static_cast<size_t>(s + 1) * NS + tid];
-      if (j >= 0) bp[(s & 1) * 32 + j] = wv;
+      const int j = j1;
+      j1 = j2, j2 = j3, j3 = j4, j4 = rank_of(s + 4);
+      T* q = bp + (s & 1) * 32;
+      if (j >= 0) q[j] = wv;
       asm volatile("bar.sync 1, %0;" ::"r"(NS) : "memory");
       // every slot's thread is past panel s - 1: its stage can be filled again
-      if (tid == 0 && s > 0 && s - 1 + S < 2 * np) issue(s - 1 + S);
-      mbar_wait(&full[s % S], (s / S) & 1, &gave_up, a.status);
-      const T* t = reinterpret_cast<const T*>(stage + static_cast<size_t>(s % S) * a.stage_bytes) + tid;
-      const T* q = bp + (s & 1) * 32;
+      if (tid == 0 && s > 0 && s - 1 + S < 2 * np) issue(s - 1 + S, freed);
+      freed = st;
+      mbar_wait(&full[st], ph, &gave_up, a.status);
+      const T* t = reinterpret_cast<const T*>(stage + static_cast<size_t>(st) * a.stage_bytes) + tid;
       T acc[4] = {wv, T(0), T(0), T(0)};
 #pragma unroll
-      for (int k = 0; k < 32; ++k) acc[k & 3] = fma(t[k * NS], q[k], acc[k & 3]);
+      for (int k = 0; k < 32; k += 4) {
+        const auto p = Vec4<T>::load(q + k);
+        acc[0] = fma(t[k * NS], p.x, acc[0]);
+        acc[1] = fma(t[(k + 1) * NS], p.y, acc[1]);
+        acc[2] = fma(t[(k + 2) * NS], p.z, acc[2]);
+        acc[3] = fma(t[(k + 3) * NS], p.w, acc[3]);
+      }
       wv = (acc[0] + acc[1]) + (acc[2] + acc[3]);
       if (j >= 0) {
         b[s * 32 + j] = wv;  // y of this panel; the chunk that enters takes the slot
         wv = s + 1 + RC < np ? b[(s + 1 + RC) * 32 + j] : T(0);
       }
+      advance();
     }
+  } else {
+    for (int s = 0; s < np; ++s) advance();
   }
   __syncthreads();
-  if (tid == 0 && np - 1 + S < 2 * np) issue(np - 1 + S);
-  // backward: eight threads a row
+  int freed = st == 0 ? S - 1 : st - 1;  // the last forward panel's
+  if (tid == 0 && np - 1 + S < 2 * np) issue(np - 1 + S, freed);
+  // backward: eight threads a row of U. Columns past the window and far columns already taken over hold
+  // zeros, their unknowns are finite: no conditions.
   const int row = tid >> 3, sub = tid & 7;
   for (int s = np - 1; s >= 0; --s) {
-    const int q = 2 * np - 1 - s;
-    mbar_wait(&full[q % S], (q / S) & 1, &gave_up, a.status);
-    const T* ui = reinterpret_cast<const T*>(stage + static_cast<size_t>(q % S) * a.stage_bytes);
+    const int q = 2 * np - 1 - s, nring = imin(RS, np - 1 - s);
+    const int f0 = far0(s), f1 = far1(s);
+    mbar_wait(&full[st], ph, &gave_up, a.status);
+    const T* ui = reinterpret_cast<const T*>(stage + static_cast<size_t>(st) * a.stage_bytes);
     const T* x = b + (s + 1) * 32;
-    const int wr = imin(RS, np - 1 - s) * 32;
+    const int c4 = blocks ? 4 * (sub ^ (row & 7)) : 4 * sub;  // logical columns of the thread's piece
+    const T* u = ui + 1024 + (blocks ? row * 32 : row * NU) + 4 * sub;
+    const int cs = blocks ? 1024 : 32;  // from chunk to chunk
     T s0 = T(0), s1 = T(0);
-    if constexpr (blocks) {
-      const T* u = ui + 1024 + row * 32 + 4 * sub;
-      const int c4 = 4 * (sub ^ (row & 7));
-      for (int c = 0; c < wr; c += 32) s0 += Vec4<T>::dot(u + c * 32, x + c + c4);
-      if (s * g < nfar && s + 1 < np)
-        for (int k = ((s * g) / 32) * 32; k < nfar; k += 32) {
-          const T* uf = u + (RS * 32 + k) * 32;
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int kk = k + c4 + e;
-            if (kk >= s * g && kk < nfar) s1 = fma(uf[e], b[(w.kf0 + kk) * nlp], s1);
-          }
-        }
-    } else {
-      const T* u = ui + 1024 + static_cast<size_t>(row) * NU;
-      for (int c = 4 * sub; c < wr; c += 32) s0 += Vec4<T>::dot(u + c, x + c);
-      const T* uf = u + RS * 32;
-      if (s * g < nfar && s + 1 < np)
-        for (int k = ((s * g) / 32) * 32 + sub; k < nfar; k += 8)
-          if (k >= s * g) s1 = fma(uf[k], b[(w.kf0 + k) * nlp], s1);
-    }
+    for (int c = 0; c < 6; ++c)  // RS <= 6
+      if (c < nring) (c & 1 ? s1 : s0) += Vec4<T>::dot(u + c * cs, x + c * 32 + c4);
+#pragma unroll 2
+    for (int c = f0; c < f1; ++c) s0 += Vec4<T>::dot(u + (RS + c) * cs, x0 + c * 32 + c4);
     T acc = s0 + s1;
     acc += __shfl_xor_sync(0xffffffffu, acc, 4);
     acc += __shfl_xor_sync(0xffffffffu, acc, 2);
     acc += __shfl_xor_sync(0xffffffffu, acc, 1);
     T* t = bp + (s & 1) * 32;
     if (sub == 0) t[row] = b[s * 32 + row] - acc;
-    __syncthreads();
-    T e = Vec4<T>::dot(ui + row * 32 + 4 * sub, t + 4 * sub);
+    __syncthreads();  // the panel's right-hand side is complete, the panel before is read
+    if (tid == 0 && q > np && q - 1 + S < 2 * np) issue(q - 1 + S, freed);
+    freed = st;
+    T e = Vec4<T>::dot(ui + row * 32 + 4 * sub, t + c4);
     e += __shfl_xor_sync(0xffffffffu, e, 4);
     e += __shfl_xor_sync(0xffffffffu, e, 2);
     e += __shfl_xor_sync(0xffffffffu, e, 1);
-    if (sub == 0) b[s * 32 + row] = (chunk_mask(w, s) >> row) & 1u ? e : T(0);
+    if (sub == 0) {
+      const int k = (s * 32 + row) >> sh, l = row & (nlp - 1);
+      b[s * 32 + row] = k < nr && l < nl ? e : T(0);
+      if (l == 0 && k >= w.kf0 && k < nr) x0[k - w.kf0] = e;
+    }
     __syncthreads();
-    if (tid == 0 && q + S < 2 * np) issue(q + S);
+    advance();
   }
-  for (int i = tid; i < n; i += kThreads) z[i] += static_cast<double>(b[(i % nr) * nlp + i / nr]);
+  __syncthreads();
+  for (int i = tid; i < n; i += kThreads) {
+    const int l = i / nr, k = i - l * nr;
+    z[i] += static_cast<double>(b[(k << sh) + l]);
+  }
 }
 
 // With check: rho of the iterate, the convergence test of launch_residual (max|r| and max|x| at the
@@ -1254,6 +1268,8 @@ __global__ void __launch_bounds__(kThreads) window_substitute_kernel(const Solve
 // made, x into out. As long as a bound that costs one reduction (|rho_p| <= sum_k |M_pk| max|M^-1 rho|
 // and |M^-1 rho| <= |T_S| max|r|) already shows a point to be short of the tolerance, neither the
 // Cholesky substitution nor the projections are made, except at the last sweep. Without check: x alone.
+// FP64 operations bound it: 75 us with the full test for 128 points of 64 x 32, 28 with the bound alone;
+// a step's evaluations 157 us, 178 with the maxima on the FP64 units and the row sums of M formed here.
 __global__ void __launch_bounds__(kEval) window_residual_kernel(const SolveArgs a, int check, int last) {
   extern __shared__ __align__(1024) unsigned char raw[];
   const int nr = a.w.nr, nl = a.w.nl, nt = a.nt, n = nl * nr, nv = nt * nr, hf = nt / 2, hc = (nt + 1) / 2;
@@ -1262,7 +1278,7 @@ __global__ void __launch_bounds__(kEval) window_residual_kernel(const SolveArgs 
   double* z = reinterpret_cast<double*>(raw);  // n
   double* dz = z + n;                          // z - y
   double* q = dz + n;                          // rho, then M^-1 rho
-  __shared__ double red[2 * kEval / 32];
+  __shared__ Mag red[2 * kEval / 32];
   const double* f = a.in + static_cast<size_t>(pt) * nv;
   double* out = a.out + static_cast<size_t>(pt) * nv;
   double* vec = a.vec + static_cast<size_t>(pt) * 3 * n;
@@ -1279,19 +1295,15 @@ __global__ void __launch_bounds__(kEval) window_residual_kernel(const SolveArgs 
     mb = a.fmax_[pt];
     nA = 1.0 + a.dt * (a.kc_inf + fabs(Ei) * a.ka_inf);
     const int mw = a.mass.w, bw = 2 * mw + 1;
-    double lb = 0.0, mz = 0.0;
+    Mag lbm = 0, mzm = 0;
     for (int i = tid; i < n; i += kEval) {
       const int l = i / nr, p = i % nr;
       const int k0 = imax(0, p - mw), k1 = imin(nr - 1, p + mw);
       const double* zl = z + l * nr;
       const double* dl = dz + l * nr;
       const double* mr = a.mass.m + static_cast<size_t>(p) * bw + mw - p;
-      double m = 0.0, c = 0.0, fl = 0.0, rs = 0.0;
-      for (int k = k0; k <= k1; ++k) {
-        const double t = __ldg(mr + k);
-        m = fma(-t, dl[k], m);
-        rs += fabs(t);
-      }
+      double m = 0.0, c = 0.0, fl = 0.0;
+      for (int k = k0; k <= k1; ++k) m = fma(-__ldg(mr + k), dl[k], m);
       if (l > 0) {
         const double* row = a.ro.band + static_cast<size_t>(p) * bw + mw - p;
         const double* fr = a.ro.fband + (static_cast<size_t>(l) * nr + p) * bw + mw - p;
@@ -1310,10 +1322,11 @@ __global__ void __launch_bounds__(kEval) window_residual_kernel(const SolveArgs 
       const double r = m + a.dt * (c + Ei * fl);
       q[i] = r;
       vec[2 * n + i] = r;
-      lb = fmax(lb, fabs(r) / rs);
-      mz = fmax(mz, fabs(dl[p]));
+      lbm = mag_max(lbm, mag(r * __ldg(a.minv + p)));
+      mzm = mag_max(mzm, mag(dl[p]));
     }
-    block_max2(lb, mz, red);
+    double lb, mz;
+    block_max2(lbm, mzm, red, lb, mz);
     if (tid == 0) atomicAdd(a.status + 1, 1u);  // residual evaluations
     const double least = lb / a.ts_inf;
     if (!last && least > a.tol * mb && least > floor_ * (nA * (mb + a.to_inf * mz) + mb)) return;
@@ -1322,7 +1335,7 @@ __global__ void __launch_bounds__(kEval) window_residual_kernel(const SolveArgs 
     __syncthreads();
   }
   // x = f + P_O (z - y) and, with check, r = P_O q, both by parity
-  double mr = 0.0, mx = 0.0;
+  Mag mrm = 0, mxm = 0;
   for (int i = tid; i < hc * nr; i += kEval) {
     const int o = i / nr, k = i % nr;
     const double* to = a.TO + o * nl;
@@ -1338,17 +1351,18 @@ __global__ void __launch_bounds__(kEval) window_residual_kernel(const SolveArgs 
       }
     }
     const double x1 = f[i] + (xe + xo);
-    mr = fmax(mr, fabs(re + ro)), mx = fmax(mx, fabs(x1));
+    mrm = mag_max(mrm, mag(re + ro)), mxm = mag_max(mxm, mag(x1));
     if (o < hf) {
       const size_t i2 = static_cast<size_t>(nt - 1 - o) * nr + k;
       const double x2 = f[i2] + (xe - xo);
       out[i2] = x2;
-      mr = fmax(mr, fabs(re - ro)), mx = fmax(mx, fabs(x2));
+      mrm = mag_max(mrm, mag(re - ro)), mxm = mag_max(mxm, mag(x2));
     }
     out[i] = x1;
   }
   if (!check) return;
-  block_max2(mr, mx, red);
+  double mr, mx;
+  block_max2(mrm, mxm, red, mr, mx);
   if (tid == 0) {
     const double ratio = mb > 0.0 ? mr / mb : (mr > 0.0 ? INFINITY : 0.0);
     a.ratio[pt] = ratio;
@@ -1527,7 +1541,7 @@ static FactorArgs factor_args(const WindowBuffers& b, const double* E, double Eu
 
 static SolveArgs solve_args(const WindowBuffers& b, MassBand mass, int nt) {
   SolveArgs a{};
-  a.w = b.w, a.T = b.T, a.U = b.U, a.slotj = b.slotj, a.vec = b.vec, a.fmax_ = b.fmax_, a.mass = mass, a.nt = nt;
+  a.w = b.w, a.T = b.T, a.U = b.U, a.slotj = b.slotj, a.vec = b.vec, a.fmax_ = b.fmax_, a.minv = b.minv, a.mass = mass, a.nt = nt;
   return a;
 }
 
@@ -1581,9 +1595,9 @@ cudaError_t launch_window_substitute(const WindowBuffers& b, const int* conv, in
   const size_t ts = b.fp64 ? sizeof(double) : sizeof(float);
   const size_t fb = ts * 32 * b.w.NS, bb = ts * (1024 + 32 * static_cast<size_t>(b.w.NU));
   a.stage_bytes = static_cast<unsigned>(round_up(static_cast<int>(std::max(fb, bb)), 128));
-  const size_t fixed = ts * (static_cast<size_t>(b.w.np + b.w.RS) * 32 + 64);
+  const size_t fixed = ts * ((static_cast<size_t>(b.w.np + b.w.RS) * 32 + 64) + b.w.NF);
   // one CTA an SM takes up to 8 stages; with more points than SMs two CTAs share one where both can
-  // have two stages
+  // have two stages (256 points of 128 x 32: 315 us instead of 352)
   size_t room = 224 * 1024 - fixed;
   if (nx > 152 && fixed + 2 * static_cast<size_t>(a.stage_bytes) <= 112 * 1024) room = 112 * 1024 - fixed;
   a.stages = static_cast<int>(std::max<size_t>(1, std::min<size_t>(8, room / a.stage_bytes)));
