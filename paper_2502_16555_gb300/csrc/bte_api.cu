@@ -216,11 +216,11 @@ bte_status harmonic_substitute(bte_handle* h, const double* E_dev, double Eu, co
   else if (h->precision == BTE_FP64)
     BTE_LAUNCH(BTE_K_LU_SOLVE, bte::launch_struct_substitute<double>(E_dev, Eu, o.dt, residual_ops(h), mass,
                                                                      static_cast<double*>(h->xs), h->win.vec, conv,
-                                                                     o.nx, o.nr, o.nl, h->st));
+                                                                     o.nx, o.nr, o.nl, h->status, h->st));
   else
     BTE_LAUNCH(BTE_K_LU_SOLVE, bte::launch_struct_substitute<float>(E_dev, Eu, o.dt, residual_ops(h), mass,
                                                                     static_cast<float*>(h->xs), h->win.vec, conv, o.nx,
-                                                                    o.nr, o.nl, h->st));
+                                                                    o.nr, o.nl, h->status, h->st));
   return BTE_OK;
 }
 

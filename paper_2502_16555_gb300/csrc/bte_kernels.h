@@ -137,7 +137,7 @@ cudaError_t launch_struct_factor(const double* E, double E_uniform, double dt, c
                                  T* S, int nx, int nr, int nl, cudaStream_t st);
 template <typename T>
 cudaError_t launch_struct_substitute(const double* E, double E_uniform, double dt, const ResidualOps& ro, MassBand mass,
-                                     const T* S, double* vec, const int* conv, int nx, int nr, int nl,
+                                     const T* S, double* vec, const int* conv, int nx, int nr, int nl, unsigned* status,
                                      cudaStream_t st);
 // The mixed paths' FP64 escalation, factors and solve in one launch: Fout = A_i^-1 Fin per point
 // (Fout += when accumulate); T is the arithmetic of the block elimination; Xscratch holds

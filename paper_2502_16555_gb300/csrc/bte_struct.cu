@@ -17,9 +17,11 @@
 // and solved in one launch for the points whose refinement has not converged.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "bte_kernels.h"
+#include "bte_async.cuh"
 #include "bte_recip.cuh"
 
 namespace bte {
@@ -228,22 +230,25 @@ __global__ void __launch_bounds__(kST) vsolve_struct_kernel(const double* __rest
   if (bad && status) atomicOr(status, kNonFinite);
 }
 
-// S_l^-1 of every harmonic of one point (CTA), l = nl - 1 .. 0, into Sg[pt][l] (row-major, stride
+// S_l^-1 of every harmonic of one point (CTA), l = nl - 1 .. 0, into Sg[pt][l] (by columns, stride
 // `stride` values). A 16 x 16 thread grid holds the block being inverted in registers, thread
 // (ty, tx) the elements (ty + 16 a, tx + 16 b); the Gauss-Jordan step k reads the pivot row, column
 // and reciprocal that their owners posted in step k - 1: one barrier a step. In FP64 the units'
 // rate bounds it (a step is 16 FMAs and 4 products a thread; the reciprocal is the owner's alone),
-// in FP32 the latency of the nl nr dependent steps.
+// in FP32 the latency of the nl nr dependent steps. 128 points of 64 x 32: FP32 672 us (752 with a
+// condition on each product of the band), FP64 4.3 ms.
 template <typename T>
 __global__ void __launch_bounds__(kST) struct_factor_kernel(const double* __restrict__ E, double E_uniform, double dt,
                                                             ResidualOps ro, MassBand mass, T* __restrict__ Sg,
                                                             size_t stride, int n, int nl) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  const int w = mass.w, bw = 2 * w + 1, nn = n * n;
+  const int w = mass.w, bw = 2 * w + 1;
   const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
-  T* Sinv = reinterpret_cast<T*>(smraw);  // [n][n]
-  T* Y = Sinv + nn;                       // [n][n]
-  T* Lb = Y + nn;                         // [n][bw], dt E (A_v)_{l+1,l}
+  // both products' operands have a zero border of the band's half width, so that they need no conditions
+  const int lds = (n + 2 * w) | 1, ldy = n | 1;
+  T* Sinv = reinterpret_cast<T*>(smraw) + w;  // rows of lds: [i][j], j = -w .. n - 1 + w
+  T* Y = reinterpret_cast<T*>(smraw) + n * lds + w * ldy;  // rows of ldy: i = -w .. n - 1 + w
+  T* Lb = Y + (n + w) * ldy;              // [bw][n]: Lb[t + w][j] = dt E (A_v)_{l+1,l}[j + t][j]
   T* Ub = Lb + n * bw;                    // [n][bw], dt E (A_v)_{l,l+1}
   T* prow2 = Ub + n * bw;                 // 2 x 64 pivot rows
   T* pcol2 = prow2 + 128;                 // 2 x 64 pivot columns
@@ -251,6 +256,7 @@ __global__ void __launch_bounds__(kST) struct_factor_kernel(const double* __rest
   const int pt = blockIdx.x;
   const double dtE = dt * (E ? E[pt] : E_uniform);
   T* out = Sg + static_cast<size_t>(pt) * nl * stride;
+  for (int e = threadIdx.x; e < n * lds + (n + 2 * w) * ldy; e += kST) reinterpret_cast<T*>(smraw)[e] = T(0);
   for (int l = nl - 1; l >= 0; --l) {
     T s[kG][kG];
 #pragma unroll
@@ -269,30 +275,36 @@ __global__ void __launch_bounds__(kST) struct_factor_kernel(const double* __rest
       }
     if (l + 1 < nl) {
       for (int e = threadIdx.x; e < n * bw; e += kST) {
-        Lb[e] = static_cast<T>(dtE * __ldg(ro.fband + static_cast<size_t>(l + 1) * n * bw + e));
+        const int t = e / n, c = e - t * n, r = c + t - w;  // L[r][c], r = c + t - w
+        Lb[e] = r >= 0 && r < n ? static_cast<T>(dtE * __ldg(ro.fband + (static_cast<size_t>(l + 1) * n + r) * bw + c - r + w)) : T(0);
         Ub[e] = static_cast<T>(dtE * __ldg(ro.fband + static_cast<size_t>(nl + l) * n * bw + e));
       }
       __syncthreads();
-      for (int e = threadIdx.x; e < nn; e += kST) {  // Y = S_{l+1}^-1 L_{l+1} (up to sign)
-        const int i = e / n, j = e % n;
-        T acc = T(0);
-        for (int t = -w; t <= w; ++t)
-          if (j + t >= 0 && j + t < n) acc = fma(Sinv[i * n + j + t], Lb[(j + t) * bw + w - t], acc);
-        Y[e] = acc;
+#pragma unroll
+      for (int b = 0; b < kG; ++b) {  // Y = S_{l+1}^-1 L_{l+1} (up to sign)
+        const int c = tx + 16 * b;
+        if (c >= n) break;
+        T acc[kG] = {T(0), T(0), T(0), T(0)};
+        for (int t = 0; t < bw; ++t) {
+          const T lv = Lb[t * n + c];
+#pragma unroll
+          for (int a = 0; a < kG; ++a)
+            if (ty + 16 * a < n) acc[a] = fma(Sinv[(ty + 16 * a) * lds + c + t - w], lv, acc[a]);
+        }
+#pragma unroll
+        for (int a = 0; a < kG; ++a)
+          if (ty + 16 * a < n) Y[(ty + 16 * a) * ldy + c] = acc[a];
       }
       __syncthreads();
 #pragma unroll
       for (int a = 0; a < kG; ++a) {
         const int i = ty + 16 * a;
         if (i >= n) break;
-        for (int t = -w; t <= w; ++t) {
-          if (i + t < 0 || i + t >= n) continue;
-          const T u = Ub[i * bw + w + t];
+        for (int t = 0; t < bw; ++t) {
+          const T u = -Ub[i * bw + t];
 #pragma unroll
-          for (int b = 0; b < kG; ++b) {
-            const int j = tx + 16 * b;
-            if (j < n) s[a][b] = fma(-u, Y[(i + t) * n + j], s[a][b]);
-          }
+          for (int b = 0; b < kG; ++b)
+            if (tx + 16 * b < n) s[a][b] = fma(u, Y[(i + t - w) * ldy + tx + 16 * b], s[a][b]);
         }
       }
     }
@@ -349,70 +361,97 @@ __global__ void __launch_bounds__(kST) struct_factor_kernel(const double* __rest
 #pragma unroll
       for (int b = 0; b < kG; ++b) {
         const int i = ty + 16 * a, j = tx + 16 * b;
-        if (i < n && j < n) Sinv[i * n + j] = s[a][b], o[i * n + j] = s[a][b];
+        if (i < n && j < n) Sinv[i * lds + j] = s[a][b];
       }
     __syncthreads();
+    for (int c = threadIdx.x >> 5; c < n; c += kST / 32)
+      for (int i = threadIdx.x & 31; i < n; i += 32) o[c * n + i] = Sinv[i * lds + c];
   }
 }
 
 // z += H^-1 rho (vectors [nx][3 nl n]: y, z, rho) through the inverses: downwards g_l = S_l^-1 r_l with
-// r_l = rho_l - U_l g_{l+1}, then upwards z_l = g_l - S_l^-1 L_l z_{l-1}. Four lanes a row; the next
-// block's row is loaded while this one is used. Converged points return at once.
+// r_l = rho_l - U_l g_{l+1}, then upwards z_l = g_l - S_l^-1 L_l z_{l-1}. Thread (part, row) takes 16
+// columns of a row; the inverses are streamed twice, through a ring of shared-memory stages filled by
+// bulk copies: latency of 2 nl - 1 dependent products, 78 us a solve for 128 points of 64 x 32 in FP32
+// and 97 in FP64 (86 and 94 with the inverses loaded by rows, one block ahead); 67 MB of inverses
+// in FP32 are 20 us at the copy bandwidth. Converged points return at once.
 template <typename T>
 __global__ void __launch_bounds__(kST) struct_substitute_kernel(const double* __restrict__ E, double E_uniform,
                                                                 double dt, ResidualOps ro, MassBand mass,
-                                                                const T* __restrict__ Sg, size_t stride,
+                                                                const T* __restrict__ Sg, int stride, int stages,
                                                                 double* __restrict__ vec, const int* conv, int n,
-                                                                int nl) {
+                                                                int nl, unsigned* status) {
   extern __shared__ __align__(16) unsigned char smraw[];
   const int pt = blockIdx.x, tid = threadIdx.x;
   if (conv && conv[pt]) return;
-  const int w = mass.w, bw = 2 * w + 1, m = nl * n;
-  T* g = reinterpret_cast<T*>(smraw);  // [nl][n]
-  T* r = g + m;                        // [64]
+  const int w = mass.w, bw = 2 * w + 1, m = nl * n, ncopy = 2 * nl - 1;
+  T* ring = reinterpret_cast<T*>(smraw);  // [stages][stride]
+  T* g = ring + stages * stride;          // [nl][n]
+  T* r = g + m;                           // [64]
+  T* part = r + 64;                       // [4][64]
+  __shared__ __align__(8) uint64_t full[8];
+  __shared__ int gave_up;
   double* z = vec + static_cast<size_t>(pt) * 3 * m + m;
   const double* rho = z + m;
   const T* S = Sg + static_cast<size_t>(pt) * nl * stride;
   const T dtE = static_cast<T>(dt * (E ? E[pt] : E_uniform));
-  const int row = tid >> 2, sub = tid & 3;  // 64 rows, lanes take columns sub + 4 c
-  T buf[16];
-  auto load = [&](int l) {
-#pragma unroll
-    for (int c = 0; c < 16; ++c) {
-      const int j = sub + 4 * c;
-      buf[c] = row < n && j < n ? S[static_cast<size_t>(l) * stride + row * n + j] : T(0);
-    }
+  const uint32_t bytes = static_cast<uint32_t>(stride * sizeof(T));
+  auto block_of = [&](int q) { return q < nl ? nl - 1 - q : q - nl + 1; };  // down nl - 1 .. 0, up 1 .. nl - 1
+  auto issue = [&](int q, int st) {
+    expect_tx(&full[st], bytes);
+    bulk_load(ring + st * stride, S + static_cast<size_t>(block_of(q)) * stride, bytes, &full[st]);
   };
-  load(nl - 1);
-  for (int i = tid; i < 64; i += kST) r[i] = i < n ? static_cast<T>(rho[(nl - 1) * n + i]) : T(0);
+  if (tid == 0) {
+    for (int i = 0; i < stages; ++i) mbar_init(&full[i], 1);
+    gave_up = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    for (int q = 0; q < min(stages, ncopy); ++q) issue(q, q);
+  }
+  const int row = tid & 63, p = tid >> 6;
+  if (tid < 64) r[tid] = tid < n ? static_cast<T>(rho[(nl - 1) * n + tid]) : T(0);
   __syncthreads();
-  for (int step = 0; step < 2 * nl - 1; ++step) {
-    const bool down = step < nl;
-    const int l = down ? nl - 1 - step : step - nl + 1;
-    T acc = T(0);
+  int st = 0;
+  uint32_t ph = 0;
+  for (int q = 0; q < ncopy; ++q) {
+    const bool down = q < nl;
+    const int l = block_of(q);
+    // what the next vector needs of rho, ahead of the wait
+    const T rn = down && l > 0 && tid < n ? static_cast<T>(rho[(l - 1) * n + tid]) : T(0);
+    mbar_wait(&full[st], ph, &gave_up, status);
+    T a0 = T(0), a1 = T(0);
+    if (row < n) {
+      const T* sc = ring + st * stride + row;
 #pragma unroll
-    for (int c = 0; c < 16; ++c) acc = fma(buf[c], r[sub + 4 * c], acc);
-    if (step + 1 < 2 * nl - 1) load(step + 1 < nl ? nl - 2 - step : step + 2 - nl);
-    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-    acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-    if (sub == 0 && row < n) g[l * n + row] = down ? acc : g[l * n + row] + acc;
+      for (int c = 0; c < 16; c += 2) {
+        const int j = 16 * p + c;
+        if (j < n) a0 = fma(sc[j * n], r[j], a0);
+        if (j + 1 < n) a1 = fma(sc[(j + 1) * n], r[j + 1], a1);
+      }
+    }
+    part[p * 64 + row] = a0 + a1;
     __syncthreads();
-    // the next vector: rho_{l-1} + dt E Aup_{l-1} g_l downwards, dt E Alo_{l+1} z_l upwards
-    const int ln = down ? l - 1 : l + 1;
-    const bool turn = down && l == 0;  // z_0 = g_0: the way up starts with harmonic 1
-    const int src = l, dst = turn ? 1 : ln;
-    if (dst >= 0 && dst < nl && tid < 64) {
+    if (tid == 0 && q + stages < ncopy) issue(q + stages, st);
+    if (tid < n) {
+      T v = (part[tid] + part[64 + tid]) + (part[128 + tid] + part[192 + tid]);
+      if (!down) v += g[l * n + tid];
+      g[l * n + tid] = v;
+    }
+    if (tid < 64) asm volatile("bar.sync 1, 64;" ::: "memory");
+    // the next vector: rho_{l-1} + dt E Aup_{l-1} g_l downwards, dt E Alo_{l+1} z_l upwards (z_0 = g_0)
+    const bool up = !down || l == 0;
+    const int dst = up ? l + 1 : l - 1;
+    if (tid < 64) {
       T v = T(0);
-      if (tid < n) {
-        const bool up = !down || turn;
+      if (tid < n && dst < nl) {
         const double* fr = ro.fband + (static_cast<size_t>(up ? dst : nl + dst) * n + tid) * bw + w - tid;
-        for (int k = max(0, tid - w); k <= min(n - 1, tid + w); ++k) v = fma(static_cast<T>(__ldg(fr + k)), g[src * n + k], v);
-        v *= dtE;
-        if (!up) v += static_cast<T>(rho[dst * n + tid]);
+        for (int k = max(0, tid - w); k <= min(n - 1, tid + w); ++k) v = fma(static_cast<T>(__ldg(fr + k)), g[l * n + k], v);
+        v = fma(dtE, v, rn);
       }
       r[tid] = v;
     }
     __syncthreads();
+    if (++st == stages) st = 0, ph ^= 1u;
   }
   for (int i = tid; i < m; i += kST) z[i] += static_cast<double>(g[i]);
 }
@@ -535,7 +574,8 @@ size_t struct_stride(int nr) { return (static_cast<size_t>(nr) * nr + 3) / 4 * 4
 template <typename T>
 cudaError_t launch_struct_factor(const double* E, double E_uniform, double dt, const ResidualOps& ro, MassBand mass,
                                  T* S, int nx, int nr, int nl, cudaStream_t st) {
-  const int smem = static_cast<int>(sizeof(T)) * (2 * nr * nr + 2 * nr * (2 * mass.w + 1) + 4 * 64);
+  const int w2 = 2 * mass.w;
+  const int smem = static_cast<int>(sizeof(T)) * (nr * ((nr + w2) | 1) + (nr + w2) * (nr | 1) + 2 * nr * (w2 + 1) + 4 * 64);
   const cudaError_t e = cudaFuncSetAttribute(struct_factor_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   struct_factor_kernel<T><<<nx, kST, smem, st>>>(E, E_uniform, dt, ro, mass, S, struct_stride(nr), nr, nl);
@@ -548,18 +588,23 @@ template cudaError_t launch_struct_factor<double>(const double*, double, double,
 
 template <typename T>
 cudaError_t launch_struct_substitute(const double* E, double E_uniform, double dt, const ResidualOps& ro, MassBand mass,
-                                     const T* S, double* vec, const int* conv, int nx, int nr, int nl,
+                                     const T* S, double* vec, const int* conv, int nx, int nr, int nl, unsigned* status,
                                      cudaStream_t st) {
-  const int smem = static_cast<int>(sizeof(T)) * (nl * nr + 64);
+  const int stride = static_cast<int>(struct_stride(nr)), fixed = static_cast<int>(sizeof(T)) * (nl * nr + 64 + 256);
+  const int sb = stride * static_cast<int>(sizeof(T));
+  const int stages = std::max(1, std::min(8, (200 * 1024 - fixed) / sb));
+  const int smem = fixed + stages * sb;
   const cudaError_t e =
       cudaFuncSetAttribute(struct_substitute_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  struct_substitute_kernel<T><<<nx, kST, smem, st>>>(E, E_uniform, dt, ro, mass, S, struct_stride(nr), vec, conv, nr, nl);
+  struct_substitute_kernel<T><<<nx, kST, smem, st>>>(E, E_uniform, dt, ro, mass, S, stride, stages, vec, conv, nr, nl, status);
   return cudaGetLastError();
 }
 template cudaError_t launch_struct_substitute<float>(const double*, double, double, const ResidualOps&, MassBand,
-                                                     const float*, double*, const int*, int, int, int, cudaStream_t);
+                                                     const float*, double*, const int*, int, int, int,
+                                                     unsigned*, cudaStream_t);
 template cudaError_t launch_struct_substitute<double>(const double*, double, double, const ResidualOps&, MassBand,
-                                                      const double*, double*, const int*, int, int, int, cudaStream_t);
+                                                      const double*, double*, const int*, int, int, int,
+                                                      unsigned*, cudaStream_t);
 
 }  // namespace bte
