@@ -233,15 +233,17 @@ __global__ void __launch_bounds__(kST) vsolve_struct_kernel(const double* __rest
 // S_l^-1 of every harmonic of one point (CTA), l = nl - 1 .. 0, into Sg[pt][l] (by columns, stride
 // `stride` values). A 16 x 16 thread grid holds the block being inverted in registers, thread
 // (ty, tx) the elements (ty + 16 a, tx + 16 b); the Gauss-Jordan step k reads the pivot row, column
-// and reciprocal that their owners posted in step k - 1: one barrier a step. In FP64 the units'
-// rate bounds it (a step is 16 FMAs and 4 products a thread; the reciprocal is the owner's alone),
-// in FP32 the latency of the nl nr dependent steps. 128 points of 64 x 32: FP32 672 us (752 with a
-// condition on each product of the band), FP64 4.3 ms.
+// and reciprocal that their owners posted in step k - 1: one barrier a step. In FP32 the latency of the
+// nl nr dependent steps bounds it: 128 points of 64 x 32 672 us (752 with a condition on each product of
+// the band). In FP64 the units' rate does (a step is 16 FMAs and 4 products a thread; the reciprocal is
+// the owner's alone), so there the blocks l >= 1, which are symmetric, are held and swept by half: 3.45 ms
+// instead of 4.30, with the same errors (in FP32 it would be 738 us: as many steps, each a little longer).
 template <typename T>
 __global__ void __launch_bounds__(kST) struct_factor_kernel(const double* __restrict__ E, double E_uniform, double dt,
                                                             ResidualOps ro, MassBand mass, T* __restrict__ Sg,
                                                             size_t stride, int n, int nl) {
   extern __shared__ __align__(16) unsigned char smraw[];
+  constexpr bool kSym = sizeof(T) == 8;
   const int w = mass.w, bw = 2 * w + 1;
   const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
   // both products' operands have a zero border of the band's half width, so that they need no conditions
@@ -258,6 +260,7 @@ __global__ void __launch_bounds__(kST) struct_factor_kernel(const double* __rest
   T* out = Sg + static_cast<size_t>(pt) * nl * stride;
   for (int e = threadIdx.x; e < n * lds + (n + 2 * w) * ldy; e += kST) reinterpret_cast<T*>(smraw)[e] = T(0);
   for (int l = nl - 1; l >= 0; --l) {
+    const bool half = kSym && l > 0;  // blocks a >= b alone
     T s[kG][kG];
 #pragma unroll
     for (int a = 0; a < kG; ++a)
@@ -285,15 +288,16 @@ __global__ void __launch_bounds__(kST) struct_factor_kernel(const double* __rest
         const int c = tx + 16 * b;
         if (c >= n) break;
         T acc[kG] = {T(0), T(0), T(0), T(0)};
+        auto rows = [&](int a) { return ty + 16 * a < n && (!half || a >= b || (a + 1 == b && ty + w >= 16)); };
         for (int t = 0; t < bw; ++t) {
           const T lv = Lb[t * n + c];
 #pragma unroll
           for (int a = 0; a < kG; ++a)
-            if (ty + 16 * a < n) acc[a] = fma(Sinv[(ty + 16 * a) * lds + c + t - w], lv, acc[a]);
+            if (rows(a)) acc[a] = fma(Sinv[(ty + 16 * a) * lds + c + t - w], lv, acc[a]);
         }
 #pragma unroll
         for (int a = 0; a < kG; ++a)
-          if (ty + 16 * a < n) Y[(ty + 16 * a) * ldy + c] = acc[a];
+          if (rows(a)) Y[(ty + 16 * a) * ldy + c] = acc[a];
       }
       __syncthreads();
 #pragma unroll
@@ -304,7 +308,7 @@ __global__ void __launch_bounds__(kST) struct_factor_kernel(const double* __rest
           const T u = -Ub[i * bw + t];
 #pragma unroll
           for (int b = 0; b < kG; ++b)
-            if (tx + 16 * b < n) s[a][b] = fma(u, Y[(i + t - w) * ldy + tx + 16 * b], s[a][b]);
+            if (tx + 16 * b < n && (b <= a || !half)) s[a][b] = fma(u, Y[(i + t - w) * ldy + tx + 16 * b], s[a][b]);
         }
       }
     }
@@ -349,19 +353,70 @@ __global__ void __launch_bounds__(kST) struct_factor_kernel(const double* __rest
         __syncthreads();
       }
     };
-    post(0, std::integral_constant<int, 0>{}, 0);
-    __syncthreads();
-    sweep(std::integral_constant<int, 0>{});
-    sweep(std::integral_constant<int, 1>{});
-    sweep(std::integral_constant<int, 2>{});
-    sweep(std::integral_constant<int, 3>{});
+    // the same on blocks a >= b alone. In place, the rows and columns already done and those still to come
+    // form symmetric blocks, and the blocks between them are each other's negative: v, the pivot row up to
+    // the pivot's block and the column below it, gives both the row and, with that sign, the column.
+    auto post_sym = [&](int o, auto q, int buf) {
+      constexpr int Q = decltype(q)::value;
+      if (ty == o)
+#pragma unroll
+        for (int b = 0; b <= Q; ++b) prow2[64 * buf + tx + 16 * b] = s[Q][b];
+      if (tx == o) {
+#pragma unroll
+        for (int a = Q + 1; a < kG; ++a) prow2[64 * buf + ty + 16 * a] = s[a][Q];
+        if (ty == o) pinv2[buf] = recip(s[Q][Q]);
+      }
+    };
+    auto sweep_sym = [&](auto q) {
+      constexpr int Q = decltype(q)::value;
+      const int kn = min(16, n - 16 * Q);
+#pragma unroll 1
+      for (int o = 0; o < kn; ++o) {
+        const int c = o & 1;
+        const T p = pinv2[c], pq = ty < o ? -p : p;
+        T pr[kG], fc[kG];
+#pragma unroll
+        for (int u = 0; u < kG; ++u) {
+          pr[u] = prow2[64 * c + tx + 16 * u];
+          fc[u] = prow2[64 * c + ty + 16 * u] * (u < Q ? -p : u == Q ? pq : p);
+        }
+#pragma unroll
+        for (int a = 0; a < kG; ++a)
+#pragma unroll
+          for (int b = 0; b <= a; ++b) s[a][b] = fma(-fc[a], pr[b], s[a][b]);
+        if (tx == o)
+#pragma unroll
+          for (int a = Q; a < kG; ++a) s[a][Q] = -fc[a];
+        if (ty == o)
+#pragma unroll
+          for (int b = 0; b <= Q; ++b) s[Q][b] = b == Q && tx == o ? p : pr[b] * p;
+        if (o + 1 < kn) post_sym(o + 1, q, c ^ 1);
+        else if (Q + 1 < kG && kn == 16 && 16 * (Q + 1) < n) post_sym(0, std::integral_constant<int, (Q + 1) % kG>{}, 0);
+        __syncthreads();
+      }
+    };
+    constexpr std::integral_constant<int, 0> q0{};
+    constexpr std::integral_constant<int, 1> q1{};
+    constexpr std::integral_constant<int, 2> q2{};
+    constexpr std::integral_constant<int, 3> q3{};
+    if (half) {
+      post_sym(0, q0, 0);
+      __syncthreads();
+      sweep_sym(q0), sweep_sym(q1), sweep_sym(q2), sweep_sym(q3);
+    } else {
+      post(0, q0, 0);
+      __syncthreads();
+      sweep(q0), sweep(q1), sweep(q2), sweep(q3);
+    }
     T* o = out + static_cast<size_t>(l) * stride;
 #pragma unroll
     for (int a = 0; a < kG; ++a)
 #pragma unroll
       for (int b = 0; b < kG; ++b) {
         const int i = ty + 16 * a, j = tx + 16 * b;
-        if (i < n && j < n) Sinv[i * lds + j] = s[a][b];
+        if (i >= n || j >= n || (half && b > a)) continue;
+        Sinv[i * lds + j] = s[a][b];
+        if (half && b < a) Sinv[j * lds + i] = s[a][b];
       }
     __syncthreads();
     for (int c = threadIdx.x >> 5; c < n; c += kST / 32)
@@ -372,9 +427,10 @@ __global__ void __launch_bounds__(kST) struct_factor_kernel(const double* __rest
 // z += H^-1 rho (vectors [nx][3 nl n]: y, z, rho) through the inverses: downwards g_l = S_l^-1 r_l with
 // r_l = rho_l - U_l g_{l+1}, then upwards z_l = g_l - S_l^-1 L_l z_{l-1}. Thread (part, row) takes 16
 // columns of a row; the inverses are streamed twice, through a ring of shared-memory stages filled by
-// bulk copies: latency of 2 nl - 1 dependent products, 78 us a solve for 128 points of 64 x 32 in FP32
-// and 97 in FP64 (86 and 94 with the inverses loaded by rows, one block ahead); 67 MB of inverses
-// in FP32 are 20 us at the copy bandwidth. Converged points return at once.
+// bulk copies; the couplings' band and rho are read a product ahead. Bound by the latency of 2 nl - 1
+// dependent products, in FP64 half by the units' rate: 128 points of 64 x 32 65 us a solve in FP32 and
+// 123 in FP64 (86 and 188 with the inverses loaded by rows, one block ahead, and the band where it is
+// used); the 67 MB of FP32 inverses, twice, are 20 us at the copy bandwidth. Converged points return at once.
 template <typename T>
 __global__ void __launch_bounds__(kST) struct_substitute_kernel(const double* __restrict__ E, double E_uniform,
                                                                 double dt, ResidualOps ro, MassBand mass,
@@ -416,8 +472,19 @@ __global__ void __launch_bounds__(kST) struct_substitute_kernel(const double* __
   for (int q = 0; q < ncopy; ++q) {
     const bool down = q < nl;
     const int l = block_of(q);
-    // what the next vector needs of rho, ahead of the wait
-    const T rn = down && l > 0 && tid < n ? static_cast<T>(rho[(l - 1) * n + tid]) : T(0);
+    // what the next vector needs of rho and of the couplings' band (w <= 3), ahead of the wait
+    const bool up = !down || l == 0;
+    const int dst = up ? l + 1 : l - 1;
+    double fb[7] = {}, rn = 0.0;
+    if (tid < n && dst < nl) {
+      if (!up) rn = rho[dst * n + tid];
+      const double* fr = ro.fband + (static_cast<size_t>(up ? dst : nl + dst) * n + tid) * bw + w - 3;
+#pragma unroll
+      for (int t = 0; t < 7; ++t) {
+        const int k = tid + t - 3;
+        if (t >= 3 - w && t <= 3 + w && k >= 0 && k < n) fb[t] = __ldg(fr + t);
+      }
+    }
     mbar_wait(&full[st], ph, &gave_up, status);
     T a0 = T(0), a1 = T(0);
     if (row < n) {
@@ -439,15 +506,14 @@ __global__ void __launch_bounds__(kST) struct_substitute_kernel(const double* __
     }
     if (tid < 64) asm volatile("bar.sync 1, 64;" ::: "memory");
     // the next vector: rho_{l-1} + dt E Aup_{l-1} g_l downwards, dt E Alo_{l+1} z_l upwards (z_0 = g_0)
-    const bool up = !down || l == 0;
-    const int dst = up ? l + 1 : l - 1;
     if (tid < 64) {
       T v = T(0);
-      if (tid < n && dst < nl) {
-        const double* fr = ro.fband + (static_cast<size_t>(up ? dst : nl + dst) * n + tid) * bw + w - tid;
-        for (int k = max(0, tid - w); k <= min(n - 1, tid + w); ++k) v = fma(static_cast<T>(__ldg(fr + k)), g[l * n + k], v);
-        v = fma(dtE, v, rn);
+#pragma unroll
+      for (int t = 0; t < 7; ++t) {
+        const int k = tid + t - 3;
+        if (k >= 0 && k < n) v = fma(static_cast<T>(fb[t]), g[l * n + k], v);
       }
+      v = tid < n ? fma(dtE, v, static_cast<T>(rn)) : T(0);
       r[tid] = v;
     }
     __syncthreads();
