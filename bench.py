@@ -2,8 +2,8 @@
 
 Workload: one discharge with Nx=128 Chebyshev points, Nr=64 B-splines, Ntheta=32 ordinates
 (Nv = 2048, 262,144 DOFs), 0.5 Torr, 150 V at 13.56 MHz, dt = T_RF/2000, four analytic processes,
-synthetic Maxwellian initial state. A step is one full bte_step: x half step, per-point dense
-LU solve of the velocity system (with FP64 refinement in the mixed path), x half step.
+synthetic Maxwellian initial state. A step is one full bte_step: x half step, per-point LU solve of
+the velocity system (in the harmonic basis, with FP64 refinement in the mixed path), x half step.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 
@@ -38,11 +38,6 @@ TF32_OVER_BF16 = 1.1 / 2.25
 # FP32 SIMT peak from unit counts and clock: 152 SMs x 128 lanes x 2 flop x 2.07 GHz (used when the
 # library FP32 GEMM measured in the run is not a plain CUDA-core GEMM).
 FP32_SIMT_UNITS_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
-# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of the first-panel launch (k0 = 0) of
-# the kernels captured with ncu on this workload (the commands are in profiles/); the per-launch
-# figure reported is scaled to the step's average launch by the algorithmic bytes. Remove an entry
-# when its kernel changes.
-TRAFFIC_K0 = {"lu_gemm": 2.584127e9 + 1.590629e9, "lu_panel": 402.5408e6 + 122.445056e6}
 
 
 def load_peaks():
@@ -191,9 +186,33 @@ def tc_pairs(nv):
     return out
 
 
-def algorithmic(cfg, precision, kernel, tc, pair=True):
+def window_plan(cfg):
+    """The windowed LU's shape for a velocity grid (window_plan in csrc/bte_window.cu), or None where
+    the dense LU runs: chunks of 32 columns, g speed indices each, a ring of RS chunks behind the
+    current one and NF columns of the far l = 0 unknowns."""
+    nr, nl = cfg["nr"], cfg.get("nl") or cfg["ntheta"]
+    nlp = 1
+    while nlp < nl:
+        nlp *= 2
+    if nlp > 32:
+        return None
+    g = 32 // nlp
+    rc = -(-3 // g)
+    rs, slots, np_ = 2 * rc, 32 * (1 + rc), -(-nr // g)
+    nfar = max(0, nr - (rs + 1) * g)
+    nf = -(-nfar // 32) * 32
+    return {"np": np_, "g": g, "rs": rs, "slots": slots, "nfar": nfar, "nf": nf} if rs * 32 + nf <= 512 else None
+
+
+def algorithmic(cfg, precision, kernel, tc, pair=True, window=None):
     """(amount, unit, bound) of the algorithmic work of one step for a kernel class (per-step sums
-    over its launches; per unit):
+    over its launches; per unit). With the windowed LU (window, the default):
+      lu_gemm      mixed: the one-launch factorisation, its factors written once (T 32 x slots, the
+                   inverse of U11 and U's ring and far columns of every panel, 4 B each);
+      lu_solve     per point solve: the same factors read once, of the far columns those still to come;
+      residual     FP64 flops of the harmonic residual per point evaluation, banded products and the
+                   dense C_0 (the projections of the final test are not counted).
+    With the dense LU:
       lu_panel     read + write of every outer panel once: 2 * 4 B * (Nv - k0) * 128 per point;
       lu_gemm      trailing updates, 2 M^2 128 flop per point and panel (M = Nv - k0 - 128); on the
                    tensor cores in panel pairs: 2 M1 kb2 128 for the first panel's update of the
@@ -216,6 +235,20 @@ def algorithmic(cfg, precision, kernel, tc, pair=True):
     esz = 8 if precision == "fp64" else 4
     nb = 64 if precision == "fp64" else 128
     panels = [(k0, min(nb, nv - k0)) for k0 in range(0, nv, nb)]
+    if window and kernel in ("lu_panel", "lu_panel_flops", "lu_swap_trsm"):
+        return None, None, None
+    if window and kernel in ("lu_gemm", "lu_solve"):
+        if kernel == "lu_gemm" and precision == "fp64":
+            return None, None, None
+        w, total = window, 0
+        for q in range(w["np"]):
+            ring = min(w["rs"], w["np"] - 1 - q)
+            far = (w["nf"] - 32 * (q * w["g"] // 32)) if q * w["g"] < w["nfar"] and q + 1 < w["np"] else 0
+            total += 32 * w["slots"] + 1024 + 32 * (32 * ring + far)
+        return (float(esz) * total * nx, "byte", "hbm") if kernel == "lu_gemm" else (float(esz) * total, "byte/point", "hbm")
+    if window and kernel == "residual":
+        b = 2 * 3 + 1
+        return 2.0 * (nr * nr + nl * nr * b + (nl - 1) * nr * b + 2 * (nl - 1) * nr * b), "flop/point", "alu"
     if kernel == "lu_panel":
         return sum(2.0 * esz * (nv - k0) * kb for k0, kb in panels) * nx, "byte", "hbm"
     if kernel == "lu_panel_flops":
@@ -251,29 +284,8 @@ def algorithmic(cfg, precision, kernel, tc, pair=True):
     return None, None, None
 
 
-def traffic_per_launch(cfg, kernel, launches_per_step):
-    """Measured DRAM bytes of the k0 = 0 launch scaled to the average launch of the step (both
-    kernels move bytes in proportion to their algorithmic bytes, which shrink with k0)."""
-    if kernel not in TRAFFIC_K0 or not launches_per_step:
-        return None
-    nv = cfg["nr"] * cfg["ntheta"]
-    nb = 128
-    if kernel == "lu_gemm":
-        # the k0 = 0 pair launch (C read and written once: 2 M2^2 words) scales the pair launches by
-        # M2^2 and the single-panel-column launches by their M1 x kb2 block
-        per = []
-        for k0, kb2, m2 in tc_pairs(nv):
-            per.append((nv - k0 - 128) * kb2)
-            if m2:
-                per.append(m2 ** 2)
-        return TRAFFIC_K0[kernel] * (sum(per) / len(per)) / (nv - 256) ** 2
-    else:
-        per = [nv - k0 for k0 in range(0, nv, nb)]
-    return TRAFFIC_K0[kernel] * (sum(per) / len(per)) / per[0]
-
-
-def roofline_of(cfg, precision, kernel, prof, steps, peaks, tc, evals=None, measured=True):
-    amount, unit, bound = algorithmic(cfg, precision, kernel, tc)
+def roofline_of(cfg, precision, kernel, prof, steps, peaks, tc, evals=None, window=None):
+    amount, unit, bound = algorithmic(cfg, precision, kernel, tc, window=window)
     ms, launches = prof.get(kernel, (0.0, 0))
     if amount is None or launches == 0 or ms <= 0:
         return None
@@ -296,17 +308,16 @@ def roofline_of(cfg, precision, kernel, prof, steps, peaks, tc, evals=None, meas
         achieved, peak, u, src = rate / 1e12, peaks["fp32_tflops"], "TFLOP/s", peaks["fp32_src"]
     out = {"kernel": kernel, "bound": bound, "achieved": achieved, "peak": peak, "unit": u,
            "frac": achieved / peak,
-           "traffic": traffic_per_launch(cfg, kernel, launches / steps) if measured else None,
            "launches_per_step": launches / steps, "ms_per_step": ms / steps, "peak_source": src}
     if unit.endswith("/point"):
         out["point_units_per_step"] = cfg["nx"] * evals
     return out
 
 
-def rooflines(cfg, precision, prof, steps, peaks, tc, evals=None, measured=True):
+def rooflines(cfg, precision, prof, steps, peaks, tc, evals=None, window=None):
     out = {}
     for k in prof:
-        r = roofline_of(cfg, precision, k, prof, steps, peaks, tc, evals, measured)
+        r = roofline_of(cfg, precision, k, prof, steps, peaks, tc, evals, window)
         if r:
             out[k] = r
     dom = max(out, key=lambda k: out[k]["ms_per_step"])
@@ -395,6 +406,7 @@ def run_ours(args, rank, world):
     # ---- mixed precision (the headline)
     s = bte.Solver(cfg, precision="mixed", panel_tc=args.panel_tc)
     tc = bool(s.info()["tensor_cores"])
+    window = window_plan(cfg) if tc and not args.panel_tc else None
     F = s.initial_state()
     F0 = F.clone()
     s.run(F, args.warmup, 0.0)
@@ -486,9 +498,8 @@ def run_ours(args, rank, world):
             del ss
 
     # ---- accuracy over the configured run (one RF cycle of 2000 steps for the default discharge):
-    # the mixed path against FP64. The dense FP64 path takes about 0.65 s per step here, so the
-    # reference is the FP64 block-tridiagonal solve of the same systems (refined in FP64), which
-    # matches the dense FP64 path to ~1e-15 over the steps compared above (structured_solve).
+    # the mixed path against FP64. The reference is the FP64 block-tridiagonal solve of the same systems (refined in FP64), which
+    # matches the FP64 LU path to ~1e-15 over the steps compared above (structured_solve).
     cycle = None
     if not args.no_cycle and cfg["nr"] <= 64 and cfg.get("steps"):
         n_cyc = int(cfg["steps"])
@@ -521,9 +532,7 @@ def run_ours(args, rank, world):
                "steps": "the device-timed plain run's %d steps: same start state and times" % args.steps,
                "matches_device_run": bool(np.array_equal(Fh, Fq.cpu().numpy()))}
 
-    # the measured DRAM traffic was captured on the default workload only
-    measured = name == WORKLOAD and not args.nx
-    rf_dom, rf_all = rooflines(cfg, "mixed", prof, args.steps, peaks, tc, evals=evals, measured=measured)
+    rf_dom, rf_all = rooflines(cfg, "mixed", prof, args.steps, peaks, tc, evals=evals, window=window)
     # kernels with a flop and a byte floor are measured against the binding one: the panel's FP32
     # flops (CUDA-core peak) and the Q apply's FP64 flops (FP64 peak) take longer than their bytes
     for kern, fkey, fpeak, fsrc in (
@@ -531,8 +540,8 @@ def run_ours(args, rank, world):
             ("x_apply_q", "x_apply_q_flops", peaks["fp64_tflops"], peaks["fp64_src"])):
         if kern not in prof or not prof[kern][1] or kern not in rf_all:
             continue
-        fl, _, _ = algorithmic(cfg, "mixed", fkey, tc)
-        by, _, _ = algorithmic(cfg, "mixed", kern, tc)
+        fl, _, _ = algorithmic(cfg, "mixed", fkey, tc, window=window)
+        by, _, _ = algorithmic(cfg, "mixed", kern, tc, window=window)
         t_alu, t_hbm = fl / (fpeak * 1e12), by / (peaks["hbm_gbs"] * 1e9)
         if t_alu <= t_hbm:
             continue
@@ -555,8 +564,9 @@ def run_ours(args, rank, world):
         "data": "synthetic",
         "config": {"workload": name, "nx": cfg["nx"], "nr": cfg["nr"], "ntheta": cfg["ntheta"],
                    "nv": cfg["nr"] * cfg["ntheta"], "dof": dof, "precision": "mixed",
-                   "l2": "working set > L2: %.1f GB of per-point FP32 factors streamed every step"
-                         % (4.0 * cfg["nx"] * (cfg["nr"] * cfg["ntheta"]) ** 2 / 1e9),
+                   "l2": "working set > L2: %.2f GB of per-point FP32 factors written and streamed every step"
+                         % (algorithmic(cfg, "mixed", "lu_gemm", tc, window=window)[0] / 1e9 if window else
+                            4.0 * cfg["nx"] * (cfg["nr"] * cfg["ntheta"]) ** 2 / 1e9),
                    "parallelism": f"replicas x{world}"},
         "fp64": fp64,
         "speedup_mixed_over_fp64": (fp64["ms_per_step"] / ms) if fp64 else None,

@@ -1101,10 +1101,10 @@ __global__ void __launch_bounds__(kEval) window_project_kernel(const SolveArgs a
 // z += H^-1 rho through the window factors, one CTA per point. The factors are streamed once, panel by
 // panel (the T forwards, then inv(U11) and U backwards), through a ring of shared-memory stages
 // filled by bulk copies; of the far blocks only those still to come are copied. On the medium grid
-// (128 points of 64 x 32, FP32) 0.40 GB a solve, 58 us at the copy bandwidth; measured 88 us, one CTA an
+// (128 points of 64 x 32, FP32) 0.40 GB a solve, 60 us at the copy bandwidth; measured 88 us, one CTA an
 // SM bound by the panels' chain (a panel 1000 cycles forwards, 1200 backwards). It was 119 us with the
 // stage found by a division, the ranks read one panel ahead and the far columns gathered from the
-// unknowns. 256 points of 128 x 32: 315 us of 295 us at the copy bandwidth (it was 366), two CTAs an
+// unknowns. 256 points of 128 x 32: 315 us of 262 us at the copy bandwidth (it was 366), two CTAs an
 // SM; one CTA with twice the stages 352 us. Vectors are read and written by rows: 1.4 times the solve
 // when each lane wrote a row of its own. Converged points return at once.
 template <typename T>
