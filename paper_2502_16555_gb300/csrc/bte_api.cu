@@ -729,8 +729,8 @@ bte_status bte_create(const bte_config* cfg, bte_handle** out) {
   {
     // The windowed LU serves every handle that refines, does not ask for a dense variant and whose
     // window fits (at most 32 harmonics, at most 512 window columns): 9 to 40 times fewer operations
-    // than the dense LU of the same systems on the workloads' grids (medium mixed step 1.8 against
-    // 12.9 ms, FP64 19 against 652 ms; 1.1 against 3.6 ms on the small FP64 grid, where launches and
+    // than the dense LU of the same systems on the workloads' grids (medium mixed step 1.5 against
+    // 12.9 ms, FP64 19 against 652 ms; 1.05 against 3.6 ms on the small FP64 grid, where launches and
     // the latency of the columns count).
     // Without refinement (refine_max 0) the result shows the factors' own accuracy, which the
     // window's order of elimination leaves up to four times lower in FP32: those keep the dense LU.

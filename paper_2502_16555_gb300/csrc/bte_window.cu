@@ -189,9 +189,11 @@ struct FactorArgs {
 // the panel's warps. Warps 4-7 meanwhile finish the panel before: the pivot rows' updated window is
 // written out as U, the rows of the entering chunk take the freed slots. The next panel waits only for
 // the update of its own 32 columns, which is issued first.
-// Bound by the latency of the 32 dependent columns of a panel (13.5 us a panel, 9.5 of them in the
-// columns), not by the tensor cores (5000 cycles a panel, hidden) or memory. Medium grid (128 points,
-// order 2048): 0.88 ms for formation and factors, where the dense LU took 10.9 ms.
+// Bound by the latency of a panel's two chains, equally long (12.6 us a panel): the 32 dependent columns, and
+// the conversion, products, rows passed on and the inverse of U11; not by the tensor cores (5000 cycles
+// a panel) or memory. Medium grid (128 points, order 2048): 0.81 ms for formation and factors, where
+// the dense LU took 11.6 ms. Every warp eliminating all 128 rows by itself (8 barriers a panel instead of
+// 40) with a ninth warp for the inverse took 0.82 ms: the second chain slows down beside it.
 __global__ void __launch_bounds__(kThreads, 2) window_lu_tc_kernel(const FactorArgs a) {
   extern __shared__ __align__(1024) unsigned char raw[];
   const WindowPlan& w = a.w;
