@@ -130,8 +130,12 @@ __global__ void ion_assemble_kernel(const double* __restrict__ Dx, const double*
 // exchanged: every warp finds the pivot of a column for itself (the magnitudes as ordered integers, so
 // that the FP64 units, whose rate bounds the kernel, do products only) and takes the rows i = warp,
 // warp + nw, ..; one barrier a column. A zero or non-finite pivot sets kZeroPivot in status.
-// n = 100: the version with row exchanges, a division and FP64 comparisons per column took 470 us.
+// A warp's FMA takes the FP64 units 16 cycles however many lanes are active, so the multipliers of 32 rows are
+// formed by one instruction, and in shared memory b is A's column n and the pivot row is in registers.
+// n = 100: 286 us; 406 with a multiplier and a right-hand side's FMA per row and warp, 470 with row
+// exchanges, a division and FP64 comparisons per column.
 constexpr int kSmemSolve = 150;
+constexpr int kChunks = (kSmemSolve + 32) / 32;  // of 32 columns of [A b]
 template <bool kShared>
 __global__ void __launch_bounds__(512) dense_solve_kernel(double* __restrict__ Ag, const double* __restrict__ bg, int n,
                                                           double* __restrict__ x, unsigned* status) {
@@ -139,11 +143,12 @@ __global__ void __launch_bounds__(512) dense_solve_kernel(double* __restrict__ A
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
   const int ld = kShared ? (n + 1) | 1 : n;  // odd: a column's entries lie in different banks
   double* A = kShared ? sm : Ag;
-  double* b = sm + (kShared ? n * ld : 0);   // n
-  double* pin = b + n;                       // n: reciprocals of the pivots
+  double* b = kShared ? sm + n : sm;         // n, stride bs: column n of A in shared memory
+  const int bs = kShared ? ld : 1;
+  double* pin = kShared ? sm + n * ld : b + n;  // n: reciprocals of the pivots
   int* slot = reinterpret_cast<int*>(pin + n);  // n: the column a row was the pivot of, -1 before
   __shared__ unsigned used_w[128];           // bit per row
-  for (int i = tid; i < n; i += nt) b[i] = bg[i], slot[i] = -1;
+  for (int i = tid; i < n; i += nt) b[i * bs] = bg[i], slot[i] = -1;
   for (int i = tid; i < 128; i += nt) used_w[i] = 0u;
   if (kShared)
     for (int i = warp; i < n; i += nw)
@@ -164,13 +169,36 @@ __global__ void __launch_bounds__(512) dense_solve_kernel(double* __restrict__ A
     const int p = static_cast<int>(__reduce_min_sync(0xffffffffu, row));
     const unsigned long long pk = (static_cast<unsigned long long>(mh) << 32) | ml;
     const double* ap = A + static_cast<size_t>(p) * ld;
-    const double inv = bte::recip(ap[k]), bp = b[p];
-    for (int i = warp; i < n; i += nw) {
-      if (i == p || ((used_w[i >> 5] >> (i & 31)) & 1u)) continue;
-      double* ai = A + static_cast<size_t>(i) * ld;
-      const double l = ai[k] * inv;
-      for (int j = k + 1 + lane; j < n; j += 32) ai[j] = fma(-l, ap[j], ai[j]);
-      if (lane == 0) b[i] = fma(-l, bp, b[i]);
+    const double inv = bte::recip(ap[k]);
+    if constexpr (kShared) {
+      double apr[kChunks];
+#pragma unroll
+      for (int c = 0; c < kChunks; ++c) apr[c] = k + 1 + lane + 32 * c <= n ? ap[k + 1 + lane + 32 * c] : 0.0;
+      for (int i0 = 0; warp + nw * i0 < n; i0 += 32) {  // 32 rows of the warp: a lane takes a row's multiplier
+        const int il = warp + nw * (i0 + lane);
+        const bool on = il < n && il != p && !((used_w[il >> 5] >> (il & 31)) & 1u);
+        const double lm = on ? A[static_cast<size_t>(il) * ld + k] * inv : 0.0;
+        for (unsigned rest = __ballot_sync(0xffffffffu, on); rest; rest &= rest - 1) {
+          const int src = __ffs(rest) - 1;
+          double* ai = A + static_cast<size_t>(warp + nw * (i0 + src)) * ld;
+          const double l = __shfl_sync(0xffffffffu, lm, src);
+#pragma unroll
+          for (int c = 0; c < kChunks; ++c) {
+            if (k + 1 + 32 * c > n) break;
+            const int j = k + 1 + lane + 32 * c;
+            if (j <= n) ai[j] = fma(-l, apr[c], ai[j]);
+          }
+        }
+      }
+    } else {
+      const double bp = b[p];
+      for (int i = warp; i < n; i += nw) {
+        if (i == p || ((used_w[i >> 5] >> (i & 31)) & 1u)) continue;
+        double* ai = A + static_cast<size_t>(i) * ld;
+        const double l = ai[k] * inv;
+        for (int j = k + 1 + lane; j < n; j += 32) ai[j] = fma(-l, ap[j], ai[j]);
+        if (lane == 0) b[i] = fma(-l, bp, b[i]);
+      }
     }
     __syncthreads();  // every warp has read the marks and the pivot row's marker of this column
     if (tid == 0) {
@@ -184,11 +212,11 @@ __global__ void __launch_bounds__(512) dense_solve_kernel(double* __restrict__ A
   // back substitution by columns, warp 0: x_k, then every earlier pivot row's right-hand side
   if (warp == 0) {
     for (int k = n - 1; k >= 0; --k) {
-      const double xk = b[slot[k]] * pin[k];
+      const double xk = b[slot[k] * bs] * pin[k];
       __syncwarp();
       for (int q = lane; q < k; q += 32) {
         const int r = slot[q];
-        b[r] = fma(-A[static_cast<size_t>(r) * ld + k], xk, b[r]);
+        b[r * bs] = fma(-A[static_cast<size_t>(r) * ld + k], xk, b[r * bs]);
       }
       if (lane == 0) x[k] = xk;
       __syncwarp();
