@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include "bte_internal.h"
+#include "bte_window_plan.h"
 
 namespace bte {
 
@@ -190,19 +191,6 @@ void launch_residual(const double* x, const double* b, const double* E, double E
 void launch_check_conv(const int* conv, int nx, unsigned* status, cudaStream_t st);
 
 // ---- the windowed LU of the harmonic system with the speed index slowest (bte_window.cu)
-// Shapes of the window for nl harmonics and nr B-splines; ok = false where it does not apply (nl > 32,
-// or a window wider than the 512 columns of tensor memory).
-struct WindowPlan {
-  int nr = 0, nl = 0;
-  int nlp = 0, g = 0;   // power of two >= nl; speed indices per 32-column chunk
-  int np = 0;           // chunks (panels)
-  int RC = 0, RS = 0;   // chunks that enter ahead of the panel; ring chunks right of it
-  int NS = 0;           // row slots in use, 32 (1 + RC)
-  int kf0 = 0, NF = 0;  // first speed index kept as a far column; far columns (a multiple of 32)
-  int NU = 0, NW = 0;   // window columns RS 32 + NF; row template length (RS + 1) 32 + NF
-  int tmem_cols = 0;
-  bool ok = false;
-};
 struct WindowBuffers {
   WindowPlan w;
   bool fp64 = false;
@@ -216,7 +204,6 @@ struct WindowBuffers {
   double* fmax_ = nullptr;                 // one value a point
   double* minv = nullptr;                  // [nr] 1 / sum_k |M_v[p][k]|
 };
-WindowPlan window_plan(int nr, int nl);
 // Templates [np 32][NW] and [np 32][(RS + 1) 32] from the unscaled blocks (M, Cg, Ag_lo, Ag_up).
 void window_tables(const WindowPlan& w, const HostOps& o, std::vector<double>& base, std::vector<double>& slope);
 // The FP32 kernel's form of the templates: [np][RS + 1 + NF / 32] blocks of 32 rows x 32 columns, the

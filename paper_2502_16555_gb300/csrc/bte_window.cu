@@ -1193,7 +1193,7 @@ __global__ void __launch_bounds__(kThreads, 2) window_substitute_kernel(const So
       if (j >= 0) q[j] = wv;
       asm volatile("bar.sync 1, %0;" ::"r"(NS) : "memory");
       // every slot's thread is past panel s - 1: its stage can be filled again
-      if (tid == 0 && s > 0 && s - 1 + S < 2 * np) issue(s - 1 + S, freed);
+      if (tid == 0 && ring_before_wait(s, np, S) >= 0) issue(ring_before_wait(s, np, S), freed);
       freed = st;
       mbar_wait(&full[st], ph, &gave_up, a.status);
       const T* t = reinterpret_cast<const T*>(stage + static_cast<size_t>(st) * a.stage_bytes) + tid;
@@ -1217,8 +1217,7 @@ __global__ void __launch_bounds__(kThreads, 2) window_substitute_kernel(const So
     for (int s = 0; s < np; ++s) advance();
   }
   __syncthreads();
-  int freed = st == 0 ? S - 1 : st - 1;  // the last forward panel's
-  if (tid == 0 && np - 1 + S < 2 * np) issue(np - 1 + S, freed);
+  if (tid == 0 && ring_after_use(np - 1, np, S) >= 0) issue(ring_after_use(np - 1, np, S), st == 0 ? S - 1 : st - 1);
   // backward: eight threads a row of U. Columns past the window and far columns already taken over hold
   // zeros, their unknowns are finite: no conditions.
   const int row = tid >> 3, sub = tid & 7;
@@ -1243,9 +1242,7 @@ __global__ void __launch_bounds__(kThreads, 2) window_substitute_kernel(const So
     acc += __shfl_xor_sync(0xffffffffu, acc, 1);
     T* t = bp + (s & 1) * 32;
     if (sub == 0) t[row] = b[s * 32 + row] - acc;
-    __syncthreads();  // the panel's right-hand side is complete, the panel before is read
-    if (tid == 0 && q > np && q - 1 + S < 2 * np) issue(q - 1 + S, freed);
-    freed = st;
+    __syncthreads();  // the panel's right-hand side is complete
     T e = Vec4<T>::dot(ui + row * 32 + 4 * sub, t + c4);
     e += __shfl_xor_sync(0xffffffffu, e, 4);
     e += __shfl_xor_sync(0xffffffffu, e, 2);
@@ -1255,7 +1252,8 @@ __global__ void __launch_bounds__(kThreads, 2) window_substitute_kernel(const So
       b[s * 32 + row] = k < nr && l < nl ? e : T(0);
       if (l == 0 && k >= w.kf0 && k < nr) x0[k - w.kf0] = e;
     }
-    __syncthreads();
+    __syncthreads();  // the panel's stage is read
+    if (tid == 0 && ring_after_use(q, np, S) >= 0) issue(ring_after_use(q, np, S), st);
     advance();
   }
   __syncthreads();
@@ -1463,30 +1461,7 @@ __global__ void __launch_bounds__(kThreads) window_solve_t_kernel(const SolveArg
   }
 }
 
-int round_up(int a, int b) { return (a + b - 1) / b * b; }
-
 }  // namespace
-
-WindowPlan window_plan(int nr, int nl) {
-  WindowPlan w;
-  w.nr = nr, w.nl = nl;
-  if (nl < 1 || nl > 32) return w;
-  w.nlp = 1;
-  while (w.nlp < nl) w.nlp *= 2;
-  w.g = kPW / w.nlp;
-  w.np = (nr + w.g - 1) / w.g;
-  w.RC = (3 + w.g - 1) / w.g;
-  w.RS = 2 * w.RC;
-  w.NS = 32 * (1 + w.RC);
-  w.kf0 = (w.RS + 1) * w.g;
-  w.NF = nr > w.kf0 ? round_up(nr - w.kf0, 32) : 0;
-  w.NU = w.RS * 32 + w.NF;
-  w.NW = (w.RS + 1) * 32 + w.NF;
-  w.tmem_cols = 32;
-  while (w.tmem_cols < w.NU) w.tmem_cols *= 2;
-  w.ok = w.NU <= 512;
-  return w;
-}
 
 void window_tables(const WindowPlan& w, const HostOps& o, std::vector<double>& base, std::vector<double>& slope) {
   const int nr = o.nr, nl = o.nl, NWR = (w.RS + 1) * 32;
@@ -1594,16 +1569,9 @@ cudaError_t launch_window_project(const WindowBuffers& b, const double* in, Mass
 cudaError_t launch_window_substitute(const WindowBuffers& b, const int* conv, int nx, unsigned* status, cudaStream_t st) {
   SolveArgs a = solve_args(b, MassBand{}, 0);
   a.conv = const_cast<int*>(conv), a.status = status;
-  const size_t ts = b.fp64 ? sizeof(double) : sizeof(float);
-  const size_t fb = ts * 32 * b.w.NS, bb = ts * (1024 + 32 * static_cast<size_t>(b.w.NU));
-  a.stage_bytes = static_cast<unsigned>(round_up(static_cast<int>(std::max(fb, bb)), 128));
-  const size_t fixed = ts * ((static_cast<size_t>(b.w.np + b.w.RS) * 32 + 64) + b.w.NF);
-  // one CTA an SM takes up to 8 stages; with more points than SMs two CTAs share one where both can
-  // have two stages (256 points of 128 x 32: 315 us instead of 352)
-  size_t room = 224 * 1024 - fixed;
-  if (nx > 152 && fixed + 2 * static_cast<size_t>(a.stage_bytes) <= 112 * 1024) room = 112 * 1024 - fixed;
-  a.stages = static_cast<int>(std::max<size_t>(1, std::min<size_t>(8, room / a.stage_bytes)));
-  const int smem = static_cast<int>(a.stages * static_cast<size_t>(a.stage_bytes) + fixed);
+  const WindowRing ring = window_ring(b.w, b.fp64 ? sizeof(double) : sizeof(float), nx, 152);
+  a.stage_bytes = static_cast<unsigned>(ring.stage_bytes), a.stages = ring.stages;
+  const int smem = static_cast<int>(ring.smem);
   auto k = b.fp64 ? window_substitute_kernel<double> : window_substitute_kernel<float>;
   const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
