@@ -96,6 +96,11 @@ typedef enum {
                                    the launch does no work and the step returns BTE_ECUDA with F
                                    unchanged. Selects the dense LU, whose kernels it tests. Never set it for
                                    real work. */
+#define BTE_FLAG_DIAG_HARMONIC_TIMEOUT 256u  /* diagnostic, the same for the windowed and the structured solves: a
+                                   wait on a barrier that nothing signals runs out (about 1 ms) in every
+                                   substitution, behind its first copies, and in every BTE_MIXED window
+                                   factorisation, behind its first products. The launch issues nothing more,
+                                   waits for what is in flight and ends; the call returns BTE_ECUDA. */
 
 typedef struct {
   int nx;            /* Chebyshev-Gauss-Lobatto points, >= 3 */

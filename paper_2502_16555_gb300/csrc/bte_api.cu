@@ -216,11 +216,11 @@ bte_status harmonic_substitute(bte_handle* h, const double* E_dev, double Eu, co
   else if (h->precision == BTE_FP64)
     BTE_LAUNCH(BTE_K_LU_SOLVE, bte::launch_struct_substitute<double>(E_dev, Eu, o.dt, residual_ops(h), mass,
                                                                      static_cast<double*>(h->xs), h->win.vec, conv,
-                                                                     o.nx, o.nr, o.nl, h->status, h->st));
+                                                                     o.nx, o.nr, o.nl, h->status, h->win.probe, h->st));
   else
     BTE_LAUNCH(BTE_K_LU_SOLVE, bte::launch_struct_substitute<float>(E_dev, Eu, o.dt, residual_ops(h), mass,
                                                                     static_cast<float*>(h->xs), h->win.vec, conv, o.nx,
-                                                                    o.nr, o.nl, h->status, h->st));
+                                                                    o.nr, o.nl, h->status, h->win.probe, h->st));
   return BTE_OK;
 }
 
@@ -711,6 +711,7 @@ bte_status bte_create(const bte_config* cfg, bte_handle** out) {
   h->structured = (cfg->flags & BTE_FLAG_STRUCTURED) != 0;
   h->tc_pair = (cfg->flags & BTE_FLAG_TC_SINGLE) == 0;
   h->tc_probe = (cfg->flags & BTE_FLAG_DIAG_TC_TIMEOUT) != 0 ? 1 : 0;
+  h->win.probe = (cfg->flags & BTE_FLAG_DIAG_HARMONIC_TIMEOUT) != 0 ? 1 : 0;
   h->tc_cg = (cfg->flags & BTE_FLAG_TC_ONE_CTA) != 0 ? 1 : 2;
   h->panel_tc = (cfg->flags & BTE_FLAG_PANEL_TC) != 0;
   {

@@ -7,7 +7,8 @@
 
 namespace bte {
 
-constexpr long long kWaitCycles = 1ll << 32;  // bounded device waits, about 2 s
+constexpr long long kWaitCycles = 1ll << 32;   // bounded device waits, about 2 s
+constexpr long long kProbeCycles = 1ll << 21;  // about 1 ms: the wait of BTE_FLAG_DIAG_HARMONIC_TIMEOUT
 
 __device__ __forceinline__ uint32_t saddr(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
 
@@ -25,18 +26,28 @@ __device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t parity) {
   return ok != 0;
 }
 
-// Bounded: on expiry the status bit is set, later waits of the CTA return at once and the kernel runs
-// to its end on whatever the buffers hold (every access stays in bounds); the step reports it.
-__device__ __forceinline__ void mbar_wait(uint64_t* b, uint32_t parity, volatile int* gave_up, unsigned* status) {
-  if (mbar_try(b, parity)) return;
+// Bounded; false if it ran out. On expiry the status bit is set, later waits of the CTA on phases that are
+// not complete return at once, and the kernel runs to its end on whatever the buffers hold (every access
+// stays in bounds); the step reports it. The thread that issues a barrier's copies or products also waits
+// for them: when its own wait fails it issues nothing more, and it waits again (mbar_drain) for what is
+// in flight, so that nothing lands in memory that the CTA has given back.
+__device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile int* gave_up, unsigned* status,
+                                          long long limit = kWaitCycles) {
+  if (mbar_try(b, parity)) return true;
   const long long t0 = clock64();
-  while (!mbar_try(b, parity)) {
-    if (*gave_up) return;
-    if (clock64() - t0 > kWaitCycles) {
+  while (!*gave_up) {
+    if (mbar_try(b, parity)) return true;
+    if (clock64() - t0 > limit) {
       *gave_up = 1;
       atomicOr(status, kTimeout);
-      return;
     }
+  }
+  return false;
+}
+
+__device__ __forceinline__ void mbar_drain(uint64_t* b, uint32_t parity) {
+  const long long t0 = clock64();
+  while (!mbar_try(b, parity) && clock64() - t0 < kWaitCycles) {
   }
 }
 

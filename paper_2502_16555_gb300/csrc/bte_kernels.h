@@ -139,7 +139,7 @@ cudaError_t launch_struct_factor(const double* E, double E_uniform, double dt, c
 template <typename T>
 cudaError_t launch_struct_substitute(const double* E, double E_uniform, double dt, const ResidualOps& ro, MassBand mass,
                                      const T* S, double* vec, const int* conv, int nx, int nr, int nl, unsigned* status,
-                                     cudaStream_t st);
+                                     int probe, cudaStream_t st);
 // The mixed paths' FP64 escalation, factors and solve in one launch: Fout = A_i^-1 Fin per point
 // (Fout += when accumulate); T is the arithmetic of the block elimination; Xscratch holds
 // nx * nl * nr * nr values of T.
@@ -194,6 +194,7 @@ void launch_check_conv(const int* conv, int nx, unsigned* status, cudaStream_t s
 struct WindowBuffers {
   WindowPlan w;
   bool fp64 = false;
+  int probe = 0;                           // a wait of every substitution and FP32 factorisation runs out
   void *base = nullptr, *slope = nullptr;  // row templates: values without and per unit of the field
                                            // (FP32: window_blocks in base)
   void *T = nullptr, *U = nullptr;         // factors, window_t_count / window_u_count values a point

@@ -436,7 +436,7 @@ __global__ void __launch_bounds__(kST) struct_substitute_kernel(const double* __
                                                                 double dt, ResidualOps ro, MassBand mass,
                                                                 const T* __restrict__ Sg, int stride, int stages,
                                                                 double* __restrict__ vec, const int* conv, int n,
-                                                                int nl, unsigned* status) {
+                                                                int nl, unsigned* status, int probe) {
   extern __shared__ __align__(16) unsigned char smraw[];
   const int pt = blockIdx.x, tid = threadIdx.x;
   if (conv && conv[pt]) return;
@@ -445,7 +445,7 @@ __global__ void __launch_bounds__(kST) struct_substitute_kernel(const double* __
   T* g = ring + stages * stride;          // [nl][n]
   T* r = g + m;                           // [64]
   T* part = r + 64;                       // [4][64]
-  __shared__ __align__(8) uint64_t full[8];
+  __shared__ __align__(8) uint64_t full[8], never;
   __shared__ int gave_up;
   double* z = vec + static_cast<size_t>(pt) * 3 * m + m;
   const double* rho = z + m;
@@ -453,16 +453,23 @@ __global__ void __launch_bounds__(kST) struct_substitute_kernel(const double* __
   const T dtE = static_cast<T>(dt * (E ? E[pt] : E_uniform));
   const uint32_t bytes = static_cast<uint32_t>(stride * sizeof(T));
   auto block_of = [&](int q) { return q < nl ? nl - 1 - q : q - nl + 1; };  // down nl - 1 .. 0, up 1 .. nl - 1
+  // by thread 0, which also waits for each copy and stops when that fails
+  bool quit = false;
+  int issued = 0;
   auto issue = [&](int q, int st) {
+    if (quit) return;
+    issued = q + 1;
     expect_tx(&full[st], bytes);
     bulk_load(ring + st * stride, S + static_cast<size_t>(block_of(q)) * stride, bytes, &full[st]);
   };
   if (tid == 0) {
     for (int i = 0; i < stages; ++i) mbar_init(&full[i], 1);
+    mbar_init(&never, 1);
     gave_up = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     for (int q = 0; q < min(stages, ncopy); ++q) issue(q, q);
+    if (probe) quit = !mbar_wait(&never, 0, &gave_up, status, kProbeCycles);
   }
   const int row = tid & 63, p = tid >> 6;
   if (tid < 64) r[tid] = tid < n ? static_cast<T>(rho[(nl - 1) * n + tid]) : T(0);
@@ -485,7 +492,7 @@ __global__ void __launch_bounds__(kST) struct_substitute_kernel(const double* __
         if (t >= 3 - w && t <= 3 + w && k >= 0 && k < n) fb[t] = __ldg(fr + t);
       }
     }
-    mbar_wait(&full[st], ph, &gave_up, status);
+    if (!mbar_wait(&full[st], ph, &gave_up, status)) quit = true;
     T a0 = T(0), a1 = T(0);
     if (row < n) {
       const T* sc = ring + st * stride + row;
@@ -520,6 +527,8 @@ __global__ void __launch_bounds__(kST) struct_substitute_kernel(const double* __
     if (++st == stages) st = 0, ph ^= 1u;
   }
   for (int i = tid; i < m; i += kST) z[i] += static_cast<double>(g[i]);
+  if (tid == 0 && quit)
+    for (int q = max(0, issued - stages); q < issued; ++q) mbar_drain(&full[q % stages], (q / stages) & 1);
 }
 
 // ---- the reduced dense system (N_l < N_theta): the same identity with I - dt B_i factored as a
@@ -655,7 +664,7 @@ template cudaError_t launch_struct_factor<double>(const double*, double, double,
 template <typename T>
 cudaError_t launch_struct_substitute(const double* E, double E_uniform, double dt, const ResidualOps& ro, MassBand mass,
                                      const T* S, double* vec, const int* conv, int nx, int nr, int nl, unsigned* status,
-                                     cudaStream_t st) {
+                                     int probe, cudaStream_t st) {
   const int stride = static_cast<int>(struct_stride(nr)), fixed = static_cast<int>(sizeof(T)) * (nl * nr + 64 + 256);
   const int sb = stride * static_cast<int>(sizeof(T));
   const int stages = std::max(1, std::min(8, (200 * 1024 - fixed) / sb));
@@ -663,14 +672,15 @@ cudaError_t launch_struct_substitute(const double* E, double E_uniform, double d
   const cudaError_t e =
       cudaFuncSetAttribute(struct_substitute_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  struct_substitute_kernel<T><<<nx, kST, smem, st>>>(E, E_uniform, dt, ro, mass, S, stride, stages, vec, conv, nr, nl, status);
+  struct_substitute_kernel<T><<<nx, kST, smem, st>>>(E, E_uniform, dt, ro, mass, S, stride, stages, vec, conv, nr, nl, status,
+                                                      probe);
   return cudaGetLastError();
 }
 template cudaError_t launch_struct_substitute<float>(const double*, double, double, const ResidualOps&, MassBand,
                                                      const float*, double*, const int*, int, int, int,
-                                                     unsigned*, cudaStream_t);
+                                                     unsigned*, int, cudaStream_t);
 template cudaError_t launch_struct_substitute<double>(const double*, double, double, const ResidualOps&, MassBand,
                                                       const double*, double*, const int*, int, int, int,
-                                                      unsigned*, cudaStream_t);
+                                                      unsigned*, int, cudaStream_t);
 
 }  // namespace bte

@@ -179,6 +179,7 @@ struct FactorArgs {
   double* W;           // FP64: the window [nx][128][NU + 32]
   int* rows;           // FP64: the padded row in each slot [nx][128]
   unsigned* status;
+  int probe;           // FP32: in the first panel, with its products in flight, a wait runs out
 };
 
 // Mixed path. The window D (128 slots x NU columns) lives in tensor memory in FP32; T and B are split
@@ -211,6 +212,7 @@ __global__ void __launch_bounds__(kThreads, 2) window_lu_tc_kernel(const FactorA
   __shared__ float ui[32 * 17];  // inverses of U11's 16 x 16 diagonal blocks
   // products of chunk s + 1, of the rest; templates of the ring and far columns, of the panel's; U11 inverted
   __shared__ __align__(8) uint64_t bar_next, bar_rest, bar_tmpl, bar_t0, bar_u;
+  __shared__ __align__(8) uint64_t never;  // the probe's
   __shared__ uint32_t tmem_base;
   __shared__ int gave_up;
 
@@ -233,6 +235,7 @@ __global__ void __launch_bounds__(kThreads, 2) window_lu_tc_kernel(const FactorA
     mbar_init(&bar_tmpl, 1);
     mbar_init(&bar_t0, 1);
     mbar_init(&bar_u, 1);
+    mbar_init(&never, 1);
     gave_up = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -281,9 +284,18 @@ __global__ void __launch_bounds__(kThreads, 2) window_lu_tc_kernel(const FactorA
     tc_fence_before();
   }
   bool bad = false;
+  // quit: a wait of this thread ran out, it issues nothing more; sent: it has issued, in this panel, what it
+  // will wait for (threads 0: bar_next, 32: bar_t0, 160: bar_tmpl)
+  bool quit = false, sent = false;
+  auto wait = [&](uint64_t* b, uint32_t ph, bool mine) {
+    if (mbar_wait(b, ph, &gave_up, a.status)) return;
+    quit = true;
+    if (mine) mbar_drain(b, ph);
+  };
 
   for (int s = 0; s < np; ++s) {
     const int par = s & 1;
+    sent = false;
     const int dmax = imin(RS, np - 1 - s);                       // ring chunks right of the panel
     const int fc0 = (s * g) / 32, nfc = s * g < nfar ? w.NF / 32 : fc0;  // far chunks [fc0, nfc)
     int pj = -1;
@@ -366,7 +378,7 @@ __global__ void __launch_bounds__(kThreads, 2) window_lu_tc_kernel(const FactorA
 #pragma unroll
           for (int k = 0; k < 8; ++k) v[24 + k] = w8[k];
         }
-        if (s > 0) mbar_wait(&bar_u, (s - 1) & 1, &gave_up, a.status);
+        if (s > 0) wait(&bar_u, (s - 1) & 1, false);
         if (pj >= 0) {
 #pragma unroll
           for (int k = 0; k < 32; ++k) u11[pj * 33 + k] = k >= pj ? v[k] : 0.f;
@@ -382,7 +394,7 @@ __global__ void __launch_bounds__(kThreads, 2) window_lu_tc_kernel(const FactorA
         sjg[static_cast<size_t>(s) * NS + slot] = static_cast<signed char>(pj);
       }
       slotj[par][slot] = static_cast<signed char>(pj);
-      if (s > 0) mbar_wait(&bar_rest, (s - 1) & 1, &gave_up, a.status);  // T and B are free again
+      if (s > 0) wait(&bar_rest, (s - 1) & 1, false);  // T and B are free again
       if (dmax > 0) {
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
@@ -405,9 +417,10 @@ __global__ void __launch_bounds__(kThreads, 2) window_lu_tc_kernel(const FactorA
     const bool enter = tnew < np, fresh = j >= 0 && enter && ((chunk_mask(w, tnew) >> j) & 1u);
     const unsigned mine = own(j & 31);
     if (dmax > 0) {
-      if (tid == 32 && enter) {
+      if (tid == 32 && enter && !quit) {
         expect_tx(&bar_t0, 4096);
         bulk_load(t0, block(tnew, 0), 4096, &bar_t0);
+        sent = true;
       }
       // the pivot rows' window, split, as the K-major B operand: chunk s + 1, which the next panel needs,
       // by the panel warps, whose product is issued at once, the others by the other half
@@ -437,7 +450,7 @@ __global__ void __launch_bounds__(kThreads, 2) window_lu_tc_kernel(const FactorA
                                (static_cast<uint32_t>(kSlots >> 4) << 24);
         const uint64_t off = static_cast<uint64_t>(col) * 8;  // 128-byte rows in units of 16 bytes
         const uint32_t d = tmem_base + col;
-        if (lane == 0) {
+        if (lane == 0 && !quit) {
 #pragma unroll 1
           for (int k = 0; k < 4; ++k) {  // 8 TF32 columns = 32 bytes inside the swizzle row
             mma_tf32(d, dal + 2 * k, dbh + off + 2 * k, idesc);
@@ -461,7 +474,7 @@ __global__ void __launch_bounds__(kThreads, 2) window_lu_tc_kernel(const FactorA
           if (warp == 0) {
             tc_fence_after();
             issue(((s + 1) % RS) * 32, 32);
-            if (lane == 0) mma_commit(&bar_next);
+            if (lane == 0 && !quit) mma_commit(&bar_next), sent = true;
             __syncwarp();
           }
         }
@@ -481,17 +494,19 @@ __global__ void __launch_bounds__(kThreads, 2) window_lu_tc_kernel(const FactorA
             if (r >= 3) col = (RS + fc0) * 32 + (r - 3) * 256, n = imin(256, (nfc - fc0) * 32 - (r - 3) * 256);
             if (n > 0) issue(col, n);
           }
-          if (lane == 0) {
+          if (lane == 0 && !quit) {
             mma_commit(&bar_rest);
-            mbar_wait(&bar_next, par, &gave_up, a.status);
-            mbar_wait(&bar_rest, par, &gave_up, a.status);
-            if (enter) {
+            if (a.probe && s == 0) quit = !mbar_wait(&never, 0, &gave_up, a.status, kProbeCycles);
+            wait(&bar_next, par, false);
+            wait(&bar_rest, par, true);
+            if (enter && !quit) {
               // the products are done: B's remainders give way to the entering rows' templates, chunk d of
               // the ring to template chunk d - 1, the chunk that enters (in the place of chunk s + 1) to RS
               const int far = nfc - fc0, last = s + 1 + RS < np ? RS + 1 : dmax;
               expect_tx(&bar_tmpl, 4096u * (last - 1 + far));
               for (int d = 2; d <= last; ++d) bulk_load(Blo + ((s + d) % RS) * 1024, block(tnew, d - 1), 4096, &bar_tmpl);
               for (int c = fc0; c < nfc; ++c) bulk_load(Blo + (RS + c) * 1024, block(tnew, RS + 1 + c), 4096, &bar_tmpl);
+              sent = true;
             }
           }
           __syncwarp();
@@ -556,13 +571,13 @@ __global__ void __launch_bounds__(kThreads, 2) window_lu_tc_kernel(const FactorA
 #pragma unroll
       for (int i = 0; i < 32; ++i) v[i] = 0.f;
       if (enter) {
-        mbar_wait(&bar_t0, par, &gave_up, a.status);
+        wait(&bar_t0, par, sent && tid == 32);
         if (fresh) {
           load_row(t0, j, v);
           scale_row(v, mine, E);
         }
       }
-      mbar_wait(&bar_next, par, &gave_up, a.status);
+      wait(&bar_next, par, sent && tid == 0);
       tc_fence_after();
       tmem_ld32(tmem + ((s + 1) % RS) * 32, r);
       if (j >= 0) {
@@ -577,9 +592,9 @@ __global__ void __launch_bounds__(kThreads, 2) window_lu_tc_kernel(const FactorA
       __syncwarp();
       asm volatile("bar.arrive 2, %0;" ::"r"(kThreads) : "memory");
     } else {
-      mbar_wait(&bar_rest, par, &gave_up, a.status);
+      wait(&bar_rest, par, false);
       tc_fence_after();
-      if (enter) mbar_wait(&bar_tmpl, par, &gave_up, a.status);
+      if (enter) wait(&bar_tmpl, par, sent);
       const int cnt = dmax - 1 + nfc - fc0;
 #pragma unroll 1
       for (int q = 0; q < cnt; ++q) {
@@ -603,7 +618,7 @@ __global__ void __launch_bounds__(kThreads, 2) window_lu_tc_kernel(const FactorA
       __syncwarp();
       asm volatile("bar.sync 2, %0;" ::"r"(kThreads) : "memory");  // U is complete; chunk s + 1 has been read
       tc_fence_after();
-      if (tid == 160) {
+      if (tid == 160 && !quit) {
         for (int d = 1; d <= dmax; ++d) bulk_store(Up + d * 1024, Bhi + ((s + d) % RS) * 1024, 4096);
         for (int c = fc0; c < nfc; ++c) bulk_store(Up + (1 + RS + c) * 1024, Bhi + (RS + c) * 1024, 4096);
         asm volatile("cp.async.bulk.commit_group;" ::: "memory");
@@ -993,6 +1008,7 @@ struct SolveArgs {
   int stages;
   unsigned stage_bytes;
   unsigned* status;
+  int probe;                // a wait runs out behind the first copies
 };
 
 template <typename T>
@@ -1127,7 +1143,7 @@ __global__ void __launch_bounds__(kThreads, 2) window_substitute_kernel(const So
   T* bp = b + npad;       // [2][32] pivot values; the backward pass's 32 partial results
   double* z = a.vec + static_cast<size_t>(pt) * 3 * n + n;
   const double* rho = z + n;
-  __shared__ __align__(8) uint64_t full[8];
+  __shared__ __align__(8) uint64_t full[8], never;
   __shared__ int gave_up;
   const T* Tg = static_cast<const T*>(a.T) + static_cast<size_t>(pt) * np * 32 * NS;
   const size_t ustride = 1024 + 32 * static_cast<size_t>(NU);
@@ -1137,8 +1153,13 @@ __global__ void __launch_bounds__(kThreads, 2) window_substitute_kernel(const So
   // the far blocks of panel s that are still to be taken over
   auto far0 = [&](int s) { return imin((s * g) >> 5, w.NF >> 5); };
   auto far1 = [&](int s) { return s * g < nfar && s + 1 < np ? w.NF >> 5 : far0(s); };
-  // the q-th copy: the T of panels 0 .. np - 1, then the U of panels np - 1 .. 0, into stage q mod S
+  // the q-th copy: the T of panels 0 .. np - 1, then the U of panels np - 1 .. 0, into stage q mod S; by thread
+  // 0, which also waits for each of them and stops when that fails
+  bool quit = false;
+  int issued = 0;
   auto issue = [&](int q, int st) {
+    if (quit) return;
+    issued = q + 1;
     T* dst = reinterpret_cast<T*>(stage + static_cast<size_t>(st) * a.stage_bytes);
     if (q < np) {
       expect_tx(&full[st], fbytes);
@@ -1160,10 +1181,12 @@ __global__ void __launch_bounds__(kThreads, 2) window_substitute_kernel(const So
   };
   if (tid == 0) {
     for (int i = 0; i < S; ++i) mbar_init(&full[i], 1);
+    mbar_init(&never, 1);
     gave_up = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     for (int q = 0; q < imin(S, 2 * np); ++q) issue(q, q);
+    if (a.probe) quit = !mbar_wait(&never, 0, &gave_up, a.status, kProbeCycles);
   }
   const int sh = 31 - __clz(nlp);
   for (int i = tid; i < npad + 64 + w.NF; i += kThreads) b[i] = T(0);  // unused unknowns stay zero
@@ -1195,7 +1218,7 @@ __global__ void __launch_bounds__(kThreads, 2) window_substitute_kernel(const So
       // every slot's thread is past panel s - 1: its stage can be filled again
       if (tid == 0 && ring_before_wait(s, np, S) >= 0) issue(ring_before_wait(s, np, S), freed);
       freed = st;
-      mbar_wait(&full[st], ph, &gave_up, a.status);
+      if (!mbar_wait(&full[st], ph, &gave_up, a.status)) quit = true;
       const T* t = reinterpret_cast<const T*>(stage + static_cast<size_t>(st) * a.stage_bytes) + tid;
       T acc[4] = {wv, T(0), T(0), T(0)};
 #pragma unroll
@@ -1224,7 +1247,7 @@ __global__ void __launch_bounds__(kThreads, 2) window_substitute_kernel(const So
   for (int s = np - 1; s >= 0; --s) {
     const int q = 2 * np - 1 - s, nring = imin(RS, np - 1 - s);
     const int f0 = far0(s), f1 = far1(s);
-    mbar_wait(&full[st], ph, &gave_up, a.status);
+    if (!mbar_wait(&full[st], ph, &gave_up, a.status)) quit = true;
     const T* ui = reinterpret_cast<const T*>(stage + static_cast<size_t>(st) * a.stage_bytes);
     const T* x = b + (s + 1) * 32;
     const int c4 = blocks ? 4 * (sub ^ (row & 7)) : 4 * sub;  // logical columns of the thread's piece
@@ -1261,6 +1284,8 @@ __global__ void __launch_bounds__(kThreads, 2) window_substitute_kernel(const So
     const int l = i / nr, k = i - l * nr;
     z[i] += static_cast<double>(b[(k << sh) + l]);
   }
+  if (tid == 0 && quit)
+    for (int q = imax(0, issued - S); q < issued; ++q) mbar_drain(&full[q % S], (q / S) & 1);
 }
 
 // With check: rho of the iterate, the convergence test of launch_residual (max|r| and max|x| at the
@@ -1512,7 +1537,7 @@ size_t window_slot_count(const WindowPlan& w) { return static_cast<size_t>(w.np)
 static FactorArgs factor_args(const WindowBuffers& b, const double* E, double Eu, unsigned* status) {
   FactorArgs a;
   a.w = b.w, a.base = b.base, a.slope = b.slope, a.E = E, a.Eu = Eu, a.T = b.T, a.U = b.U, a.slotj = b.slotj;
-  a.W = b.W, a.rows = b.rows, a.status = status;
+  a.W = b.W, a.rows = b.rows, a.status = status, a.probe = b.probe;
   return a;
 }
 
@@ -1568,7 +1593,7 @@ cudaError_t launch_window_project(const WindowBuffers& b, const double* in, Mass
 
 cudaError_t launch_window_substitute(const WindowBuffers& b, const int* conv, int nx, unsigned* status, cudaStream_t st) {
   SolveArgs a = solve_args(b, MassBand{}, 0);
-  a.conv = const_cast<int*>(conv), a.status = status;
+  a.conv = const_cast<int*>(conv), a.status = status, a.probe = b.probe;
   const WindowRing ring = window_ring(b.w, b.fp64 ? sizeof(double) : sizeof(float), nx, 152);
   a.stage_bytes = static_cast<unsigned>(ring.stage_bytes), a.stages = ring.stages;
   const int smem = static_cast<int>(ring.smem);
