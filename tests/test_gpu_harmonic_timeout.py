@@ -46,3 +46,17 @@ def test_step_reports_an_expired_wait_and_keeps_the_state(precision, structured)
     ref = O.Operators(cfg).step(F0, t, E=E.cpu().numpy())
     err = float(np.linalg.norm(F.cpu().numpy() - ref) / np.linalg.norm(ref))
     assert err <= (1e-10 if precision == "fp64" else 1e-9)
+
+
+def test_adjoint_reports_an_expired_wait():
+    """F* of an expired substitution is no solution: the sensitivities must not come back as good."""
+    from paper_2502_16555_gb300 import bte
+    cfg = W.scaled(W.SMALL, nx=5, nr=20, ntheta=9)
+    s = bte.Solver(cfg, precision="fp64", diag_harmonic_timeout=True)
+    F = torch.from_numpy(W.random_state(5, 9, 20, seed=74)).cuda()
+    lam = torch.ones_like(F)
+    SC = torch.zeros((180, 180), dtype=torch.float64, device="cuda")
+    with pytest.raises(bte.BteError) as e:
+        s.step_adjoint(F, lam, 0.2 / W.RF_FREQ_HZ, SC=SC)
+    assert e.value.status == bte.ECUDA
+    assert "wait expired" in str(e.value)
