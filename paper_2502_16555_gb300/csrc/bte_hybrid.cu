@@ -374,14 +374,16 @@ __global__ void __launch_bounds__(kDotBlock) multi_dot_kernel(const double* __re
 }
 
 // out[j] = sum over blocks of partial[blk][j]: one CTA per j, strided partial sums then a tree
-// (a fixed order, so the result is reproducible)
-__global__ void sum_partials_kernel(const double* __restrict__ partial, int nblk, int k, double* __restrict__ out) {
+// (a fixed order, so the result is reproducible); with status its word goes to out[k]
+__global__ void sum_partials_kernel(const double* __restrict__ partial, int nblk, int k, double* __restrict__ out,
+                                    const unsigned* status) {
   __shared__ double red[32];
   const int j = blockIdx.x;
   double s = 0.0;
   for (int b = threadIdx.x; b < nblk; b += blockDim.x) s += partial[static_cast<size_t>(b) * k + j];
   s = block_sum(s, red);
   if (threadIdx.x == 0) out[j] = s;
+  if (status && j == 0 && threadIdx.x == 0) out[k] = *status;
 }
 
 // w = a w + sg sum_{j<k} c_j V_j   (c in device memory)
@@ -532,18 +534,20 @@ void enqueue_vapply(bte_handle* h, const double* X, const double* E, double c, d
                                           h->Aup, h->TO, h->TS, out, o.nt, o.nr, o.nl);
 }
 
-// out_dev[j] = V_j . w for j < k on the device (stream-ordered; no host synchronisation)
-void enqueue_dots(bte_handle* h, const double* V, size_t ld, int k, const double* w, double* out_dev) {
+// out_dev[j] = V_j . w for j < k on the device (stream-ordered; no host synchronisation); with status the
+// handle's status word follows as out_dev[k]
+void enqueue_dots(bte_handle* h, const double* V, size_t ld, int k, const double* w, double* out_dev,
+                  bool status = false) {
   const size_t D = static_cast<size_t>(h->ops.nx) * h->ops.nv;
   multi_dot_kernel<<<dim3(dot_grid(D), (k + kDotVec - 1) / kDotVec), kDotBlock, 0, h->st>>>(V, ld, k, w, D, h->part);
-  sum_partials_kernel<<<k, 128, 0, h->st>>>(h->part, dot_grid(D), k, out_dev);
+  sum_partials_kernel<<<k, 128, 0, h->st>>>(h->part, dot_grid(D), k, out_dev, status ? h->status : nullptr);
 }
 
 // dots[j] = V_j . w for j < k into the pinned host array (synchronises the stream)
 bte_status host_dots(bte_handle* h, const double* V, size_t ld, int k, const double* w, std::vector<double>& out) {
   const size_t D = static_cast<size_t>(h->ops.nx) * h->ops.nv;
   multi_dot_kernel<<<dim3(dot_grid(D), (k + kDotVec - 1) / kDotVec), kDotBlock, 0, h->st>>>(V, ld, k, w, D, h->part);
-  sum_partials_kernel<<<k, 128, 0, h->st>>>(h->part, dot_grid(D), k, h->dsum);
+  sum_partials_kernel<<<k, 128, 0, h->st>>>(h->part, dot_grid(D), k, h->dsum, nullptr);
   BH_CUDA(h, cudaMemcpyAsync(h->dsum_host, h->dsum, k * sizeof(double), cudaMemcpyDeviceToHost, h->st));
   BH_CUDA(h, cudaStreamSynchronize(h->st));
   out.assign(h->dsum_host, h->dsum_host + k);
@@ -678,14 +682,14 @@ bte_status bte_step_implicit(bte_handle* h, double* F_dev, const double* ni_dev,
   unsigned long long launches = 0;
 
   // F^n, and the initial iterate: the semi-implicit self-consistent step from F^n (F^n itself if
-  // that step flags anything)
+  // that step does not factor or converge)
   BH_CUDA(h, cudaMemsetAsync(h->status, 0, 2 * sizeof(unsigned), st));
   BH_CUDA(h, cudaMemcpyAsync(h->Fn, F_dev, D * sizeof(double), cudaMemcpyDeviceToDevice, st));
   BH_CUDA(h, cudaMemcpyAsync(h->Fk, F_dev, D * sizeof(double), cudaMemcpyDeviceToDevice, st));
   s = bte::handle_enqueue_sc_step(h, h->Fk, ni_dev, t_s, V0, freq_Hz);
   if (s != BTE_OK) return s;
   s = bte::handle_read_status(h);
-  if (s == BTE_ENONFINITE) return s;
+  if (s == BTE_ENONFINITE || s == BTE_ECUDA) return s;
   BH_CUDA(h, cudaMemsetAsync(h->status, 0, 2 * sizeof(unsigned), st));
 
   auto residual = [&](const double* X, double* R) {
@@ -791,10 +795,12 @@ bte_status bte_step_implicit(bte_handle* h, double* F_dev, const double* ni_dev,
           multi_axpy_kernel<<<vg, 256, 0, st>>>(Vn, 1.0, h->Vb, D, j + 1, dp, -1.0, D);
           launches += 3;
         }
-        bte::enqueue_dots(h, Vn, 0, 1, Vn, h->dsum + 2 * stride);
+        bte::enqueue_dots(h, Vn, 0, 1, Vn, h->dsum + 2 * stride, true);
         launches += 2;
         BH_CUDA(h, cudaMemcpyAsync(h->dsum_host, h->dsum, 3 * stride * sizeof(double), cudaMemcpyDeviceToHost, st));
         BH_CUDA(h, cudaStreamSynchronize(st));
+        // an expired wait: every further solve would take its 2 s too, for nothing
+        if (static_cast<unsigned>(h->dsum_host[2 * stride + 1]) & bte::kTimeout) return bte::handle_read_status(h);
         for (int i = 0; i <= j; ++i) H[static_cast<size_t>(i) * m + j] += h->dsum_host[i] + h->dsum_host[stride + i];
         const double hn = std::sqrt(h->dsum_host[2 * stride]);
         H[static_cast<size_t>(j + 1) * m + j] = hn;

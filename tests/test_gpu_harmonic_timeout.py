@@ -60,3 +60,21 @@ def test_adjoint_reports_an_expired_wait():
         s.step_adjoint(F, lam, 0.2 / W.RF_FREQ_HZ, SC=SC)
     assert e.value.status == bte.ECUDA
     assert "wait expired" in str(e.value)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_implicit_step_stops_at_an_expired_wait(precision):
+    """Its first step already meets the expired wait: no Newton iteration may follow (each Krylov iteration would
+    wait again). The semi-implicit step launches fewer than 100 kernels here."""
+    from paper_2502_16555_gb300 import bte
+    cfg = W.scaled(W.SMALL, nx=5, nr=12, ntheta=6)
+    s = bte.Solver(cfg, precision=precision, diag_harmonic_timeout=True)
+    F = s.initial_state()
+    F0 = F.clone()
+    ni = torch.full((5,), 1e15, dtype=torch.float64, device="cuda")
+    before = s.info()["launches"]
+    with pytest.raises(bte.BteError) as e:
+        s.step_implicit(F, ni, 0.0)
+    assert e.value.status == bte.ECUDA
+    assert torch.equal(F, F0)
+    assert s.info()["launches"] - before < 100
