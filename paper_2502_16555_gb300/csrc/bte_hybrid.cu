@@ -136,6 +136,9 @@ __global__ void ion_assemble_kernel(const double* __restrict__ Dx, const double*
 // exchanges, a division and FP64 comparisons per column.
 constexpr int kSmemSolve = 150;
 constexpr int kChunks = (kSmemSolve + 32) / 32;  // of 32 columns of [A b]
+size_t ion_smem(size_t n, bool shared) {
+  return (shared ? sizeof(double) * n * ((n + 1) | 1) : 0) + n * (2 * sizeof(double) + sizeof(int));
+}
 template <bool kShared>
 __global__ void __launch_bounds__(512) dense_solve_kernel(double* __restrict__ Ag, const double* __restrict__ bg, int n,
                                                           double* __restrict__ x, unsigned* status) {
@@ -619,9 +622,9 @@ bte_status bte_ion_step(bte_handle* h, double* ni_dev, const double* F_dev, doub
                                            o.dt, o.nx, h->ionA, h->ionb);
   {
     const bool fits = o.nx <= kSmemSolve;
-    const size_t smem = (fits ? sizeof(double) * o.nx * ((o.nx + 1) | 1) : 0) + o.nx * (2 * sizeof(double) + sizeof(int));
+    const size_t smem = ion_smem(o.nx, fits);
     auto solve = fits ? dense_solve_kernel<true> : dense_solve_kernel<false>;
-    BH_CUDA(h, cudaFuncSetAttribute(solve, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+    BH_CUDA(h, bte::set_smem_limit(solve, fits ? ion_smem(kSmemSolve, true) : ion_smem(4096, false)));  // nx <= 4096
     solve<<<1, fits ? 256 : 512, smem, st>>>(h->ionA, h->ionb, o.nx, h->ned, h->status);
   }
   bte::launch_commit(h->ned, ni_dev, o.nx, h->status, st);

@@ -16,6 +16,15 @@ enum StatusBits : unsigned {
   kNonFiniteIn = 16u,  // NaN/Inf in an input: the state handed in, or the field array
 };
 
+// A kernel's limit of dynamic shared memory belongs to the kernel, not to a handle, and handles step on several
+// host threads: a launcher that raised it to its own launch's size could lower it between another
+// thread's raise and launch, which is then rejected. So it is always set to the same value, the most that any
+// handle that bte_create accepts asks for.
+template <typename K>
+cudaError_t set_smem_limit(K* kernel, size_t most) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(most));
+}
+
 // The block-diagonal Galerkin mass matrix I (x) M_v acting on one point's vector, in blocks of nr
 // (one block per ordinate, or per harmonic in the reduced form). M_v is banded with half width w and
 // stored as m[p * (2 w + 1) + k - p + w] = M_v[p][k]. m == nullptr stands for the identity.

@@ -28,6 +28,8 @@ namespace bte {
 namespace {
 
 constexpr int kST = 256;  // threads per CTA
+constexpr int kSubstituteRoom = 200 * 1024;  // shared memory of the substitution: bte_create's check of
+                                             // struct_smem_bytes leaves it at least one stage
 constexpr int kG = 4;     // elements per thread and dimension (Nr <= 16 kG)
 
 // acc(a, b) += sum_k AT[k][ty + 16 a] B[k][tx + 16 b] over k < n: AT is the left factor stored
@@ -649,9 +651,9 @@ size_t struct_stride(int nr) { return (static_cast<size_t>(nr) * nr + 3) / 4 * 4
 template <typename T>
 cudaError_t launch_struct_factor(const double* E, double E_uniform, double dt, const ResidualOps& ro, MassBand mass,
                                  T* S, int nx, int nr, int nl, cudaStream_t st) {
-  const int w2 = 2 * mass.w;
-  const int smem = static_cast<int>(sizeof(T)) * (nr * ((nr + w2) | 1) + (nr + w2) * (nr | 1) + 2 * nr * (w2 + 1) + 4 * 64);
-  const cudaError_t e = cudaFuncSetAttribute(struct_factor_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  auto values = [w2 = 2 * mass.w](int n) { return n * ((n + w2) | 1) + (n + w2) * (n | 1) + 2 * n * (w2 + 1) + 4 * 64; };
+  const int smem = static_cast<int>(sizeof(T)) * values(nr);
+  const cudaError_t e = set_smem_limit(struct_factor_kernel<T>, sizeof(T) * values(16 * kG));  // nr <= 64
   if (e != cudaSuccess) return e;
   struct_factor_kernel<T><<<nx, kST, smem, st>>>(E, E_uniform, dt, ro, mass, S, struct_stride(nr), nr, nl);
   return cudaGetLastError();
@@ -667,10 +669,9 @@ cudaError_t launch_struct_substitute(const double* E, double E_uniform, double d
                                      int probe, cudaStream_t st) {
   const int stride = static_cast<int>(struct_stride(nr)), fixed = static_cast<int>(sizeof(T)) * (nl * nr + 64 + 256);
   const int sb = stride * static_cast<int>(sizeof(T));
-  const int stages = std::max(1, std::min(8, (200 * 1024 - fixed) / sb));
+  const int stages = std::max(1, std::min(8, (kSubstituteRoom - fixed) / sb));
   const int smem = fixed + stages * sb;
-  const cudaError_t e =
-      cudaFuncSetAttribute(struct_substitute_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  const cudaError_t e = set_smem_limit(struct_substitute_kernel<T>, kSubstituteRoom);
   if (e != cudaSuccess) return e;
   struct_substitute_kernel<T><<<nx, kST, smem, st>>>(E, E_uniform, dt, ro, mass, S, stride, stages, vec, conv, nr, nl, status,
                                                       probe);

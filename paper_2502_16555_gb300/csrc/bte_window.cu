@@ -1551,7 +1551,7 @@ cudaError_t launch_window_factor(const WindowBuffers& b, const double* E, double
                                  cudaStream_t st) {
   const FactorArgs a = factor_args(b, E, Eu, status);
   const int smem = 1024 + 4096 + static_cast<int>(sizeof(float)) * kPW * 2 * (kSlots + b.w.NU);
-  const cudaError_t e = cudaFuncSetAttribute(window_lu_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  const cudaError_t e = set_smem_limit(window_lu_tc_kernel, 1024 + 4096 + sizeof(float) * kPW * 2 * (kSlots + 512));
   if (e != cudaSuccess) return e;
   window_lu_tc_kernel<<<nx, kThreads, smem, st>>>(a);
   return cudaGetLastError();
@@ -1585,7 +1585,8 @@ cudaError_t launch_window_project(const WindowBuffers& b, const double* in, Mass
   SolveArgs a = solve_args(b, mass, nt);
   a.in = in, a.TS = TS, a.conv = conv;
   const int smem = static_cast<int>(sizeof(double)) * (2 * ((nt + 1) / 2) + b.w.nl) * b.w.nr;
-  const cudaError_t e = cudaFuncSetAttribute(window_project_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  // (nt + 1 + nl) nr values, nl <= nt, nr <= 544
+  const cudaError_t e = set_smem_limit(window_project_kernel, sizeof(double) * (2 * kMaxNv + 544));
   if (e != cudaSuccess) return e;
   window_project_kernel<<<nx, kEval, smem, st>>>(a);
   return cudaGetLastError();
@@ -1598,7 +1599,7 @@ cudaError_t launch_window_substitute(const WindowBuffers& b, const int* conv, in
   a.stage_bytes = static_cast<unsigned>(ring.stage_bytes), a.stages = ring.stages;
   const int smem = static_cast<int>(ring.smem);
   auto k = b.fp64 ? window_substitute_kernel<double> : window_substitute_kernel<float>;
-  const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  const cudaError_t e = set_smem_limit(k, kRingRoom);
   if (e != cudaSuccess) return e;
   k<<<nx, kThreads, smem, st>>>(a);
   return cudaGetLastError();
@@ -1612,7 +1613,7 @@ cudaError_t launch_window_residual(const WindowBuffers& b, const double* in, dou
   a.in = in, a.out = out, a.E = E, a.Eu = Eu, a.dt = dt, a.ro = ro, a.TO = TO, a.ts_inf = ts_inf, a.to_inf = to_inf;
   a.ratio = ratio, a.conv = conv, a.tol = tol, a.kc_inf = kc_inf, a.ka_inf = ka_inf, a.status = status;
   const int smem = static_cast<int>(sizeof(double)) * 3 * b.w.nl * b.w.nr;
-  const cudaError_t e = cudaFuncSetAttribute(window_residual_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  const cudaError_t e = set_smem_limit(window_residual_kernel, sizeof(double) * 3 * kMaxNv);
   if (e != cudaSuccess) return e;
   window_residual_kernel<<<nx, kEval, smem, st>>>(a, check ? 1 : 0, last ? 1 : 0);
   return cudaGetLastError();
@@ -1623,7 +1624,8 @@ cudaError_t launch_window_solve_t(const WindowBuffers& b, const double* in, doub
   SolveArgs a = solve_args(b, mass, nt);
   a.in = in, a.out = out, a.TO = TO, a.TS = TS;
   const int smem = static_cast<int>(sizeof(double)) * ((b.w.np + b.w.RS) * 32 + kSlots + 32);
-  const cudaError_t e = cudaFuncSetAttribute(window_solve_t_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  // np <= 327 (one speed index a chunk), RS <= 6
+  const cudaError_t e = set_smem_limit(window_solve_t_kernel, sizeof(double) * ((327 + 6) * 32 + kSlots + 32));
   if (e != cudaSuccess) return e;
   window_solve_t_kernel<<<nx, kThreads, smem, st>>>(a);
   return cudaGetLastError();
