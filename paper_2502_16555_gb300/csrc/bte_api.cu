@@ -740,7 +740,7 @@ bte_status bte_create(const bte_config* cfg, bte_handle** out) {
     h->win.w = bte::window_plan(cfg->nr, cfg->nl > 0 ? cfg->nl : cfg->ntheta);
     h->win.fp64 = cfg->precision == BTE_FP64;
     h->windowed = !h->structured && !h->host_only && cfg->refine_max != 0 && (cfg->flags & dense_flags) == 0 && h->win.w.ok &&
-                  bte::window_ring(h->win.w, h->win.fp64 ? 8 : 4, cfg->nx, 152).stages >= 1 &&
+                  bte::window_ring(h->win.w, h->win.fp64 ? 8 : 4, 1, 1).stages >= 1 &&
                   (h->win.fp64 || bte::tc_available());
   }
   h->tol = cfg->refine_tol > 0 ? cfg->refine_tol : (cfg->precision == BTE_FP64 ? 1e-13 : 1e-12);

@@ -51,6 +51,7 @@ struct ResidualOps {
 // 0-1 L21 split, 2-3 (P A12)^T split, 4-5 one panel's inv(L11) split, 6-7 U12^T split, 8-9 a
 // two-panel block's inv(L11) split (layout in bte_tc.cu)
 bool tc_available();
+int sm_count();  // SMs of the current device
 // Tensor map (128 bytes into map) of the per-point FP32 matrices as a 3-D array [nx][n][n], boxes of
 // 128 rows x 32 columns, 128-byte swizzle: the K-major operand tiles the tensor cores read.
 bool tc_matrix_map(void* map, float* fac, int nx, int n);

@@ -657,16 +657,6 @@ Maps& maps_for(float* fac, void* ws, int nx, int n) {
   return maps;
 }
 
-int sm_count() {
-  static int sms = 0;
-  if (!sms) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  }
-  return sms;
-}
-
 void launch(const Maps& mp, int ia, int ib, const TcArgs& a, cudaStream_t st) {
   const int grid = a.total < sm_count() ? a.total : sm_count();
   tc_gemm_kernel<1><<<grid, NTHREADS, sizeof(Smem) + 1024, st>>>(mp.m[ia], mp.m[ia + 1], mp.m[ib], mp.m[ib + 1],
@@ -788,6 +778,16 @@ float* tc_ws_part(void* ws, int nx, int n, int part) {
 bool tc_matrix_map(void* map, float* fac, int nx, int n) {
   static_assert(sizeof(CUtensorMap) == 128, "tensor map size");
   return CW == 32 && make_cmap(static_cast<CUtensorMap*>(map), fac, nx, n);
+}
+
+int sm_count() {
+  static int sms = 0;
+  if (!sms) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  }
+  return sms;
 }
 
 bool tc_available() {

@@ -1595,7 +1595,7 @@ cudaError_t launch_window_project(const WindowBuffers& b, const double* in, Mass
 cudaError_t launch_window_substitute(const WindowBuffers& b, const int* conv, int nx, unsigned* status, cudaStream_t st) {
   SolveArgs a = solve_args(b, MassBand{}, 0);
   a.conv = const_cast<int*>(conv), a.status = status, a.probe = b.probe;
-  const WindowRing ring = window_ring(b.w, b.fp64 ? sizeof(double) : sizeof(float), nx, 152);
+  const WindowRing ring = window_ring(b.w, b.fp64 ? sizeof(double) : sizeof(float), nx, sm_count());
   a.stage_bytes = static_cast<unsigned>(ring.stage_bytes), a.stages = ring.stages;
   const int smem = static_cast<int>(ring.smem);
   auto k = b.fp64 ? window_substitute_kernel<double> : window_substitute_kernel<float>;
