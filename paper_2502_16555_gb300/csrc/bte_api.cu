@@ -179,6 +179,17 @@ bte::ResidualOps residual_ops(const bte_handle* h) {
   return ro;
 }
 
+// Structured handles that hardly refine: out_i (+)= A_i^-1 in_i at the points with conv[i] == 0, factors and all.
+bte_status scaled_solve(bte_handle* h, const double* in, double* out, const double* E_dev, double Eu, const int* conv,
+                        int accumulate) {
+  const HostOps& o = h->ops;
+  BTE_LAUNCH(BTE_K_LU_SOLVE, bte::launch_vsolve_struct<float>(in, out, E_dev, Eu, o.dt, h->Cs, h->Alo, h->Aup, h->TO,
+                                                              h->TS, static_cast<float*>(h->xs), o.nx, o.nt, o.nr,
+                                                              o.nl, conv, accumulate, accumulate ? nullptr : h->status,
+                                                              h->st));
+  return BTE_OK;
+}
+
 // The window factors of H_i at every point.
 bte_status window_factor(bte_handle* h, const double* E_dev, double Eu) {
   const int nx = h->ops.nx, np = h->win.w.np;
@@ -254,6 +265,7 @@ bte_status enqueue_vsolve(bte_handle* h, const double* in, double* out, const do
   const int nx = o.nx;
   cudaStream_t st = h->st;
   const int n = h->nlu, nb = h->nb;
+  if (h->struct_scaled) return scaled_solve(h, in, out, E_dev, Eu, nullptr, 0);
   if (h->windowed || h->structured) {
     if (factor) BTE_TRY(h->structured ? struct_factor(h, E_dev, Eu) : window_factor(h, E_dev, Eu));
     return harmonic_solve(h, in, out, E_dev, Eu, 0);
@@ -374,7 +386,7 @@ bte_status enqueue_step(bte_handle* h, const double* F_in, double* F_out, const 
   // velocity step (eq. "bte_semi_implicit_vspace" / "vspace_batched_system"); a caller's field
   // array is checked like the state
   if (E_dev && !ni_dev) BTE_LAUNCH(BTE_K_OTHER, bte::launch_check_field(E_dev, nx, h->status, st));
-  const bool harmonic = h->windowed || h->structured;
+  const bool harmonic = h->windowed || (h->structured && !h->struct_scaled);
   if (harmonic) {
     BTE_TRY(h->structured ? struct_factor(h, E_dev, Eu) : window_factor(h, E_dev, Eu));
     BTE_TRY(harmonic_solve(h, h->Fa, h->Fb, E_dev, Eu, h->refine_max));
@@ -391,7 +403,8 @@ bte_status enqueue_step(bte_handle* h, const double* F_in, double* F_out, const 
                                                       h->conv, h->tol, o.kc_inf, o.ka_inf, nx, nt, nr, nl, h->status,
                                                       st));
       if (s == h->refine_max) break;
-      BTE_TRY(enqueue_lu_solve(h, h->R, h->Fb, h->conv, 1));
+      if (h->struct_scaled) BTE_TRY(scaled_solve(h, h->R, h->Fb, E_dev, Eu, h->conv, 1));
+      else BTE_TRY(enqueue_lu_solve(h, h->R, h->Fb, h->conv, 1));
     }
     if (h->xs64) {
       // points whose refinement with the FP32 factors has not converged (cond(A_i) * eps_32 near or
@@ -745,6 +758,11 @@ bte_status bte_create(const bte_config* cfg, bte_handle** out) {
   }
   h->tol = cfg->refine_tol > 0 ? cfg->refine_tol : (cfg->precision == BTE_FP64 ? 1e-13 : 1e-12);
   h->refine_max = cfg->refine_max >= 0 ? cfg->refine_max : (cfg->precision == BTE_FP64 ? 2 : 4);
+  // The FP32 block solve is 18 times more accurate on the mass-scaled blocks (168 steps of small grids, unrefined:
+  // 1.2e-7 against 2.1e-6). From two refinement sweeps on both reach the tolerance (2.0 and 2.8 residuals a point)
+  // and the banded form takes a third of the time; with none the result shows the difference, with one some points
+  // would be left to the FP64 escalation.
+  h->struct_scaled = h->structured && cfg->precision == BTE_MIXED && h->refine_max <= 1;
   std::string e = bte::assemble_x(*cfg, h->ops);
   // handles that factor the Nv x Nv form keep its unscaled operators
   h->ops.want_kg = !h->reduced && !h->structured;

@@ -21,6 +21,7 @@ struct bte_handle {
   double tol = 0.0;
   int refine_max = 0;
   bool structured = false;  // block-tridiagonal velocity solve instead of the dense LU
+  bool struct_scaled = false;  // its mixed solve on the mass-scaled blocks, in one launch (refine_max <= 1)
   void* xs = nullptr;       // its per-point scratch (nx * nl * nr * nr values)
   double* xs64 = nullptr;   // mixed path: FP64 scratch of the structured solve that takes over points
                             // whose refinement with the FP32 factors stalls (nx * nl * nr * nr)

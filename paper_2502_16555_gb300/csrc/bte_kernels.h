@@ -150,7 +150,8 @@ template <typename T>
 cudaError_t launch_struct_substitute(const double* E, double E_uniform, double dt, const ResidualOps& ro, MassBand mass,
                                      const T* S, double* vec, const int* conv, int nx, int nr, int nl, unsigned* status,
                                      int probe, cudaStream_t st);
-// The mixed paths' FP64 escalation, factors and solve in one launch: Fout = A_i^-1 Fin per point
+// The same solve on the mass-scaled blocks, factors and solve in one launch (the mixed paths' FP64 escalation,
+// and in FP32 structured handles that hardly refine): Fout = A_i^-1 Fin per point
 // (Fout += when accumulate); T is the arithmetic of the block elimination; Xscratch holds
 // nx * nl * nr * nr values of T.
 size_t struct_smem_bytes(int nr, int nl, size_t tsize);

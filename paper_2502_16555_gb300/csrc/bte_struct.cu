@@ -13,8 +13,10 @@
 // semidefinite matrix and its inversion needs no pivoting; S_0 comes last. The products with L and U
 // cost 7 operations an element. The inverses are kept for the refinement's solves.
 //
-// The mixed paths' escalation (vsolve_struct_kernel, FP64): the mass-scaled blocks, eliminated upwards
-// and solved in one launch for the points whose refinement has not converged.
+// vsolve_struct_kernel: the mass-scaled blocks I - dt B_i, eliminated upwards and solved in one launch. In
+// FP64 it is the mixed paths' escalation, for the points whose refinement has not converged; in FP32 the
+// structured solve of handles with at most one refinement sweep, whose results show the solve's own accuracy
+// (1.2e-7 of f; 2.1e-6 through H_i, whose elimination meets the condition of M_v).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -642,6 +644,9 @@ void launch_vsolve_struct(const double* Fin, double* Fout, const double* E, doub
                                                  conv, accumulate, status);
 }
 
+template void launch_vsolve_struct<float>(const double*, double*, const double*, double, double, const double*,
+                                          const double*, const double*, const double*, const double*, float*, int,
+                                          int, int, int, const int*, int, unsigned*, cudaStream_t);
 template void launch_vsolve_struct<double>(const double*, double*, const double*, double, double, const double*,
                                            const double*, const double*, const double*, const double*, double*, int,
                                            int, int, int, const int*, int, unsigned*, cudaStream_t);
