@@ -601,6 +601,10 @@ bte_status alloc_window(bte_handle* h) {
     BTE_TRY(dalloc(h, &b.rows, nx * 128));
   }
   b.base = base, b.slope = slope, b.T = T, b.U = U;
+  BTE_TRY(dalloc(h, &b.rscale, o.nr));
+  const std::vector<double> scale = bte::window_row_scale(o, b.levelled);
+  BTE_TRY(upload(h, b.rscale, scale));
+  BTE_CUDA(h, cudaStreamSynchronize(h->st));
   BTE_CUDA(h, cudaMemsetAsync(U, 0, ts * nx * bte::window_u_count(w), h->st));
   return BTE_OK;
 }
@@ -608,7 +612,7 @@ bte_status alloc_window(bte_handle* h) {
 // Row templates of the windowed LU for the current cross sections, in the factors' type.
 bte_status upload_window(bte_handle* h) {
   std::vector<double> base, slope;
-  bte::window_tables(h->win.w, h->ops, base, slope);
+  bte::window_tables(h->win.w, h->ops, bte::window_row_scale(h->ops, h->win.levelled), base, slope);
   if (h->win.fp64) {
     BTE_TRY(upload(h, static_cast<double*>(h->win.base), base));
     BTE_TRY(upload(h, static_cast<double*>(h->win.slope), slope));
@@ -823,6 +827,7 @@ bte_status bte_create(const bte_config* cfg, bte_handle** out) {
       // the mixed path's escalation for ill-conditioned points: the FP64 block-tridiagonal solve
       if (h->precision == BTE_MIXED && o.nr <= 64 && bte::struct_smem_bytes(o.nr, o.nl, sizeof(double)) <= 200 * 1024)
         ok = chk(dalloc(h, &h->xs64, static_cast<size_t>(o.nx) * o.nl * o.nr * o.nr));
+      h->win.levelled = h->precision == BTE_FP64 || !h->xs64;
       if (h->windowed) {
         ok = ok && chk(alloc_window(h));
       } else if (h->reduced)

@@ -215,9 +215,16 @@ struct WindowBuffers {
   double* vec = nullptr;                   // 3 nl nr values a point
   double* fmax_ = nullptr;                 // one value a point
   double* minv = nullptr;                  // [nr] 1 / sum_k |M_v[p][k]|
+  bool levelled = false;                   // the rows are multiplied by window_row_scale
+  double* rscale = nullptr;                // [nr] the rows' factors
 };
-// Templates [np 32][NW] and [np 32][(RS + 1) 32] from the unscaled blocks (M, Cg, Ag_lo, Ag_up).
-void window_tables(const WindowPlan& w, const HostOps& o, std::vector<double>& base, std::vector<double>& slope);
+// Powers of two by which the rows of speed index p are multiplied before the elimination: the row sums of M_v
+// grow as v^2 (by 1e5 over 256 B-splines), and pivoting by magnitude across them would take the highest row of
+// a column's window for its size alone. The largest row's factor is 1 (so is every row's, if not levelled).
+std::vector<double> window_row_scale(const HostOps& o, bool levelled);
+// Templates [np 32][NW] and [np 32][(RS + 1) 32] from the unscaled blocks (M, Cg, Ag_lo, Ag_up) and the rows' factors.
+void window_tables(const WindowPlan& w, const HostOps& o, const std::vector<double>& scale, std::vector<double>& base,
+                   std::vector<double>& slope);
 // The FP32 kernel's form of the templates: [np][RS + 1 + NF / 32] blocks of 32 rows x 32 columns, the
 // 16-byte pieces of row r exchanged by r & 7; a column of another harmonic holds the value per unit field.
 std::vector<float> window_blocks(const WindowPlan& w, const std::vector<double>& base, const std::vector<double>& slope);

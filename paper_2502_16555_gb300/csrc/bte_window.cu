@@ -25,6 +25,15 @@
 // any other row holds t = -L21 inv(L11). The whole window is then updated by one product,
 // D += T B with B the pivot rows (T's pivot rows: inv(L11) - I), and the forward substitution is
 // one matrix-vector product with T per panel.
+//
+// Levelled rows (FP64, and mixed handles without the FP64 escalation): the rows are multiplied by powers of two that
+// level the row sums of M_v (window_row_scale), which changes nothing but the choice of pivots. Without it the
+// FP32 factors of fine speed grids at strong fields took the error only 1e-3 down a refinement sweep, and some steps
+// that the dense LU refined in time did not converge (256 x 7, 1.1e6 V/m, FP32 LU on the host, error after each
+// sweep: 2.1e-2, 8.8e-5, 3.0e-7; levelled 3.5e-5, 7.9e-9, 7.9e-13; the dense LU, harmonic slowest, 4.4e-2, 6.1e-7,
+// 1.3e-11). FP64 steps of 168 small grids need 1.0 residual evaluations a point instead of 1.7, with errors 0.6 of what
+// they were. Mixed handles with the escalation need it less and stay as they are: levelled they end a sweep earlier
+// and further off (a batch of eight: 1.3e-12 instead of 4.6e-13).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -1001,9 +1010,11 @@ struct SolveArgs {
   double* vec;              // [nx][3 n]: y, z, rho
   double* fmax_;            // [nx] max|f|
   const double* minv;       // [nr] 1 / sum_k |M_pk|
+  const double* rscale;     // [nr] the factors' row scale
   double* ratio;
   int* conv;
   double tol, kc_inf, ka_inf;
+  double skip_tol, skip_floor;  // launch_window_residual
   int nt;
   int stages;
   unsigned stage_bytes;
@@ -1194,7 +1205,7 @@ __global__ void __launch_bounds__(kThreads, 2) window_substitute_kernel(const So
   // rho and z by rows, whole lines at a time; the columns' conflicts in shared memory cost less
   for (int i = tid; i < n; i += kThreads) {
     const int l = i / nr, k = i - l * nr;
-    b[(k << sh) + l] = static_cast<T>(rho[i]);
+    b[(k << sh) + l] = static_cast<T>(__ldg(a.rscale + k) * rho[i]);
   }
   __syncthreads();
   // the stage and phase of the copy in use, advanced by hand (a division by S costs as much as the product)
@@ -1354,7 +1365,7 @@ __global__ void __launch_bounds__(kEval) window_residual_kernel(const SolveArgs 
     block_max2(lbm, mzm, red, lb, mz);
     if (tid == 0) atomicAdd(a.status + 1, 1u);  // residual evaluations
     const double least = lb / a.ts_inf;
-    if (!last && least > a.tol * mb && least > floor_ * (nA * (mb + a.to_inf * mz) + mb)) return;
+    if (!last && least > a.skip_tol * mb && least > a.skip_floor * (nA * (mb + a.to_inf * mz) + mb)) return;
     // q_l <- M^-1 q_l by the banded Cholesky factor, one thread a harmonic
     for (int l = tid; l < nl; l += kEval) mass_solve(q + l * nr, a.ro.chol, a.ro.cinv, nr, mw);
     __syncthreads();
@@ -1469,6 +1480,8 @@ __global__ void __launch_bounds__(kThreads) window_solve_t_kernel(const SolveArg
   }
   if (tid < NS && tid < np * 32) x[tid] = wv[tid];
   __syncthreads();
+  for (int i = tid; i < nr * nlp; i += kThreads) x[i] *= __ldg(a.rscale + i / nlp);  // H^T = (factors)^T / scale
+  __syncthreads();
   const int mw = a.mass.w, bw = 2 * mw + 1;
   for (int i = tid; i < n; i += kThreads) {
     const int l = i / nr, p = i % nr;
@@ -1488,7 +1501,20 @@ __global__ void __launch_bounds__(kThreads) window_solve_t_kernel(const SolveArg
 
 }  // namespace
 
-void window_tables(const WindowPlan& w, const HostOps& o, std::vector<double>& base, std::vector<double>& slope) {
+std::vector<double> window_row_scale(const HostOps& o, bool levelled) {
+  if (!levelled) return std::vector<double>(o.nr, 1.0);
+  std::vector<double> s(o.nr);
+  double most = 0.0;
+  for (int p = 0; p < o.nr; ++p) {
+    for (int k = 0; k < o.nr; ++k) s[p] += std::fabs(o.M[static_cast<size_t>(p) * o.nr + k]);
+    most = std::max(most, s[p]);
+  }
+  for (double& v : s) v = std::exp2(std::round(std::log2(most / v)));
+  return s;
+}
+
+void window_tables(const WindowPlan& w, const HostOps& o, const std::vector<double>& scale, std::vector<double>& base,
+                   std::vector<double>& slope) {
   const int nr = o.nr, nl = o.nl, NWR = (w.RS + 1) * 32;
   base.assign(static_cast<size_t>(w.np) * 32 * w.NW, 0.0);
   slope.assign(static_cast<size_t>(w.np) * 32 * NWR, 0.0);
@@ -1504,12 +1530,12 @@ void window_tables(const WindowPlan& w, const HostOps& o, std::vector<double>& b
         const int d = k / w.g - c0, col = d <= w.RS ? d * 32 + (k % w.g) * w.nlp : -1;
         const size_t e = (static_cast<size_t>(l) * nr + p) * nr + k;
         const double m = std::abs(p - k) <= 3 ? o.M[p * nr + k] : 0.0;
-        const double v = m - o.dt * o.Cg[e];
+        const double v = scale[p] * (m - o.dt * o.Cg[e]), f = -o.dt * scale[p];
         if (col >= 0) br[col + l] = v;
         else br[NWR + k - w.kf0] = v;
         if (k <= p + 3) {
-          if (l > 0) sr[col + l - 1] = -o.dt * o.Ag_lo[e];
-          if (l + 1 < nl) sr[col + l + 1] = -o.dt * o.Ag_up[e];
+          if (l > 0) sr[col + l - 1] = f * o.Ag_lo[e];
+          if (l + 1 < nl) sr[col + l + 1] = f * o.Ag_up[e];
         }
       }
     }
@@ -1543,7 +1569,7 @@ static FactorArgs factor_args(const WindowBuffers& b, const double* E, double Eu
 
 static SolveArgs solve_args(const WindowBuffers& b, MassBand mass, int nt) {
   SolveArgs a{};
-  a.w = b.w, a.T = b.T, a.U = b.U, a.slotj = b.slotj, a.vec = b.vec, a.fmax_ = b.fmax_, a.minv = b.minv, a.mass = mass, a.nt = nt;
+  a.w = b.w, a.T = b.T, a.U = b.U, a.slotj = b.slotj, a.vec = b.vec, a.fmax_ = b.fmax_, a.minv = b.minv, a.rscale = b.rscale, a.mass = mass, a.nt = nt;
   return a;
 }
 
@@ -1611,6 +1637,12 @@ cudaError_t launch_window_residual(const WindowBuffers& b, const double* in, dou
                                    int nx, int nt, bool check, bool last, unsigned* status, cudaStream_t st) {
   SolveArgs a = solve_args(b, mass, nt);
   a.in = in, a.out = out, a.E = E, a.Eu = Eu, a.dt = dt, a.ro = ro, a.TO = TO, a.ts_inf = ts_inf, a.to_inf = to_inf;
+  // A point whose bound is above these goes on without the full test. Levelled FP32 factors are near the tolerance one
+  // sweep before they are below it: with a point or two of a launch tested in full for nothing there, 100 points of
+  // 128 x 3 took 182 us of residuals a step, with what is within 256 of it (down to rounding) going on unasked 131,
+  // as with rows as they come. A point that goes on ends at 1e-14, not just below 1e-12.
+  const double fl = std::min(kBackwardFloor, tol), part = b.levelled && !b.fp64 ? 1.0 / 256 : 1.0;
+  a.skip_tol = std::max(tol * part, fl), a.skip_floor = std::min(fl, std::max(fl * part, kBackwardFloor / 256));
   a.ratio = ratio, a.conv = conv, a.tol = tol, a.kc_inf = kc_inf, a.ka_inf = ka_inf, a.status = status;
   const int smem = static_cast<int>(sizeof(double)) * 3 * b.w.nl * b.w.nr;
   const cudaError_t e = set_smem_limit(window_residual_kernel, sizeof(double) * 3 * kMaxNv);
