@@ -94,19 +94,22 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
                : "memory");
 }
 
+// Loads from tensor memory and their wait in one statement: the registers hold nothing before the wait, and between
+// two statements the compiler may copy or spill them.
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
   uint32_t r[32];
   __syncwarp();
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
+      " tcgen05.wait::ld.sync.aligned;"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
         "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
         "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]),
         "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),
         "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      : "r"(taddr)
+      : "memory");
 #pragma unroll
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
@@ -130,8 +133,10 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const float (&v)[32]) 
 __device__ __forceinline__ float tmem_ld1(uint32_t taddr) {
   uint32_t r;
   __syncwarp();
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];\n tcgen05.wait::ld.sync.aligned;"
+               : "=r"(r)
+               : "r"(taddr)
+               : "memory");
   return __uint_as_float(r);
 }
 
@@ -452,7 +457,10 @@ __global__ void __launch_bounds__(kThreads, 2) window_lu_tc_kernel(const FactorA
         }
       };
       // warp 0 issues the first product, warp 5 the rest (not a panel warp: the tensor cores' queue holds
-      // the issuing thread up)
+      // the issuing thread up). Both loops stay rolled: unrolled over k inside the rolled loop over column groups
+      // the products came out wrong, the same every time; with both rolled, or both unrolled, they are right. The
+      // cause was not found (the loads from tensor memory and their wait were two statements then, see
+      // tmem_ld32; the form has not been run again). Speed is no reason: the queue bounds the issue.
       auto issue = [&](int col, int ncol) {
         const uint64_t dah = sdesc(saddr(Thi)), dal = sdesc(saddr(Tlo)), dbh = sdesc(saddr(Bhi)), dbl = sdesc(saddr(Blo));
         const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | (static_cast<uint32_t>(ncol >> 3) << 17) |
