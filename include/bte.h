@@ -54,9 +54,9 @@ typedef enum {
 } bte_precision;
 
 /* How the velocity systems are factored. By default, with at most 32 harmonics, refinement on
- * (refine_max != 0) and a window of at most 512 columns (nr <= 320 with more than 16 harmonics, up to
- * 544 with fewer), through a windowed LU with partial pivoting: the system in the harmonic basis with
- * the speed index slowest, which is a band matrix but for the l = 0 columns that inelastic gain
+ * (refine_max != 0) and a window of at most 512 columns (nr up to 327 with 17 to 32 harmonics, 394 with
+ * 9 to 16, 460 with 5 to 8, 472 with 3 and 4, 496 with 2, 544 with 1; in both precisions), through a
+ * windowed LU with partial pivoting: the system in the harmonic basis with the speed index slowest, which is a band matrix but for the l = 0 columns that inelastic gain
  * reaches (Section 3.3; csrc/bte_window.cu). Otherwise, and with any of the flags below that select a
  * variant of it, through a dense LU per point. Both eliminate with partial pivoting and are refined
  * against the same system. */
@@ -71,7 +71,9 @@ typedef enum {
                                    instead of the dense per-point LU: the same solution with about
                                    Nv^3 / (5 N_l Nr^3) fewer flops and no dense factors in memory. The
                                    block elimination runs in FP64 (BTE_FP64) or FP32 with the FP64
-                                   refinement (BTE_MIXED). Requires nr <= 64. */
+                                   refinement (BTE_MIXED; with refine_max <= 1 on the
+                                   mass-scaled blocks, whose FP32 solve is more accurate as it
+                                   is). Requires nr <= 64. */
 #define BTE_FLAG_TC_SINGLE 8u   /* BTE_MIXED on the tensor cores: apply each 128-column panel to the
                                    trailing matrix on its own (K = 128) instead of two panels at a time
                                    (K = 256, half the trailing-matrix traffic); same factors up to
@@ -120,7 +122,9 @@ typedef struct {
   double refine_tol; /* stop refining a point when max|r| <= refine_tol * max|b|, or when its normwise
                         backward error is at FP64 rounding level: max|r| <= min(256 eps, refine_tol)
                         (|A_i| max|x| + max|b|), |A_i| bounded by the infinity norms of dt K_C, dt K_A
-                        (<= 0: default 1e-13 FP64, 1e-12 mixed) */
+                        (<= 0: default 1e-13 FP64, 1e-12 mixed). While sweeps are left a windowed
+                        BTE_MIXED handle without the escalation below corrects a point that a bound
+                        shows to be close to these limits once more instead of testing it in full */
   int refine_max;    /* maximum refinement sweeps per step (< 0: default: 2 FP64, 4 mixed). The dense
                         paths factor (I (x) M_v) A_i, not A_i itself; their first FP64 solve is
                         accurate to about cond(M_v) eps, one FP64 sweep restores the backward error
@@ -240,7 +244,8 @@ bte_status bte_moments(bte_handle* h, const double* F_dev, double* ne_dev, doubl
  * 10 density moment vector [nv], 11 energy moment vector [nv], 12 rate vectors [n_proc][nv],
  * 13 Clenshaw-Curtis weights of the collocation points on [0, L] [nx], 14 P_O C P_S[nv][nv] and
  * 15 P_O A_v P_S[nv][nv] (before the mass scaling: (I (x) M_v) K_C and (I (x) M_v) K_A, the operators
- * of the matrices the dense Nv x Nv path factors; formed only for handles on that path).
+ * of the matrices the dense Nv x Nv path factors; formed for handles with nl == ntheta or
+ * BTE_FLAG_FULL_V and without BTE_FLAG_STRUCTURED, whichever LU they take).
  * Returns BTE_EINVAL if count does not match, BTE_ESTATE if the operator is not assembled yet
  * (or, for 14 and 15, not formed for this handle). */
 bte_status bte_get_operator(const bte_handle* h, int which, double* host_out, size_t count);

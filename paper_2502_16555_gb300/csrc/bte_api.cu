@@ -548,7 +548,7 @@ bte_status read_status(bte_handle* h, int steps = 1) {
   }
   // a non-finite input explains whatever follows from it; otherwise a failed factorisation explains
   // a non-finite result
-  if (f & bte::kTimeout) return fail(h, BTE_ECUDA, "a bounded device-side wait expired in the tensor-core update");
+  if (f & bte::kTimeout) return fail(h, BTE_ECUDA, "a bounded device-side wait expired");
   if (f & bte::kNonFiniteIn) return fail(h, BTE_ENONFINITE, "non-finite values in the state or field handed in");
   if (f & bte::kZeroPivot) return fail(h, BTE_ESINGULAR, "zero or non-finite pivot in a per-point factorisation");
   if (f & bte::kNonFinite) return fail(h, BTE_ENONFINITE, "non-finite values in the result of a step");

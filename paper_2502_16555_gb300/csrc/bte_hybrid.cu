@@ -73,9 +73,6 @@ __global__ void field_kernel(const double* __restrict__ Lop, const double* __res
   if (lane == 0) E[warp] = s + vleft * E1[warp];
 }
 
-// The ion system of eq. "fluid_step", row i per CTA: A = I/dt + D_x diag(mu E) - d D_x D_x,
-// b = ni/dt + src; the wall rows are the flux conditions J(0) = n max(0, -mu E(0)) and
-// J(L) = -n max(0, mu E(L)) with J = mu E n - d D_x n (right-hand side 0).
 // D2 = D_x D_x, once per handle (row i per CTA).
 __global__ void square_kernel(const double* __restrict__ Dx, int nx, double* __restrict__ D2) {
   const int i = blockIdx.x;
@@ -87,6 +84,9 @@ __global__ void square_kernel(const double* __restrict__ Dx, int nx, double* __r
   }
 }
 
+// The ion system of eq. "fluid_step", row i per CTA: A = I/dt + D_x diag(mu E) - d D_x D_x,
+// b = ni/dt + src; the wall rows are the flux conditions J(0) = n max(0, -mu E(0)) and
+// J(L) = -n max(0, mu E(L)) with J = mu E n - d D_x n (right-hand side 0).
 __global__ void ion_assemble_kernel(const double* __restrict__ Dx, const double* __restrict__ D2,
                                     const double* __restrict__ E,
                                     const double* __restrict__ ni, const double* __restrict__ src, double mu,

@@ -258,7 +258,8 @@ __global__ void __launch_bounds__(kThreads, 2) window_lu_tc_kernel(const FactorA
                  "r"(static_cast<uint32_t>(w.tmem_cols)));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
-  // K columns of unused unknowns stay zero in B for the whole factorisation
+  // K columns of unused unknowns are never converted: they hold zeros, later rows of U or of templates, all finite,
+  // and T's columns for them are zero
   for (int i = tid; i < w.NU * kPW; i += kThreads) Bhi[i] = Blo[i] = 0.f;
   for (int i = tid; i < 2 * 8 * 24; i += kThreads) (&pblk[0][0][0])[i] = 0.f;
   if (tid < 8) (&keys[0][0])[tid] = make_uint2(0u, 0u);
@@ -1415,7 +1416,7 @@ __global__ void __launch_bounds__(kEval) window_residual_kernel(const SolveArgs 
 }
 
 // out = A^-T in for the adjoint (FP64 factors, no refinement): the transposed passes of
-// window_solve_kernel in reverse order. A^-1 = I + P_O (H^-1 M - I) P_S, so
+// window_substitute_kernel in reverse order. A^-1 = I + P_O (H^-1 M - I) P_S, so
 // A^-T g = g + P_S^T (M H^-T - I) P_O^T g (M symmetric).
 __global__ void __launch_bounds__(kThreads) window_solve_t_kernel(const SolveArgs a) {
   extern __shared__ __align__(1024) unsigned char raw[];
