@@ -1142,8 +1142,8 @@ __global__ void __launch_bounds__(kEval) window_project_kernel(const SolveArgs a
 // (128 points of 64 x 32, FP32) 0.40 GB a solve, 60 us at the copy bandwidth; measured 88 us, one CTA an
 // SM bound by the panels' chain (a panel 1000 cycles forwards, 1200 backwards). It was 119 us with the
 // stage found by a division, the ranks read one panel ahead and the far columns gathered from the
-// unknowns. 256 points of 128 x 32: 315 us of 262 us at the copy bandwidth (it was 366), two CTAs an
-// SM; one CTA with twice the stages 352 us. Vectors are read and written by rows: 1.4 times the solve
+// unknowns. 256 points of 128 x 32: 274 us of 262 us at the copy bandwidth, two CTAs an SM (314 with the copy of the
+// next block issued half a panel later; one CTA with twice the stages was slower by a tenth). Vectors are read and written by rows: 1.4 times the solve
 // when each lane wrote a row of its own. Converged points return at once.
 template <typename T>
 __global__ void __launch_bounds__(kThreads, 2) window_substitute_kernel(const SolveArgs a) {

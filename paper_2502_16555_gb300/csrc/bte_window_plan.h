@@ -57,7 +57,7 @@ struct WindowRing {
 constexpr size_t kRingRoom = 224 * 1024;
 
 // ts: bytes of a factor's value. One CTA an SM takes up to 8 stages; with more points than SMs two CTAs
-// share one where both can have two stages (256 points of 128 x 32: 315 us instead of 352). FP64 factors
+// share one where both can have two stages (256 points of 128 x 32: 315 us instead of 352, now 274). FP64 factors
 // of fine speed grids (nr >= 136 with 17 to 32 harmonics) leave room for one stage.
 inline WindowRing window_ring(const WindowPlan& w, size_t ts, int nx, int sms) {
   WindowRing r;
